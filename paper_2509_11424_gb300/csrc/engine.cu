@@ -393,7 +393,8 @@ void Engine::free_hierarchy() {
     dfree(L.Dinv32);
     if (l > 0) {
       dfree(L.A64);
-      dfree(L.AT64);
+      dfree(L.AF);
+      dfree(L.AFu);
       dfree(L.AT32);
       dfree(L.ATC);
       if (L.ATCB) cudaFree(L.ATCB);
@@ -467,7 +468,7 @@ void Engine::stencil_run(int l, int v, const float2 *in, float2 *out, int nrhs) 
   else if (v == 3 && L.ATB16 && pipe) stencil_apply_pipe(in, out, L.ATB16, true, L.g, nrhs, flag_dev_ + 1, stream);
   else if ((v == 6 || v == 7) && L.ATS && nrhs <= 8) stencil_apply_stream(in, out, L.ATS, L.g, nrhs, v == 7, stream);
   else if (pipe) stencil_apply_pipe(in, out, L.AT32, false, L.g, nrhs, flag_dev_ + 1, stream);
-  else stencil_apply<float>(in, out, L.AT32, L.g, nrhs, flag_dev_ + 1, stream);
+  else stencil_apply(in, out, L.AT32, L.g, nrhs, flag_dev_ + 1, stream);
 }
 
 // the tensor-core variants compute TF32 products, so the variant changes the
@@ -555,7 +556,7 @@ template <typename T> void Engine::apply_D(int l, const C<T> *in, C<T> *out, int
     // bytes of one complex block entry as stored (BF16 variants: 4)
     double bs = cs;
     if constexpr (sizeof(T) == 8) {
-      stencil_apply<T>(in, out, L.AT64, L.g, nrhs, flag_dev_ + 1, stream);
+      stencil_apply_fx(in, out, L.AF, L.AFu, L.g, nrhs, stream);
     } else {
       const int v = stencil_pick(l, nrhs, in, out);
       stencil_run(l, v, in, out, nrhs);
@@ -1106,7 +1107,8 @@ void Engine::galerkin(int l) {
   double2 *cols = ws<double>("galc", l, (size_t)9 * nc);
   const size_t acnt = (size_t)c.g.V * 9 * dofc * dofc;
   c.A64 = dalloc<double2>(acnt);
-  c.AT64 = dalloc<double2>(acnt);
+  c.AF = dalloc<int4>(acnt);
+  c.AFu = dalloc<short>((size_t)c.g.V * dofc);
   c.AT32 = dalloc<float2>(acnt);
   for (int col = 0; col < dofc; ++col) {
     probe_column(probe, f.P64, m, col, stream);
@@ -1115,8 +1117,8 @@ void Engine::galerkin(int l) {
     restrict_op<double>(out9, cols, f.P64, m, 9, stream);
     galerkin_scatter(cols, c.A64, c.g, col, stream);
   }
-  stencil_transpose<double>(c.A64, c.AT64, (int64_t)c.g.V * 9, dofc, stream);
-  stencil_transpose<float>(c.A64, c.AT32, (int64_t)c.g.V * 9, dofc, stream);
+  stencil_digits(c.A64, c.AF, c.AFu, c.g, stream);
+  stencil_transpose(c.A64, c.AT32, (int64_t)c.g.V * 9, dofc, stream);
   if (stencil_tc_supported(c.g)) {
     c.ATC = dalloc<float>(stencil_tc_elems(c.g));
     stencil_tile_tc(c.A64, c.ATC, false, c.g, stream);

@@ -21,7 +21,8 @@ struct Level {
   float2 *UD32 = nullptr;  // FP32 links structure-of-arrays [4][3][3][V] (FP32 kernels)
   float *Ub16 = nullptr;   // bf16 links structure-of-arrays (one bf16 pair per float slot)
   double2 *A64 = nullptr;   // coarse stencil, canonical [V][9][dof][dof]
-  double2 *AT64 = nullptr;  // the same blocks transposed [V][9][j][i] (apply)
+  int4 *AF = nullptr;       // the same blocks transposed [V][9][j][i] as fixed-point digits (FP64 apply)
+  short *AFu = nullptr;     // exponent of each row's unit [V][dof]
   float2 *AT32 = nullptr;
   float *ATC = nullptr;     // tensor-core tiles (32 dofs per site only), see stencil_tile_tc
   void *ATCB = nullptr;     // the same tiles in BF16 (kind::f16 MMAs)

@@ -121,12 +121,17 @@ void link_soa(const float2 *U, float2 *UDs, int V, cudaStream_t s);
 template <typename T>
 void wilson_split(const C<T> *in, C<T> *out9, const C<T> *U, Geom g, double m0, const int b[4],
                   cudaStream_t s);
-// coarse stencil with transposed blocks AT[X][d][j][i]; when they fit, the 9
-// blocks of a site are staged by one TMA bulk copy; err[0] = 2 if a copy
-// does not complete within the bounded wait
-template <typename T>
-void stencil_apply(const C<T> *in, C<T> *out, const C<T> *AT, Geom g, int nrhs, int *err,
+// FP32 coarse stencil with transposed blocks AT[X][d][j][i]; when they fit,
+// the 9 blocks of a site are staged by one TMA bulk copy; err[0] = 2 if a
+// copy does not complete within the bounded wait
+void stencil_apply(const float2 *in, float2 *out, const float2 *AT, Geom g, int nrhs, int *err,
                    cudaStream_t s);
+// FP64 coarse stencil in fixed point on the integer pipe (fixed.cuh), up to
+// 256 dofs per site: AF, unit from stencil_digits (transposed like AT, 16
+// bytes per entry, one exponent per row)
+void stencil_digits(const double2 *A, int4 *AF, short *unit, const Geom &g, cudaStream_t s);
+void stencil_apply_fx(const double2 *in, double2 *out, const int4 *AF, const short *unit, Geom g, int nrhs,
+                      cudaStream_t s);
 // Tensor-core (tcgen05 kind::tf32) coarse stencil for 32 dofs per site:
 // ATC holds each site's nine stacked [Re A_d; Im A_d] tiles in the MMA's
 // shared-memory image (stencil_tile_tc builds it from the canonical A);
@@ -157,8 +162,7 @@ void stencil_apply_stream(const float2 *in, float2 *out, const void *AS, Geom g,
                           cudaStream_t s);
 void stencil_to_stream(const float2 *AT32, void *AS, int64_t count, cudaStream_t s);
 // AT = blockwise transpose of the canonical A[X][d][i][j] (nblocks = 9 V)
-template <typename To>
-void stencil_transpose(const double2 *A, C<To> *AT, int64_t nblocks, int m, cudaStream_t s);
+void stencil_transpose(const double2 *A, float2 *AT, int64_t nblocks, int m, cudaStream_t s);
 // (<q, r>, <q, q>) for every rhs in one pass: out_qr[r], out_qq[r]
 template <typename T>
 void dot_qr(const C<T> *q, const C<T> *r, int64_t n, int nrhs, double2 *out_qr, double2 *out_qq,

@@ -33,31 +33,31 @@ template <typename V> __device__ __forceinline__ V warp_csum(V v) {
 // vectors staged in shared memory; the 9 partial rows are then summed in
 // shared memory by the d = 0 threads.  Each block entry is read once per RG
 // right-hand sides.
-template <typename T, int RG>
-__global__ void stencil_t_kernel(const C<T> *__restrict__ in, C<T> *__restrict__ out,
-                                 const C<T> *__restrict__ AT, Geom g, int nrhs) {
+template <int RG>
+__global__ void stencil_t_kernel(const float2 *__restrict__ in, float2 *__restrict__ out,
+                                 const float2 *__restrict__ AT, Geom g, int nrhs) {
   extern __shared__ unsigned char smem_raw[];
   const int m = g.dof;
-  C<T> *xs = reinterpret_cast<C<T> *>(smem_raw);  // [9][RG][m]
-  C<T> *part = xs + 9 * RG * m;                   // [9][RG][m]
+  float2 *xs = reinterpret_cast<float2 *>(smem_raw);  // [9][RG][m]
+  float2 *part = xs + 9 * RG * m;                   // [9][RG][m]
   const int X = blockIdx.x;
   const int i = threadIdx.x, d = threadIdx.y;
   const int64_t n = g.n();
   const int nb = g.neighbor(X, d);
-  const C<T> *Ad = AT + ((int64_t)X * 9 + d) * m * m;
+  const float2 *Ad = AT + ((int64_t)X * 9 + d) * m * m;
   for (int r0 = 0; r0 < nrhs; r0 += RG) {
     const int rg = nrhs - r0 < RG ? nrhs - r0 : RG;
 #pragma unroll
     for (int r = 0; r < RG; ++r)
       if (r < rg) xs[(d * RG + r) * m + i] = in[(int64_t)(r0 + r) * n + (int64_t)nb * m + i];
     __syncthreads();
-    C<T> acc[RG];
+    float2 acc[RG];
 #pragma unroll
-    for (int r = 0; r < RG; ++r) acc[r] = mk<T>((T)0, (T)0);
-    const C<T> *xd = xs + d * RG * m;
+    for (int r = 0; r < RG; ++r) acc[r] = make_float2(0.f, 0.f);
+    const float2 *xd = xs + d * RG * m;
 #pragma unroll 4
     for (int j = 0; j < m; ++j) {
-      const C<T> a = __ldg(Ad + (int64_t)j * m + i);
+      const float2 a = __ldg(Ad + (int64_t)j * m + i);
 #pragma unroll
       for (int r = 0; r < RG; ++r) acc[r] = cfma(a, xd[r * m + j], acc[r]);
     }
@@ -66,7 +66,7 @@ __global__ void stencil_t_kernel(const C<T> *__restrict__ in, C<T> *__restrict__
     __syncthreads();
     if (d == 0) {
       for (int r = 0; r < rg; ++r) {
-        C<T> v = part[r * m + i];
+        float2 v = part[r * m + i];
 #pragma unroll
         for (int dd = 1; dd < 9; ++dd) v = cadd(v, part[(dd * RG + r) * m + i]);
         out[(int64_t)(r0 + r) * n + (int64_t)X * m + i] = v;
@@ -82,15 +82,15 @@ __global__ void stencil_t_kernel(const C<T> *__restrict__ in, C<T> *__restrict__
 // takes the columns j = w, w + 8, ... of every direction.  The neighbour
 // vectors of the 9 directions for RG right-hand sides are staged in shared
 // memory; the 8 warp partials of a row are added in warp order.
-template <typename T, int RG>
-__global__ void __launch_bounds__(256) stencil_wide_kernel(const C<T> *__restrict__ in,
-                                                           C<T> *__restrict__ out,
-                                                           const C<T> *__restrict__ AT, Geom g,
+template <int RG>
+__global__ void __launch_bounds__(256) stencil_wide_kernel(const float2 *__restrict__ in,
+                                                           float2 *__restrict__ out,
+                                                           const float2 *__restrict__ AT, Geom g,
                                                            int nrhs) {
   extern __shared__ unsigned char smem_raw[];
   const int m = g.dof;
-  C<T> *xs = reinterpret_cast<C<T> *>(smem_raw);  // [9][RG][m]
-  C<T> *part = xs + 9 * RG * m;                   // [8 warps][RG][32]
+  float2 *xs = reinterpret_cast<float2 *>(smem_raw);  // [9][RG][m]
+  float2 *part = xs + 9 * RG * m;                   // [8 warps][RG][32]
   const int X = blockIdx.x, i0 = blockIdx.y * 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = i0 + lane;
@@ -101,18 +101,18 @@ __global__ void __launch_bounds__(256) stencil_wide_kernel(const C<T> *__restric
     __syncthreads();
     for (int e = threadIdx.x; e < 9 * RG * m; e += blockDim.x) {
       const int d = e / (RG * m), rem = e - d * RG * m, r = rem / m, j = rem - r * m;
-      xs[e] = r < rg ? in[(int64_t)(r0 + r) * n + (int64_t)g.neighbor(X, d) * m + j] : mk<T>((T)0, (T)0);
+      xs[e] = r < rg ? in[(int64_t)(r0 + r) * n + (int64_t)g.neighbor(X, d) * m + j] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    C<T> acc[RG];
+    float2 acc[RG];
 #pragma unroll
-    for (int r = 0; r < RG; ++r) acc[r] = mk<T>((T)0, (T)0);
+    for (int r = 0; r < RG; ++r) acc[r] = make_float2(0.f, 0.f);
     if (row_ok) {
       for (int d = 0; d < 9; ++d) {
-        const C<T> *Ad = AT + ((int64_t)X * 9 + d) * m * m;
-        const C<T> *xd = xs + d * RG * m;
+        const float2 *Ad = AT + ((int64_t)X * 9 + d) * m * m;
+        const float2 *xd = xs + d * RG * m;
         for (int j = w; j < m; j += 8) {
-          const C<T> a = __ldg(Ad + (int64_t)j * m + i);
+          const float2 a = __ldg(Ad + (int64_t)j * m + i);
 #pragma unroll
           for (int r = 0; r < RG; ++r) acc[r] = cfma(a, xd[r * m + j], acc[r]);
         }
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(256) stencil_wide_kernel(const C<T> *__restric
     __syncthreads();
     if (w == 0 && row_ok) {
       for (int r = 0; r < rg; ++r) {
-        C<T> v = part[r * 32 + lane];
+        float2 v = part[r * 32 + lane];
 #pragma unroll
         for (int ww = 1; ww < 8; ++ww) v = cadd(v, part[(ww * RG + r) * 32 + lane]);
         out[(int64_t)(r0 + r) * n + (int64_t)X * m + i] = v;
@@ -132,13 +132,13 @@ __global__ void __launch_bounds__(256) stencil_wide_kernel(const C<T> *__restric
   }
 }
 
-template <typename T, int RG>
-void launch_wide(const C<T> *in, C<T> *out, const C<T> *AT, Geom g, int nrhs, cudaStream_t s) {
+template <int RG>
+void launch_wide(const float2 *in, float2 *out, const float2 *AT, Geom g, int nrhs, cudaStream_t s) {
   const int m = g.dof;
-  const size_t sm = (size_t)(9 * RG * m + 8 * RG * 32) * sizeof(C<T>);
-  smem_optin((const void *)stencil_wide_kernel<T, RG>, 200 * 1024);
+  const size_t sm = (size_t)(9 * RG * m + 8 * RG * 32) * sizeof(float2);
+  smem_optin((const void *)stencil_wide_kernel<RG>, 200 * 1024);
   if (sm > 200 * 1024) throw Error(1, "coarse stencil: too many dofs per site");
-  stencil_wide_kernel<T, RG><<<dim3(g.V, (m + 31) / 32), 256, sm, s>>>(in, out, AT, g, nrhs);
+  stencil_wide_kernel<RG><<<dim3(g.V, (m + 31) / 32), 256, sm, s>>>(in, out, AT, g, nrhs);
   MG_LAUNCH_CHECK();
 }
 
@@ -187,21 +187,21 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *mbar, unsigned parit
 // (9 m^2 complex, contiguous) brought into shared memory by one TMA bulk copy
 // issued by thread 0 while the others stage the neighbour vectors; every
 // block entry is then read from shared memory for all right-hand sides.
-template <typename T, int RG>
-__global__ void stencil_tma_kernel(const C<T> *__restrict__ in, C<T> *__restrict__ out,
-                                   const C<T> *__restrict__ AT, Geom g, int nrhs, int *err,
+template <int RG>
+__global__ void stencil_tma_kernel(const float2 *__restrict__ in, float2 *__restrict__ out,
+                                   const float2 *__restrict__ AT, Geom g, int nrhs, int *err,
                                    unsigned extra_tx) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t mbar;
   const int m = g.dof;
-  C<T> *As = reinterpret_cast<C<T> *>(smem_raw);  // [9][j][i]
-  C<T> *xs = As + 9 * m * m;                        // [9][RG][m]
-  C<T> *part = xs + 9 * RG * m;                     // [9][RG][m]
+  float2 *As = reinterpret_cast<float2 *>(smem_raw);  // [9][j][i]
+  float2 *xs = As + 9 * m * m;                        // [9][RG][m]
+  float2 *part = xs + 9 * RG * m;                     // [9][RG][m]
   const int X = blockIdx.x;
   const int i = threadIdx.x, d = threadIdx.y;
   const int tid = d * blockDim.x + i;
   const int64_t n = g.n();
-  const unsigned bytes = (unsigned)(9u * m * m * sizeof(C<T>));
+  const unsigned bytes = (unsigned)(9u * m * m * sizeof(float2));
   if (tid == 0) mbar_init(&mbar, 1);
   __syncthreads();
   if (tid == 0) {
@@ -225,14 +225,14 @@ __global__ void stencil_tma_kernel(const C<T> *__restrict__ in, C<T> *__restrict
       }
     }
     __syncthreads();
-    C<T> acc[RG];
+    float2 acc[RG];
 #pragma unroll
-    for (int r = 0; r < RG; ++r) acc[r] = mk<T>((T)0, (T)0);
-    const C<T> *xd = xs + d * RG * m;
-    const C<T> *Ad = As + d * m * m;
+    for (int r = 0; r < RG; ++r) acc[r] = make_float2(0.f, 0.f);
+    const float2 *xd = xs + d * RG * m;
+    const float2 *Ad = As + d * m * m;
 #pragma unroll 4
     for (int j = 0; j < m; ++j) {
-      const C<T> a = Ad[j * m + i];
+      const float2 a = Ad[j * m + i];
 #pragma unroll
       for (int r = 0; r < RG; ++r) acc[r] = cfma(a, xd[r * m + j], acc[r]);
     }
@@ -241,7 +241,7 @@ __global__ void stencil_tma_kernel(const C<T> *__restrict__ in, C<T> *__restrict
     __syncthreads();
     if (d == 0) {
       for (int r = 0; r < rg; ++r) {
-        C<T> v = part[r * m + i];
+        float2 v = part[r * m + i];
 #pragma unroll
         for (int dd = 1; dd < 9; ++dd) v = cadd(v, part[(dd * RG + r) * m + i]);
         out[(int64_t)(r0 + r) * n + (int64_t)X * m + i] = v;
@@ -575,9 +575,8 @@ void launch_pipe(const float2 *in, float2 *out, const S *AT, Geom g, int nrhs, i
   MG_LAUNCH_CHECK();
 }
 
-// AT[X][d][j][i] = A[X][d][i][j], converted to the storage type To.
-template <typename To>
-__global__ void stencil_transpose_kernel(const double2 *__restrict__ A, C<To> *__restrict__ AT,
+// AT[X][d][j][i] = A[X][d][i][j] in FP32
+__global__ void stencil_transpose_kernel(const double2 *__restrict__ A, float2 *__restrict__ AT,
                                          int64_t nblocks, int m) {
   const int64_t total = nblocks * m * m;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
@@ -585,7 +584,7 @@ __global__ void stencil_transpose_kernel(const double2 *__restrict__ A, C<To> *_
     const int64_t blk = e / ((int64_t)m * m);
     const int rem = (int)(e - blk * m * m);
     const int j = rem / m, i = rem - j * m;  // e indexes AT[blk][j][i]
-    AT[e] = cvt<To>(A[blk * m * m + (int64_t)i * m + j]);
+    AT[e] = cvt<float>(A[blk * m * m + (int64_t)i * m + j]);
   }
 }
 
@@ -940,32 +939,31 @@ int sm_count() {
   return n;
 }
 
-template <typename T>
-void stencil_apply(const C<T> *in, C<T> *out, const C<T> *AT, Geom g, int nrhs, int *err,
+void stencil_apply(const float2 *in, float2 *out, const float2 *AT, Geom g, int nrhs, int *err,
                    cudaStream_t s) {
-  constexpr int RG = sizeof(T) == 4 ? 8 : 4;
+  constexpr int RG = 8;
   const int m = g.dof;
   // the (m, 9)-thread kernels below need 9 m threads of ~80 registers, which
   // one SM holds only up to m ~ 91; wider operators take the tiled kernel
   if (m > 64) {
     // wide operators: as many right-hand sides per pass as ~96 KB of staged
     // neighbour vectors allow
-    const size_t per = (size_t)9 * m * sizeof(C<T>);
-    if (per * 4 <= 96 * 1024) launch_wide<T, 4>(in, out, AT, g, nrhs, s);
-    else if (per * 2 <= 96 * 1024) launch_wide<T, 2>(in, out, AT, g, nrhs, s);
-    else launch_wide<T, 1>(in, out, AT, g, nrhs, s);
+    const size_t per = (size_t)9 * m * sizeof(float2);
+    if (per * 4 <= 96 * 1024) launch_wide<4>(in, out, AT, g, nrhs, s);
+    else if (per * 2 <= 96 * 1024) launch_wide<2>(in, out, AT, g, nrhs, s);
+    else launch_wide<1>(in, out, AT, g, nrhs, s);
     return;
   }
-  const size_t sm_tma = (size_t)(9 * m * m + 2 * 9 * RG * m) * sizeof(C<T>);
+  const size_t sm_tma = (size_t)(9 * m * m + 2 * 9 * RG * m) * sizeof(float2);
   if (sm_tma <= 200 * 1024) {
-    smem_optin((const void *)stencil_tma_kernel<T, RG>, 200 * 1024);
-    stencil_tma_kernel<T, RG><<<g.V, dim3(m, 9), sm_tma, s>>>(in, out, AT, g, nrhs, err, staging_extra_bytes());
+    smem_optin((const void *)stencil_tma_kernel<RG>, 200 * 1024);
+    stencil_tma_kernel<RG><<<g.V, dim3(m, 9), sm_tma, s>>>(in, out, AT, g, nrhs, err, staging_extra_bytes());
     MG_LAUNCH_CHECK();
     return;
   }
-  const size_t sm = (size_t)2 * 9 * RG * m * sizeof(C<T>);
-  smem_optin((const void *)stencil_t_kernel<T, RG>, 200 * 1024);
-  stencil_t_kernel<T, RG><<<g.V, dim3(m, 9), sm, s>>>(in, out, AT, g, nrhs);
+  const size_t sm = (size_t)2 * 9 * RG * m * sizeof(float2);
+  smem_optin((const void *)stencil_t_kernel<RG>, 200 * 1024);
+  stencil_t_kernel<RG><<<g.V, dim3(m, 9), sm, s>>>(in, out, AT, g, nrhs);
   MG_LAUNCH_CHECK();
 }
 
@@ -1020,13 +1018,10 @@ void stencil_to_bf16(const float2 *AT32, void *ATB, int64_t count, cudaStream_t 
   MG_LAUNCH_CHECK();
 }
 
-template <typename To>
-void stencil_transpose(const double2 *A, C<To> *AT, int64_t nblocks, int m, cudaStream_t s) {
-  stencil_transpose_kernel<To><<<grid_for(nblocks * m * m), 256, 0, s>>>(A, AT, nblocks, m);
+void stencil_transpose(const double2 *A, float2 *AT, int64_t nblocks, int m, cudaStream_t s) {
+  stencil_transpose_kernel<<<grid_for(nblocks * m * m), 256, 0, s>>>(A, AT, nblocks, m);
   MG_LAUNCH_CHECK();
 }
-template void stencil_transpose<double>(const double2 *, C<double> *, int64_t, int, cudaStream_t);
-template void stencil_transpose<float>(const double2 *, C<float> *, int64_t, int, cudaStream_t);
 
 template <typename T>
 void stencil_split(const C<T> *in, C<T> *out9, const C<T> *A, Geom g, const int b[4],
@@ -1135,8 +1130,6 @@ void dense_trace(const double2 *M, int n, double2 *out, cudaStream_t s) {
 }
 
 #define INST(T)                                                                                 \
-  template void stencil_apply<T>(const C<T> *, C<T> *, const C<T> *, Geom, int, int *,         \
-                                 cudaStream_t);                                                 \
   template void stencil_split<T>(const C<T> *, C<T> *, const C<T> *, Geom, const int *,         \
                                  cudaStream_t);                                                 \
   template void restrict_op<T>(const C<T> *, C<T> *, const C<T> *, const AggMap &, int,         \
