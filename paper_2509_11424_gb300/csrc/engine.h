@@ -18,6 +18,8 @@ struct Level {
   Geom g{};
   bool fine = false;
   double2 *U64 = nullptr;  // fine links [V][4][3][3]
+  int4 *UF = nullptr;      // fine links as fixed-point digits (FP64 apply), tiled by 32 sites
+  int UFe = 0;             // exponent field of their unit, 0: the links need the FP64 kernel
   float2 *UD32 = nullptr;  // FP32 links structure-of-arrays [4][3][3][V] (FP32 kernels)
   float *Ub16 = nullptr;   // bf16 links structure-of-arrays (one bf16 pair per float slot)
   double2 *A64 = nullptr;   // coarse stencil, canonical [V][9][dof][dof]

@@ -46,15 +46,16 @@ FX_HD int64_t bits_of(double v) {
 // below 2^(e - 1022)
 FX_HD int exp_field(double v) { return (int)((bits_of(v) >> 52) & 0x7ff); }
 
-// round toward zero of v 2^(kVecBits - (E - 1022)); |result| < 2^kVecBits for
-// every v whose exponent field is at most E (1 <= E < 2047)
-FX_HD int64_t to_fixed(double v, int E) {
+// round toward zero of v 2^(BITS - (E - 1022)), BITS = 53 .. 62; |result| <
+// 2^BITS for every v whose exponent field is at most E (1 <= E < 2047)
+template <int BITS = kVecBits> FX_HD int64_t to_fixed(double v, int E) {
   const int64_t b = bits_of(v);
   int e = (int)((b >> 52) & 0x7ff);
   const uint64_t m = ((uint64_t)b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
   if (e == 0) e = 1;
-  // m 2^(e - E + 4): the mantissa left-aligned below the sign, then one shift
-  int s = E - e + 6;
+  // m 2^(e - E + BITS - 53): the mantissa left-aligned below the sign, then
+  // one shift
+  int s = E - e + 63 - BITS;
   if (s > 63) s = 63;
   const int64_t x = (int64_t)((m << 10) >> s);
   const int64_t sg = b >> 63;

@@ -106,6 +106,15 @@ int wilson_fp32_variants();
 // (seed): Philox4x64-10 words -> Box-Muller normals A -> H = (A + A^H)/2 -
 // tr/3 -> matrix exponential; U row-major per link, canonical link order
 void gauge_generate(double2 *U, int64_t nlinks, double eps, uint64_t seed, cudaStream_t s);
+// D psi in FP64 on the integer pipe (fixed.cuh): UF, EU from link_digits,
+// work of wilson_fx_elems complex doubles.  link_digits returns the exponent
+// field of the links' unit, or 0 where the links differ too much in size for
+// one (range: two ints of device scratch; synchronises).
+size_t link_digits_elems(int V);
+int link_digits(const double2 *U, int4 *UF, int *range, int V, cudaStream_t s);
+size_t wilson_fx_elems(int V, int nrhs);
+void wilson_apply_fx(const double2 *in, double2 *out, const int4 *UF, const double2 *U, int EU, double2 *work, Geom g,
+                     double m0, int nrhs, cudaStream_t s);
 // BF16 storage, FP32 arithmetic: D psi for nrhs vectors of complex bf16 in
 // the chunked structure-of-arrays order (pair ((i/4) V + s) * 4 + i % 4),
 // links Ub from link_bf16; 16-byte aligned

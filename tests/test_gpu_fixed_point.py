@@ -11,6 +11,7 @@ max|x|, and typically the square root of K of it.  Asserted: 1e-13 of
 import numpy as np
 import pytest
 
+from oracle import dirac
 from paper_2509_11424_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -81,3 +82,75 @@ def test_coarse_stencil_fp64_special_values():
             assert not got[5].any()
     finally:
         s.close()
+
+
+def _wilson(dims, U, x, m0):
+    from gpu_util import require_lib
+    M = require_lib()
+    ctx = M.mgmlmc_create(dims, torch.cuda.current_stream())
+    try:
+        M.mgmlmc_set_gauge(ctx, U)
+        M.mgmlmc_set_mass(ctx, m0)
+        xd = dev(x)
+        yd = torch.full_like(xd, float('nan'))
+        M.mgmlmc_apply(ctx, M.OP_D, 0, M.FP64, xd, yd, x.shape[0])
+        return host(yd)
+    finally:
+        M.mgmlmc_destroy(ctx)
+
+
+# sites: fewer than a tile of 32, no multiple of the 64 of a block, extents of
+# 2 and 3, more right-hand sides than one converted group on small lattices
+# (2^18 sites / V) never are, so the group of 4 is crossed with a larger one
+@pytest.mark.parametrize('dims,nrhs', [((2, 2, 2, 2), 1), ((3, 2, 2, 5), 3), ((5, 4, 3, 7), 2), ((8, 4, 2, 6), 5),
+                                       ((28, 28, 28, 28), 5)])
+def test_wilson_fp64_fixed_point(dims, nrhs):
+    """Sites of very different size (each is kept in units of its own largest
+    entry): entry by entry within 2e-15 of the largest entry among the site
+    and its neighbours (7 bits of a 61-bit unit summed over 8 hops is far
+    less; the FP64 diagonal term rounds at 2^-53 x 4)."""
+    V = dirac.volume(dims)
+    U = synth.gauge_field(dims, 0.4, 71)
+    x = synth.complex_normal((nrhs, V, 12), 72)
+    x *= 2.0 ** np.random.default_rng(73).integers(-30, 30, (nrhs, V, 1))
+    got = _wilson(dims, U, x.reshape(nrhs, -1), -0.3).reshape(nrhs, V, 12)
+    top = np.abs(x).max(2).reshape(nrhs, *dims[::-1])
+    near = np.max([np.roll(top, k, a) for a in range(1, 5) for k in (-1, 0, 1)], 0).reshape(nrhs, V)
+    for r in range(nrhs):
+        want = dirac.apply_wilson(U, x[r].reshape(-1), -0.3, dims).reshape(V, 12)
+        assert np.all(np.abs(got[r] - want).max(1) <= 4e-15 * near[r])
+
+
+def test_wilson_fp64_special_values():
+    """Inf / NaN stay with the sites that touch them; subnormal, huge and zero
+    vectors keep their values; links of very different size take the FP64
+    kernel."""
+    dims = (4, 6, 4, 4)
+    V = dirac.volume(dims)
+    U = synth.gauge_field(dims, 0.4, 74)
+    x = synth.complex_normal((6, V * 12), 75)
+    x[1, 7] = np.nan
+    x[2, 30] = np.inf
+    x[3] *= 2.0 ** -1040
+    x[4] *= 2.0 ** 1010
+    x[5] = 0.0
+    got = _wilson(dims, U, x, -0.3)
+    with np.errstate(all='ignore'):
+        for r, j in ((1, 7), (2, 30)):
+            hit = ~np.isfinite(got[r]).reshape(V, 12).all(1)
+            c = x[r].copy()
+            c[j] = 0.0
+            e = np.zeros_like(c)
+            e[j] = 1.0
+            touched = np.abs(dirac.apply_wilson(U, e, -0.3, dims)).reshape(V, 12).max(1) > 0
+            assert np.array_equal(hit, touched)
+            want = dirac.apply_wilson(U, c, -0.3, dims)
+            assert np.abs(got[r] - want).reshape(V, 12)[~touched].max() < 1e-14
+        assert np.abs(got[3] - dirac.apply_wilson(U, x[3], -0.3, dims)).max() <= 2.0 ** -1074 * 64
+        want = dirac.apply_wilson(U, x[4] * 2.0 ** -1010, -0.3, dims)
+        assert np.abs(got[4] * 2.0 ** -1010 - want).max() < 1e-13
+        assert not got[5].any()
+    U2 = U.copy()
+    U2[:9] *= 1e-9
+    y = _wilson(dims, U2, x[:1], -0.3)
+    assert np.abs(y[0] - dirac.apply_wilson(U2, x[0], -0.3, dims)).max() < 1e-13
