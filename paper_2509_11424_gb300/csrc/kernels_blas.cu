@@ -3,10 +3,16 @@
 //
 // Reductions are deterministic: a fixed number of blocks (a function of n
 // only) writes partial sums that the last block to finish adds in block
-// order, so a result never depends on scheduling.  Sums are accumulated in
-// FP64 for both storage precisions.
+// order, so a result never depends on scheduling.  FP32 products are summed
+// in FP32 within a thread, FP64 ones as integers (fixed.cuh); the sums over
+// the lanes of a warp are exact integer ones (52 bits of the largest lane for
+// FP32), and across warps and blocks FP64.  FP64 additions are kept to those:
+// a warp's shuffle reduction of one complex number in FP64 takes 640 cycles
+// of the FP64 pipe, as long as 64 FP32 multiply-adds per lane.
+#include "fixed.cuh"
 #include "kernels.h"
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -15,30 +21,6 @@ namespace mg {
 
 namespace {
 constexpr int RB = 256;  // reduction block size
-
-__device__ __forceinline__ double2 warp_sum(double2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-    v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-  }
-  return v;
-}
-
-// block-wide sum; valid in thread 0
-__device__ __forceinline__ double2 block_sum(double2 v) {
-  __shared__ double2 sh[RB / 32];
-  v = warp_sum(v);
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  if (w == 0) {
-    v = (l < (int)(blockDim.x >> 5)) ? sh[l] : make_double2(0.0, 0.0);
-    v = warp_sum(v);
-  }
-  __syncthreads();
-  return v;
-}
 
 // Single-pass reductions.  Block b of output g sums its chunk, writes the
 // partial, and takes a ticket; the block that draws the last ticket adds the
@@ -54,156 +36,529 @@ __device__ __forceinline__ bool last_block(unsigned *ticket) {
   return last;
 }
 
-__device__ __forceinline__ double2 sum_partials(const double2 *p, int NB) {
+// 2^e as a double, also outside the normal range
+__device__ __forceinline__ double scaled(double v, int e) {
+  return e > -1000 && e < 1000 ? v * __longlong_as_double((long long)(e + 1023) << 52) : scalbn(v, e);
+}
+
+// ---- exact sums over a warp.  Every lane calls add() for value 0, 1, ... in
+// turn; get() then gives lane v the sum of value v.
+//
+// FP32 lanes: integers of 51 bits in the unit of the largest lane's exponent,
+// as two words whose 32-fold sums fit 32 bits.
+struct WarpSumF {
+  unsigned lo = 0;
+  int hi = 0, e = 0;
+  __device__ __forceinline__ void add(int v, float p) {
+    const unsigned b = __float_as_uint(p);
+    int x = (b >> 23) & 0xff;
+    const int E = __reduce_max_sync(0xffffffffu, x);
+    const unsigned m = (b & 0x7fffffu) | (x ? 0x800000u : 0u);
+    x = x ? x : 1;
+    const int s = min(max(E, 1) - x, 60);
+    long long X = (long long)(((unsigned long long)m << 27) >> s);
+    X = (int)b < 0 ? -X : X;
+    const unsigned l = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
+    const int h = __reduce_add_sync(0xffffffffu, (int)(X >> 26));
+    if ((int)(threadIdx.x & 31) == v) {
+      lo = l;
+      hi = h;
+      e = E;
+    }
+  }
+  __device__ __forceinline__ double get() const {
+    const double d = scaled((double)(((long long)hi << 26) + lo), max(e, 1) - (127 + 23 + 27));
+    return e == 0xff ? __longlong_as_double(0x7ff8000000000000ll) : d;
+  }
+};
+// 64-bit integers in units of 2^unit (the same in every lane): three words
+struct WarpSumI {
+  unsigned w0 = 0, w1 = 0;
+  int w2 = 0, e = 0;
+  __device__ __forceinline__ void add(int v, long long X, int unit, bool bad) {
+    const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
+    const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(X >> 26) & 0x3ffffffu);
+    const int c = __reduce_add_sync(0xffffffffu, (int)(X >> 52));
+    if ((int)(threadIdx.x & 31) == v) {
+      w0 = a;
+      w1 = b;
+      w2 = c;
+      e = bad ? 1 << 20 : unit;
+    }
+  }
+  __device__ __forceinline__ double get() const {
+    const double d = fma((double)w2, 0x1p52, (double)(((long long)w1 << 26) + w0));
+    return e == 1 << 20 ? __longlong_as_double(0x7ff8000000000000ll) : scaled(d, e);
+  }
+};
+
+__device__ __forceinline__ int warp_exp(int e) { return max(__reduce_max_sync(0xffffffffu, e), 1); }
+__device__ __forceinline__ int exp2of(double2 v) { return max(fx::exp_field(v.x), fx::exp_field(v.y)); }
+__device__ __forceinline__ int4 digits(double2 v, int E) {
+  const long long a = fx::to_fixed(v.x, E), b = fx::to_fixed(v.y, E);
+  return make_int4(fx::digit_hi(a), fx::digit_lo(a), fx::digit_hi(b), fx::digit_lo(b));
+}
+
+// The block's NV sums (lane v of every warp holds value v) to partial[v * NB +
+// b] (doubles, pv apart); the block that finishes group g last adds the NB
+// partials of every value in block order and returns true with value v in
+// thread v < NV.
+template <int NV>
+__device__ __forceinline__ bool block_finish(double mine, double *__restrict__ partial, unsigned *__restrict__ ticket,
+                                             int nv, double &out) {
+  __shared__ double red[RB / 32][NV];
+  __shared__ double tail[RB / NV][NV];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, NB = gridDim.x;
+  if (lane < NV) red[wp][lane] = mine;
+  __syncthreads();
+  if ((int)threadIdx.x < nv) {
+    double t = red[0][threadIdx.x];
+#pragma unroll
+    for (int q = 1; q < RB / 32; ++q) t += red[q][threadIdx.x];
+    if (NB == 1) out = t;
+    else partial[(int64_t)threadIdx.x * NB + blockIdx.x] = t;
+  }
+  if (NB == 1) return true;
   __threadfence();
-  double2 acc = make_double2(0.0, 0.0);
-  for (int b = threadIdx.x; b < NB; b += blockDim.x) {
-    const double2 v = __ldcg(p + b);
-    acc.x += v.x;
-    acc.y += v.y;
+  __syncthreads();
+  if (!last_block(ticket)) return false;
+  __threadfence();
+  const int v = threadIdx.x % NV, c = threadIdx.x / NV;
+  if (c < RB / NV) {
+    double t = 0.0;
+    if (v < nv) {
+      // RB / NV threads per value, each over consecutive blocks
+      const int per = (NB + RB / NV - 1) / (RB / NV), b0 = c * per, b1 = min(NB, b0 + per);
+      for (int q = b0; q < b1; ++q) t += __ldcg(partial + (int64_t)v * NB + q);
+    }
+    tail[c][v] = t;
   }
-  return block_sum(acc);
+  __syncthreads();
+  if ((int)threadIdx.x < nv) {
+    double t = tail[0][threadIdx.x];
+    for (int q = 1; q < RB / NV; ++q) t += tail[q][threadIdx.x];
+    out = t;
+  }
+  if (threadIdx.x == 0) *ticket = 0u;
+  return true;
 }
 
-// out[r * ldh + j] = sum conj(x_j,r) y_r; output g = j * nrhs + r, its NB
-// partials at partial[g * NB ..]
-template <typename T>
-__global__ void dot_kernel(const C<T> *__restrict__ x, int64_t xstride, const C<T> *__restrict__ y,
-                           int64_t n, int64_t chunk, double2 *__restrict__ partial,
-                           unsigned *__restrict__ ticket, double2 *__restrict__ out, int ldh) {
-  const int b = blockIdx.x, r = blockIdx.y, j = blockIdx.z;
-  const int64_t g = (int64_t)j * gridDim.y + r;
-  const C<T> *xr = x + j * xstride + r * n;
-  const C<T> *yr = y + r * n;
-  const int64_t beg = (int64_t)b * chunk;
-  const int64_t end = beg + chunk < n ? beg + chunk : n;
-  // per-thread partial in the storage precision over the few elements a
-  // thread visits (reduce_blocks keeps that short; FP32 FMAs run ~58x faster
-  // than FP64 ones on this part), then FP64 across threads and blocks
-  C<T> acc = mk<T>((T)0, (T)0);
-  for (int64_t i = beg + threadIdx.x; i < end; i += blockDim.x) {
-    const C<T> a = xr[i], c = yr[i];
-    acc = cfmac(a, c, acc);
+// element pairs of FP32 vectors as one 16-byte load where the operands allow
+template <bool VEC>
+__device__ __forceinline__ float4 ld2(const float2 *__restrict__ p, int64_t i, int64_t end) {
+  if (VEC) return i < end ? __ldg(reinterpret_cast<const float4 *>(p + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (i < end) { v.x = p[i].x; v.y = p[i].y; }
+  if (i + 1 < end) { v.z = p[i + 1].x; v.w = p[i + 1].y; }
+  return v;
+}
+
+// out[r * ldh + j] = sum conj(x_j,r) y_r, JG vectors x_j per block (grid z),
+// y read once for them.  Block (b, r, z): elements [b chunk, (b + 1) chunk).
+// Bound: memory (x once, y once per JG of them; 5.4 TB/s at n = 786 k, 8
+// right-hand sides, 15 vectors), latency below n ~ 10^5: short chunks, so that
+// a right-hand side of 8192 entries has 8 blocks.
+template <int JG, bool VEC>
+__global__ void __launch_bounds__(RB) dot_f32_kernel(const float2 *__restrict__ x, int64_t xstride, int k,
+                                                     const float2 *__restrict__ y, int64_t n, int64_t chunk,
+                                                     double2 *__restrict__ partial, unsigned *__restrict__ ticket,
+                                                     double2 *__restrict__ out, int ldh) {
+  constexpr int U = 2;  // element pairs per thread and step
+  const int r = blockIdx.y, j0 = blockIdx.z * JG, kg = min(JG, k - j0);
+  const float2 *xr = x + j0 * xstride + r * n, *yr = y + r * n;
+  const int64_t beg = (int64_t)blockIdx.x * chunk, end = min(beg + chunk, n);
+  float ar[JG], ai[JG];
+#pragma unroll
+  for (int j = 0; j < JG; ++j) ar[j] = ai[j] = 0.f;
+  for (int64_t i0 = beg + 2 * threadIdx.x; i0 < end; i0 += 2 * RB * U) {
+    float4 c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = ld2<VEC>(yr, i0 + 2 * RB * u, end);
+#pragma unroll
+    for (int j = 0; j < JG; ++j) {
+      if (j < kg) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float4 a = ld2<VEC>(xr + j * xstride, i0 + 2 * RB * u, end);
+          ar[j] = fmaf(a.x, c[u].x, fmaf(a.y, c[u].y, fmaf(a.z, c[u].z, fmaf(a.w, c[u].w, ar[j]))));
+          ai[j] = fmaf(a.x, c[u].y, fmaf(-a.y, c[u].x, fmaf(a.z, c[u].w, fmaf(-a.w, c[u].z, ai[j]))));
+        }
+      }
+    }
   }
-  const double2 tot = block_sum(make_double2((double)acc.x, (double)acc.y));
-  if (threadIdx.x == 0) partial[g * gridDim.x + b] = tot;
-  if (!last_block(ticket + g)) return;
-  const double2 s = sum_partials(partial + g * gridDim.x, gridDim.x);
-  if (threadIdx.x == 0) {
-    out[r * ldh + j] = s;
-    ticket[g] = 0u;
+  WarpSumF ws;
+#pragma unroll
+  for (int j = 0; j < JG; ++j) {
+    if (j < kg) {
+      ws.add(2 * j, ar[j]);
+      ws.add(2 * j + 1, ai[j]);
+    }
+  }
+  double s;
+  const int64_t g = (int64_t)r * gridDim.z + blockIdx.z;
+  double *part = reinterpret_cast<double *>(partial) + ((int64_t)r * k + j0) * 2 * gridDim.x;
+  if (block_finish<2 * JG>(ws.get(), part, ticket + g, 2 * kg, s) && (int)threadIdx.x < 2 * kg)
+    reinterpret_cast<double *>(out + r * ldh + j0)[threadIdx.x] = s;
+}
+
+// The same for FP64 vectors on the integer pipe: every warp scales its 128
+// elements of y and of each x_j by their own largest entry; 12 integer
+// multiply-adds per element and vector, exact sums, one conversion per warp,
+// vector and 128 elements.  n = 786 k, 16 right-hand sides, 20 vectors: 1.20
+// ms, 3.8 TB/s; 4 FP64 FMAs per element took 1.97 ms, y read for every vector.
+template <int JG>
+__global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__ x, int64_t xstride, int k,
+                                                     const double2 *__restrict__ y, int64_t n, int64_t chunk,
+                                                     double2 *__restrict__ partial, unsigned *__restrict__ ticket,
+                                                     double2 *__restrict__ out, int ldh) {
+  constexpr int U = 4;  // elements per thread and step
+  const int r = blockIdx.y, j0 = blockIdx.z * JG, kg = min(JG, k - j0);
+  const double2 *xr = x + j0 * xstride + r * n, *yr = y + r * n;
+  const int64_t beg = (int64_t)blockIdx.x * chunk, end = min(beg + chunk, n);
+  const double2 zero = make_double2(0.0, 0.0);
+  double acc = 0.0;
+  for (int64_t t0 = beg; t0 < end; t0 += RB * U) {
+    const int64_t i0 = t0 + threadIdx.x;
+    double2 a[U];
+    int4 c[U];
+    int Ey = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      a[u] = i0 + RB * u < end ? __ldg(yr + i0 + RB * u) : zero;
+      Ey = max(Ey, exp2of(a[u]));
+    }
+    Ey = warp_exp(Ey);
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = digits(a[u], min(Ey, fx::kBadExp - 1));
+#pragma unroll
+    for (int u = 0; u < U; ++u) a[u] = i0 + RB * u < end ? __ldg(xr + i0 + RB * u) : zero;
+    WarpSumI ws;
+#pragma unroll
+    for (int j = 0; j < JG; ++j) {
+      if (j < kg) {
+        double2 b[U];
+        int Ex = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          b[u] = a[u];
+          Ex = max(Ex, exp2of(b[u]));
+        }
+        if (j + 1 < kg) {  // the next vector's elements while this one is used
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            a[u] = i0 + RB * u < end ? __ldg(xr + (j + 1) * xstride + i0 + RB * u) : zero;
+        }
+        Ex = warp_exp(Ex);
+        long long hr = 0, hi = 0, mr = 0, mi = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          // conj(x) y
+          const int4 q = digits(b[u], min(Ex, fx::kBadExp - 1));
+          const int n1 = -q.z, n0 = -q.w;
+          hr = fx::madw(q.z, c[u].z, fx::madw(q.x, c[u].x, hr));
+          hi = fx::madw(n1, c[u].x, fx::madw(q.x, c[u].z, hi));
+          mr = fx::madw(q.w, c[u].z, fx::madw(q.z, c[u].w, fx::madw(q.y, c[u].x, fx::madw(q.x, c[u].y, mr))));
+          mi = fx::madw(n0, c[u].x, fx::madw(n1, c[u].y, fx::madw(q.y, c[u].z, fx::madw(q.x, c[u].w, mi))));
+        }
+        const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
+        const bool bad = Ex == fx::kBadExp || Ey == fx::kBadExp;
+        ws.add(2 * j, fx::fold(hr, mr), e, bad);
+        ws.add(2 * j + 1, fx::fold(hi, mi), e, bad);
+      }
+    }
+    acc += ws.get();
+  }
+  double s;
+  const int64_t g = (int64_t)r * gridDim.z + blockIdx.z;
+  double *part = reinterpret_cast<double *>(partial) + ((int64_t)r * k + j0) * 2 * gridDim.x;
+  if (block_finish<2 * JG>(acc, part, ticket + g, 2 * kg, s) && (int)threadIdx.x < 2 * kg)
+    reinterpret_cast<double *>(out + r * ldh + j0)[threadIdx.x] = s;
+}
+
+// oqr[r] = <q_r, r_r>, oqq[r] = <q_r, q_r>
+template <bool VEC>
+__global__ void __launch_bounds__(RB) dot_qr_f32_kernel(const float2 *__restrict__ q, const float2 *__restrict__ rr,
+                                                        int64_t n, int64_t chunk, double2 *__restrict__ partial,
+                                                        unsigned *__restrict__ ticket, double2 *__restrict__ oqr,
+                                                        double2 *__restrict__ oqq) {
+  constexpr int U = 2;
+  const int r = blockIdx.y;
+  const float2 *qr = q + r * n, *xr = rr + r * n;
+  const int64_t beg = (int64_t)blockIdx.x * chunk, end = min(beg + chunk, n);
+  float sr = 0.f, si = 0.f, sq = 0.f;
+  for (int64_t i0 = beg + 2 * threadIdx.x; i0 < end; i0 += 2 * RB * U) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float4 a = ld2<VEC>(qr, i0 + 2 * RB * u, end), c = ld2<VEC>(xr, i0 + 2 * RB * u, end);
+      sr = fmaf(a.x, c.x, fmaf(a.y, c.y, fmaf(a.z, c.z, fmaf(a.w, c.w, sr))));
+      si = fmaf(a.x, c.y, fmaf(-a.y, c.x, fmaf(a.z, c.w, fmaf(-a.w, c.z, si))));
+      sq = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, sq))));
+    }
+  }
+  WarpSumF ws;
+  ws.add(0, sr);
+  ws.add(1, si);
+  ws.add(2, sq);
+  double s;
+  double *part = reinterpret_cast<double *>(partial) + (int64_t)r * 4 * gridDim.x;
+  if (block_finish<4>(ws.get(), part, ticket + r, 3, s) && threadIdx.x < 3) {
+    if (threadIdx.x == 0) oqr[r].x = s;
+    else if (threadIdx.x == 1) oqr[r].y = s;
+    else oqq[r] = make_double2(s, 0.0);
   }
 }
 
-// oqr[r] = <q_r, r_r>, oqq[r] = <q_r, q_r>; output r, partials at
-// partial[(2 r + o) * NB ..]
-template <typename T>
-__global__ void dot_qr_kernel(const C<T> *__restrict__ q, const C<T> *__restrict__ rr, int64_t n,
-                              int64_t chunk, double2 *__restrict__ partial,
-                              unsigned *__restrict__ ticket, double2 *__restrict__ oqr,
-                              double2 *__restrict__ oqq) {
-  const int b = blockIdx.x, r = blockIdx.y;
-  const C<T> *qr = q + r * n;
-  const C<T> *xr = rr + r * n;
-  const int64_t beg = (int64_t)b * chunk;
-  const int64_t end = beg + chunk < n ? beg + chunk : n;
-  C<T> ta = mk<T>((T)0, (T)0);
-  T tc = (T)0;
-  for (int64_t i = beg + threadIdx.x; i < end; i += blockDim.x) {
-    const C<T> u = qr[i], v = xr[i];
-    ta = cfmac(u, v, ta);
-    tc = fma(u.x, u.x, fma(u.y, u.y, tc));
+__global__ void __launch_bounds__(RB) dot_qr_f64_kernel(const double2 *__restrict__ q, const double2 *__restrict__ rr,
+                                                        int64_t n, int64_t chunk, double2 *__restrict__ partial,
+                                                        unsigned *__restrict__ ticket, double2 *__restrict__ oqr,
+                                                        double2 *__restrict__ oqq) {
+  constexpr int U = 4;
+  const int r = blockIdx.y;
+  const double2 *qr = q + r * n, *xr = rr + r * n;
+  const int64_t beg = (int64_t)blockIdx.x * chunk, end = min(beg + chunk, n);
+  const double2 zero = make_double2(0.0, 0.0);
+  double acc = 0.0;
+  for (int64_t t0 = beg; t0 < end; t0 += RB * U) {
+    double2 a[U], c[U];
+    int Ea = 0, Ec = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = t0 + threadIdx.x + RB * u;
+      a[u] = i < end ? __ldg(qr + i) : zero;
+      c[u] = i < end ? __ldg(xr + i) : zero;
+      Ea = max(Ea, exp2of(a[u]));
+      Ec = max(Ec, exp2of(c[u]));
+    }
+    Ea = warp_exp(Ea);
+    Ec = warp_exp(Ec);
+    long long hr = 0, hi = 0, mr = 0, mi = 0, hq = 0, mq = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int4 p = digits(a[u], min(Ea, fx::kBadExp - 1)), w = digits(c[u], min(Ec, fx::kBadExp - 1));
+      const int n1 = -p.z, n0 = -p.w;
+      hr = fx::madw(p.z, w.z, fx::madw(p.x, w.x, hr));
+      hi = fx::madw(n1, w.x, fx::madw(p.x, w.z, hi));
+      mr = fx::madw(p.w, w.z, fx::madw(p.z, w.w, fx::madw(p.y, w.x, fx::madw(p.x, w.y, mr))));
+      mi = fx::madw(n0, w.x, fx::madw(n1, w.y, fx::madw(p.y, w.z, fx::madw(p.x, w.w, mi))));
+      hq = fx::madw(p.z, p.z, fx::madw(p.x, p.x, hq));
+      mq = fx::madw(2 * p.w, p.z, fx::madw(2 * p.y, p.x, mq));
+    }
+    const int e = 2 * fx::kDigit + Ea + Ec - 2 * (1022 + fx::kVecBits);
+    const int eq = 2 * fx::kDigit + 2 * Ea - 2 * (1022 + fx::kVecBits);
+    const bool ba = Ea == fx::kBadExp, bc = ba || Ec == fx::kBadExp;
+    WarpSumI ws;
+    ws.add(0, fx::fold(hr, mr), e, bc);
+    ws.add(1, fx::fold(hi, mi), e, bc);
+    ws.add(2, fx::fold(hq, mq), eq, ba);
+    acc += ws.get();
   }
-  const double2 a = block_sum(make_double2((double)ta.x, (double)ta.y));
-  const double2 c = block_sum(make_double2((double)tc, 0.0));
-  if (threadIdx.x == 0) {
-    partial[((int64_t)r * 2 + 0) * gridDim.x + b] = a;
-    partial[((int64_t)r * 2 + 1) * gridDim.x + b] = c;
-  }
-  if (!last_block(ticket + r)) return;
-  const double2 sa = sum_partials(partial + ((int64_t)r * 2 + 0) * gridDim.x, gridDim.x);
-  const double2 sc = sum_partials(partial + ((int64_t)r * 2 + 1) * gridDim.x, gridDim.x);
-  if (threadIdx.x == 0) {
-    oqr[r] = sa;
-    oqq[r] = sc;
-    ticket[r] = 0u;
+  double s;
+  double *part = reinterpret_cast<double *>(partial) + (int64_t)r * 4 * gridDim.x;
+  if (block_finish<4>(acc, part, ticket + r, 3, s) && threadIdx.x < 3) {
+    if (threadIdx.x == 0) oqr[r].x = s;
+    else if (threadIdx.x == 1) oqr[r].y = s;
+    else oqq[r] = make_double2(s, 0.0);
   }
 }
 
-template <typename T>
-__global__ void multi_axpy_kernel(const C<T> *__restrict__ V, int64_t vstride, int k,
-                                  C<T> *__restrict__ w, int64_t n, const double2 *__restrict__ h,
-                                  int ldh, double sign) {
-  __shared__ C<T> coef[128];
+// w_r += sign sum_j h[r * ldh + j] V_j,r
+template <bool VEC>
+__global__ void __launch_bounds__(256) multi_axpy_f32_kernel(const float2 *__restrict__ V, int64_t vstride, int k,
+                                                             float2 *__restrict__ w, int64_t n,
+                                                             const double2 *__restrict__ h, int ldh, double sign) {
+  __shared__ float2 coef[128];
+  const int r = blockIdx.y;
+  for (int j = threadIdx.x; j < k; j += blockDim.x) {
+    const double2 c = h[r * ldh + j];
+    coef[j] = make_float2((float)(sign * c.x), (float)(sign * c.y));
+  }
+  __syncthreads();
+  float2 *wr = w + r * n;
+  const float2 *Vr = V + r * n;
+  for (int64_t i = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); i < n; i += 2 * (int64_t)gridDim.x * blockDim.x) {
+    float4 t = ld2<VEC>(wr, i, n);
+    float2 a = make_float2(t.x, t.y), b = make_float2(t.z, t.w);
+#pragma unroll 4
+    for (int j = 0; j < k; ++j) {
+      const float4 v = ld2<VEC>(Vr + j * vstride, i, n);
+      a = cfma(coef[j], make_float2(v.x, v.y), a);
+      b = cfma(coef[j], make_float2(v.z, v.w), b);
+    }
+    if (VEC) {
+      *reinterpret_cast<float4 *>(wr + i) = make_float4(a.x, a.y, b.x, b.y);
+    } else {
+      wr[i] = a;
+      if (i + 1 < n) wr[i + 1] = b;
+    }
+  }
+}
+
+// The same for FP64 vectors on the integer pipe: JG vectors at a time are
+// added as integers in the unit of the largest coefficient times entry of
+// the warp's 64 elements, then once to w in FP64.  n = 786 k, 16 right-hand
+// sides, 1 .. 20 vectors: 705 us on average (3.6 TB/s) against 931 us in FP64.
+__global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__restrict__ V, int64_t vstride, int k,
+                                                             double2 *__restrict__ w, int64_t n,
+                                                             const double2 *__restrict__ h, int ldh, double sign) {
+  constexpr int JG = 8, U = 2;
+  __shared__ int4 cd[128];
+  __shared__ int ce[128];
+  __shared__ double2 coef[128];
   const int r = blockIdx.y;
   for (int j = threadIdx.x; j < k; j += blockDim.x) {
     double2 c = h[r * ldh + j];
-    coef[j] = mk<T>((T)(sign * c.x), (T)(sign * c.y));
+    c = make_double2(sign * c.x, sign * c.y);
+    const int E = max(exp2of(c), 1);
+    coef[j] = c;
+    ce[j] = E;
+    cd[j] = digits(c, min(E, fx::kBadExp - 1));
   }
   __syncthreads();
-  C<T> *wr = w + r * n;
-  const C<T> *Vr = V + r * n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    C<T> acc = wr[i];
-    for (int j = 0; j < k; ++j) acc = cfma(coef[j], Vr[j * vstride + i], acc);
-    wr[i] = acc;
+  double2 *wr = w + r * n;
+  const double2 *Vr = V + r * n;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x * U;
+  for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x * U; t0 < n; t0 += step) {
+    // lanes past the end work on zeros (the warp scales together)
+    const int64_t i0 = t0 + threadIdx.x;
+    double2 acc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + (int64_t)u * blockDim.x;
+      acc[u] = i < n ? wr[i] : make_double2(0.0, 0.0);
+    }
+    for (int j0 = 0; j0 < k; j0 += JG) {
+      const int kg = min(JG, k - j0);
+      double2 v[JG][U];
+#pragma unroll
+      for (int j = 0; j < JG; ++j)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t i = i0 + (int64_t)u * blockDim.x;
+          v[j][u] = j < kg && i < n ? __ldg(Vr + (j0 + j) * vstride + i) : make_double2(0.0, 0.0);
+        }
+      int S = 2;  // largest exponent sum of a coefficient and its entries
+      bool bad = false;
+#pragma unroll
+      for (int j = 0; j < JG; ++j) {
+        if (j < kg) {
+          int e = 1;
+#pragma unroll
+          for (int u = 0; u < U; ++u) e = max(e, exp2of(v[j][u]));
+          bad |= e == fx::kBadExp || ce[j0 + j] == fx::kBadExp;
+          S = max(S, e + ce[j0 + j]);
+        }
+      }
+      S = __reduce_max_sync(0xffffffffu, S);
+      const int ex = S - 2 * (1022 + fx::kVecBits) + 2 * fx::kDigit;
+      if (__any_sync(0xffffffffu, bad) || ex < -1000 || ex > 900) {
+#pragma unroll
+        for (int j = 0; j < JG; ++j)
+          if (j < kg)
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc[u] = cfma(coef[j0 + j], v[j][u], acc[u]);
+        continue;
+      }
+      long long hr[U], hi[U], mr[U], mi[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) hr[u] = hi[u] = mr[u] = mi[u] = 0;
+#pragma unroll
+      for (int j = 0; j < JG; ++j) {
+        if (j < kg) {
+          const int4 c = cd[j0 + j];
+          const int n1 = -c.z, n0 = -c.w;
+          // the entries in the unit that makes c v come out in units of 2^ex;
+          // a far smaller product vanishes against the largest
+          const int E = S - ce[j0 + j];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int4 q = digits(v[j][u], E);
+            hr[u] = fx::madw(n1, q.z, fx::madw(c.x, q.x, hr[u]));
+            hi[u] = fx::madw(c.z, q.x, fx::madw(c.x, q.z, hi[u]));
+            mr[u] = fx::madw(n0, q.z, fx::madw(n1, q.w, fx::madw(c.y, q.x, fx::madw(c.x, q.y, mr[u]))));
+            mi[u] = fx::madw(c.w, q.x, fx::madw(c.z, q.y, fx::madw(c.y, q.z, fx::madw(c.x, q.w, mi[u]))));
+          }
+        }
+      }
+      const double f = __longlong_as_double((long long)(ex + 1023) << 52);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        acc[u].x = fma(f, (double)fx::fold(hr[u], mr[u]), acc[u].x);
+        acc[u].y = fma(f, (double)fx::fold(hi[u], mi[u]), acc[u].y);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + (int64_t)u * blockDim.x;
+      if (i < n) wr[i] = acc[u];
+    }
   }
 }
 
-template <typename T>
-__global__ void axpby_kernel(T a, const C<T> *__restrict__ x, T b, C<T> *__restrict__ y,
-                             int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    C<T> xv = x[i], yv = y[i];
-    yv.x = a * xv.x + b * yv.x;
-    yv.y = a * xv.y + b * yv.y;
-    y[i] = yv;
+// W complex entries moved by one access (16 bytes: 2 FP32 or 1 FP64 ones)
+template <typename T, int W> struct alignas(W * sizeof(C<T>)) Pack {
+  C<T> v[W];
+};
+template <typename T, int W> __device__ __forceinline__ Pack<T, W> ldp(const C<T> *p) {
+  return *reinterpret_cast<const Pack<T, W> *>(p);
+}
+template <typename T, int W> __device__ __forceinline__ void stp(C<T> *p, const Pack<T, W> &v) {
+  *reinterpret_cast<Pack<T, W> *>(p) = v;
+}
+// first entry of the thread's pack, entries between its packs
+#define MG_PACKS(i, W, n)                                                                          \
+  for (int64_t i = (int64_t)(W) * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); i < (n);       \
+       i += (int64_t)(W)*gridDim.x * blockDim.x)
+
+template <typename T, int W>
+__global__ void axpby_kernel(T a, const C<T> *__restrict__ x, T b, C<T> *__restrict__ y, int64_t n) {
+  MG_PACKS(i, W, n) {
+    const Pack<T, W> xv = ldp<T, W>(x + i);
+    Pack<T, W> yv = ldp<T, W>(y + i);
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+      yv.v[q].x = a * xv.v[q].x + b * yv.v[q].x;
+      yv.v[q].y = a * xv.v[q].y + b * yv.v[q].y;
+    }
+    stp<T, W>(y + i, yv);
   }
 }
 
-template <typename T>
+template <typename T, int W>
 __global__ void scale_rhs_kernel(const C<T> *x, C<T> *y,  // may alias (in-place scaling)
                                  const double *__restrict__ scal, int64_t n) {
-  const int r = blockIdx.y;
-  const T f = (T)scal[r];
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    y[r * n + i] = cscale(x[r * n + i], f);
-}
-
-template <typename T>
-__global__ void mr_update_kernel(C<T> *__restrict__ z, C<T> *__restrict__ res,
-                                 const C<T> *__restrict__ q, const double2 *__restrict__ dqr,
-                                 const double2 *__restrict__ nq, int64_t n) {
-  const int r = blockIdx.y;
-  const double qq = nq[r].x;
-  const double2 d = dqr[r];
-  const C<T> al = qq > 0.0 ? mk<T>((T)(d.x / qq), (T)(d.y / qq)) : mk<T>((T)0, (T)0);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t o = r * n + i;
-    C<T> rv = res[o];
-    z[o] = cfma(al, rv, z[o]);
-    res[o] = cfma(cneg(al), q[o], rv);
+  const int64_t o = blockIdx.y * n;
+  const T f = (T)scal[blockIdx.y];
+  MG_PACKS(i, W, n) {
+    Pack<T, W> v = ldp<T, W>(x + o + i);
+#pragma unroll
+    for (int q = 0; q < W; ++q) v.v[q] = cscale(v.v[q], f);
+    stp<T, W>(y + o + i, v);
   }
 }
 
-// z += alpha e; r -= alpha q with alpha = <q, r> / <q, q> per rhs
-template <typename T>
-__global__ void mr_dir_kernel(C<T> *__restrict__ z, C<T> *__restrict__ res, const C<T> *__restrict__ e,
-                              const C<T> *__restrict__ q, const double2 *__restrict__ dqr,
-                              const double2 *__restrict__ nq, int64_t n) {
+// z += alpha e; r -= alpha q with alpha = <q, r> / <q, q> per rhs, alpha = 0
+// where <q, q> is not above `tiny`.  DIR: along a given direction e; else
+// along the residual itself.
+template <typename T, int W, bool DIR>
+__global__ void mr_update_kernel(C<T> *__restrict__ z, C<T> *__restrict__ res, const C<T> *__restrict__ e,
+                                 const C<T> *__restrict__ q, const double2 *__restrict__ dqr,
+                                 const double2 *__restrict__ nq, int64_t n, double tiny) {
   const int r = blockIdx.y;
   const double qq = nq[r].x;
   const double2 d = dqr[r];
-  const C<T> al = qq > 1e-280 ? mk<T>((T)(d.x / qq), (T)(d.y / qq)) : mk<T>((T)0, (T)0);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t o = r * n + i;
-    z[o] = cfma(al, e[o], z[o]);
-    res[o] = cfma(cneg(al), q[o], res[o]);
+  const C<T> al = qq > tiny ? mk<T>((T)(d.x / qq), (T)(d.y / qq)) : mk<T>((T)0, (T)0);
+  const int64_t o = r * n;
+  MG_PACKS(i, W, n) {
+    Pack<T, W> zv = ldp<T, W>(z + o + i), rv = ldp<T, W>(res + o + i);
+    const Pack<T, W> qv = ldp<T, W>(q + o + i);
+    const Pack<T, W> ev = DIR ? ldp<T, W>(e + o + i) : rv;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      zv.v[k] = cfma(al, ev.v[k], zv.v[k]);
+      rv.v[k] = cfma(cneg(al), qv.v[k], rv.v[k]);
+    }
+    stp<T, W>(z + o + i, zv);
+    stp<T, W>(res + o + i, rv);
   }
 }
 
@@ -401,44 +756,76 @@ void smem_optin(const void *func, int bytes) {
   done[key] = bytes;
 }
 
-// blocks of the first reduction stage: chunks of >= 4096 elements, at most
-// 4096 blocks, so a thread of a 256-wide block sums at most ~16 elements for
-// vectors up to 16.7 M entries (and proportionally more beyond)
+// blocks of a reduction: chunks of 1024 elements (one step of a block), at
+// most 1024 blocks, whose blocks then take several steps
 int reduce_blocks(int64_t n) {
-  int64_t b = (n + 4095) / 4096;
+  int64_t b = (n + 1023) / 1024;
   if (b < 1) b = 1;
-  if (b > 4096) b = 4096;
+  if (b > 1024) b = 1024;
   return (int)b;
 }
+
+namespace {
+// elements per block, a multiple of one step's
+int64_t reduce_chunk(int64_t n) {
+  const int64_t c = (n + reduce_blocks(n) - 1) / reduce_blocks(n);
+  return (c + 1023) / 1024 * 1024;
+}
+// blocks that have elements at that chunk
+int blocks_of(int64_t n) { return div_up(n, reduce_chunk(n)); }
+template <typename... P> bool aligned16(int64_t stride, P... p) {
+  uintptr_t a = 0;
+  ((a |= (uintptr_t)p), ...);
+  return (a & 15) == 0 && stride % 2 == 0;
+}
+
+template <typename T, int JG>
+void launch_dot(const C<T> *V, int64_t vstride, int k, const C<T> *w, int64_t n, int nrhs, double2 *h, int ldh,
+                RedScratch scr, cudaStream_t s) {
+  const dim3 grid(blocks_of(n), nrhs, (k + JG - 1) / JG);
+  const int64_t chunk = reduce_chunk(n);
+  if constexpr (sizeof(T) == 8) {
+    dot_f64_kernel<JG><<<grid, RB, 0, s>>>(V, vstride, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
+  } else if (aligned16(n | vstride, V, w)) {
+    dot_f32_kernel<JG, true><<<grid, RB, 0, s>>>(V, vstride, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
+  } else {
+    dot_f32_kernel<JG, false><<<grid, RB, 0, s>>>(V, vstride, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
+  }
+  MG_LAUNCH_CHECK();
+}
+}  // namespace
 
 template <typename T>
 void dot(const C<T> *x, const C<T> *y, int64_t n, int nrhs, double2 *out, RedScratch scr,
          cudaStream_t s) {
-  const int NB = reduce_blocks(n);
-  const int64_t chunk = (n + NB - 1) / NB;
   if (nrhs > kTickets) throw Error(1, "reduction: too many outputs for the ticket array");
-  dot_kernel<T><<<dim3(NB, nrhs, 1), RB, 0, s>>>(x, 0, y, n, chunk, scr.partial, scr.ticket, out, 1);
-  MG_LAUNCH_CHECK();
+  launch_dot<T, 1>(x, 0, 1, y, n, nrhs, out, 1, scr, s);
 }
 
 template <typename T>
 void dot_qr(const C<T> *q, const C<T> *r, int64_t n, int nrhs, double2 *out_qr, double2 *out_qq,
             RedScratch scr, cudaStream_t s) {
-  const int NB = reduce_blocks(n);
-  const int64_t chunk = (n + NB - 1) / NB;
   if (nrhs > kTickets) throw Error(1, "reduction: too many outputs for the ticket array");
-  dot_qr_kernel<T><<<dim3(NB, nrhs), RB, 0, s>>>(q, r, n, chunk, scr.partial, scr.ticket, out_qr, out_qq);
+  const dim3 grid(blocks_of(n), nrhs);
+  const int64_t chunk = reduce_chunk(n);
+  if constexpr (sizeof(T) == 8) {
+    dot_qr_f64_kernel<<<grid, RB, 0, s>>>(q, r, n, chunk, scr.partial, scr.ticket, out_qr, out_qq);
+  } else if (aligned16(n, q, r)) {
+    dot_qr_f32_kernel<true><<<grid, RB, 0, s>>>(q, r, n, chunk, scr.partial, scr.ticket, out_qr, out_qq);
+  } else {
+    dot_qr_f32_kernel<false><<<grid, RB, 0, s>>>(q, r, n, chunk, scr.partial, scr.ticket, out_qr, out_qq);
+  }
   MG_LAUNCH_CHECK();
 }
 
 template <typename T>
 void multi_dot(const C<T> *V, int64_t vstride, int k, const C<T> *w, int64_t n, int nrhs,
                double2 *h, int ldh, RedScratch scr, cudaStream_t s) {
-  const int NB = reduce_blocks(n);
-  const int64_t chunk = (n + NB - 1) / NB;
   if ((int64_t)k * nrhs > kTickets) throw Error(1, "reduction: too many outputs for the ticket array");
-  dot_kernel<T><<<dim3(NB, nrhs, k), RB, 0, s>>>(V, vstride, w, n, chunk, scr.partial, scr.ticket, h, ldh);
-  MG_LAUNCH_CHECK();
+  // vectors per block: w is read once for that many
+  if (k == 1) launch_dot<T, 1>(V, vstride, k, w, n, nrhs, h, ldh, scr, s);
+  else if (k <= 4) launch_dot<T, 4>(V, vstride, k, w, n, nrhs, h, ldh, scr, s);
+  else launch_dot<T, 8>(V, vstride, k, w, n, nrhs, h, ldh, scr, s);
 }
 
 template <typename T>
@@ -446,37 +833,57 @@ void multi_axpy(const C<T> *V, int64_t vstride, int k, C<T> *w, int64_t n, int n
                 const double2 *h, int ldh, double sign, cudaStream_t s) {
   if (k <= 0) return;
   if (k > 128) throw Error(1, "multi_axpy: k > 128");
-  const int gx = (grid_for(n) + nrhs - 1) / nrhs + 1;
-  multi_axpy_kernel<T><<<dim3(gx, nrhs), 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
+  // two elements per thread, at most 32 blocks per SM over all right-hand sides
+  const dim3 grid((unsigned)std::min<int64_t>(div_up(n, 512), std::max(1, sm_count() * 32 / nrhs)), nrhs);
+  if constexpr (sizeof(T) == 8) {
+    multi_axpy_f64_kernel<<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
+  } else if (aligned16(n | vstride, V, w)) {
+    multi_axpy_f32_kernel<true><<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
+  } else {
+    multi_axpy_f32_kernel<false><<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
+  }
   MG_LAUNCH_CHECK();
 }
 
+namespace {
+// blocks per right-hand side of an elementwise pass over n / W packs: one
+// pack per thread, at most 32 blocks per SM over all right-hand sides
+dim3 pack_grid(int64_t packs, int nrhs) {
+  return dim3((unsigned)std::min<int64_t>(div_up(packs, 256), std::max(1, sm_count() * 32 / nrhs)), nrhs);
+}
+template <typename T, typename... P> bool packs16(int64_t n, P... p) { return sizeof(T) == 4 && aligned16(n, p...); }
+}  // namespace
+
 template <typename T>
 void axpby(double a, const C<T> *x, double b, C<T> *y, int64_t n, int nrhs, cudaStream_t s) {
-  axpby_kernel<T><<<grid_for(n * nrhs), 256, 0, s>>>((T)a, x, (T)b, y, n * nrhs);
+  const int64_t tot = n * nrhs;
+  if (packs16<T>(tot, x, y)) axpby_kernel<T, 2><<<pack_grid(tot / 2, 1), 256, 0, s>>>((T)a, x, (T)b, y, tot);
+  else axpby_kernel<T, 1><<<pack_grid(tot, 1), 256, 0, s>>>((T)a, x, (T)b, y, tot);
   MG_LAUNCH_CHECK();
 }
 
 template <typename T>
 void scale_rhs(const C<T> *x, C<T> *y, const double *scal, int64_t n, int nrhs, cudaStream_t s) {
-  const int gx = (grid_for(n) + nrhs - 1) / nrhs + 1;
-  scale_rhs_kernel<T><<<dim3(gx, nrhs), 256, 0, s>>>(x, y, scal, n);
+  if (packs16<T>(n, x, y)) scale_rhs_kernel<T, 2><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(x, y, scal, n);
+  else scale_rhs_kernel<T, 1><<<pack_grid(n, nrhs), 256, 0, s>>>(x, y, scal, n);
   MG_LAUNCH_CHECK();
 }
 
 template <typename T>
 void mr_update(C<T> *z, C<T> *r, const C<T> *q, const double2 *dqr, const double2 *nq, int64_t n,
                int nrhs, cudaStream_t s) {
-  const int gx = (grid_for(n) + nrhs - 1) / nrhs + 1;
-  mr_update_kernel<T><<<dim3(gx, nrhs), 256, 0, s>>>(z, r, q, dqr, nq, n);
+  if (packs16<T>(n, z, r, q))
+    mr_update_kernel<T, 2, false><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(z, r, r, q, dqr, nq, n, 0.0);
+  else mr_update_kernel<T, 1, false><<<pack_grid(n, nrhs), 256, 0, s>>>(z, r, r, q, dqr, nq, n, 0.0);
   MG_LAUNCH_CHECK();
 }
 
 template <typename T>
 void mr_dir_update(C<T> *z, C<T> *r, const C<T> *e, const C<T> *q, const double2 *dqr,
                    const double2 *nq, int64_t n, int nrhs, cudaStream_t s) {
-  const int gx = (grid_for(n) + nrhs - 1) / nrhs + 1;
-  mr_dir_kernel<T><<<dim3(gx, nrhs), 256, 0, s>>>(z, r, e, q, dqr, nq, n);
+  if (packs16<T>(n, z, r, e, q))
+    mr_update_kernel<T, 2, true><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(z, r, e, q, dqr, nq, n, 1e-280);
+  else mr_update_kernel<T, 1, true><<<pack_grid(n, nrhs), 256, 0, s>>>(z, r, e, q, dqr, nq, n, 1e-280);
   MG_LAUNCH_CHECK();
 }
 
