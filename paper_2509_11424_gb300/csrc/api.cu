@@ -309,28 +309,26 @@ mgmlmc_status mgmlmc_apply(mgmlmc_ctx *ctx, int op_flags, int level, int precisi
     const bool fine_op = op == MGMLMC_OP_D || op == MGMLMC_OP_RESTRICT || op == MGMLMC_OP_PROLONG ||
                          op == MGMLMC_OP_PROJECT || op == MGMLMC_OP_SMOOTH || op == MGMLMC_OP_NET;
     if (!dp && level == 0 && fine_op && !internal) {
-      // FP32 level-0 vectors live structure-of-arrays inside the library:
-      // the caller's canonical buffers are reordered in and out
-      const mg::Geom &g = e.level(0).g;
-      const size_t cnt = (size_t)g.n() * nrhs;
-      const bool fin = op != MGMLMC_OP_PROLONG, fout = op != MGMLMC_OP_RESTRICT;
+      // FP32 level-0 vectors live structure-of-arrays inside the library.  The
+      // transfers read and write the caller's order as it is; D and the
+      // smoother reorder where they gain by it, the network always
       const float2 *src = (const float2 *)in;
       float2 *dst = (float2 *)out;
-      if (fin) {
-        float2 *t = e.scratch32("api_in32", cnt);
-        mg::relayout<float, float>(src, t, nullptr, g.V, nrhs, true, e.stream);
-        src = t;
-      }
-      if (fout) dst = e.scratch32("api_out32", cnt);
       switch (op) {
-        case MGMLMC_OP_D: e.apply_D<float>(0, src, dst, nrhs); break;
-        case MGMLMC_OP_RESTRICT: e.restrict_to<float>(0, src, dst, nrhs); break;
-        case MGMLMC_OP_PROLONG: e.prolong_from<float>(0, src, dst, nrhs, 0.0); break;
-        case MGMLMC_OP_PROJECT: e.project_out<float>(0, src, dst, nrhs); break;
-        case MGMLMC_OP_SMOOTH: e.smooth_apply<float>(0, src, dst, nrhs); break;
-        default: e.net_forward<float>(src, dst, nrhs); break;
+        case MGMLMC_OP_D: e.apply_D_canonical(src, dst, nrhs); break;
+        case MGMLMC_OP_RESTRICT: e.restrict_to<float>(0, src, dst, nrhs, true); break;
+        case MGMLMC_OP_PROLONG: e.prolong_from<float>(0, src, dst, nrhs, 0.0, true); break;
+        case MGMLMC_OP_PROJECT: e.project_out<float>(0, src, dst, nrhs, true); break;
+        case MGMLMC_OP_SMOOTH: e.smooth_apply<float>(0, src, dst, nrhs, true); break;
+        default: {
+          const mg::Geom &g = e.level(0).g;
+          const size_t cnt = (size_t)g.n() * nrhs;
+          float2 *x = e.scratch32("api_in32", cnt), *y = e.scratch32("api_out32", cnt);
+          mg::relayout<float, float>(src, x, nullptr, g.V, nrhs, true, e.stream);
+          e.net_forward<float>(x, y, nrhs);
+          mg::relayout<float, float>(y, dst, nullptr, g.V, nrhs, false, e.stream);
+        }
       }
-      if (fout) mg::relayout<float, float>(dst, (float2 *)out, nullptr, g.V, nrhs, false, e.stream);
       MG_CUDA(cudaGetLastError());
       return;
     }

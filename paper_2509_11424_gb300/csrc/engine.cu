@@ -307,6 +307,7 @@ template <> const C<float> *Engine::Dinv<float>(int l) const { return levels_[l]
 // ------------------------------------------------------------------ inputs
 void Engine::set_gauge(const double *U, bool on_device) {
   const size_t cnt = (size_t)fine_.V * 36;
+  levels_[0].UFe = 0;  // digits of the old links, should this call fail
   MG_CUDA(cudaMemcpyAsync(levels_[0].U64, U, cnt * sizeof(double2),
                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream));
   MG_CUDA(cudaMemsetAsync(flag_dev_, 0, sizeof(int), stream));
@@ -330,6 +331,7 @@ void Engine::get_gauge(double *U, bool on_device) {
 
 void Engine::gen_gauge(double eps, uint64_t seed) {
   if (!std::isfinite(eps)) throw Error(MGMLMC_ERR_ARG, "eps must be finite");
+  levels_[0].UFe = 0;
   gauge_generate(levels_[0].U64, (int64_t)fine_.V * 4, eps, seed, stream);
   gauge_derived();
 }
@@ -585,6 +587,27 @@ template <typename T> void Engine::apply_D(int l, const C<T> *in, C<T> *out, int
   }
 }
 
+// The caller's order in one launch where the two reordering passes around the
+// operator would cost more than its strided accesses: up to kDirectSites
+// sites times right-hand sides, once the autotuned choice for nrhs is made
+// (it stays what mgmlmc_get_kernel_variant reports), 16-byte aligned.
+void Engine::apply_D_canonical(const float2 *in, float2 *out, int nrhs) {
+  const Level &L = levels_[0];
+  const int64_t n = L.g.n();
+  const bool direct = (int64_t)L.g.V * nrhs <= kDirectSites && dslash_force_ == -2 && dslash_tuned_.count(nrhs) &&
+                      (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
+  if (direct) {
+    cudaEvent_t a = prof_begin();
+    wilson_apply_canonical(in, out, L.UD32, L.g, m0_, nrhs, stream);
+    prof_end(a, K_WILSON32, (double)L.g.V * (24.0 * nrhs + 36.0) * sizeof(float2), 1368.0 * L.g.V * nrhs);
+    return;
+  }
+  float2 *x = scratch32("api_in32", (size_t)n * nrhs), *y = scratch32("api_out32", (size_t)n * nrhs);
+  relayout<float, float>(in, x, nullptr, L.g.V, nrhs, true, stream);
+  apply_D<float>(0, x, y, nrhs);
+  relayout<float, float>(y, out, nullptr, L.g.V, nrhs, false, stream);
+}
+
 void Engine::apply_D_bf16(const void *in, void *out, int nrhs) {
   if (!have_gauge_) throw Error(MGMLMC_ERR_STATE, "no gauge field");
   const Level &L = levels_[0];
@@ -612,35 +635,36 @@ template <typename T> void Engine::coarsest_apply(const C<T> *Minv, const C<T> *
 template void Engine::coarsest_apply<float>(const float2 *, const float2 *, float2 *, int, int);
 template void Engine::coarsest_apply<double>(const double2 *, const double2 *, double2 *, int, int);
 
-template <typename T> AggMap Engine::agg_of(int l) const {
+template <typename T> AggMap Engine::agg_of(int l, bool canonical) const {
   AggMap m = levels_.at(l).agg;
-  m.soa = (sizeof(T) == 4 && l == 0) ? 1 : 0;  // FP32 fine vectors are structure-of-arrays
+  // FP32 fine vectors are structure-of-arrays inside the library
+  m.soa = (sizeof(T) == 4 && l == 0 && !canonical) ? 1 : 0;
   return m;
 }
-template <typename T> void Engine::restrict_to(int l, const C<T> *in, C<T> *out, int nrhs) {
+template <typename T> void Engine::restrict_to(int l, const C<T> *in, C<T> *out, int nrhs, bool canonical) {
   if constexpr (sizeof(T) == 4) {
     if (transfer_variant_ == 1 && levels_[l].PB16) {
-      restrict_op_bf16(in, out, levels_[l].PB16, agg_of<T>(l), nrhs, stream);
+      restrict_op_bf16(in, out, levels_[l].PB16, agg_of<T>(l, canonical), nrhs, stream);
       return;
     }
   }
-  restrict_op<T>(in, out, Pmat<T>(l), agg_of<T>(l), nrhs, stream);
+  restrict_op<T>(in, out, Pmat<T>(l), agg_of<T>(l, canonical), nrhs, stream);
 }
 template <typename T>
-void Engine::prolong_from(int l, const C<T> *in, C<T> *out, int nrhs, double beta) {
+void Engine::prolong_from(int l, const C<T> *in, C<T> *out, int nrhs, double beta, bool canonical) {
   if constexpr (sizeof(T) == 4) {
     if (transfer_variant_ == 1 && levels_[l].PB16) {
-      prolong_op_bf16(in, out, levels_[l].PB16, agg_of<T>(l), nrhs, beta, stream);
+      prolong_op_bf16(in, out, levels_[l].PB16, agg_of<T>(l, canonical), nrhs, beta, stream);
       return;
     }
   }
-  prolong_op<T>(in, out, Pmat<T>(l), agg_of<T>(l), nrhs, beta, stream);
+  prolong_op<T>(in, out, Pmat<T>(l), agg_of<T>(l, canonical), nrhs, beta, stream);
 }
-template <typename T> void Engine::project_out(int l, const C<T> *in, C<T> *out, int nrhs) {
+template <typename T> void Engine::project_out(int l, const C<T> *in, C<T> *out, int nrhs, bool canonical) {
   const int64_t n = levels_[l].g.n(), nc = levels_[l + 1].g.n();
   C<T> *xc = ws<T>("proj_c", l + 1, (size_t)nc * nrhs);
-  restrict_op<T>(in, xc, Pmat<T>(l), agg_of<T>(l), nrhs, stream);
-  prolong_op<T>(xc, out, Pmat<T>(l), agg_of<T>(l), nrhs, 0.0, stream);
+  restrict_op<T>(in, xc, Pmat<T>(l), agg_of<T>(l, canonical), nrhs, stream);
+  prolong_op<T>(xc, out, Pmat<T>(l), agg_of<T>(l, canonical), nrhs, 0.0, stream);
   axpby<T>(1.0, in, -1.0, out, n, nrhs, stream);
 }
 
@@ -719,15 +743,26 @@ template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs) {
   }
 }
 
-template <typename T> void Engine::smooth_apply(int l, const C<T> *in, C<T> *out, int nrhs) {
+template <typename T> void Engine::smooth_apply(int l, const C<T> *in, C<T> *out, int nrhs, bool canonical) {
   const int64_t n = levels_.at(l).g.n();
   C<T> *res = ws<T>("smres", l, (size_t)n * nrhs);
+  if constexpr (sizeof(T) == 4) {
+    if (canonical) {
+      // the reordering of the right-hand side makes the residual
+      C<T> *z = ws<T>("api_out32", 0, (size_t)n * nrhs);
+      relayout<float, float>(in, res, nullptr, levels_[l].g.V, nrhs, true, stream);
+      MG_CUDA(cudaMemsetAsync(z, 0, sizeof(C<T>) * n * nrhs, stream));
+      smooth<T>(l, z, res, nrhs);
+      relayout<float, float>(z, out, nullptr, levels_[l].g.V, nrhs, false, stream);
+      return;
+    }
+  }
   MG_CUDA(cudaMemcpyAsync(res, in, sizeof(C<T>) * n * nrhs, cudaMemcpyDeviceToDevice, stream));
   MG_CUDA(cudaMemsetAsync(out, 0, sizeof(C<T>) * n * nrhs, stream));
   smooth<T>(l, out, res, nrhs);
 }
-template void Engine::smooth_apply<double>(int, const C<double> *, C<double> *, int);
-template void Engine::smooth_apply<float>(int, const C<float> *, C<float> *, int);
+template void Engine::smooth_apply<double>(int, const C<double> *, C<double> *, int, bool);
+template void Engine::smooth_apply<float>(int, const C<float> *, C<float> *, int, bool);
 
 // z = M r: pre-smoothing, coarse-grid correction (recursive K-cycle: a few
 // FGMRES iterations on the next level, exact dense solve on the coarsest),
@@ -1807,12 +1842,12 @@ void Engine::get_coarse_op(int l, double *host) {
 
 template void Engine::apply_D<double>(int, const C<double> *, C<double> *, int);
 template void Engine::apply_D<float>(int, const C<float> *, C<float> *, int);
-template void Engine::restrict_to<double>(int, const C<double> *, C<double> *, int);
-template void Engine::restrict_to<float>(int, const C<float> *, C<float> *, int);
-template void Engine::prolong_from<double>(int, const C<double> *, C<double> *, int, double);
-template void Engine::prolong_from<float>(int, const C<float> *, C<float> *, int, double);
-template void Engine::project_out<double>(int, const C<double> *, C<double> *, int);
-template void Engine::project_out<float>(int, const C<float> *, C<float> *, int);
+template void Engine::restrict_to<double>(int, const C<double> *, C<double> *, int, bool);
+template void Engine::restrict_to<float>(int, const C<float> *, C<float> *, int, bool);
+template void Engine::prolong_from<double>(int, const C<double> *, C<double> *, int, double, bool);
+template void Engine::prolong_from<float>(int, const C<float> *, C<float> *, int, double, bool);
+template void Engine::project_out<double>(int, const C<double> *, C<double> *, int, bool);
+template void Engine::project_out<float>(int, const C<float> *, C<float> *, int, bool);
 
 }  // namespace mg
 

@@ -115,10 +115,14 @@ class Engine {
   template <typename T> void apply_D(int l, const C<T> *in, C<T> *out, int nrhs);
   // level-0 D on complex-bf16 vectors in the chunked internal order
   void apply_D_bf16(const void *in, void *out, int nrhs);
-  template <typename T> void restrict_to(int l, const C<T> *in, C<T> *out, int nrhs);
-  template <typename T> void prolong_from(int l, const C<T> *in, C<T> *out, int nrhs, double beta);
-  template <typename T> void project_out(int l, const C<T> *in, C<T> *out, int nrhs);
-  template <typename T> void smooth_apply(int l, const C<T> *in, C<T> *out, int nrhs);
+  // canonical: FP32 level-0 vectors in the caller's order (else internal)
+  template <typename T> void restrict_to(int l, const C<T> *in, C<T> *out, int nrhs, bool canonical = false);
+  template <typename T>
+  void prolong_from(int l, const C<T> *in, C<T> *out, int nrhs, double beta, bool canonical = false);
+  template <typename T> void project_out(int l, const C<T> *in, C<T> *out, int nrhs, bool canonical = false);
+  template <typename T> void smooth_apply(int l, const C<T> *in, C<T> *out, int nrhs, bool canonical = false);
+  // level-0 FP32 D on canonical vectors
+  void apply_D_canonical(const float2 *in, float2 *out, int nrhs);
   // z = D_l^-1 b (FP64 interface; the solver precision is set by set_solver)
   SolveInfo solve(int l, const double2 *b, double2 *x, int nrhs);
   void noise(int l, uint64_t seed, uint64_t sample0, uint64_t term, uint64_t aux, int slice,
@@ -217,7 +221,7 @@ class Engine {
   template <typename T> const C<T> *Pmat(int l) const;
   // the aggregation map of level l for vectors of type T (FP32 level-0
   // vectors are structure-of-arrays)
-  template <typename T> AggMap agg_of(int l) const;
+  template <typename T> AggMap agg_of(int l, bool canonical = false) const;
   template <typename T> const C<T> *Dinv(int l) const;
 
   template <typename T> void smooth(int l, C<T> *z, C<T> *res, int nrhs);
@@ -312,6 +316,7 @@ class Engine {
   int stencil_pick(int l, int nrhs, const float2 *in, float2 *out);
   void stencil_run(int l, int v, const float2 *in, float2 *out, int nrhs);
   int dslash_pick(int nrhs, const float2 *in, float2 *out);
+  static constexpr int64_t kDirectSites = 1 << 15;
 };
 
 }  // namespace mg

@@ -102,6 +102,9 @@ template <typename T>
 void wilson_apply(const C<T> *in, C<T> *out, const C<T> *U, const C<T> *UDs, Geom g, double m0,
                   int nrhs, int variant, cudaStream_t s);
 int wilson_fp32_variants();
+// D on FP32 vectors in the canonical order, 16-byte aligned; same sums
+void wilson_apply_canonical(const float2 *in, float2 *out, const float2 *UDs, Geom g, double m0, int nrhs,
+                            cudaStream_t s);
 // nlinks synthetic SU(3) links U = exp(i eps H) from a counter-based draw
 // (seed): Philox4x64-10 words -> Box-Muller normals A -> H = (A + A^H)/2 -
 // tr/3 -> matrix exponential; U row-major per link, canonical link order

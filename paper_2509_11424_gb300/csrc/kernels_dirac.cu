@@ -230,14 +230,15 @@ template <int I, int R> __device__ __forceinline__ int item_site(const Ctx<R> &t
   return t.g.index(cn);
 }
 
-template <int I, int R>
+// CANON: spinors in the caller's order, [site][12], six chunks per site
+template <int I, int R, bool CANON = false>
 __device__ __forceinline__ void load_item(const Ctx<R> &t, float4 (&p)[R][6], float2 (&u)[9]) {
   const int sn = item_site<I, R>(t);
 #pragma unroll
   for (int q = 0; q < R; ++q)
     if (q < t.nr) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) p[q][k] = __ldg(t.P[q] + k * t.V + sn);
+      for (int k = 0; k < 6; ++k) p[q][k] = __ldg(t.P[q] + (CANON ? (int64_t)sn * 6 + k : k * t.V + sn));
     }
   if constexpr (I > 0) {
     constexpr int mu = (I - 1) / 2;
@@ -281,12 +282,12 @@ __device__ __forceinline__ void step(Ctx<R> &t, float4 (&pc)[R][6], float2 (&uc)
 }
 // the same sets one after the other: load, consume (scheduling left to the
 // compiler, fewer registers)
-template <int I, int R> __device__ __forceinline__ void serial(Ctx<R> &t) {
+template <int I, int R, bool CANON = false> __device__ __forceinline__ void serial(Ctx<R> &t) {
   float4 p[R][6];
   float2 u[9];
-  load_item<I, R>(t, p, u);
+  load_item<I, R, CANON>(t, p, u);
   use_item<I, R>(t, p, u);
-  if constexpr (I < 8) serial<I + 1, R>(t);
+  if constexpr (I < 8) serial<I + 1, R, CANON>(t);
 }
 }  // namespace soa
 
@@ -332,6 +333,27 @@ __global__ void __launch_bounds__(BS, MINB) wilson_soa_kernel(const float2 *__re
                                      t.acc[q][2 * k + 1].y);
     }
   }
+}
+
+// D on FP32 vectors in the caller's order in one launch, for small calls:
+// same sums as the kernels above.
+__global__ void __launch_bounds__(64) wilson_canonical_kernel(const float2 *__restrict__ in,
+                                                              float2 *__restrict__ out,
+                                                              const float2 *__restrict__ UDs, Geom g, float diag) {
+  const int s = blockIdx.x * 64 + threadIdx.x;
+  if (s >= g.V) return;
+  const int64_t n = (int64_t)g.V * 12;
+  soa::Ctx<1> t;
+  t.nr = 1;
+  t.P[0] = reinterpret_cast<const float4 *>(in + blockIdx.y * n);
+  t.UDs = UDs;
+  t.g = g;
+  t.V = g.V;
+  t.s = s;
+  t.diag = diag;
+  g.coords(s, t.c);
+  soa::serial<0, 1, true>(t);
+  store_spinor<float>(out + blockIdx.y * n + (int64_t)s * 12, t.acc[0]);
 }
 
 // The right-hand sides of a group in the warps of one CTA: warp w of a CTA
@@ -464,6 +486,28 @@ __global__ void relayout_bf16_kernel(const __nv_bfloat162 *__restrict__ x, __nv_
     const int64_t is = ((int64_t)(i >> 2) * V + s) * 4 + (i & 3);
     if (to_soa) yr[is] = xr[e];
     else yr[e] = xr[is];
+  }
+}
+
+// The same for buffers aligned to 16 bytes: whole 16-byte chunks (three per
+// site) through shared memory, 256 sites per block.
+__global__ void __launch_bounds__(256) relayout_bf16_chunk_kernel(const uint4 *__restrict__ x, uint4 *__restrict__ y,
+                                                                  int64_t V, bool to_soa) {
+  __shared__ uint4 sh[3][257];
+  const int64_t s0 = (int64_t)blockIdx.x * 256;
+  const int ns = (int)(V - s0 < 256 ? V - s0 : 256);
+  x += blockIdx.y * 3 * V;
+  y += blockIdx.y * 3 * V;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int p = q * 256 + threadIdx.x, site = to_soa ? p / 3 : (int)threadIdx.x, k = to_soa ? p - site * 3 : q;
+    if (site < ns) sh[k][site] = __ldg(x + (to_soa ? s0 * 3 + p : k * V + s0 + site));
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int p = q * 256 + threadIdx.x, site = to_soa ? (int)threadIdx.x : p / 3, k = to_soa ? q : p - site * 3;
+    if (site < ns) y[to_soa ? k * V + s0 + site : s0 * 3 + p] = sh[k][site];
   }
 }
 
@@ -674,6 +718,12 @@ void launch_soa(const float2 *in, float2 *out, const float2 *UDs, Geom g, float 
 
 int wilson_fp32_variants() { return 7; }
 
+void wilson_apply_canonical(const float2 *in, float2 *out, const float2 *UDs, Geom g, double m0, int nrhs,
+                            cudaStream_t s) {
+  wilson_canonical_kernel<<<dim3(div_up(g.V, 64), nrhs), 64, 0, s>>>(in, out, UDs, g, (float)(4.0 + m0));
+  MG_LAUNCH_CHECK();
+}
+
 template <typename T>
 void wilson_apply(const C<T> *in, C<T> *out, const C<T> *U, const C<T> *UDs, Geom g, double m0,
                   int nrhs, int variant, cudaStream_t s) {
@@ -717,6 +767,12 @@ void link_bf16(const float2 *U, void *Ub, int V, cudaStream_t s) {
 }
 
 void relayout_bf16(const void *x, void *y, int64_t V, int nrhs, bool to_soa, cudaStream_t s) {
+  if ((((uintptr_t)x | (uintptr_t)y) & 15) == 0) {
+    relayout_bf16_chunk_kernel<<<dim3(div_up(V, 256), nrhs), 256, 0, s>>>(static_cast<const uint4 *>(x),
+                                                                          static_cast<uint4 *>(y), V, to_soa);
+    MG_LAUNCH_CHECK();
+    return;
+  }
   const int gx = (grid_for(V * 12) + nrhs - 1) / nrhs + 1;
   relayout_bf16_kernel<<<dim3(gx, nrhs), 256, 0, s>>>(static_cast<const __nv_bfloat162 *>(x),
                                                       static_cast<__nv_bfloat162 *>(y), V, to_soa);
