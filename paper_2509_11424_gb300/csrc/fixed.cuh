@@ -82,6 +82,75 @@ __device__ __forceinline__ long long madw(int a, int b, long long c) {
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
   return r;
 }
+
+// 2^e as a double, also outside the normal range
+__device__ __forceinline__ double scaled(double v, int e) {
+  return e > -1000 && e < 1000 ? v * __longlong_as_double((long long)(e + 1023) << 52) : scalbn(v, e);
+}
+
+// ---- exact sums over a warp.  Every lane calls add() for value 0, 1, ... in
+// turn; get() then gives lane v the sum of value v.
+//
+// FP32 lanes: integers of 51 bits in the unit of the largest lane's exponent,
+// as two words whose 32-fold sums fit 32 bits.
+struct WarpSumF {
+  unsigned lo = 0;
+  int hi = 0, e = 0;
+  __device__ __forceinline__ void add(int v, float p) {
+    const unsigned b = __float_as_uint(p);
+    int x = (b >> 23) & 0xff;
+    const int E = __reduce_max_sync(0xffffffffu, x);
+    const unsigned m = (b & 0x7fffffu) | (x ? 0x800000u : 0u);
+    x = x ? x : 1;
+    const int s = min(max(E, 1) - x, 60);
+    long long X = (long long)(((unsigned long long)m << 27) >> s);
+    X = (int)b < 0 ? -X : X;
+    const unsigned l = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
+    const int h = __reduce_add_sync(0xffffffffu, (int)(X >> 26));
+    if ((int)(threadIdx.x & 31) == v) {
+      lo = l;
+      hi = h;
+      e = E;
+    }
+  }
+  __device__ __forceinline__ double get() const {
+    const double d = scaled((double)(((long long)hi << 26) + lo), max(e, 1) - (127 + 23 + 27));
+    return e == 0xff ? __longlong_as_double(0x7ff8000000000000ll) : d;
+  }
+};
+// 64-bit integers in units of 2^unit (the same in every lane): three words
+struct WarpSumI {
+  unsigned w0 = 0, w1 = 0;
+  int w2 = 0, e = 0;
+  __device__ __forceinline__ void add(int v, long long X, int unit, bool bad) {
+    const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
+    const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(X >> 26) & 0x3ffffffu);
+    const int c = __reduce_add_sync(0xffffffffu, (int)(X >> 52));
+    if ((int)(threadIdx.x & 31) == v) {
+      w0 = a;
+      w1 = b;
+      w2 = c;
+      e = bad ? 1 << 20 : unit;
+    }
+  }
+  __device__ __forceinline__ double get() const {
+    const double d = fma((double)w2, 0x1p52, (double)(((long long)w1 << 26) + w0));
+    return e == 1 << 20 ? __longlong_as_double(0x7ff8000000000000ll) : scaled(d, e);
+  }
+};
+
+__device__ __forceinline__ int warp_exp(int e) { return max(__reduce_max_sync(0xffffffffu, e), 1); }
+// the sum over a warp's lanes of FP64 values, value v to lane v
+struct WarpSumD : WarpSumI {
+  __device__ __forceinline__ void add(int v, double p) {
+    const int E = max(__reduce_max_sync(0xffffffffu, exp_field(p)), 1);
+    WarpSumI::add(v, to_fixed(p, min(E, kBadExp - 1)), E - 1022 - kVecBits, E == kBadExp);
+  }
+};
+__device__ __forceinline__ int4 digits(double2 v, int E) {
+  const long long a = to_fixed(v.x, E), b = to_fixed(v.y, E);
+  return make_int4(digit_hi(a), digit_lo(a), digit_hi(b), digit_lo(b));
+}
 #endif
 
 }  // namespace fx

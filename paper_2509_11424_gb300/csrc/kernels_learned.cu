@@ -10,6 +10,7 @@
 // structure-of-arrays links, FP64 canonical [site][12]); weights
 // [h][o][c][4][4].  The adjoint uses that
 // the adjoint of hop h is the reversed hop and the adjoint of W is W^H.
+#include "fixed.cuh"
 #include "kernels.h"
 
 namespace mg {
@@ -69,8 +70,11 @@ __device__ __forceinline__ void transported(const C<T> *__restrict__ psi, const 
 // transported input T_h psi[c] is formed once for the whole group;
 // blockIdx.x = (site range, sample) with the sample fastest, so the blocks
 // of one site range run together and read its links from L2 after the
-// first; blockIdx.y = output group
-template <typename T, int OG>
+// first; blockIdx.y = output group.
+// ADJ: the adjoint layer, out[c] = sum_o sum_h W[h][o][c]^H T_rev(h) gin[o]:
+// the same sums with the weights W'[rev(h)][c][o] = W[h][o][c]^H, which the
+// staging makes (Cin, Cout: channels read and written).
+template <typename T, int OG, bool ADJ>
 __global__ void __launch_bounds__(128) glayer_forward_kernel(const C<T> *__restrict__ in,
                                                              C<T> *__restrict__ out,
                                                              const C<T> *__restrict__ W,
@@ -83,7 +87,13 @@ __global__ void __launch_bounds__(128) glayer_forward_kernel(const C<T> *__restr
   for (int e = threadIdx.x; e < 9 * Cin * OG * 16; e += blockDim.x) {
     const int h = e / (Cin * OG * 16), rem = e - h * Cin * OG * 16;
     const int c = rem / (OG * 16), rem2 = rem - c * OG * 16, k = rem2 / 16, q = rem2 % 16;
-    Ws[e] = k < og ? W[(((int64_t)h * Cout + o0 + k) * Cin + c) * 16 + q] : mk<T>((T)0, (T)0);
+    C<T> w = mk<T>((T)0, (T)0);
+    if (k < og && !ADJ) w = W[(((int64_t)h * Cout + o0 + k) * Cin + c) * 16 + q];
+    if (k < og && ADJ) {
+      const int hr = h == 0 ? 0 : ((h & 1) ? h + 1 : h - 1);
+      w = cconj(W[(((int64_t)hr * Cin + c) * Cout + o0 + k) * 16 + (q & 3) * 4 + (q >> 2)]);
+    }
+    Ws[e] = w;
   }
   __syncthreads();
   const int s = (int)(blockIdx.x / (unsigned)nb) * blockDim.x + threadIdx.x;
@@ -123,75 +133,31 @@ __global__ void __launch_bounds__(128) glayer_forward_kernel(const C<T> *__restr
   }
 }
 
-// adjoint: out[c](x) = sum_o sum_h W[h][o][c]^H (T_rev(h) gin[o])(x)
-template <typename T>
-__global__ void __launch_bounds__(128) glayer_adjoint_kernel(const C<T> *__restrict__ gin,
-                                                             C<T> *__restrict__ out,
-                                                             const C<T> *__restrict__ W,
-                                                             const C<T> *__restrict__ U, Geom g,
-                                                             int Cin, int Cout, int nb) {
-  extern __shared__ unsigned char smem_raw[];
-  C<T> *Ws = reinterpret_cast<C<T> *>(smem_raw);  // [h][o][16] for this c
-  // blockIdx.x = (site range, sample), the sample fastest (as the forward)
-  const int c = blockIdx.y, b = (int)(blockIdx.x % (unsigned)nb);
-  for (int e = threadIdx.x; e < 9 * Cout * 16; e += blockDim.x) {
-    const int h = e / (Cout * 16), rem = e - h * Cout * 16, o = rem / 16, k = rem % 16;
-    Ws[e] = W[(((int64_t)h * Cout + o) * Cin + c) * 16 + k];
-  }
-  __syncthreads();
-  const int s = (int)(blockIdx.x / (unsigned)nb) * blockDim.x + threadIdx.x;
-  if (s >= g.V) return;
-  const int64_t n = g.n();
-  int cc[4];
-  g.coords(s, cc);
-  C<T> acc[12];
-#pragma unroll
-  for (int i = 0; i < 12; ++i) acc[i] = mk<T>((T)0, (T)0);
-  for (int o = 0; o < Cout; ++o) {
-    const C<T> *gp = gin + ((int64_t)b * Cout + o) * n;
-    for (int h = 0; h < 9; ++h) {
-      const int hr = h == 0 ? 0 : ((h & 1) ? h + 1 : h - 1);
-      C<T> t[12];
-      transported<T>(gp, U, g, s, cc, hr, t);
-      const C<T> *w = Ws + (h * Cout + o) * 16;
-#pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int sq = 0; sq < 4; ++sq) {
-          const C<T> wv = w[sq * 4 + sp];  // (W^H)[sp][sq] = conj(W[sq][sp])
-#pragma unroll
-          for (int a = 0; a < 3; ++a) acc[sp * 3 + a] = cfmac(wv, t[sq * 3 + a], acc[sp * 3 + a]);
-        }
-    }
-  }
-  C<T> *o_ = out + ((int64_t)b * Cin + c) * n;
-#pragma unroll
-  for (int i = 0; i < 12; ++i) o_[fidx<kSoa<T>>(s, i, g.V)] = acc[i];
-}
+// weight-gradient partials: block (chunk, c * 9 + h, output pair) sums over its
+// sites and all samples g[o](x) (T_h psi[c])(x)^H (16 spin entries, colour
+// summed) for OG outputs, the transported input formed once for them.  Bound:
+// FP64 pipe (FP64) / FMAs; the chunks are short so that a small lattice fills
+// the GPU (4096 sites in one block took 2.2 ms whatever the layer), and the
+// sums over a warp are integer ones (fixed.cuh).
+constexpr int kWgradThreads = 128;
+// sites per block; longer on large lattices, whose partials would outgrow use
+inline int wgrad_chunk(const Geom &g) { return g.V <= (1 << 18) ? 512 : 4096; }
 
-__device__ __forceinline__ double2 warp_sum2(double2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-    v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-  }
-  return v;
-}
-
-// weight-gradient partials: block (chunk, c*9 + h, o) sums over its sites
-// and all samples g[o](x) (T_h psi[c])(x)^H (16 spin entries, colour summed)
-template <typename T>
-__global__ void __launch_bounds__(256) glayer_wgrad_kernel(const C<T> *__restrict__ gin,
+template <typename T, int OG>
+__global__ void __launch_bounds__(kWgradThreads) glayer_wgrad_kernel(const C<T> *__restrict__ gin,
                                                            const C<T> *__restrict__ in,
                                                            const C<T> *__restrict__ U, Geom g,
                                                            int Cin, int Cout, int B, int chunk,
                                                            double2 *__restrict__ partial) {
-  __shared__ double2 sh[16][8];
-  const int ch = blockIdx.y / 9, h = blockIdx.y % 9, o = blockIdx.z;
+  constexpr int NW = kWgradThreads / 32;
+  __shared__ double sh[OG][32][NW];
+  const int ch = blockIdx.y / 9, h = blockIdx.y % 9, o0 = blockIdx.z * OG;
   const int64_t n = g.n();
-  C<T> acc[16];
+  C<T> acc[OG][16];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) acc[k] = mk<T>((T)0, (T)0);
+  for (int q = 0; q < OG; ++q)
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc[q][k] = mk<T>((T)0, (T)0);
   const int beg = blockIdx.x * chunk, end = min(g.V, beg + chunk);
   for (int s = beg + threadIdx.x; s < end; s += blockDim.x) {
     int cc[4];
@@ -199,34 +165,51 @@ __global__ void __launch_bounds__(256) glayer_wgrad_kernel(const C<T> *__restric
     for (int b = 0; b < B; ++b) {
       C<T> t[12];
       transported<T>(in + ((int64_t)b * Cin + ch) * n, U, g, s, cc, h, t);
-      const C<T> *gp = gin + ((int64_t)b * Cout + o) * n;
-      C<T> gv[12];
 #pragma unroll
-      for (int i = 0; i < 12; ++i) gv[i] = gp[fidx<kSoa<T>>(s, i, g.V)];
+      for (int q = 0; q < OG; ++q) {
+        if (o0 + q >= Cout) break;
+        const C<T> *gp = gin + ((int64_t)b * Cout + o0 + q) * n;
+        C<T> gv[12];
+        load_fine_site<T>(gp, s, g.V, gv);
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
+        for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
-        for (int sq = 0; sq < 4; ++sq)
+          for (int sq = 0; sq < 4; ++sq)
 #pragma unroll
-          for (int a = 0; a < 3; ++a)
-            acc[sp * 4 + sq] = cfmac(t[sq * 3 + a], gv[sp * 3 + a], acc[sp * 4 + sq]);  // g conj(t)
+            for (int a = 0; a < 3; ++a)
+              acc[q][sp * 4 + sq] = cfmac(t[sq * 3 + a], gv[sp * 3 + a], acc[q][sp * 4 + sq]);  // g conj(t)
+      }
     }
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    double2 v = warp_sum2(make_double2((double)acc[k].x, (double)acc[k].y));
-    if (l == 0) sh[k][w] = v;
+  for (int q = 0; q < OG; ++q) {
+    if constexpr (sizeof(T) == 4) {
+      fx::WarpSumF ws;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        ws.add(2 * k, acc[q][k].x);
+        ws.add(2 * k + 1, acc[q][k].y);
+      }
+      sh[q][l][w] = ws.get();
+    } else {
+      fx::WarpSumD ws;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        ws.add(2 * k, acc[q][k].x);
+        ws.add(2 * k + 1, acc[q][k].y);
+      }
+      sh[q][l][w] = ws.get();
+    }
   }
   __syncthreads();
-  if (threadIdx.x < 16) {
-    double2 t = make_double2(0.0, 0.0);
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-      t.x += sh[threadIdx.x][i].x;
-      t.y += sh[threadIdx.x][i].y;
-    }
+  for (int e = threadIdx.x; e < OG * 32; e += blockDim.x) {
+    const int q = e >> 5, v = e & 31;
+    if (o0 + q >= Cout) continue;
+    double t = 0.0;
+    for (int i = 0; i < NW; ++i) t += sh[q][v][i];
     // layout [chunk][h][o][c][16]
-    partial[((((int64_t)blockIdx.x * 9 + h) * Cout + o) * Cin + ch) * 16 + threadIdx.x] = t;
+    reinterpret_cast<double *>(partial)[((((int64_t)blockIdx.x * 9 + h) * Cout + o0 + q) * Cin + ch) * 32 + v] = t;
   }
 }
 
@@ -270,46 +253,53 @@ __global__ void adam_kernel(double2 *__restrict__ W, const double2 *__restrict__
 
 }  // namespace
 
-template <typename T, int OG>
-static void glayer_forward_og(const C<T> *in, C<T> *out, const C<T> *W, const C<T> *U, Geom g, int Cin,
-                              int Cout, int B, cudaStream_t s) {
+template <typename T, int OG, bool ADJ>
+static void glayer_og(const C<T> *in, C<T> *out, const C<T> *W, const C<T> *U, Geom g, int Cin, int Cout, int B,
+                      cudaStream_t s) {
   const size_t sm = (size_t)9 * Cin * OG * 16 * sizeof(C<T>);
-  smem_optin((const void *)glayer_forward_kernel<T, OG>, 160 * 1024);
-  glayer_forward_kernel<T, OG><<<dim3((unsigned)div_up(g.V, 128) * (unsigned)B, div_up(Cout, OG), 1), 128, sm,
-                                 s>>>(in, out, W, U, g, Cin, Cout, B);
+  smem_optin((const void *)glayer_forward_kernel<T, OG, ADJ>, 160 * 1024);
+  glayer_forward_kernel<T, OG, ADJ>
+      <<<dim3((unsigned)div_up(g.V, 128) * (unsigned)B, div_up(Cout, OG), 1), 128, sm, s>>>(in, out, W, U, g, Cin,
+                                                                                          Cout, B);
   MG_LAUNCH_CHECK();
+}
+
+template <typename T, bool ADJ>
+static void glayer(const C<T> *in, C<T> *out, const C<T> *W, const C<T> *U, Geom g, int Cin, int Cout, int B,
+                   cudaStream_t s) {
+  // four output channels share a transported input; their weights stay within
+  // the shared memory (32 input channels in FP64: two)
+  if (Cout == 1) glayer_og<T, 1, ADJ>(in, out, W, U, g, Cin, Cout, B, s);
+  else if (Cout == 2 || (size_t)9 * Cin * 64 * sizeof(C<T>) > 160 * 1024)
+    glayer_og<T, 2, ADJ>(in, out, W, U, g, Cin, Cout, B, s);
+  else glayer_og<T, 4, ADJ>(in, out, W, U, g, Cin, Cout, B, s);
 }
 
 template <typename T>
 void glayer_forward(const C<T> *in, C<T> *out, const C<T> *W, const C<T> *U, Geom g, int Cin,
                     int Cout, int B, cudaStream_t s) {
-  if (Cout == 1) glayer_forward_og<T, 1>(in, out, W, U, g, Cin, Cout, B, s);
-  else if (Cout == 2) glayer_forward_og<T, 2>(in, out, W, U, g, Cin, Cout, B, s);
-  else glayer_forward_og<T, 4>(in, out, W, U, g, Cin, Cout, B, s);
+  glayer<T, false>(in, out, W, U, g, Cin, Cout, B, s);
 }
 
 template <typename T>
 void glayer_adjoint(const C<T> *gin, C<T> *out, const C<T> *W, const C<T> *U, Geom g, int Cin,
                     int Cout, int B, cudaStream_t s) {
-  const size_t sm = (size_t)9 * Cout * 16 * sizeof(C<T>);
-  smem_optin((const void *)glayer_adjoint_kernel<T>, 100 * 1024);
-  glayer_adjoint_kernel<T><<<dim3((unsigned)div_up(g.V, 128) * (unsigned)B, Cin, 1), 128, sm, s>>>(gin, out, W, U,
-                                                                                                  g, Cin, Cout, B);
-  MG_LAUNCH_CHECK();
+  glayer<T, true>(gin, out, W, U, g, Cout, Cin, B, s);
 }
 
-int glayer_wgrad_chunks(const Geom &g) {
-  const int chunk = 4096;
-  return div_up(g.V, chunk);
-}
+int glayer_wgrad_chunks(const Geom &g) { return div_up(g.V, wgrad_chunk(g)); }
 
 template <typename T>
 void glayer_wgrad(const C<T> *gin, const C<T> *in, const C<T> *U, Geom g, int Cin, int Cout, int B,
                   double2 *partial, double2 *out, cudaStream_t s) {
-  const int chunk = 4096;
-  const int nchunks = div_up(g.V, chunk);
-  glayer_wgrad_kernel<T><<<dim3(nchunks, Cin * 9, Cout), 256, 0, s>>>(gin, in, U, g, Cin, Cout, B, chunk,
-                                                                        partial);
+  const int nchunks = glayer_wgrad_chunks(g);
+  if (Cout == 1)
+    glayer_wgrad_kernel<T, 1><<<dim3(nchunks, Cin * 9, 1), kWgradThreads, 0, s>>>(gin, in, U, g, Cin, Cout, B,
+                                                                                 wgrad_chunk(g), partial);
+  else
+    glayer_wgrad_kernel<T, 2><<<dim3(nchunks, Cin * 9, div_up(Cout, 2)), kWgradThreads, 0, s>>>(gin, in, U, g, Cin,
+                                                                                               Cout, B, wgrad_chunk(g),
+                                                                                               partial);
   MG_LAUNCH_CHECK();
   const int64_t count = (int64_t)9 * Cout * Cin * 16;
   wgrad_sum_kernel<<<grid_for(count), 256, 0, s>>>(partial, nchunks, count, out);
