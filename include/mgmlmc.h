@@ -584,13 +584,12 @@ mgmlmc_status mgmlmc_profile_stats(mgmlmc_ctx *ctx, int kernel_class, int64_t *l
  * correction decides convergence with the true residual either way. */
 #define MGMLMC_VARIANT_STENCIL_FP32 1
 /* The FP32 SAP sweep on the fine level (the smoother of Sec. 4's
- * DD-alpha-AMG solver).  With two or more right-hand sides and blocks of
- * 8 x 4 x 4 x 2 or 4^4 sites, one block and two right-hand sides per thread
- * block: 0 (default) = one thread per site and right-hand side, the block's
- * links and the solution it updates staged in shared memory by asynchronous
- * copies that overlap the residual load; 1 = one thread per site carrying
- * both right-hand sides in packed FP32 pairs (.f32x2 instructions).  Other
- * cases, and 2 = throughout, the general kernels.  Every variant updates the
+ * DD-alpha-AMG solver).  With blocks of 8 x 4 x 4 x 2 or 4^4 sites: 0
+ * (default) = one block and right-hand side per thread block, one thread per
+ * site, the block's links staged in shared memory by asynchronous copies that
+ * overlap the residual load; 1 = with two or more right-hand sides, one
+ * thread per site carrying two of them in packed FP32 pairs (.f32x2
+ * instructions).  Other cases, and 2 = throughout, the general kernels.  Every variant updates the
  * faces of each colour in a separate pass over that colour's sites, and all
  * compute the same sums in the same order: identical results. */
 #define MGMLMC_VARIANT_SAP_FP32 2

@@ -680,10 +680,16 @@ void Engine::noise(int l, uint64_t seed, uint64_t sample0, uint64_t term, uint64
 // (MGMLMC_SMOOTHER_SAP), followed for MGMLMC_SMOOTHER_LEARNED by one learned
 // step z += alpha N(res) with the residual-minimising alpha (so the step can
 // only lower ||res||); other levels / MR: minimal-residual steps.
-template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs) {
+template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs, const C<T> *r0) {
   const int64_t n = levels_[l].g.n();
   const bool learned = l == 0 && sp_.smoother == MGMLMC_SMOOTHER_LEARNED;
-  if (l == 0 && sp_.smoother == MGMLMC_SMOOTHER_NET) {
+  const int n_steps = l == 0 ? sp_.smoother_steps : sp_.coarse_smoother_steps;
+  const bool net = l == 0 && sp_.smoother == MGMLMC_SMOOTHER_NET;
+  if (r0 && (net || n_steps == 0)) {
+    MG_CUDA(cudaMemcpyAsync(res, r0, sizeof(C<T>) * n * nrhs, cudaMemcpyDeviceToDevice, stream));
+    MG_CUDA(cudaMemsetAsync(z, 0, sizeof(C<T>) * n * nrhs, stream));
+  }
+  if (net) {
     // the network in place of SAP: smoother_steps residual-minimising steps
     // z += alpha N(res), res -= alpha D N(res)
     if (!net_.C) throw Error(MGMLMC_ERR_STATE, "network smoother selected but the network is not initialised");
@@ -714,7 +720,7 @@ template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs) {
     const double flops = (double)g.V * nrhs * (1368.0 * sp_.sap_iters + 684.0);
     for (int s = 0; s < sp_.smoother_steps; ++s) {
       cudaEvent_t a = prof_begin();
-      sap_sweep<T>(res, z, e, U, g, sap_b_, m0_, sp_.sap_iters, nrhs, stream, sap_variant_);
+      sap_sweep<T>(res, z, e, U, g, sap_b_, m0_, sp_.sap_iters, nrhs, stream, sap_variant_, s == 0 ? r0 : nullptr);
       prof_end(a, sizeof(T) == 8 ? K_SAP64 : K_SAP32, bytes, flops);
     }
     // training pairs: the residuals the learned step will see -- after SAP,
@@ -735,11 +741,11 @@ template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs) {
   }
   C<T> *q = ws<T>("smq", l, (size_t)n * nrhs);
   double2 *d = ws<double>("smd", l, 2 * (size_t)nrhs);
-  const int steps = l == 0 ? sp_.smoother_steps : sp_.coarse_smoother_steps;
-  for (int s = 0; s < steps; ++s) {
-    apply_D<T>(l, res, q, nrhs);
-    dot_qr<T>(q, res, n, nrhs, d, d + nrhs, partials((size_t)reduce_blocks(n) * nrhs * 2), stream);
-    mr_update<T>(z, res, q, d, d + nrhs, n, nrhs, stream);
+  for (int s = 0; s < n_steps; ++s) {
+    const C<T> *first = s == 0 ? r0 : nullptr, *x = first ? first : res;
+    apply_D<T>(l, x, q, nrhs);
+    dot_qr<T>(q, x, n, nrhs, d, d + nrhs, partials((size_t)reduce_blocks(n) * nrhs * 2), stream);
+    mr_update<T>(z, res, q, d, d + nrhs, n, nrhs, stream, first);
   }
 }
 
@@ -748,18 +754,14 @@ template <typename T> void Engine::smooth_apply(int l, const C<T> *in, C<T> *out
   C<T> *res = ws<T>("smres", l, (size_t)n * nrhs);
   if constexpr (sizeof(T) == 4) {
     if (canonical) {
-      // the reordering of the right-hand side makes the residual
-      C<T> *z = ws<T>("api_out32", 0, (size_t)n * nrhs);
-      relayout<float, float>(in, res, nullptr, levels_[l].g.V, nrhs, true, stream);
-      MG_CUDA(cudaMemsetAsync(z, 0, sizeof(C<T>) * n * nrhs, stream));
-      smooth<T>(l, z, res, nrhs);
+      C<T> *x = ws<T>("api_in32", 0, (size_t)n * nrhs), *z = ws<T>("api_out32", 0, (size_t)n * nrhs);
+      relayout<float, float>(in, x, nullptr, levels_[l].g.V, nrhs, true, stream);
+      smooth<T>(l, z, res, nrhs, x);
       relayout<float, float>(z, out, nullptr, levels_[l].g.V, nrhs, false, stream);
       return;
     }
   }
-  MG_CUDA(cudaMemcpyAsync(res, in, sizeof(C<T>) * n * nrhs, cudaMemcpyDeviceToDevice, stream));
-  MG_CUDA(cudaMemsetAsync(out, 0, sizeof(C<T>) * n * nrhs, stream));
-  smooth<T>(l, out, res, nrhs);
+  smooth<T>(l, out, res, nrhs, in);
 }
 template void Engine::smooth_apply<double>(int, const C<double> *, C<double> *, int, bool);
 template void Engine::smooth_apply<float>(int, const C<float> *, C<float> *, int, bool);
@@ -782,17 +784,18 @@ template <typename T> void Engine::precond(int l, const C<T> *r, C<T> *z, int nr
     return;
   }
   const int64_t nc = levels_[l + 1].g.n();
+  const int n_steps = l == 0 ? sp_.smoother_steps : sp_.coarse_smoother_steps;
   C<T> *res = ws<T>("mgres", l, (size_t)n * nrhs);
   // q = D z of the post-smoothing residual shares the smoothers' work vector
   // (dead whenever the smoother runs)
   C<T> *q = ws<T>("smq", l, (size_t)n * nrhs);
   C<T> *rc = ws<T>("mgrc", l + 1, (size_t)nc * nrhs);
   C<T> *ec = ws<T>("mgec", l + 1, (size_t)nc * nrhs);
-  MG_CUDA(cudaMemsetAsync(z, 0, sizeof(C<T>) * n * nrhs, stream));
-  MG_CUDA(cudaMemcpyAsync(res, r, sizeof(C<T>) * n * nrhs, cudaMemcpyDeviceToDevice, stream));
-  if (!(sp_.post_smoothing_only && l == 0)) smooth<T>(l, z, res, nrhs);
+  // without pre-smoothing the residual is r itself and z = 0 is never stored
+  const bool pre = !(sp_.post_smoothing_only && l == 0) && n_steps > 0;
+  if (pre) smooth<T>(l, z, res, nrhs, r);
   cudaEvent_t pr = prof_begin();
-  restrict_to<T>(l, res, rc, nrhs);
+  restrict_to<T>(l, pre ? res : r, rc, nrhs);
   prof_end(pr, K_TRANSFER, 0.0, 0.0);
   if (l + 1 == n_levels() - 1) {
     cudaEvent_t pd = prof_begin();
@@ -802,12 +805,11 @@ template <typename T> void Engine::precond(int l, const C<T> *r, C<T> *z, int nr
     fgmres<T>(l + 1, rc, ec, nrhs, 0.0, sp_.coarse_iters, sp_.coarse_iters, true, true);
   }
   cudaEvent_t pp = prof_begin();
-  prolong_from<T>(l, ec, z, nrhs, 1.0);
+  prolong_from<T>(l, ec, z, nrhs, pre ? 1.0 : 0.0);
   prof_end(pp, K_TRANSFER, 0.0, 0.0);
-  if ((l == 0 ? sp_.smoother_steps : sp_.coarse_smoother_steps) > 0) {
+  if (n_steps > 0) {
     apply_D<T>(l, z, q, nrhs);
-    MG_CUDA(cudaMemcpyAsync(res, r, sizeof(C<T>) * n * nrhs, cudaMemcpyDeviceToDevice, stream));
-    axpby<T>(-1.0, q, 1.0, res, n, nrhs, stream);
+    subtract<T>(r, q, res, n * nrhs, stream);
     post_smooth_ = true;
     smooth<T>(l, z, res, nrhs);
     post_smooth_ = false;
@@ -957,8 +959,7 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
     if (fixed && total >= max_iter) break;
     // true residual (V_1 as the work vector: the cycle's basis is spent)
     apply_D<T>(l, x, V + vs, nrhs);
-    MG_CUDA(cudaMemcpyAsync(V, b, sizeof(C<T>) * vs, cudaMemcpyDeviceToDevice, stream));
-    axpby<T>(-1.0, V + vs, 1.0, V, n, nrhs, stream);
+    subtract<T>(b, V + vs, V, vs, stream);
     if (fixed) continue;
     dot<T>(V, V, n, nrhs, st.nrm, part(1), stream);
     double2 *h = static_cast<double2 *>(pinned(sizeof(double2) * nrhs));

@@ -224,7 +224,9 @@ class Engine {
   template <typename T> AggMap agg_of(int l, bool canonical = false) const;
   template <typename T> const C<T> *Dinv(int l) const;
 
-  template <typename T> void smooth(int l, C<T> *z, C<T> *res, int nrhs);
+  // r0: the smoothing starts from z = 0 with the residual r0 (left as it is;
+  // z and res hold nothing yet)
+  template <typename T> void smooth(int l, C<T> *z, C<T> *res, int nrhs, const C<T> *r0 = nullptr);
   template <typename T> void precond(int l, const C<T> *r, C<T> *z, int nrhs);
   // out = Minv in for the dense coarsest-level inverse (n x n, row-major) and
   // nrhs vectors of n: one complex GEMM in cuBLAS (FP32 or FP64 arithmetic,

@@ -33,6 +33,9 @@ void multi_dot(const C<T> *V, int64_t vstride, int k, const C<T> *w, int64_t n, 
 template <typename T>
 void multi_axpy(const C<T> *V, int64_t vstride, int k, C<T> *w, int64_t n, int nrhs,
                 const double2 *h, int ldh, double sign, cudaStream_t s);
+// d = a - b
+template <typename T>
+void subtract(const C<T> *a, const C<T> *b, C<T> *d, int64_t n, cudaStream_t s);
 // y = a x + b y   (host scalars, all rhs)
 template <typename T>
 void axpby(double a, const C<T> *x, double b, C<T> *y, int64_t n, int nrhs, cudaStream_t s);
@@ -40,10 +43,11 @@ void axpby(double a, const C<T> *x, double b, C<T> *y, int64_t n, int nrhs, cuda
 template <typename T>
 void scale_rhs(const C<T> *x, C<T> *y, const double *scal, int64_t n, int nrhs, cudaStream_t s);
 // minimal-residual step for every rhs: alpha = <q, r> / <q, q>;
-// z += alpha r; r -= alpha q.  dots[r] = <q, r>, nq[r].x = <q, q>
+// z += alpha r; r -= alpha q.  dots[r] = <q, r>, nq[r].x = <q, q>.  r0: the
+// first step from z = 0, z = alpha r0; r = r0 - alpha q (neither z nor r read)
 template <typename T>
 void mr_update(C<T> *z, C<T> *r, const C<T> *q, const double2 *dqr, const double2 *nq,
-               int64_t n, int nrhs, cudaStream_t s);
+               int64_t n, int nrhs, cudaStream_t s, const C<T> *r0 = nullptr);
 // minimal-residual step along a given direction e with q = D e:
 // alpha = <q, r> / <q, q>; z += alpha e; r -= alpha q
 template <typename T>
@@ -195,11 +199,13 @@ template <typename T> size_t sap_smem_bytes(const int b[4], int rs);
 // FP32: structure-of-arrays vectors and links (UDs), FP64: canonical.
 // variant 0: the staged FP32 block kernels where they apply (two or more
 // right-hand sides, blocks 8 x 4 x 4 x 2 or 4^4), 1: the paired ones there,
-// 2: the general kernels throughout; all give identical results
+// 2: the general kernels throughout; all give identical results.  r0: the
+// residual of z = 0, read in r's place and left as it is, z being written
+// without a read (no copy of r0 and no clearing of z before the first sweep)
 int sap_variants();
 template <typename T>
 void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4], double m0,
-               int block_iters, int nrhs, cudaStream_t s, int variant = 0);
+               int block_iters, int nrhs, cudaStream_t s, int variant = 0, const C<T> *r0 = nullptr);
 
 // ------------------------------------------------------------------ learned smoother
 // gauge-covariant layer phi[o] = sum_c sum_h W[h][o][c] T_h psi[c]; activations

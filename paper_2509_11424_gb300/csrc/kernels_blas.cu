@@ -479,10 +479,23 @@ __global__ void scale_rhs_kernel(const C<T> *x, C<T> *y,  // may alias (in-place
   }
 }
 
+template <typename T, int W>
+__global__ void subtract_kernel(const C<T> *__restrict__ a, const C<T> *__restrict__ b, C<T> *__restrict__ d, int64_t n) {
+  MG_PACKS(i, W, n) {
+    Pack<T, W> v = ldp<T, W>(a + i);
+    const Pack<T, W> w = ldp<T, W>(b + i);
+#pragma unroll
+    for (int q = 0; q < W; ++q) v.v[q] = csub(v.v[q], w.v[q]);
+    stp<T, W>(d + i, v);
+  }
+}
+
 // z += alpha e; r -= alpha q with alpha = <q, r> / <q, q> per rhs, alpha = 0
-// where <q, q> is not above `tiny`.  DIR: along a given direction e; else
-// along the residual itself.
-template <typename T, int W, bool DIR>
+// where <q, q> is not above `tiny`.  MR_RES: along the residual itself;
+// MR_DIR: along a given direction e; MR_FIRST: along the residual e of z = 0,
+// neither z nor r holding anything yet.
+enum MrMode { MR_RES, MR_DIR, MR_FIRST };
+template <typename T, int W, MrMode MODE>
 __global__ void mr_update_kernel(C<T> *__restrict__ z, C<T> *__restrict__ res, const C<T> *__restrict__ e,
                                  const C<T> *__restrict__ q, const double2 *__restrict__ dqr,
                                  const double2 *__restrict__ nq, int64_t n, double tiny) {
@@ -492,12 +505,13 @@ __global__ void mr_update_kernel(C<T> *__restrict__ z, C<T> *__restrict__ res, c
   const C<T> al = qq > tiny ? mk<T>((T)(d.x / qq), (T)(d.y / qq)) : mk<T>((T)0, (T)0);
   const int64_t o = r * n;
   MG_PACKS(i, W, n) {
-    Pack<T, W> zv = ldp<T, W>(z + o + i), rv = ldp<T, W>(res + o + i);
+    Pack<T, W> zv, rv = ldp<T, W>((MODE == MR_FIRST ? e : res) + o + i);
     const Pack<T, W> qv = ldp<T, W>(q + o + i);
-    const Pack<T, W> ev = DIR ? ldp<T, W>(e + o + i) : rv;
+    const Pack<T, W> ev = MODE == MR_DIR ? ldp<T, W>(e + o + i) : rv;
+    if (MODE != MR_FIRST) zv = ldp<T, W>(z + o + i);
 #pragma unroll
     for (int k = 0; k < W; ++k) {
-      zv.v[k] = cfma(al, ev.v[k], zv.v[k]);
+      zv.v[k] = cfma(al, ev.v[k], MODE == MR_FIRST ? mk<T>((T)0, (T)0) : zv.v[k]);
       rv.v[k] = cfma(cneg(al), qv.v[k], rv.v[k]);
     }
     stp<T, W>(z + o + i, zv);
@@ -842,6 +856,13 @@ void axpby(double a, const C<T> *x, double b, C<T> *y, int64_t n, int nrhs, cuda
 }
 
 template <typename T>
+void subtract(const C<T> *a, const C<T> *b, C<T> *d, int64_t n, cudaStream_t s) {
+  if (packs16<T>(n, a, b, d)) subtract_kernel<T, 2><<<pack_grid(n / 2, 1), 256, 0, s>>>(a, b, d, n);
+  else subtract_kernel<T, 1><<<pack_grid(n, 1), 256, 0, s>>>(a, b, d, n);
+  MG_LAUNCH_CHECK();
+}
+
+template <typename T>
 void scale_rhs(const C<T> *x, C<T> *y, const double *scal, int64_t n, int nrhs, cudaStream_t s) {
   if (packs16<T>(n, x, y)) scale_rhs_kernel<T, 2><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(x, y, scal, n);
   else scale_rhs_kernel<T, 1><<<pack_grid(n, nrhs), 256, 0, s>>>(x, y, scal, n);
@@ -850,10 +871,16 @@ void scale_rhs(const C<T> *x, C<T> *y, const double *scal, int64_t n, int nrhs, 
 
 template <typename T>
 void mr_update(C<T> *z, C<T> *r, const C<T> *q, const double2 *dqr, const double2 *nq, int64_t n,
-               int nrhs, cudaStream_t s) {
-  if (packs16<T>(n, z, r, q))
-    mr_update_kernel<T, 2, false><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(z, r, r, q, dqr, nq, n, 0.0);
-  else mr_update_kernel<T, 1, false><<<pack_grid(n, nrhs), 256, 0, s>>>(z, r, r, q, dqr, nq, n, 0.0);
+               int nrhs, cudaStream_t s, const C<T> *r0) {
+  if (r0) {
+    if (packs16<T>(n, z, r, q, r0))
+      mr_update_kernel<T, 2, MR_FIRST><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(z, r, r0, q, dqr, nq, n, 0.0);
+    else mr_update_kernel<T, 1, MR_FIRST><<<pack_grid(n, nrhs), 256, 0, s>>>(z, r, r0, q, dqr, nq, n, 0.0);
+  } else if (packs16<T>(n, z, r, q)) {
+    mr_update_kernel<T, 2, MR_RES><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(z, r, nullptr, q, dqr, nq, n, 0.0);
+  } else {
+    mr_update_kernel<T, 1, MR_RES><<<pack_grid(n, nrhs), 256, 0, s>>>(z, r, nullptr, q, dqr, nq, n, 0.0);
+  }
   MG_LAUNCH_CHECK();
 }
 
@@ -861,8 +888,8 @@ template <typename T>
 void mr_dir_update(C<T> *z, C<T> *r, const C<T> *e, const C<T> *q, const double2 *dqr,
                    const double2 *nq, int64_t n, int nrhs, cudaStream_t s) {
   if (packs16<T>(n, z, r, e, q))
-    mr_update_kernel<T, 2, true><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(z, r, e, q, dqr, nq, n, 1e-280);
-  else mr_update_kernel<T, 1, true><<<pack_grid(n, nrhs), 256, 0, s>>>(z, r, e, q, dqr, nq, n, 1e-280);
+    mr_update_kernel<T, 2, MR_DIR><<<pack_grid(n / 2, nrhs), 256, 0, s>>>(z, r, e, q, dqr, nq, n, 1e-280);
+  else mr_update_kernel<T, 1, MR_DIR><<<pack_grid(n, nrhs), 256, 0, s>>>(z, r, e, q, dqr, nq, n, 1e-280);
   MG_LAUNCH_CHECK();
 }
 
@@ -924,7 +951,8 @@ void gmres_solve(GmresState st, cudaStream_t s) {
   template void axpby<T>(double, const C<T> *, double, C<T> *, int64_t, int, cudaStream_t);      \
   template void scale_rhs<T>(const C<T> *, C<T> *, const double *, int64_t, int, cudaStream_t);  \
   template void mr_update<T>(C<T> *, C<T> *, const C<T> *, const double2 *, const double2 *,     \
-                             int64_t, int, cudaStream_t);                                        \
+                             int64_t, int, cudaStream_t, const C<T> *);                          \
+  template void subtract<T>(const C<T> *, const C<T> *, C<T> *, int64_t, cudaStream_t);           \
   template void check_finite<T>(const C<T> *, int64_t, int *, cudaStream_t);               \
   template void dot_qr<T>(const C<T> *, const C<T> *, int64_t, int, double2 *, double2 *,        \
                           RedScratch, cudaStream_t);                                           \

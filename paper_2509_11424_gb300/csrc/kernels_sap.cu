@@ -16,16 +16,15 @@
 // sites, black blocks, face pass on the red sites (four launches per sweep).
 //
 // Three block kernels, for FP32 blocks of 256 sites with every extent >= 2
-// (8 x 4 x 4 x 2 and 4^4) and two or more right-hand sides: the staged one
-// (the default) gives each thread one (site, right-hand side), the block's
-// links and the z it updates arriving in shared memory by asynchronous
-// copies that overlap the residual load; the paired one gives each thread
-// one site and two right-hand sides held in the two lanes of packed
-// registers (.f32x2 arithmetic: one instruction and one link read from
-// shared memory serve both; fewer instructions, but its 197 KB of shared
-// memory leaves 8 warps per SM).  The general one below serves FP64, other
-// block shapes and single right-hand sides.  All compute the same sums in
-// the same order.
+// (8 x 4 x 4 x 2 and 4^4): the staged one (the default) takes one block and
+// right-hand side per CTA, two CTAs per SM, the links arriving in shared
+// memory by asynchronous copies that overlap the residual load; the paired
+// one (two or more right-hand sides) gives each thread one site and two
+// right-hand sides held in the two lanes of packed registers (.f32x2
+// arithmetic: one instruction and one link read from shared memory serve
+// both; fewer instructions, but its 197 KB of shared memory leaves 8 warps
+// per SM).  The general one below serves FP64 and other block shapes.  All
+// compute the same sums in the same order.
 //
 // One CTA per (active block, rhs), one thread per site of the block; the
 // right-hand side varies fastest over the grid, so the CTAs of a block share
@@ -50,6 +49,20 @@ __device__ __forceinline__ void link_at(const C<T> *__restrict__ U, int64_t V, i
 #pragma unroll
   for (int k = 0; k < 9; ++k)
     u[k] = kSoa<T> ? U[(int64_t)(mu * 9 + k) * V + site] : U[(site * 4 + mu) * 9 + k];
+}
+
+// z += e at one site, or z = e where z still is zero (`zero`: not even set)
+template <typename T>
+__device__ __forceinline__ void add_to_z(C<T> *z, int64_t s, int64_t V, const C<T> (&e)[12], bool zero) {
+  if (zero) {
+    store_fine_site<T>(z, s, V, e);
+    return;
+  }
+  C<T> zz[12];
+  load_fine_site<T>(z, s, V, zz);
+#pragma unroll
+  for (int i = 0; i < 12; ++i) zz[i] = cadd(zz[i], e[i]);
+  store_fine_site<T>(z, s, V, zz);
 }
 
 struct SapGeom {
@@ -325,40 +338,40 @@ __device__ __forceinline__ void staged_hops(const float4 *rho, const float2 *Us,
   }
 }
 
-// Staged FP32 block kernel: one CTA per (active block, pair of right-hand
-// sides), one thread per (site, right-hand side).  Shared memory: links
-// [36][S] float2, residuals [2][6][S] float4, the z being updated [2][6][S]
-// float4, reduction partials (172 KB at S = 256).  The links (shared by both
-// slots) and z are asynchronous copies issued before the residual load and
-// the face terms, awaited before the first block iteration; the MR iterations
-// and every sum follow sap_block_kernel exactly (bit-identical results).
+// Staged FP32 block kernel: one CTA per (active block, right-hand side), one
+// thread per site.  Shared memory: links [36][S] float2, residual [6][S]
+// float4, reduction partials (98 KB at S = 256).  The links are asynchronous
+// copies issued before the residual load and awaited before the first block
+// iteration; the MR iterations and every sum follow sap_block_kernel exactly
+// (bit-identical results).
+//
+// Bound: shared memory (42 wavefronts per hop of a warp) and issue slots while
+// it iterates, memory while it loads and stores.  Two CTAs per SM do one
+// while the other does the other: a sweep of 32^4 sites and 4 right-hand
+// sides takes 1.20 ms, against 1.40 ms with both right-hand sides of a pair
+// in one CTA (links read once for both, z staged; one CTA per SM, so its
+// phases followed one another: issue 50%, shared memory 53%, DRAM 33%).
 template <int B0, int B1, int B2, int B3>
-__global__ void __launch_bounds__(2 * B0 * B1 * B2 * B3, 1)
-    sap_block_staged_kernel(float2 *__restrict__ r, float2 *__restrict__ z, float2 *e_out,
+__global__ void __launch_bounds__(B0 * B1 * B2 * B3, 2)
+    sap_block_staged_kernel(const float2 *rin, float2 *r, float2 *__restrict__ z, float2 *e_out,
                             const float2 *__restrict__ U, SapGeom sg, float diag, int color, int iters,
-                            int nrhs) {
+                            int nrhs, bool zero) {
   using SH = SapShape<B0, B1, B2, B3>;
   constexpr int S = SH::S, NW = S / 32;
   static_assert(S % 32 == 0 && B0 % 2 == 0 && B1 >= 2 && B2 >= 2 && B3 >= 2, "staged SAP block shape");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2 *Us = reinterpret_cast<float2 *>(smem_raw);
-  float4 *vbase = reinterpret_cast<float4 *>(Us + 36 * S);
-  const int slot = (int)threadIdx.x / S;
-  const int ls = (int)threadIdx.x - slot * S;
-  float4 *rho = vbase + slot * 6 * S;
-  float4 *zs = vbase + (2 + slot) * 6 * S;
-  float *red = reinterpret_cast<float *>(vbase + 4 * 6 * S) + slot * 3 * NW;
+  float4 *rho = reinterpret_cast<float4 *>(Us + 36 * S);
+  float *red = reinterpret_cast<float *>(rho + 6 * S);
+  const int ls = (int)threadIdx.x;
   const Geom &g = sg.g;
   const int64_t n = g.n(), V = g.V;
-  const int ngr = (nrhs + 1) >> 1;
-  const int rq = (int)(blockIdx.x % (unsigned)ngr) * 2 + slot;
-  const bool live = rq < nrhs;  // a slot past the last right-hand side computes on zeros
-  const int rr = live ? rq : nrhs - 1;
+  const int rr = (int)(blockIdx.x % (unsigned)nrhs);
   float2 *rv = r + rr * n;
   float2 *zv = z + rr * n;
   float2 *ev = e_out + rr * n;
   int bc[4];
-  active_block(sg, (int)(blockIdx.x / (unsigned)ngr), color, bc);
+  active_block(sg, (int)(blockIdx.x / (unsigned)nrhs), color, bc);
   const int lc[4] = {ls % B0, (ls / B0) % B1, (ls / (B0 * B1)) % B2, ls / (B0 * B1 * B2)};
   int gc[4];
 #pragma unroll
@@ -366,32 +379,21 @@ __global__ void __launch_bounds__(2 * B0 * B1 * B2 * B3, 1)
   const int s = g.index(gc);
   {
     // links: 16-byte copies of site pairs (x rows hold an even number of
-    // sites starting at an even x), 9 per thread at S = 256
+    // sites starting at an even x), 18 per thread
     int oc[4] = {bc[0] * B0, bc[1] * B1, bc[2] * B2, bc[3] * B3};
     const int64_t s0 = g.index(oc);
-    static_assert((18 * S) % (2 * S) == 0, "link chunks per thread");
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      const int j = q * 2 * S + (int)threadIdx.x;
+    for (int q = 0; q < 18; ++q) {
+      const int j = q * S + ls;
       const int comp = j / (S / 2), l0 = 2 * (j - comp * (S / 2));
       const int lx = l0 % B0, ly = (l0 / B0) % B1, lz = (l0 / (B0 * B1)) % B2, lt = l0 / (B0 * B1 * B2);
       const int64_t gs = s0 + lx + (int64_t)g.L[0] * (ly + g.L[1] * (lz + (int64_t)g.L[2] * lt));
       cp_async16(Us + comp * S + l0, U + (int64_t)comp * V + gs);
     }
-    if (live) {
-      const float4 *zc = reinterpret_cast<const float4 *>(zv);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) cp_async16(zs + k * S + ls, zc + (int64_t)k * V + s);
-    }
     cp_async_commit();
   }
   float2 rh[12];
-  if (live) {
-    load_fine_site<float>(rv, s, V, rh);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 12; ++i) rh[i] = make_float2(0.f, 0.f);
-  }
+  load_fine_site<float>(rin + rr * n, s, V, rh);
 #pragma unroll
   for (int k = 0; k < 6; ++k)
     rho[k * S + ls] = make_float4(rh[2 * k].x, rh[2 * k].y, rh[2 * k + 1].x, rh[2 * k + 1].y);
@@ -449,16 +451,9 @@ __global__ void __launch_bounds__(2 * B0 * B1 * B2 * B3, 1)
       rho[k * S + ls] = make_float4(rh[2 * k].x, rh[2 * k].y, rh[2 * k + 1].x, rh[2 * k + 1].y);
     __syncthreads();
   }
-  if (!live) return;
-  {
-    float2 zz[12];
-    chunk_site<S>(zs, ls, zz);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) zz[i] = cadd(zz[i], e[i]);
-    store_fine_site<float>(zv, s, V, zz);
-  }
   store_fine_site<float>(ev, s, V, e);
   store_fine_site<float>(rv, s, V, rh);
+  add_to_z<float>(zv, s, V, e, zero);
 }
 
 // ---- paired FP32 arithmetic (P2 and the p2* helpers of common.cuh): the
@@ -598,9 +593,9 @@ __device__ __forceinline__ void pair_hops(const ulonglong2 *rho, const ulonglong
 // partials (197 KB at S = 256).  Same sums as sap_block_kernel.
 template <int B0, int B1, int B2, int B3>
 __global__ void __launch_bounds__(B0 * B1 * B2 * B3, 1)
-    sap_block_pair_kernel(float2 *__restrict__ r, float2 *__restrict__ z, float2 *e_out,
+    sap_block_pair_kernel(const float2 *rin, float2 *r, float2 *__restrict__ z, float2 *e_out,
                           const float2 *__restrict__ U, SapGeom sg, float diag, int color, int iters,
-                          int nrhs) {
+                          int nrhs, bool zero) {
   using SH = SapShape<B0, B1, B2, B3>;
   constexpr int S = SH::S, NW = S / 32;
   static_assert(S % 32 == 0 && B0 >= 2 && B1 >= 2 && B2 >= 2 && B3 >= 2, "paired SAP block shape");
@@ -628,9 +623,9 @@ __global__ void __launch_bounds__(B0 * B1 * B2 * B3, 1)
     Us[k * S + ls] = make_ulonglong2(p2(u.x, u.x).v, p2(u.y, u.y).v);
   }
   float2 rh0[12], rh1[12];
-  load_fine_site<float>(r + r0 * n, s, V, rh0);
+  load_fine_site<float>(rin + r0 * n, s, V, rh0);
   if (live1) {
-    load_fine_site<float>(r + (r0 + 1) * n, s, V, rh1);
+    load_fine_site<float>(rin + (r0 + 1) * n, s, V, rh1);
   } else {
 #pragma unroll
     for (int i = 0; i < 12; ++i) rh1[i] = make_float2(0.f, 0.f);
@@ -714,21 +709,11 @@ __global__ void __launch_bounds__(B0 * B1 * B2 * B3, 1)
     rh0[i] = make_float2(rr_.x, ri.x);
     rh1[i] = make_float2(rr_.y, ri.y);
   }
-  {
-    float2 zz[12];
-    load_fine_site<float>(z + r0 * n, s, V, zz);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) zz[i] = cadd(zz[i], e0[i]);
-    store_fine_site<float>(z + r0 * n, s, V, zz);
-    store_fine_site<float>(e_out + r0 * n, s, V, e0);
-    store_fine_site<float>(r + r0 * n, s, V, rh0);
-  }
+  add_to_z<float>(z + r0 * n, s, V, e0, zero);
+  store_fine_site<float>(e_out + r0 * n, s, V, e0);
+  store_fine_site<float>(r + r0 * n, s, V, rh0);
   if (live1) {
-    float2 zz[12];
-    load_fine_site<float>(z + (r0 + 1) * n, s, V, zz);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) zz[i] = cadd(zz[i], e1[i]);
-    store_fine_site<float>(z + (r0 + 1) * n, s, V, zz);
+    add_to_z<float>(z + (r0 + 1) * n, s, V, e1, zero);
     store_fine_site<float>(e_out + (r0 + 1) * n, s, V, e1);
     store_fine_site<float>(r + (r0 + 1) * n, s, V, rh1);
   }
@@ -744,8 +729,8 @@ __global__ void __launch_bounds__(B0 * B1 * B2 * B3, 1)
 // (123 KB); FP64 (196 KB) fits one, so it takes the whole register file.
 template <typename T, int RS>
 __global__ void __launch_bounds__(256 * RS, (sizeof(T) == 4 && RS == 1) ? 2 : 1)
-    sap_block_kernel(C<T> *__restrict__ r, C<T> *__restrict__ z, C<T> *e_out, const C<T> *__restrict__ U,
-                     SapGeom sg, T diag, int color, int iters, int nrhs) {
+    sap_block_kernel(const C<T> *rin, C<T> *r, C<T> *__restrict__ z, C<T> *e_out, const C<T> *__restrict__ U,
+                     SapGeom sg, T diag, int color, int iters, int nrhs, bool zero) {
   extern __shared__ unsigned char smem_raw[];
   const int sites = sg.sites;
   const int slot = RS == 1 ? 0 : (int)threadIdx.x / sites;
@@ -784,7 +769,7 @@ __global__ void __launch_bounds__(256 * RS, (sizeof(T) == 4 && RS == 1) ? 2 : 1)
   C<T> rh[12];  // this site's residual, kept in registers (its slot in rho is for the neighbours)
   {
     if (live) {
-      load_fine_site<T>(rv, s, V, rh);
+      load_fine_site<T>(rin + rr * n, s, V, rh);
     } else {
 #pragma unroll
       for (int i = 0; i < 12; ++i) rh[i] = mk<T>((T)0, (T)0);
@@ -827,13 +812,7 @@ __global__ void __launch_bounds__(256 * RS, (sizeof(T) == 4 && RS == 1) ? 2 : 1)
     __syncthreads();
   }
   if (!live) return;
-  {
-    C<T> zz[12];
-    load_fine_site<T>(zv, s, V, zz);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) zz[i] = cadd(zz[i], e[i]);
-    store_fine_site<T>(zv, s, V, zz);
-  }
+  add_to_z<T>(zv, s, V, e, zero);
   store_fine_site<T>(ev, s, V, e);
   store_fine_site<T>(rv, s, V, rh);
 }
@@ -843,7 +822,7 @@ __global__ void __launch_bounds__(256 * RS, (sizeof(T) == 4 && RS == 1) ? 2 : 1)
 // one load set per direction where the block extent allows it; the same sum
 // as sap_boundary_kernel.  Right-hand side fastest over the grid.
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) sap_face_kernel(C<T> *__restrict__ r, const C<T> *__restrict__ e,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) sap_face_kernel(const C<T> *rin, C<T> *r, const C<T> *__restrict__ e,
                                                        const C<T> *__restrict__ U, SapGeom sg, int color,
                                                        int nrhs) {
   const int rr = (int)(blockIdx.x % (unsigned)nrhs);
@@ -875,28 +854,29 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) sap_face_kernel(C
   cross_dir<2, T>(ev, U, sg, s, c, lc[2], acc, (T)1);
   cross_dir<3, T>(ev, U, sg, s, c, lc[3], acc, (T)1);
   C<T> res[12];
-  load_fine_site<T>(rv, s, sg.g.V, res);
+  load_fine_site<T>(rin + rr * n, s, sg.g.V, res);
 #pragma unroll
   for (int i = 0; i < 12; ++i) res[i] = csub(res[i], acc[i]);
   store_fine_site<T>(rv, s, sg.g.V, res);
 }
 
 template <int B0, int B1, int B2, int B3>
-void launch_pair(float2 *r, float2 *z, float2 *e, const float2 *U, const SapGeom &sg, float diag, int color,
-                 int iters, int nrhs, unsigned grid, cudaStream_t st) {
+void launch_pair(const float2 *rin, float2 *r, float2 *z, float2 *e, const float2 *U, const SapGeom &sg, float diag,
+                 int color, int iters, int nrhs, bool zero, unsigned grid, cudaStream_t st) {
   constexpr int S = B0 * B1 * B2 * B3;
   const int sm = 48 * S * 16 + 6 * (S / 32) * 4;
   smem_optin((const void *)sap_block_pair_kernel<B0, B1, B2, B3>, sm);
-  sap_block_pair_kernel<B0, B1, B2, B3><<<grid, S, sm, st>>>(r, z, e, U, sg, diag, color, iters, nrhs);
+  sap_block_pair_kernel<B0, B1, B2, B3><<<grid, S, sm, st>>>(rin, r, z, e, U, sg, diag, color, iters, nrhs, zero);
 }
 
 template <int B0, int B1, int B2, int B3>
-void launch_staged(float2 *r, float2 *z, float2 *e, const float2 *U, const SapGeom &sg, float diag, int color,
-                   int iters, int nrhs, unsigned grid, cudaStream_t st) {
+void launch_staged(const float2 *rin, float2 *r, float2 *z, float2 *e, const float2 *U, const SapGeom &sg, float diag,
+                   int color, int iters, int nrhs, bool zero, unsigned blocks, cudaStream_t st) {
   constexpr int S = B0 * B1 * B2 * B3;
-  const int sm = 36 * S * 8 + 4 * 6 * S * 16 + 2 * 3 * (S / 32) * 4;
+  const int sm = 36 * S * 8 + 6 * S * 16 + 3 * (S / 32) * 4;
   smem_optin((const void *)sap_block_staged_kernel<B0, B1, B2, B3>, sm);
-  sap_block_staged_kernel<B0, B1, B2, B3><<<grid, 2 * S, sm, st>>>(r, z, e, U, sg, diag, color, iters, nrhs);
+  sap_block_staged_kernel<B0, B1, B2, B3>
+      <<<blocks * (unsigned)nrhs, S, sm, st>>>(rin, r, z, e, U, sg, diag, color, iters, nrhs, zero);
 }
 
 }  // namespace
@@ -921,7 +901,8 @@ size_t sap_smem_bytes(const int b[4], int rs) {
 
 template <typename T>
 void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4], double m0,
-               int block_iters, int nrhs, cudaStream_t s, int variant) {
+               int block_iters, int nrhs, cudaStream_t s, int variant, const C<T> *r0) {
+  const bool zero = r0 != nullptr;
   SapGeom sg;
   sg.g = g;
   sg.sites = 1;
@@ -941,45 +922,51 @@ void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4],
   const unsigned grid = (unsigned)(nblocks / 2) * (unsigned)((nrhs + rs - 1) / rs);
   const float dg = (float)(4.0 + m0);
   bool b8 = false, b4 = false;
+  const unsigned half = (unsigned)(nblocks / 2);
   if constexpr (sizeof(T) == 4) {
-    b8 = two && b[0] == 8 && b[1] == 4 && b[2] == 4 && b[3] == 2;
-    b4 = two && b[0] == 4 && b[1] == 4 && b[2] == 4 && b[3] == 4;
+    // the staged kernel's copies and its 16-byte chunks want aligned vectors
+    b8 = b[0] == 8 && b[1] == 4 && b[2] == 4 && b[3] == 2;
+    b4 = b[0] == 4 && b[1] == 4 && b[2] == 4 && b[3] == 4;
   }
   // red blocks; the black sites take the red corrections across their
   // faces; black blocks; the red sites take the black corrections (r exact
   // again).  The face updates run over one colour's sites at a time in their
   // own kernel, where many resident warps hide the latency of the gathers.
+  // The first pass over each colour reads r0 where it is given: the red blocks
+  // and the face pass on the black sites.
   for (int color = 0; color < 2; ++color) {
+    const C<T> *rin = r0 && color == 0 ? r0 : r;
     if (color == 1) {
-      sap_face_kernel<T><<<(unsigned)div_up(g.V / 2, 256) * (unsigned)nrhs, 256, 0, s>>>(r, e, U, sg, 1, nrhs);
+      sap_face_kernel<T><<<(unsigned)div_up(g.V / 2, 256) * (unsigned)nrhs, 256, 0, s>>>(r0 ? r0 : r, r, e, U, sg, 1,
+                                                                                        nrhs);
       MG_LAUNCH_CHECK();
     }
     if constexpr (sizeof(T) == 4) {
-      if (variant == 0 && b8) launch_staged<8, 4, 4, 2>(r, z, e, U, sg, dg, color, block_iters, nrhs, grid, s);
-      else if (variant == 0 && b4) launch_staged<4, 4, 4, 4>(r, z, e, U, sg, dg, color, block_iters, nrhs, grid, s);
-      else if (variant == 1 && b8) launch_pair<8, 4, 4, 2>(r, z, e, U, sg, dg, color, block_iters, nrhs, grid, s);
-      else if (variant == 1 && b4) launch_pair<4, 4, 4, 4>(r, z, e, U, sg, dg, color, block_iters, nrhs, grid, s);
+      if (variant == 0 && b8) launch_staged<8, 4, 4, 2>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, half, s);
+      else if (variant == 0 && b4) launch_staged<4, 4, 4, 4>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, half, s);
+      else if (variant == 1 && two && b8) launch_pair<8, 4, 4, 2>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, grid, s);
+      else if (variant == 1 && two && b4) launch_pair<4, 4, 4, 4>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, grid, s);
       else if (two) {
         smem_optin((const void *)sap_block_kernel<T, 2>, (int)sm);
-        sap_block_kernel<T, 2><<<grid, 2 * sg.sites, sm, s>>>(r, z, e, U, sg, (T)dg, color, block_iters, nrhs);
+        sap_block_kernel<T, 2><<<grid, 2 * sg.sites, sm, s>>>(rin, r, z, e, U, sg, (T)dg, color, block_iters, nrhs, zero);
       } else {
         smem_optin((const void *)sap_block_kernel<T, 1>, (int)sm);
-        sap_block_kernel<T, 1><<<grid, sg.sites, sm, s>>>(r, z, e, U, sg, (T)dg, color, block_iters, nrhs);
+        sap_block_kernel<T, 1><<<grid, sg.sites, sm, s>>>(rin, r, z, e, U, sg, (T)dg, color, block_iters, nrhs, zero);
       }
     } else {
       smem_optin((const void *)sap_block_kernel<T, 1>, (int)sm);
-      sap_block_kernel<T, 1><<<grid, sg.sites, sm, s>>>(r, z, e, U, sg, (T)(4.0 + m0), color, block_iters, nrhs);
+      sap_block_kernel<T, 1><<<grid, sg.sites, sm, s>>>(rin, r, z, e, U, sg, (T)(4.0 + m0), color, block_iters, nrhs, zero);
     }
     MG_LAUNCH_CHECK();
   }
-  sap_face_kernel<T><<<(unsigned)div_up(g.V / 2, 256) * (unsigned)nrhs, 256, 0, s>>>(r, e, U, sg, 0, nrhs);
+  sap_face_kernel<T><<<(unsigned)div_up(g.V / 2, 256) * (unsigned)nrhs, 256, 0, s>>>(r, r, e, U, sg, 0, nrhs);
   MG_LAUNCH_CHECK();
 }
 
 template void sap_sweep<double>(C<double> *, C<double> *, C<double> *, const C<double> *, Geom,
-                                const int *, double, int, int, cudaStream_t, int);
+                                const int *, double, int, int, cudaStream_t, int, const C<double> *);
 template void sap_sweep<float>(C<float> *, C<float> *, C<float> *, const C<float> *, Geom,
-                               const int *, double, int, int, cudaStream_t, int);
+                               const int *, double, int, int, cudaStream_t, int, const C<float> *);
 template size_t sap_smem_bytes<double>(const int *, int);
 template size_t sap_smem_bytes<float>(const int *, int);
 
