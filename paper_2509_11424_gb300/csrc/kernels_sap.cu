@@ -456,6 +456,122 @@ __global__ void __launch_bounds__(B0 * B1 * B2 * B3, 2)
   add_to_z<float>(zv, s, V, e, zero);
 }
 
+// FP32 blocks of 2^4 sites: one half warp per (active block, right-hand side),
+// everything in registers.  A site has one hop inside the block per direction,
+// to the lane that differs in that bit, through the link of the pair's lower
+// site: the lower site uses U and sg = -1, the upper one U^H and sg = +1, so
+// each lane keeps the matrix it needs (four per site, for all iterations) and
+// the hops are the same code for both.  The neighbour's half-spinor comes by
+// shuffles, and so do the block sums (butterflies: every lane has them).
+// Bound: latency on the lattices that have such blocks; one 16-thread CTA per
+// block took 16 us per colour at 12^3 x 20.
+template <int MU>
+__device__ __forceinline__ void pair_hop(const float2 (&rh)[12], const float2 (&m)[9], float sg, float2 (&q)[12]) {
+  // what the partner needs of this site: u + sg' B l with the partner's sign
+  float2 h[2][3];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float2 t = cadd(rh[3 * a + c], cscale(sBl<MU>(a, rh[6 + c], rh[9 + c]), -sg));
+      h[a][c].x = __shfl_xor_sync(0xffffffffu, t.x, 1 << MU);
+      h[a][c].y = __shfl_xor_sync(0xffffffffu, t.y, 1 << MU);
+    }
+  float2 v[2][3];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int b = 0; b < 3; ++b) z = cfma(m[3 * c + b], h[a][b], z);
+      v[a][c] = z;
+    }
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      q[3 * a + c].x = fmaf(-0.5f, v[a][c].x, q[3 * a + c].x);
+      q[3 * a + c].y = fmaf(-0.5f, v[a][c].y, q[3 * a + c].y);
+      const float2 w = sBh<MU>(a, v[0][c], v[1][c]);
+      q[6 + 3 * a + c].x = fmaf(-0.5f * sg, w.x, q[6 + 3 * a + c].x);
+      q[6 + 3 * a + c].y = fmaf(-0.5f * sg, w.y, q[6 + 3 * a + c].y);
+    }
+}
+
+__global__ void __launch_bounds__(128, 2)
+    sap_small_kernel(const float2 *rin, float2 *r, float2 *__restrict__ z, float2 *e_out,
+                     const float2 *__restrict__ U, SapGeom sg, float diag, int color, int iters, int nrhs,
+                     bool zero) {
+  const int64_t id = ((int64_t)blockIdx.x * 128 + threadIdx.x) >> 4;  // (block, right-hand side), the latter fastest
+  const int ls = threadIdx.x & 15;
+  const bool live = id < (int64_t)(sg.g.V / 32) * nrhs;  // a half warp past the end computes on the last block
+  const int64_t it_ = live ? id : (int64_t)(sg.g.V / 32) * nrhs - 1;
+  const int rr = (int)(it_ % nrhs);
+  int bc[4];
+  active_block(sg, (int)(it_ / nrhs), color, bc);
+  const Geom &g = sg.g;
+  const int64_t V = g.V, n = g.n();
+  int gc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) gc[i] = 2 * bc[i] + ((ls >> i) & 1);
+  const int s = g.index(gc);
+  const int st[4] = {1, g.L[0], g.L[0] * g.L[1], g.L[0] * g.L[1] * g.L[2]};
+  float2 rh[12], m[4][9];
+  load_fine_site<float>(rin + rr * n, s, V, rh);
+  float sgn[4];
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const bool up = (ls >> mu) & 1;
+    sgn[mu] = up ? 1.f : -1.f;
+    const float2 *u = U + (int64_t)mu * 9 * V + (up ? s - st[mu] : s);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const float2 t = __ldg(u + (int64_t)(up ? 3 * b + a : 3 * a + b) * V);
+        m[mu][3 * a + b] = up ? cconj(t) : t;
+      }
+  }
+  float2 e[12];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) e[i] = make_float2(0.f, 0.f);
+  for (int it = 0; it < iters; ++it) {
+    float2 q[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) q[i] = cscale(rh[i], diag);
+    pair_hop<0>(rh, m[0], sgn[0], q);
+    pair_hop<1>(rh, m[1], sgn[1], q);
+    pair_hop<2>(rh, m[2], sgn[2], q);
+    pair_hop<3>(rh, m[3], sgn[3], q);
+    float qr_re = 0.f, qr_im = 0.f, qq = 0.f;
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      const float2 p = rh[i];
+      qr_re = fmaf(q[i].x, p.x, fmaf(q[i].y, p.y, qr_re));
+      qr_im = fmaf(q[i].x, p.y, fmaf(-q[i].y, p.x, qr_im));
+      qq = fmaf(q[i].x, q[i].x, fmaf(q[i].y, q[i].y, qq));
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      qr_re += __shfl_xor_sync(0xffffffffu, qr_re, o);
+      qr_im += __shfl_xor_sync(0xffffffffu, qr_im, o);
+      qq += __shfl_xor_sync(0xffffffffu, qq, o);
+    }
+    const float2 al = qq > 1e-30f ? make_float2(qr_re / qq, qr_im / qq) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      const float2 p = rh[i];
+      e[i] = cfma(al, p, e[i]);
+      rh[i] = cfma(cneg(al), q[i], p);
+    }
+  }
+  if (!live) return;
+  store_fine_site<float>(e_out + rr * n, s, V, e);
+  store_fine_site<float>(r + rr * n, s, V, rh);
+  add_to_z<float>(z + rr * n, s, V, e, zero);
+}
+
 // ---- paired FP32 arithmetic (P2 and the p2* helpers of common.cuh): the
 // same component of two right-hand sides in the two lanes of a register pair
 
@@ -921,13 +1037,17 @@ void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4],
   if (sm > 220 * 1024) throw Error(1, "SAP block too large for shared memory");
   const unsigned grid = (unsigned)(nblocks / 2) * (unsigned)((nrhs + rs - 1) / rs);
   const float dg = (float)(4.0 + m0);
-  bool b8 = false, b4 = false;
+  bool b8 = false, b4 = false, b2 = false;
   const unsigned half = (unsigned)(nblocks / 2);
   if constexpr (sizeof(T) == 4) {
     // the staged kernel's copies and its 16-byte chunks want aligned vectors
     b8 = b[0] == 8 && b[1] == 4 && b[2] == 4 && b[3] == 2;
     b4 = b[0] == 4 && b[1] == 4 && b[2] == 4 && b[3] == 4;
+    b2 = b[0] == 2 && b[1] == 2 && b[2] == 2 && b[3] == 2;
   }
+  // small lattices spread their face sites over more, smaller blocks
+  const int face = (int64_t)g.V / 2 * nrhs < (int64_t)sm_count() * 512 ? 64 : 256;
+  const unsigned face_grid = (unsigned)div_up(g.V / 2, face) * (unsigned)nrhs;
   // red blocks; the black sites take the red corrections across their
   // faces; black blocks; the red sites take the black corrections (r exact
   // again).  The face updates run over one colour's sites at a time in their
@@ -937,8 +1057,7 @@ void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4],
   for (int color = 0; color < 2; ++color) {
     const C<T> *rin = r0 && color == 0 ? r0 : r;
     if (color == 1) {
-      sap_face_kernel<T><<<(unsigned)div_up(g.V / 2, 256) * (unsigned)nrhs, 256, 0, s>>>(r0 ? r0 : r, r, e, U, sg, 1,
-                                                                                        nrhs);
+      sap_face_kernel<T><<<face_grid, face, 0, s>>>(r0 ? r0 : r, r, e, U, sg, 1, nrhs);
       MG_LAUNCH_CHECK();
     }
     if constexpr (sizeof(T) == 4) {
@@ -946,7 +1065,10 @@ void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4],
       else if (variant == 0 && b4) launch_staged<4, 4, 4, 4>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, half, s);
       else if (variant == 1 && two && b8) launch_pair<8, 4, 4, 2>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, grid, s);
       else if (variant == 1 && two && b4) launch_pair<4, 4, 4, 4>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, grid, s);
-      else if (two) {
+      else if (b2) {
+        sap_small_kernel<<<(unsigned)div_up((int64_t)half * nrhs, 8), 128, 0, s>>>(rin, r, z, e, U, sg, dg, color,
+                                                                                  block_iters, nrhs, zero);
+      } else if (two) {
         smem_optin((const void *)sap_block_kernel<T, 2>, (int)sm);
         sap_block_kernel<T, 2><<<grid, 2 * sg.sites, sm, s>>>(rin, r, z, e, U, sg, (T)dg, color, block_iters, nrhs, zero);
       } else {
@@ -959,7 +1081,7 @@ void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4],
     }
     MG_LAUNCH_CHECK();
   }
-  sap_face_kernel<T><<<(unsigned)div_up(g.V / 2, 256) * (unsigned)nrhs, 256, 0, s>>>(r, r, e, U, sg, 0, nrhs);
+  sap_face_kernel<T><<<face_grid, face, 0, s>>>(r, r, e, U, sg, 0, nrhs);
   MG_LAUNCH_CHECK();
 }
 
