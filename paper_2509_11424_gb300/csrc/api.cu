@@ -336,8 +336,8 @@ mgmlmc_status mgmlmc_apply(mgmlmc_ctx *ctx, int op_flags, int level, int precisi
       case MGMLMC_OP_D:
         if (dp) e.apply_D<double>(level, (const double2 *)in, (double2 *)out, nrhs);
         else e.apply_D<float>(level, (const float2 *)in, (float2 *)out, nrhs);
-        // a bounded wait of the FP32 stencil ran out (the FP64 one has none)
-        if (level > 0 && !dp) e.check_staging();
+        // a bounded wait of the stencil ran out (kernels that have none need no check)
+        if (level > 0 && !dp && e.stencil_waits(level, nrhs)) e.check_staging();
         break;
       case MGMLMC_OP_RESTRICT:
         if (dp) e.restrict_to<double>(level, (const double2 *)in, (double2 *)out, nrhs);

@@ -401,6 +401,7 @@ void Engine::free_hierarchy() {
       dfree(L.AF);
       dfree(L.AFu);
       dfree(L.AT32);
+      dfree(L.AR32);
       dfree(L.ATC);
       if (L.ATCB) cudaFree(L.ATCB);
       L.ATCB = nullptr;
@@ -472,8 +473,16 @@ void Engine::stencil_run(int l, int v, const float2 *in, float2 *out, int nrhs) 
   else if (v == 5 && L.ATCB) stencil_apply_tc(in, out, L.ATCB, L.g, nrhs, flag_dev_ + 1, 3, stream);
   else if (v == 3 && L.ATB16 && pipe) stencil_apply_pipe(in, out, L.ATB16, true, L.g, nrhs, flag_dev_ + 1, stream);
   else if ((v == 6 || v == 7) && L.ATS && nrhs <= 8) stencil_apply_stream(in, out, L.ATS, L.g, nrhs, v == 7, stream);
+  else if (L.AR32 && stencil_rows_supported(L.g, nrhs)) stencil_apply_rows(in, out, L.AR32, L.g, nrhs, stream);
   else if (pipe) stencil_apply_pipe(in, out, L.AT32, false, L.g, nrhs, flag_dev_ + 1, stream);
   else stencil_apply(in, out, L.AT32, L.g, nrhs, flag_dev_ + 1, stream);
+}
+
+bool Engine::stencil_waits(int l, int nrhs) const {
+  const Level &L = levels_.at(l);
+  const int v = stencil_variant(l, nrhs);
+  return !(v == 0 && L.AR32 && stencil_rows_supported(L.g, nrhs)) &&
+         !((v == 6 || v == 7) && L.ATS && nrhs <= 8);
 }
 
 // the tensor-core variants compute TF32 products, so the variant changes the
@@ -680,6 +689,25 @@ void Engine::noise(int l, uint64_t seed, uint64_t sample0, uint64_t term, uint64
 // (MGMLMC_SMOOTHER_SAP), followed for MGMLMC_SMOOTHER_LEARNED by one learned
 // step z += alpha N(res) with the residual-minimising alpha (so the step can
 // only lower ||res||); other levels / MR: minimal-residual steps.
+// One launch where the FP32 row-chunked stencil applies and its last block can
+// add every site's sums in the time of another launch (V <= 2048), else two.
+template <typename T> void Engine::apply_D_dots(int l, const C<T> *x, C<T> *q, int nrhs, double2 *d) {
+  const Level &L = levels_[l];
+  const int64_t n = L.g.n();
+  if constexpr (sizeof(T) == 4) {
+    if (!L.fine && L.AR32 && stencil_rows_supported(L.g, nrhs) && L.g.V <= 2048 && stencil_pick(l, nrhs, x, q) == 0) {
+      cudaEvent_t a = prof_begin();
+      stencil_apply_rows_dots(x, q, L.AR32, L.g, nrhs, partials(stencil_dots_scratch(L.g, nrhs)), d, d + nrhs, stream);
+      const double m = L.g.dof;
+      prof_end(a, K_STENCIL32, (double)L.g.V * (9.0 * m * m + 2.0 * m * nrhs) * sizeof(float2),
+               72.0 * m * m * L.g.V * nrhs);
+      return;
+    }
+  }
+  apply_D<T>(l, x, q, nrhs);
+  dot_qr<T>(q, x, n, nrhs, d, d + nrhs, partials((size_t)reduce_blocks(n) * nrhs * 2), stream);
+}
+
 template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs, const C<T> *r0) {
   const int64_t n = levels_[l].g.n();
   const bool learned = l == 0 && sp_.smoother == MGMLMC_SMOOTHER_LEARNED;
@@ -743,8 +771,7 @@ template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs, c
   double2 *d = ws<double>("smd", l, 2 * (size_t)nrhs);
   for (int s = 0; s < n_steps; ++s) {
     const C<T> *first = s == 0 ? r0 : nullptr, *x = first ? first : res;
-    apply_D<T>(l, x, q, nrhs);
-    dot_qr<T>(q, x, n, nrhs, d, d + nrhs, partials((size_t)reduce_blocks(n) * nrhs * 2), stream);
+    apply_D_dots<T>(l, x, q, nrhs, d);
     mr_update<T>(z, res, q, d, d + nrhs, n, nrhs, stream, first);
   }
 }
@@ -1170,6 +1197,10 @@ void Engine::galerkin(int l) {
     stencil_tile_tc(c.A64, c.ATC, false, c.g, stream);
     c.ATCB = dalloc<float>((stencil_tc_elems(c.g) + 1) / 2);  // BF16 elements, two per float slot
     stencil_tile_tc(c.A64, c.ATCB, true, c.g, stream);
+  }
+  if (stencil_rows_supported(c.g, 1)) {
+    c.AR32 = dalloc<float4>((acnt + 1) / 2);
+    stencil_to_rows(c.A64, c.AR32, (int64_t)acnt, stream);
   }
   if (stencil_pipe_supported(c.g)) {
     c.ATB16 = dalloc<float>(acnt);  // one bf16 pair (4 bytes) per complex entry

@@ -26,6 +26,7 @@ struct Level {
   int4 *AF = nullptr;       // the same blocks transposed [V][9][j][i] as fixed-point digits (FP64 apply)
   short *AFu = nullptr;     // exponent of each row's unit [V][dof]
   float2 *AT32 = nullptr;
+  float4 *AR32 = nullptr;   // the FP32 blocks row-chunked (32 dofs per site only), see stencil_apply_rows
   float *ATC = nullptr;     // tensor-core tiles (32 dofs per site only), see stencil_tile_tc
   void *ATCB = nullptr;     // the same tiles in BF16 (kind::f16 MMAs)
   float *ATB16 = nullptr;   // AT32 as bf16 pairs (32 dofs per site only), preconditioner variant
@@ -179,6 +180,9 @@ class Engine {
   // free every workspace (and the graphs that use them) except the levels'
   // test vectors; later calls allocate what they need again
   void release_workspaces();
+  // whether the FP32 stencil of level l waits for staging copies (then a call
+  // that applied it has to check)
+  bool stencil_waits(int l, int nrhs) const;
   // MGMLMC_ERR_CUDA (and the flag cleared) if a coarse-stencil kernel's
   // bounded staging wait ran out since the last check; synchronises
   void check_staging();
@@ -224,6 +228,9 @@ class Engine {
   template <typename T> AggMap agg_of(int l, bool canonical = false) const;
   template <typename T> const C<T> *Dinv(int l) const;
 
+  // q = D_l x and the two dots of a minimal-residual step, d[r] = <q_r, x_r>,
+  // d[nrhs + r] = <q_r, q_r>
+  template <typename T> void apply_D_dots(int l, const C<T> *x, C<T> *q, int nrhs, double2 *d);
   // r0: the smoothing starts from z = 0 with the residual r0 (left as it is;
   // z and res hold nothing yet)
   template <typename T> void smooth(int l, C<T> *z, C<T> *res, int nrhs, const C<T> *r0 = nullptr);

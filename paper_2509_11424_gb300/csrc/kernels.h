@@ -177,6 +177,17 @@ void stencil_to_bf16(const float2 *AT32, void *ATB, int64_t count, cudaStream_t 
 void stencil_apply_stream(const float2 *in, float2 *out, const void *AS, Geom g, int nrhs, bool per_site,
                           cudaStream_t s);
 void stencil_to_stream(const float2 *AT32, void *AS, int64_t count, cudaStream_t s);
+// FP32 coarse stencil for 32 dofs per site, 1 .. 8 right-hand sides and at
+// least one site per SM: one block per site, the blocks row-chunked (AR from
+// stencil_to_rows, count complex entries).  Identical results to
+// stencil_apply.  _dots: also out_qx[r] = <q_r, x_r>, out_qq[r] = <q_r, q_r> of
+// the result q and the input x (scr: stencil_dots_scratch partials).
+bool stencil_rows_supported(const Geom &g, int nrhs);
+void stencil_apply_rows(const float2 *in, float2 *out, const float4 *AR, Geom g, int nrhs, cudaStream_t s);
+void stencil_apply_rows_dots(const float2 *in, float2 *out, const float4 *AR, Geom g, int nrhs, RedScratch scr,
+                             double2 *out_qx, double2 *out_qq, cudaStream_t s);
+size_t stencil_dots_scratch(const Geom &g, int nrhs);
+void stencil_to_rows(const double2 *A, float4 *AR, int64_t count, cudaStream_t s);
 // AT = blockwise transpose of the canonical A[X][d][i][j] (nblocks = 9 V)
 void stencil_transpose(const double2 *A, float2 *AT, int64_t nblocks, int m, cudaStream_t s);
 // (<q, r>, <q, q>) for every rhs in one pass: out_qr[r], out_qq[r]

@@ -2,6 +2,7 @@
 // 2.2) stored as 9 dense (2 N_tv)^2 blocks per coarse site, the transfer
 // operators P_l / P_l^H built per aggregate and chirality, the Galerkin
 // construction, and the dense coarsest-level inverse.
+#include "fixed.cuh"
 #include "kernels.h"
 
 #include <cuda_bf16.h>
@@ -550,6 +551,148 @@ __global__ void __launch_bounds__(288) stencil_stream_site_kernel(const float2 *
   }
 }
 
+// ---- FP32 coarse stencil for 32 dofs per site and up to 8 right-hand sides:
+// one thread block per coarse site, a warp per direction, lane i forming row
+// i.  The blocks are stored row-chunked, AR[X][d][c][i][q] = A(X, d)[i][2c +
+// q], so that a lane's two entries of a chunk are one 16-byte load and a
+// warp's load is 512 contiguous bytes; a warp issues the 16 loads of its 8 KB
+// before the first use, so an SM has 147 KB in flight from two blocks without
+// a shared-memory stage, an mbarrier or a wait.  Same sums in the same order
+// as the kernels above: identical results.
+//
+// DOTS: also <q, x> and <q, q> of the result q with the input x, per
+// right-hand side (a minimal-residual step needs them): every block leaves
+// its site's sums, the last block adds them in site order.
+//
+// Bound: memory above ~10^3 sites (2592 sites, 4 right-hand sides: 36 us, 5.6
+// TB/s; the pipelined kernel, one block per SM with two sites in flight, 45
+// us and a wait for its error flag), latency below.
+template <int RP, bool DOTS>
+__global__ void __launch_bounds__(288, 2)
+    stencil_site_kernel(const float2 *__restrict__ in, float2 *__restrict__ out, const float4 *__restrict__ AR, Geom g,
+                        int nrhs, double *__restrict__ partial, unsigned *__restrict__ ticket,
+                        double2 *__restrict__ oqx, double2 *__restrict__ oqq) {
+  __shared__ __align__(16) float4 xbuf[9][32 * RP];  // [j][rhs pair], then the partial rows
+  const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
+  const int X = blockIdx.x;
+  const int64_t n = g.n();
+  const float4 *src = AR + ((int64_t)X * 9 + d) * 512 + lane;
+  float4 a[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) a[c] = __ldg(src + c * 32);
+  float4 *xs = xbuf[d];
+  {
+    const float2 *xn = in + (int64_t)stream_neighbor(g, X, d) * 32 + lane;
+#pragma unroll
+    for (int rp = 0; rp < RP; ++rp) {
+      const float2 u = 2 * rp < nrhs ? __ldg(xn + (2 * rp) * n) : make_float2(0.f, 0.f);
+      const float2 w = 2 * rp + 1 < nrhs ? __ldg(xn + (2 * rp + 1) * n) : make_float2(0.f, 0.f);
+      xs[lane * RP + rp] = make_float4(u.x, w.x, u.y, w.y);
+    }
+  }
+  __syncwarp();
+  P2 accR[RP], accI[RP];
+#pragma unroll
+  for (int rp = 0; rp < RP; ++rp) accR[rp] = accI[rp] = p2(0.f, 0.f);
+#pragma unroll
+  for (int c = 0; c < 16; ++c) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float ar = q ? a[c].z : a[c].x, ai = q ? a[c].w : a[c].y;
+      const P2 AX = p2(ar, ar), NAY = p2(-ai, -ai), AY = p2(ai, ai);
+#pragma unroll
+      for (int rp = 0; rp < RP; ++rp) {
+        const float4 x4 = xs[(2 * c + q) * RP + rp];
+        const P2 XR = p2(x4.x, x4.y), XI = p2(x4.z, x4.w);
+        // cfma: re += ar xr, re += -ai xi; im += ar xi, im += ai xr
+        accR[rp] = p2fma(AX, XR, accR[rp]);
+        accR[rp] = p2fma(NAY, XI, accR[rp]);
+        accI[rp] = p2fma(AX, XI, accI[rp]);
+        accI[rp] = p2fma(AY, XR, accI[rp]);
+      }
+    }
+  }
+  float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (DOTS) {
+    __syncthreads();
+    if (d < RP) x0 = xbuf[0][lane * RP + d];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int rp = 0; rp < RP; ++rp) {
+    const float2 re = p2split(accR[rp]), im = p2split(accI[rp]);
+    xs[rp * 32 + lane] = make_float4(re.x, re.y, im.x, im.y);
+  }
+  __syncthreads();
+  if (d < RP) {
+    // warp rp adds the nine partial rows of right-hand sides 2 rp, 2 rp + 1
+    const int rp = d;
+    float4 v = xbuf[0][rp * 32 + lane];
+    P2 totR = p2(v.x, v.y), totI = p2(v.z, v.w);
+#pragma unroll
+    for (int dd = 1; dd < 9; ++dd) {
+      v = xbuf[dd][rp * 32 + lane];
+      totR = p2add(totR, p2(v.x, v.y));
+      totI = p2add(totI, p2(v.z, v.w));
+    }
+    const float2 re = p2split(totR), im = p2split(totI);
+    if (2 * rp < nrhs) out[(int64_t)(2 * rp) * n + (int64_t)X * 32 + lane] = make_float2(re.x, im.x);
+    if (2 * rp + 1 < nrhs) out[(int64_t)(2 * rp + 1) * n + (int64_t)X * 32 + lane] = make_float2(re.y, im.y);
+    if (DOTS) {
+      fx::WarpSumF ws;
+      ws.add(0, fmaf(re.x, x0.x, im.x * x0.z));  // conj(q) x, then |q|^2, of both right-hand sides
+      ws.add(1, fmaf(re.x, x0.z, -im.x * x0.x));
+      ws.add(2, fmaf(re.x, re.x, im.x * im.x));
+      ws.add(3, fmaf(re.y, x0.y, im.y * x0.w));
+      ws.add(4, fmaf(re.y, x0.w, -im.y * x0.y));
+      ws.add(5, fmaf(re.y, re.y, im.y * im.y));
+      if (lane < 6) partial[((int64_t)rp * 6 + lane) * g.V + X] = ws.get();
+    }
+  }
+  if constexpr (DOTS) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // 288 / (6 RP) threads per value, each over consecutive sites
+    constexpr int NV = 6 * RP, K = 288 / NV;
+    static_assert(K <= 48, "threads per value");
+    double *tail = reinterpret_cast<double *>(&xbuf[0][0]);  // [K][NV]
+    const int v = threadIdx.x % NV, c = threadIdx.x / NV;
+    if (c < K) {
+      const int per = (g.V + K - 1) / K, b0 = c * per, b1 = min(g.V, b0 + per);
+      double t = 0.0;
+      for (int q = b0; q < b1; ++q) t += __ldcg(partial + (int64_t)v * g.V + q);
+      tail[c * NV + v] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < NV) {
+      double t = tail[threadIdx.x];
+      for (int q = 1; q < K; ++q) t += tail[q * NV + threadIdx.x];
+      const int r = 2 * (threadIdx.x / 6) + (threadIdx.x % 6) / 3, w = threadIdx.x % 3;
+      if (r < nrhs) {
+        if (w == 0) oqx[r].x = t;
+        else if (w == 1) oqx[r].y = t;
+        else oqq[r] = make_double2(t, 0.0);
+      }
+    }
+    if (threadIdx.x == 0) *ticket = 0u;
+  }
+}
+
+// AR[blk][c][i][q] = A[blk][i][2c + q] in FP32, blk = 9 X + d
+__global__ void stencil_rows_layout_kernel(const double2 *__restrict__ A, float2 *__restrict__ AR, int64_t total) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t blk = e >> 10;
+    const int w = (int)(e & 1023), q = w & 1, i = (w >> 1) & 31, c = w >> 6;
+    AR[e] = cvt<float>(A[(blk << 10) + i * 32 + 2 * c + q]);
+  }
+}
+
 // AS[blk][c][i][q] = AT32[blk][4c + q][i] as a BF16 pair (round to nearest),
 // blk = 9 X + d
 __global__ void stencil_stream_layout_kernel(const float2 *__restrict__ AT32, __nv_bfloat162 *__restrict__ AS,
@@ -1005,6 +1148,40 @@ void stencil_apply_stream(const float2 *in, float2 *out, const void *AS, Geom g,
   if (nrhs <= 2) stencil_stream_kernel<1><<<grid, 256, 0, s>>>(in, out, a, g, nrhs);
   else if (nrhs <= 4) stencil_stream_kernel<2><<<grid, 256, 0, s>>>(in, out, a, g, nrhs);
   else stencil_stream_kernel<4><<<grid, 256, 0, s>>>(in, out, a, g, nrhs);
+  MG_LAUNCH_CHECK();
+}
+
+namespace {
+template <bool DOTS>
+void launch_site(const float2 *in, float2 *out, const float4 *AR, Geom g, int nrhs, RedScratch scr, double2 *oqx,
+                 double2 *oqq, cudaStream_t s) {
+  double *part = reinterpret_cast<double *>(scr.partial);
+  if (nrhs <= 2) stencil_site_kernel<1, DOTS><<<g.V, 288, 0, s>>>(in, out, AR, g, nrhs, part, scr.ticket, oqx, oqq);
+  else if (nrhs <= 4) stencil_site_kernel<2, DOTS><<<g.V, 288, 0, s>>>(in, out, AR, g, nrhs, part, scr.ticket, oqx, oqq);
+  else stencil_site_kernel<4, DOTS><<<g.V, 288, 0, s>>>(in, out, AR, g, nrhs, part, scr.ticket, oqx, oqq);
+  MG_LAUNCH_CHECK();
+}
+}  // namespace
+
+// One block per site pays from one site per SM on (below, the bulk copies of
+// the staged kernels bring a site's 74 KB with fewer requests); up to 8
+// right-hand sides.
+bool stencil_rows_supported(const Geom &g, int nrhs) {
+  return g.dof == 32 && nrhs >= 1 && nrhs <= 8 && g.V >= sm_count();
+}
+
+void stencil_apply_rows(const float2 *in, float2 *out, const float4 *AR, Geom g, int nrhs, cudaStream_t s) {
+  launch_site<false>(in, out, AR, g, nrhs, RedScratch{nullptr, nullptr}, nullptr, nullptr, s);
+}
+
+void stencil_apply_rows_dots(const float2 *in, float2 *out, const float4 *AR, Geom g, int nrhs, RedScratch scr,
+                             double2 *oqx, double2 *oqq, cudaStream_t s) {
+  launch_site<true>(in, out, AR, g, nrhs, scr, oqx, oqq, s);
+}
+size_t stencil_dots_scratch(const Geom &g, int nrhs) { return (size_t)g.V * 3 * (nrhs <= 2 ? 2 : nrhs <= 4 ? 4 : 8); }
+
+void stencil_to_rows(const double2 *A, float4 *AR, int64_t count, cudaStream_t s) {
+  stencil_rows_layout_kernel<<<grid_for(count), 256, 0, s>>>(A, reinterpret_cast<float2 *>(AR), count);
   MG_LAUNCH_CHECK();
 }
 
