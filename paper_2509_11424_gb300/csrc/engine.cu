@@ -893,9 +893,31 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
   const int64_t n = L.g.n();
   const int64_t vs = n * nrhs;
   const std::string tag = fixed ? "k" : "t";
-  // basis V_0..V_m; the new direction of iteration i is formed in V_{i+1}
-  // itself (orthogonalised and normalised in place), so no extra work vector
-  C<T> *V = ws<T>("gmV" + tag, l, (size_t)(m + 1) * vs);
+  // basis V_0..V_m.  FP32: the new direction of iteration i is formed in
+  // V_{i+1} itself (orthogonalised and normalised in place), so no extra work
+  // vector.  FP64: the basis is kept as digits (16 bytes per entry, B), and two
+  // FP64 vectors hold the current direction (V) and the next (V + vs).
+  constexpr bool dig = sizeof(T) == 8;
+  C<T> *V = ws<T>("gmV" + tag, l, (size_t)(dig ? 2 : m + 1) * vs);
+  DigitBasis B{nullptr, nullptr};
+  if (dig) {
+    B.v = reinterpret_cast<int4 *>(ws<double>("gmD" + tag, l, (size_t)(m + 1) * vs));
+    B.e = reinterpret_cast<short *>(ws<double>("gmE" + tag, l, ((size_t)(m + 1) * nrhs * digit_tiles(n) + 7) / 8));
+  }
+  auto vec = [&](int i) { return dig ? V + (i & 1) * vs : V + i * vs; };
+  // h = V^H w over the first k vectors; w += sign V h
+  auto basis_dot = [&](int k, const C<T> *w, double2 *h, RedScratch scr) {
+    if constexpr (dig) multi_dot_digits(B, k, w, n, nrhs, h, m + 1, scr, stream);
+    else multi_dot<T>(V, vs, k, w, n, nrhs, h, m + 1, scr, stream);
+  };
+  auto basis_axpy = [&](int k, C<T> *w, const double2 *h, int ldh, double sign) {
+    if constexpr (dig) multi_axpy_digits(B, k, w, n, nrhs, h, ldh, sign, stream);
+    else multi_axpy<T>(V, vs, k, w, n, nrhs, h, ldh, sign, stream);
+  };
+  auto normalise = [&](int i, const double *inv) {
+    if constexpr (dig) normalise_digits(vec(i), vec(i), B, i, inv, n, nrhs, stream);
+    else scale_rhs<T>(vec(i), vec(i), inv, n, nrhs, stream);
+  };
   C<T> *Z = use_precond ? ws<T>("gmZ" + tag, l, (size_t)m * vs) : nullptr;
   GmresState st;
   st.m = m;
@@ -944,23 +966,23 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
   for (;;) {
     dot<T>(V, V, n, nrhs, st.nrm, part(1), stream);
     gmres_start(st, stream);
-    scale_rhs<T>(V, V, st.inv, n, nrhs, stream);
+    normalise(0, st.inv);
     int it = 0;
     for (int i = 0; i < m; ++i) {
-      C<T> *vi = V + i * vs;
+      C<T> *vi = vec(i);
       C<T> *zi = use_precond ? Z + i * vs : vi;
-      C<T> *w = V + (i + 1) * vs;
+      C<T> *w = vec(i + 1);
       if (use_precond) {
         if (fixed) precond<T>(l, vi, zi, nrhs);
         else precond_top<T>(l, vi, zi, nrhs);
       }
       apply_D<T>(l, zi, w, nrhs);
       cudaEvent_t po = prof_begin();
-      multi_dot<T>(V, vs, i + 1, w, n, nrhs, st.h1, m + 1, part(i + 1), stream);
-      multi_axpy<T>(V, vs, i + 1, w, n, nrhs, st.h1, m + 1, -1.0, stream);
+      basis_dot(i + 1, w, st.h1, part(i + 1));
+      basis_axpy(i + 1, w, st.h1, m + 1, -1.0);
       if (two_pass) {
-        multi_dot<T>(V, vs, i + 1, w, n, nrhs, st.h2, m + 1, part(i + 1), stream);
-        multi_axpy<T>(V, vs, i + 1, w, n, nrhs, st.h2, m + 1, -1.0, stream);
+        basis_dot(i + 1, w, st.h2, part(i + 1));
+        basis_axpy(i + 1, w, st.h2, m + 1, -1.0);
       }
       dot<T>(w, w, n, nrhs, st.nrm, part(1), stream);
       // unique data of CGS2 (CGS1): the i+1 basis vectors twice (once) for the
@@ -968,7 +990,7 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
       prof_end(po, K_ORTHO,
                (double)vs * sizeof(C<T>) * (two_pass ? 4.0 * (i + 1) + 9.0 : 2.0 * (i + 1) + 5.0), 0.0);
       gmres_arnoldi(st, i, stream);
-      scale_rhs<T>(w, w, st.inv, n, nrhs, stream);
+      normalise(i + 1, st.inv);
       ++it;
       ++total;
       if (total >= max_iter) break;
@@ -982,7 +1004,8 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
       }
     }
     gmres_solve(st, stream);
-    multi_axpy<T>(use_precond ? Z : V, vs, it, x, n, nrhs, st.y, m, 1.0, stream);
+    if (use_precond) multi_axpy<T>(Z, vs, it, x, n, nrhs, st.y, m, 1.0, stream);
+    else basis_axpy(it, x, st.y, m, 1.0);
     if (fixed && total >= max_iter) break;
     // true residual (V_1 as the work vector: the cycle's basis is spent)
     apply_D<T>(l, x, V + vs, nrhs);
@@ -1332,8 +1355,9 @@ void Engine::setup_test_vectors(int l, double2 *V, int ntv, const mgmlmc_mg_para
   const double es = fp32 ? sizeof(float2) : sizeof(double2);
   size_t freeb = 0, totalb = 0;
   MG_CUDA(cudaMemGetInfo(&freeb, &totalb));
-  // per column: the basis (m + 1), the iterate, the converted input
-  const double per_col = (double)n * es * (m + 3);
+  // per column: the basis (m + 1), the iterate, the converted input, in FP64
+  // the two work vectors beside the basis
+  const double per_col = (double)n * es * (m + (fp32 ? 3 : 5));
   const int group = std::max(1, std::min(ntv, (int)(0.7 * (double)freeb / per_col)));
   double *inv = reinterpret_cast<double *>(ws<double>("tvinv", l, (size_t)ntv));
   double *nr = reinterpret_cast<double *>(ws<double>("tvnr", l, (size_t)ntv));
@@ -1364,7 +1388,7 @@ void Engine::setup_test_vectors(int l, double2 *V, int ntv, const mgmlmc_mg_para
     }
   }
   // the fixed-length GMRES workspaces of the setup (recreated on demand)
-  for (const char *name : {"gmVk", "gmZk", "gsHk", "gsh1k", "gsh2k", "gssnk", "gsgk", "gsyk", "gsnrmk",
+  for (const char *name : {"gmVk", "gmDk", "gmEk", "gmZk", "gsHk", "gsh1k", "gsh2k", "gssnk", "gsgk", "gsyk", "gsnrmk",
                            "gssck", "gsik"}) {
     ws_release(name, l, true);
     ws_release(name, l, false);

@@ -36,6 +36,22 @@ void multi_axpy(const C<T> *V, int64_t vstride, int k, C<T> *w, int64_t n, int n
 // d = a - b
 template <typename T>
 void subtract(const C<T> *a, const C<T> *b, C<T> *d, int64_t n, cudaStream_t s);
+// A Krylov basis of FP64 vectors as fixed-point digits (fixed.cuh): slot j,
+// right-hand side r at v + (j nrhs + r) n, the exponents of its tiles at e +
+// (j nrhs + r) digit_tiles(n).  normalise_digits: v_r = w_r inv[r] (may be in
+// place) and the same into `slot`; the products are those of multi_dot and
+// multi_axpy.
+struct DigitBasis {
+  int4 *v;
+  short *e;
+};
+int64_t digit_tiles(int64_t n);
+void normalise_digits(const double2 *w, double2 *v, DigitBasis b, int slot, const double *inv, int64_t n, int nrhs,
+                      cudaStream_t s);
+void multi_dot_digits(DigitBasis V, int k, const double2 *w, int64_t n, int nrhs, double2 *h, int ldh, RedScratch scr,
+                      cudaStream_t s);
+void multi_axpy_digits(DigitBasis V, int k, double2 *w, int64_t n, int nrhs, const double2 *h, int ldh, double sign,
+                       cudaStream_t s);
 // y = a x + b y   (host scalars, all rhs)
 template <typename T>
 void axpby(double a, const C<T> *x, double b, C<T> *y, int64_t n, int nrhs, cudaStream_t s);

@@ -41,6 +41,22 @@ using fx::WarpSumI;
 using fx::warp_exp;
 using fx::digits;
 __device__ __forceinline__ int exp2of(double2 v) { return max(fx::exp_field(v.x), fx::exp_field(v.y)); }
+// conj(a) b for the digits a, b: high and middle sums
+__device__ __forceinline__ void macc(int4 a, int4 b, long long &hr, long long &hi, long long &mr, long long &mi) {
+  const int n1 = -a.z, n0 = -a.w;
+  hr = fx::madw(a.z, b.z, fx::madw(a.x, b.x, hr));
+  hi = fx::madw(n1, b.x, fx::madw(a.x, b.z, hi));
+  mr = fx::madw(a.w, b.z, fx::madw(a.z, b.w, fx::madw(a.y, b.x, fx::madw(a.x, b.y, mr))));
+  mi = fx::madw(n0, b.x, fx::madw(n1, b.y, fx::madw(a.y, b.z, fx::madw(a.x, b.w, mi))));
+}
+// a b
+__device__ __forceinline__ void mac(int4 a, int4 b, long long &hr, long long &hi, long long &mr, long long &mi) {
+  const int n1 = -a.z, n0 = -a.w;
+  hr = fx::madw(n1, b.z, fx::madw(a.x, b.x, hr));
+  hi = fx::madw(a.z, b.x, fx::madw(a.x, b.z, hi));
+  mr = fx::madw(n0, b.z, fx::madw(n1, b.w, fx::madw(a.y, b.x, fx::madw(a.x, b.y, mr))));
+  mi = fx::madw(a.w, b.x, fx::madw(a.z, b.y, fx::madw(a.y, b.z, fx::madw(a.x, b.w, mi))));
+}
 
 // The block's NV sums (lane v of every warp holds value v) to partial[v * NB +
 // b] (doubles, pv apart); the block that finishes group g last adds the NB
@@ -195,14 +211,138 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
         long long hr = 0, hi = 0, mr = 0, mi = 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          // conj(x) y
-          const int4 q = digits(b[u], min(Ex, fx::kBadExp - 1));
-          const int n1 = -q.z, n0 = -q.w;
-          hr = fx::madw(q.z, c[u].z, fx::madw(q.x, c[u].x, hr));
-          hi = fx::madw(n1, c[u].x, fx::madw(q.x, c[u].z, hi));
-          mr = fx::madw(q.w, c[u].z, fx::madw(q.z, c[u].w, fx::madw(q.y, c[u].x, fx::madw(q.x, c[u].y, mr))));
-          mi = fx::madw(n0, c[u].x, fx::madw(n1, c[u].y, fx::madw(q.y, c[u].z, fx::madw(q.x, c[u].w, mi))));
+          macc(digits(b[u], min(Ex, fx::kBadExp - 1)), c[u], hr, hi, mr, mi);
         }
+        const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
+        const bool bad = Ex == fx::kBadExp || Ey == fx::kBadExp;
+        ws.add(2 * j, fx::fold(hr, mr), e, bad);
+        ws.add(2 * j + 1, fx::fold(hi, mi), e, bad);
+      }
+    }
+    acc += ws.get();
+  }
+  double s;
+  const int64_t g = (int64_t)r * gridDim.z + blockIdx.z;
+  double *part = reinterpret_cast<double *>(partial) + ((int64_t)r * k + j0) * 2 * gridDim.x;
+  if (block_finish<2 * JG>(acc, part, ticket + g, 2 * kg, s) && (int)threadIdx.x < 2 * kg)
+    reinterpret_cast<double *>(out + r * ldh + j0)[threadIdx.x] = s;
+}
+
+// ---- Krylov bases of FP64 solves are kept as digits (16 bytes per entry, as
+// much as the FP64 entries), 57 bits of the largest entry of every tile of
+// kTile entries: the vector is converted once, when it is normalised, instead
+// of in each of the four passes of its every later orthogonalisation (the
+// conversions took two thirds of the instructions of the kernels above).
+constexpr int kTile = 1024;
+
+// A thread's own entries of the vectors j, j + 1, ... pass through a ring of
+// kRing slots in shared memory by asynchronous copies: kRing vectors' entries
+// are in flight per thread (64 KB per block, three blocks per SM) without a
+// register for them, and without a barrier, since every thread reads only
+// what it copied.  n = 786 k, 16 right-hand sides, 1 .. 20 vectors: updates 364
+// us on average, 6.9 TB/s, 20 dots 756 us; with the loads of one vector at a
+// time in registers 707 and 1225 us, waiting for memory.
+constexpr int kRing = 4;
+struct Ring {
+  int4 *slot;  // [kRing][kTile]
+  __device__ __forceinline__ void fetch(int s, const int4 *src, int64_t left) const {
+#pragma unroll
+    for (int u = 0; u < kTile / RB; ++u) {
+      int4 *d = slot + s * kTile + u * RB + threadIdx.x;
+      if (u * RB + (int)threadIdx.x < left)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(d)),
+                     "l"(src + u * RB + threadIdx.x)
+                     : "memory");
+      else *d = make_int4(0, 0, 0, 0);
+    }
+  }
+  __device__ __forceinline__ static void commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+  // the oldest of the last kRing groups has landed
+  __device__ __forceinline__ static void wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 1) : "memory"); }
+  __device__ __forceinline__ int4 get(int s, int u) const { return slot[s * kTile + u * RB + threadIdx.x]; }
+};
+
+// v = w inv[r], its digits and the exponent field of each tile's unit
+__global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2 *v, int4 *__restrict__ vf,
+                                                       short *__restrict__ ev, const double *__restrict__ inv,
+                                                       int64_t n) {
+  constexpr int U = kTile / RB;
+  __shared__ int top[RB / 32];
+  const int r = blockIdx.y;
+  const double f = inv[r];
+  const int64_t i0 = (int64_t)blockIdx.x * kTile + threadIdx.x;
+  double2 x[U];
+  int E = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t i = i0 + u * RB;
+    x[u] = i < n ? cscale(w[r * n + i], f) : make_double2(0.0, 0.0);
+    E = max(E, exp2of(x[u]));
+  }
+  E = warp_exp(E);
+  if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = E;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < RB / 32; ++q) E = max(E, top[q]);
+  if (threadIdx.x == 0) ev[(int64_t)r * gridDim.x + blockIdx.x] = (short)E;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t i = i0 + u * RB;
+    if (i < n) {
+      v[r * n + i] = x[u];
+      vf[r * n + i] = digits(x[u], min(E, fx::kBadExp - 1));
+    }
+  }
+}
+
+// dot_f64_kernel with the vectors x_j as digits (ev: their tiles' exponents,
+// [j][r][tile])
+template <int JG>
+__global__ void __launch_bounds__(RB) dot_digits_kernel(const int4 *__restrict__ x, const short *__restrict__ ev,
+                                                        int64_t xstride, int k, const double2 *__restrict__ y,
+                                                        int64_t n, int64_t chunk, double2 *__restrict__ partial,
+                                                        unsigned *__restrict__ ticket, double2 *__restrict__ out,
+                                                        int ldh) {
+  constexpr int U = kTile / RB;
+  const int r = blockIdx.y, nrhs = gridDim.y, j0 = blockIdx.z * JG, kg = min(JG, k - j0);
+  const int64_t nt = (n + kTile - 1) / kTile;
+  const int4 *xr = x + j0 * xstride + r * n;
+  const double2 *yr = y + r * n;
+  const int64_t beg = (int64_t)blockIdx.x * chunk, end = min(beg + chunk, n);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const Ring ring{reinterpret_cast<int4 *>(smem_raw)};
+  double acc = 0.0;
+  for (int64_t t0 = beg; t0 < end; t0 += kTile) {
+    const int64_t i0 = t0 + threadIdx.x, tile = t0 / kTile;
+#pragma unroll
+    for (int j = 0; j < kRing; ++j) {
+      if (j < kg) ring.fetch(j, xr + j * xstride + t0, end - t0);
+      Ring::commit();
+    }
+    int4 c[U];
+    int Ey = 0;
+    {
+      double2 a[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a[u] = i0 + RB * u < end ? __ldg(yr + i0 + RB * u) : make_double2(0.0, 0.0);
+        Ey = max(Ey, exp2of(a[u]));
+      }
+      Ey = warp_exp(Ey);
+#pragma unroll
+      for (int u = 0; u < U; ++u) c[u] = digits(a[u], min(Ey, fx::kBadExp - 1));
+    }
+    WarpSumI ws;
+#pragma unroll
+    for (int j = 0; j < JG; ++j) {
+      if (j < kg) {
+        const int Ex = ev[((int64_t)(j0 + j) * nrhs + r) * nt + tile];
+        long long hr = 0, hi = 0, mr = 0, mi = 0;
+        Ring::wait();
+#pragma unroll
+        for (int u = 0; u < U; ++u) macc(ring.get(j % kRing, u), c[u], hr, hi, mr, mi);
+        if (j + kRing < kg) ring.fetch(j % kRing, xr + (j + kRing) * xstride + t0, end - t0);
+        Ring::commit();
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
         const bool bad = Ex == fx::kBadExp || Ey == fx::kBadExp;
         ws.add(2 * j, fx::fold(hr, mr), e, bad);
@@ -278,11 +418,7 @@ __global__ void __launch_bounds__(RB) dot_qr_f64_kernel(const double2 *__restric
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int4 p = digits(a[u], min(Ea, fx::kBadExp - 1)), w = digits(c[u], min(Ec, fx::kBadExp - 1));
-      const int n1 = -p.z, n0 = -p.w;
-      hr = fx::madw(p.z, w.z, fx::madw(p.x, w.x, hr));
-      hi = fx::madw(n1, w.x, fx::madw(p.x, w.z, hi));
-      mr = fx::madw(p.w, w.z, fx::madw(p.z, w.w, fx::madw(p.y, w.x, fx::madw(p.x, w.y, mr))));
-      mi = fx::madw(n0, w.x, fx::madw(n1, w.y, fx::madw(p.y, w.z, fx::madw(p.x, w.w, mi))));
+      macc(p, w, hr, hi, mr, mi);
       hq = fx::madw(p.z, p.z, fx::madw(p.x, p.x, hq));
       mq = fx::madw(2 * p.w, p.z, fx::madw(2 * p.y, p.x, mq));
     }
@@ -408,17 +544,12 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
       for (int j = 0; j < JG; ++j) {
         if (j < kg) {
           const int4 c = cd[j0 + j];
-          const int n1 = -c.z, n0 = -c.w;
           // the entries in the unit that makes c v come out in units of 2^ex;
           // a far smaller product vanishes against the largest
           const int E = S - ce[j0 + j];
 #pragma unroll
           for (int u = 0; u < U; ++u) {
-            const int4 q = digits(v[j][u], E);
-            hr[u] = fx::madw(n1, q.z, fx::madw(c.x, q.x, hr[u]));
-            hi[u] = fx::madw(c.z, q.x, fx::madw(c.x, q.z, hi[u]));
-            mr[u] = fx::madw(n0, q.z, fx::madw(n1, q.w, fx::madw(c.y, q.x, fx::madw(c.x, q.y, mr[u]))));
-            mi[u] = fx::madw(c.w, q.x, fx::madw(c.z, q.y, fx::madw(c.y, q.z, fx::madw(c.x, q.w, mi[u]))));
+            mac(c, digits(v[j][u], E), hr[u], hi[u], mr[u], mi[u]);
           }
         }
       }
@@ -435,6 +566,99 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
       if (i < n) wr[i] = acc[u];
     }
   }
+}
+
+// The same with the vectors as digits: one tile of kTile elements per block,
+// whose units are the vectors' own, so a product is shifted to the largest
+// unit of its group of JG before it is added.
+__global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__restrict__ V, const short *__restrict__ ev,
+                                                               int64_t vs, int k, double2 *__restrict__ w, int64_t n,
+                                                               const double2 *__restrict__ h, int ldh, double sign) {
+  constexpr int JG = 8, U = kTile / RB;
+  __shared__ int4 cd[128];
+  __shared__ int ce[128];  // exponent of coefficient times tile
+  __shared__ double2 coef[128];
+  const int r = blockIdx.y, nrhs = gridDim.y;
+  const int64_t nt = gridDim.x;
+  for (int j = threadIdx.x; j < k; j += blockDim.x) {
+    double2 c = h[r * ldh + j];
+    c = make_double2(sign * c.x, sign * c.y);
+    const int E = max(exp2of(c), 1), Ev = ev[((int64_t)j * nrhs + r) * nt + blockIdx.x];
+    coef[j] = c;
+    ce[j] = E == fx::kBadExp || Ev == fx::kBadExp ? 1 << 20 : E + Ev;
+    cd[j] = digits(c, min(E, fx::kBadExp - 1));
+  }
+  __syncthreads();
+  const int64_t t0 = (int64_t)blockIdx.x * kTile, i0 = t0 + threadIdx.x;
+  double2 *wr = w + r * n;
+  const int4 *Vr = V + r * n;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const Ring ring{reinterpret_cast<int4 *>(smem_raw)};
+#pragma unroll
+  for (int j = 0; j < kRing; ++j) {
+    if (j < k) ring.fetch(j, Vr + j * vs + t0, n - t0);
+    Ring::commit();
+  }
+  double2 acc[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) acc[u] = i0 + u * RB < n ? wr[i0 + u * RB] : make_double2(0.0, 0.0);
+  for (int j0 = 0; j0 < k; j0 += JG) {
+    const int kg = min(JG, k - j0);
+    int S = 2;
+    for (int j = 0; j < kg; ++j) S = max(S, ce[j0 + j]);
+    const int ex = S - 2 * (1022 + fx::kVecBits) + 2 * fx::kDigit;
+    if (S >= 1 << 20 || ex < -1000 || ex > 900) {
+      // Inf or NaN among them, or products near the ends of the range: in
+      // FP64 from the digits (an entry is then NaN or scaled twice)
+      for (int j = 0; j < kg; ++j) {
+        // the ring keeps its order
+        Ring::wait();
+        if (j0 + j + kRing < k) ring.fetch((j0 + j) % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
+        Ring::commit();
+        const bool bad = ce[j0 + j] >= 1 << 20;
+        const int Ev = ev[((int64_t)(j0 + j) * nrhs + r) * nt + blockIdx.x] - 1022 - fx::kVecBits;
+        for (int u = 0; u < U; ++u) {
+          if (i0 + u * RB >= n) continue;
+          const int4 q = Vr[(j0 + j) * vs + i0 + u * RB];
+          double2 x = make_double2(scalbn((double)(((long long)q.x << fx::kDigit) + q.y), Ev),
+                                   scalbn((double)(((long long)q.z << fx::kDigit) + q.w), Ev));
+          if (bad) x.x = x.y = __longlong_as_double(0x7ff8000000000000ll);
+          acc[u] = cfma(coef[j0 + j], x, acc[u]);
+        }
+      }
+      continue;
+    }
+    long long sr[U], si[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) sr[u] = si[u] = 0;
+#pragma unroll
+    for (int j = 0; j < JG; ++j) {
+      if (j < kg) {
+        const int4 c = cd[j0 + j];
+        const int sh = min(S - ce[j0 + j], 63);
+        Ring::wait();
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          long long hr = 0, hi = 0, mr = 0, mi = 0;
+          mac(c, ring.get(j % kRing, u), hr, hi, mr, mi);  // j0 is a multiple of kRing
+          sr[u] += fx::fold(hr, mr) >> sh;
+          si[u] += fx::fold(hi, mi) >> sh;
+        }
+        if (j0 + j + kRing < k) ring.fetch(j % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
+        Ring::commit();
+      }
+    }
+    static_assert(JG % kRing == 0, "ring slots of a group");
+    const double f = __longlong_as_double((long long)(ex + 1023) << 52);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      acc[u].x = fma(f, (double)sr[u], acc[u].x);
+      acc[u].y = fma(f, (double)si[u], acc[u].y);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (i0 + u * RB < n) wr[i0 + u * RB] = acc[u];
 }
 
 // W complex entries moved by one access (16 bytes: 2 FP32 or 1 FP64 ones)
@@ -787,6 +1011,42 @@ void launch_dot(const C<T> *V, int64_t vstride, int k, const C<T> *w, int64_t n,
   MG_LAUNCH_CHECK();
 }
 }  // namespace
+
+void normalise_digits(const double2 *w, double2 *v, DigitBasis b, int slot, const double *inv, int64_t n, int nrhs,
+                      cudaStream_t s) {
+  const int nt = div_up(n, kTile);
+  normalise_kernel<<<dim3(nt, nrhs), RB, 0, s>>>(w, v, b.v + (int64_t)slot * n * nrhs,
+                                                 b.e + (int64_t)slot * nt * nrhs, inv, n);
+  MG_LAUNCH_CHECK();
+}
+int64_t digit_tiles(int64_t n) { return (n + kTile - 1) / kTile; }
+
+void multi_dot_digits(DigitBasis V, int k, const double2 *w, int64_t n, int nrhs, double2 *h, int ldh, RedScratch scr,
+                      cudaStream_t s) {
+  if ((int64_t)k * nrhs > kTickets) throw Error(1, "reduction: too many outputs for the ticket array");
+  const int64_t chunk = reduce_chunk(n), vs = n * nrhs;
+  const int JG = k == 1 ? 1 : k <= 4 ? 4 : 8;
+  const dim3 grid(blocks_of(n), nrhs, (k + JG - 1) / JG);
+  constexpr int sm = kRing * kTile * (int)sizeof(int4);
+  auto go = [&](auto kernel) {
+    smem_optin((const void *)kernel, sm);
+    kernel<<<grid, RB, sm, s>>>(V.v, V.e, vs, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
+  };
+  if (JG == 1) go(dot_digits_kernel<1>);
+  else if (JG == 4) go(dot_digits_kernel<4>);
+  else go(dot_digits_kernel<8>);
+  MG_LAUNCH_CHECK();
+}
+
+void multi_axpy_digits(DigitBasis V, int k, double2 *w, int64_t n, int nrhs, const double2 *h, int ldh, double sign,
+                       cudaStream_t s) {
+  if (k <= 0) return;
+  if (k > 128) throw Error(1, "multi_axpy: k > 128");
+  constexpr int sm = kRing * kTile * (int)sizeof(int4);
+  smem_optin((const void *)multi_axpy_digits_kernel, sm);
+  multi_axpy_digits_kernel<<<dim3(div_up(n, kTile), nrhs), RB, sm, s>>>(V.v, V.e, n * nrhs, k, w, n, h, ldh, sign);
+  MG_LAUNCH_CHECK();
+}
 
 template <typename T>
 void dot(const C<T> *x, const C<T> *y, int64_t n, int nrhs, double2 *out, RedScratch scr,
