@@ -910,9 +910,15 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
     if constexpr (dig) multi_dot_digits(B, k, w, n, nrhs, h, m + 1, scr, stream);
     else multi_dot<T>(V, vs, k, w, n, nrhs, h, m + 1, scr, stream);
   };
-  auto basis_axpy = [&](int k, C<T> *w, const double2 *h, int ldh, double sign) {
-    if constexpr (dig) multi_axpy_digits(B, k, w, n, nrhs, h, ldh, sign, stream);
-    else multi_axpy<T>(V, vs, k, w, n, nrhs, h, ldh, sign, stream);
+  // nrm: also the norms of the updated w
+  auto basis_axpy = [&](int k, C<T> *w, const double2 *h, int ldh, double sign, double2 *nrm) {
+    if constexpr (dig) {
+      multi_axpy_digits(B, k, w, n, nrhs, h, ldh, sign, stream, nrm,
+                        partials((size_t)std::max<int64_t>(reduce_blocks(n), (digit_tiles(n) + 1) / 2) * nrhs));
+    } else {
+      multi_axpy<T>(V, vs, k, w, n, nrhs, h, ldh, sign, stream);
+      if (nrm) dot<T>(w, w, n, nrhs, nrm, partials((size_t)reduce_blocks(n) * nrhs), stream);
+    }
   };
   auto normalise = [&](int i, const double *inv) {
     if constexpr (dig) normalise_digits(vec(i), vec(i), B, i, inv, n, nrhs, stream);
@@ -979,12 +985,11 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
       apply_D<T>(l, zi, w, nrhs);
       cudaEvent_t po = prof_begin();
       basis_dot(i + 1, w, st.h1, part(i + 1));
-      basis_axpy(i + 1, w, st.h1, m + 1, -1.0);
+      basis_axpy(i + 1, w, st.h1, m + 1, -1.0, two_pass ? nullptr : st.nrm);
       if (two_pass) {
         basis_dot(i + 1, w, st.h2, part(i + 1));
-        basis_axpy(i + 1, w, st.h2, m + 1, -1.0);
+        basis_axpy(i + 1, w, st.h2, m + 1, -1.0, st.nrm);
       }
-      dot<T>(w, w, n, nrhs, st.nrm, part(1), stream);
       // unique data of CGS2 (CGS1): the i+1 basis vectors twice (once) for the
       // dots and twice (once) for the updates, w read/written 9 (5) times
       prof_end(po, K_ORTHO,
@@ -1005,7 +1010,7 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
     }
     gmres_solve(st, stream);
     if (use_precond) multi_axpy<T>(Z, vs, it, x, n, nrhs, st.y, m, 1.0, stream);
-    else basis_axpy(it, x, st.y, m, 1.0);
+    else basis_axpy(it, x, st.y, m, 1.0, nullptr);
     if (fixed && total >= max_iter) break;
     // true residual (V_1 as the work vector: the cycle's basis is spent)
     apply_D<T>(l, x, V + vs, nrhs);

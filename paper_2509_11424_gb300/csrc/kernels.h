@@ -40,7 +40,8 @@ void subtract(const C<T> *a, const C<T> *b, C<T> *d, int64_t n, cudaStream_t s);
 // right-hand side r at v + (j nrhs + r) n, the exponents of its tiles at e +
 // (j nrhs + r) digit_tiles(n).  normalise_digits: v_r = w_r inv[r] (may be in
 // place) and the same into `slot`; the products are those of multi_dot and
-// multi_axpy.
+// multi_axpy, nrm (may be null) receives <w_r, w_r> of the updated w (scr:
+// digit_tiles(n) doubles per right-hand side).
 struct DigitBasis {
   int4 *v;
   short *e;
@@ -51,7 +52,7 @@ void normalise_digits(const double2 *w, double2 *v, DigitBasis b, int slot, cons
 void multi_dot_digits(DigitBasis V, int k, const double2 *w, int64_t n, int nrhs, double2 *h, int ldh, RedScratch scr,
                       cudaStream_t s);
 void multi_axpy_digits(DigitBasis V, int k, double2 *w, int64_t n, int nrhs, const double2 *h, int ldh, double sign,
-                       cudaStream_t s);
+                       cudaStream_t s, double2 *nrm, RedScratch scr);
 // y = a x + b y   (host scalars, all rhs)
 template <typename T>
 void axpby(double a, const C<T> *x, double b, C<T> *y, int64_t n, int nrhs, cudaStream_t s);

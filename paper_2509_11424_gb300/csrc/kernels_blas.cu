@@ -570,10 +570,16 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
 
 // The same with the vectors as digits: one tile of kTile elements per block,
 // whose units are the vectors' own, so a product is shifted to the largest
-// unit of its group of JG before it is added.
+// unit of its group of JG before it is added.  NORM: also nrm[r].x = <w_r, w_r>
+// of the result (one pass over w less, 133 us of 560 at n = 786 k and 16
+// right-hand sides; partial, ticket as for the dots).
+template <bool NORM>
 __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__restrict__ V, const short *__restrict__ ev,
                                                                int64_t vs, int k, double2 *__restrict__ w, int64_t n,
-                                                               const double2 *__restrict__ h, int ldh, double sign) {
+                                                               const double2 *__restrict__ h, int ldh, double sign,
+                                                               double *__restrict__ partial,
+                                                               unsigned *__restrict__ ticket,
+                                                               double2 *__restrict__ nrm) {
   constexpr int JG = 8, U = kTile / RB;
   __shared__ int4 cd[128];
   __shared__ int ce[128];  // exponent of coefficient times tile
@@ -659,6 +665,27 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
 #pragma unroll
   for (int u = 0; u < U; ++u)
     if (i0 + u * RB < n) wr[i0 + u * RB] = acc[u];
+  if constexpr (NORM) {
+    int E = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (i0 + u * RB >= n) acc[u] = make_double2(0.0, 0.0);
+      E = max(E, exp2of(acc[u]));
+    }
+    E = warp_exp(E);
+    long long hq = 0, mq = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int4 q = digits(acc[u], min(E, fx::kBadExp - 1));
+      hq = fx::madw(q.z, q.z, fx::madw(q.x, q.x, hq));
+      mq = fx::madw(2 * q.w, q.z, fx::madw(2 * q.y, q.x, mq));
+    }
+    WarpSumI ws;
+    ws.add(0, fx::fold(hq, mq), 2 * fx::kDigit + 2 * E - 2 * (1022 + fx::kVecBits), E == fx::kBadExp);
+    double s;
+    if (block_finish<4>(ws.get(), partial + (int64_t)r * nt, ticket + r, 1, s) && threadIdx.x == 0)
+      nrm[r] = make_double2(s, 0.0);
+  }
 }
 
 // W complex entries moved by one access (16 bytes: 2 FP32 or 1 FP64 ones)
@@ -870,81 +897,99 @@ __global__ void gmres_start_kernel(GmresState st) {
   st.inv[r] = (act && beta > 0.0) ? 1.0 / beta : 0.0;
 }
 
-__global__ void gmres_arnoldi_kernel(GmresState st, int i) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= st.nrhs || !st.active[r]) return;
+// One warp per right-hand side: its lanes bring the coefficients and the
+// previous rotations in and the column out together, lane 0 rotates (a chain
+// of FP64 operations; with every operand of it loaded in turn from memory an
+// iteration with 20 vectors took 20 us).
+__global__ void __launch_bounds__(32) gmres_arnoldi_kernel(GmresState st, int i) {
+  __shared__ double2 col[66], sn[64];
+  __shared__ double cs[64];
+  const int r = blockIdx.x, lane = threadIdx.x;
+  if (!st.active[r]) return;
   const int m = st.m;
-  double2 *H = st.H + (int64_t)r * (m + 1) * m;
-  double2 *col = H + i * (m + 1);
-  for (int j = 0; j <= i; ++j) {
-    double2 a = st.h1[r * (m + 1) + j], b = st.h2[r * (m + 1) + j];
+  double2 *out = st.H + (int64_t)r * (m + 1) * m + i * (m + 1);
+  for (int j = lane; j <= i; j += 32) {
+    const double2 a = st.h1[r * (m + 1) + j], b = st.h2[r * (m + 1) + j];
     col[j] = make_double2(a.x + b.x, a.y + b.y);
+    if (j < i) {
+      cs[j] = st.cs[r * m + j];
+      sn[j] = st.sn[r * m + j];
+    }
   }
+  __syncwarp();
   const double hn = sqrt(fmax(st.nrm[r].x, 0.0));
-  col[i + 1] = make_double2(hn, 0.0);
-  // previous rotations
-  for (int j = 0; j < i; ++j) {
-    const double c = st.cs[r * m + j];
-    const double2 s = st.sn[r * m + j];
-    const double2 a = col[j], b = col[j + 1];
-    col[j] = cadd(cscale(a, c), dcmul(s, b));
-    col[j + 1] = csub(cscale(b, c), dcmul(cconj(s), a));
+  if (lane == 0) {
+    col[i + 1] = make_double2(hn, 0.0);
+    // previous rotations
+    for (int j = 0; j < i; ++j) {
+      const double c = cs[j];
+      const double2 s = sn[j];
+      const double2 a = col[j], b = col[j + 1];
+      col[j] = cadd(cscale(a, c), dcmul(s, b));
+      col[j + 1] = csub(cscale(b, c), dcmul(cconj(s), a));
+    }
+    // new rotation zeroing col[i+1] (real, >= 0)
+    const double2 a = col[i];
+    const double b = col[i + 1].x;
+    const double aa = sqrt(cabs2(a));
+    const double rr = sqrt(aa * aa + b * b);
+    double c;
+    double2 s;
+    if (rr == 0.0) {
+      c = 1.0;
+      s = make_double2(0.0, 0.0);
+    } else if (aa == 0.0) {
+      c = 0.0;
+      s = make_double2(1.0, 0.0);
+      col[i] = make_double2(rr, 0.0);
+    } else {
+      c = aa / rr;
+      const double2 ph = make_double2(a.x / aa, a.y / aa);
+      s = cscale(ph, b / rr);
+      col[i] = cscale(ph, rr);
+    }
+    col[i + 1] = make_double2(0.0, 0.0);
+    st.cs[r * m + i] = c;
+    st.sn[r * m + i] = s;
+    double2 *g = st.g + r * (m + 1);
+    const double2 gi = g[i];
+    g[i + 1] = cneg(dcmul(cconj(s), gi));
+    g[i] = cscale(gi, c);
+    const double res = sqrt(cabs2(g[i + 1]));
+    st.res[r] = res;
+    st.nit[r] = i + 1;
+    const bool done = !(res > st.target[r]) || hn == 0.0 || !isfinite(res) || rr == 0.0;
+    if (done) {
+      st.active[r] = 0;
+      st.inv[r] = 0.0;
+    } else {
+      st.inv[r] = 1.0 / hn;
+    }
   }
-  // new rotation zeroing col[i+1] (real, >= 0)
-  const double2 a = col[i];
-  const double b = col[i + 1].x;
-  const double aa = sqrt(cabs2(a));
-  const double rr = sqrt(aa * aa + b * b);
-  double c;
-  double2 s;
-  if (rr == 0.0) {
-    c = 1.0;
-    s = make_double2(0.0, 0.0);
-  } else if (aa == 0.0) {
-    c = 0.0;
-    s = make_double2(1.0, 0.0);
-    col[i] = make_double2(rr, 0.0);
-  } else {
-    c = aa / rr;
-    const double2 ph = make_double2(a.x / aa, a.y / aa);
-    s = cscale(ph, b / rr);
-    col[i] = cscale(ph, rr);
-  }
-  col[i + 1] = make_double2(0.0, 0.0);
-  st.cs[r * m + i] = c;
-  st.sn[r * m + i] = s;
-  double2 *g = st.g + r * (m + 1);
-  const double2 gi = g[i];
-  g[i + 1] = cneg(dcmul(cconj(s), gi));
-  g[i] = cscale(gi, c);
-  const double res = sqrt(cabs2(g[i + 1]));
-  st.res[r] = res;
-  st.nit[r] = i + 1;
-  const bool done = !(res > st.target[r]) || hn == 0.0 || !isfinite(res) || rr == 0.0;
-  if (done) {
-    st.active[r] = 0;
-    st.inv[r] = 0.0;
-  } else {
-    st.inv[r] = 1.0 / hn;
-  }
+  __syncwarp();
+  for (int j = lane; j <= i + 1; j += 32) out[j] = col[j];
 }
 
-__global__ void gmres_solve_kernel(GmresState st) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= st.nrhs) return;
+// Back substitution with one warp per right-hand side: the right-hand side in
+// shared memory, each solved entry taken from all others at once.
+__global__ void __launch_bounds__(32) gmres_solve_kernel(GmresState st) {
+  __shared__ double2 acc[64];
+  const int r = blockIdx.x, lane = threadIdx.x;
   const int m = st.m;
   const int k = st.nit[r];
   const double2 *H = st.H + (int64_t)r * (m + 1) * m;
-  const double2 *g = st.g + r * (m + 1);
   double2 *y = st.y + r * m;
-  for (int j = k; j < m; ++j) y[j] = make_double2(0.0, 0.0);
+  for (int j = lane; j < k; j += 32) acc[j] = st.g[r * (m + 1) + j];
+  for (int j = k + lane; j < m; j += 32) y[j] = make_double2(0.0, 0.0);
   for (int j = k - 1; j >= 0; --j) {
-    double2 acc = g[j];
-    for (int l = j + 1; l < k; ++l) acc = csub(acc, dcmul(H[l * (m + 1) + j], y[l]));
-    const double2 d = H[j * (m + 1) + j];
+    const double2 *col = H + j * (m + 1);
+    __syncwarp();
+    const double2 a = acc[j], d = col[j];
     const double dd = cabs2(d);
-    y[j] = dd > 0.0 ? make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd)
-                    : make_double2(0.0, 0.0);
+    const double2 yj = dd > 0.0 ? make_double2((a.x * d.x + a.y * d.y) / dd, (a.y * d.x - a.x * d.y) / dd)
+                                : make_double2(0.0, 0.0);
+    if (lane == 0) y[j] = yj;
+    for (int l = lane; l < j; l += 32) acc[l] = csub(acc[l], dcmul(col[l], yj));
   }
 }
 }  // namespace
@@ -1039,12 +1084,17 @@ void multi_dot_digits(DigitBasis V, int k, const double2 *w, int64_t n, int nrhs
 }
 
 void multi_axpy_digits(DigitBasis V, int k, double2 *w, int64_t n, int nrhs, const double2 *h, int ldh, double sign,
-                       cudaStream_t s) {
+                       cudaStream_t s, double2 *nrm, RedScratch scr) {
   if (k <= 0) return;
   if (k > 128) throw Error(1, "multi_axpy: k > 128");
   constexpr int sm = kRing * kTile * (int)sizeof(int4);
-  smem_optin((const void *)multi_axpy_digits_kernel, sm);
-  multi_axpy_digits_kernel<<<dim3(div_up(n, kTile), nrhs), RB, sm, s>>>(V.v, V.e, n * nrhs, k, w, n, h, ldh, sign);
+  auto go = [&](auto kernel) {
+    smem_optin((const void *)kernel, sm);
+    kernel<<<dim3(div_up(n, kTile), nrhs), RB, sm, s>>>(V.v, V.e, n * nrhs, k, w, n, h, ldh, sign,
+                                                       reinterpret_cast<double *>(scr.partial), scr.ticket, nrm);
+  };
+  if (nrm) go(multi_axpy_digits_kernel<true>);
+  else go(multi_axpy_digits_kernel<false>);
   MG_LAUNCH_CHECK();
 }
 
@@ -1193,11 +1243,11 @@ void gmres_start(GmresState st, cudaStream_t s) {
   MG_LAUNCH_CHECK();
 }
 void gmres_arnoldi(GmresState st, int i, cudaStream_t s) {
-  gmres_arnoldi_kernel<<<(st.nrhs + 63) / 64, 64, 0, s>>>(st, i);
+  gmres_arnoldi_kernel<<<st.nrhs, 32, 0, s>>>(st, i);
   MG_LAUNCH_CHECK();
 }
 void gmres_solve(GmresState st, cudaStream_t s) {
-  gmres_solve_kernel<<<(st.nrhs + 63) / 64, 64, 0, s>>>(st);
+  gmres_solve_kernel<<<st.nrhs, 32, 0, s>>>(st);
   MG_LAUNCH_CHECK();
 }
 
