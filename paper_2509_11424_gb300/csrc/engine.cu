@@ -1215,7 +1215,7 @@ void Engine::galerkin(int l) {
     probe_column(probe, f.P64, m, col, stream);
     if (f.fine) wilson_split<double>(probe, out9, f.U64, f.g, m0_, m.b, stream);
     else stencil_split<double>(probe, out9, f.A64, f.g, m.b, stream);
-    restrict_op<double>(out9, cols, f.P64, m, 9, stream);
+    galerkin_restrict(out9, cols, f.P64, m, stream);
     galerkin_scatter(cols, c.A64, c.g, col, stream);
   }
   stencil_digits(c.A64, c.AF, c.AFu, c.g, stream);

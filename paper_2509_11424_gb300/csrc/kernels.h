@@ -276,6 +276,10 @@ void probe_column(double2 *out, const double2 *P, const AggMap &m, int col, cuda
 // Gram-Schmidt run twice in k order.  status[0] set to 1 on a zero norm.
 void build_prolongator(const double2 *V, double2 *P, const AggMap &m, int *status,
                        cudaStream_t s);
+// cols[h] = P^H out9[h] for the nine hop-class parts of one probe column: the
+// hops that leave an aggregate live on one of its faces, whose rows alone are
+// read and summed
+void galerkin_restrict(const double2 *out9, double2 *cols, const double2 *P, const AggMap &m, cudaStream_t s);
 // A[X][h][i][col] = cols[h][X * dof + i] for h = 0..8
 void galerkin_scatter(const double2 *cols, double2 *A, Geom coarse, int col, cudaStream_t s);
 // convert / transpose P to the canonical host order [X][c][row][k]
