@@ -912,13 +912,9 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
   };
   // nrm: also the norms of the updated w
   auto basis_axpy = [&](int k, C<T> *w, const double2 *h, int ldh, double sign, double2 *nrm) {
-    if constexpr (dig) {
-      multi_axpy_digits(B, k, w, n, nrhs, h, ldh, sign, stream, nrm,
-                        partials((size_t)std::max<int64_t>(reduce_blocks(n), (digit_tiles(n) + 1) / 2) * nrhs));
-    } else {
-      multi_axpy<T>(V, vs, k, w, n, nrhs, h, ldh, sign, stream);
-      if (nrm) dot<T>(w, w, n, nrhs, nrm, partials((size_t)reduce_blocks(n) * nrhs), stream);
-    }
+    const RedScratch scr = nrm ? partials((size_t)norm_scratch(n) * nrhs) : RedScratch{};
+    if constexpr (dig) multi_axpy_digits(B, k, w, n, nrhs, h, ldh, sign, stream, nrm, scr);
+    else multi_axpy<T>(V, vs, k, w, n, nrhs, h, ldh, sign, stream, nrm, scr);
   };
   auto normalise = [&](int i, const double *inv) {
     if constexpr (dig) normalise_digits(vec(i), vec(i), B, i, inv, n, nrhs, stream);
@@ -991,9 +987,9 @@ SolveInfo Engine::fgmres(int l, const C<T> *b, C<T> *x, int nrhs, double tol, in
         basis_axpy(i + 1, w, st.h2, m + 1, -1.0, st.nrm);
       }
       // unique data of CGS2 (CGS1): the i+1 basis vectors twice (once) for the
-      // dots and twice (once) for the updates, w read/written 9 (5) times
+      // dots and twice (once) for the updates, w read/written 8 (4) times
       prof_end(po, K_ORTHO,
-               (double)vs * sizeof(C<T>) * (two_pass ? 4.0 * (i + 1) + 9.0 : 2.0 * (i + 1) + 5.0), 0.0);
+               (double)vs * sizeof(C<T>) * (two_pass ? 4.0 * (i + 1) + 8.0 : 2.0 * (i + 1) + 4.0), 0.0);
       gmres_arnoldi(st, i, stream);
       normalise(i + 1, st.inv);
       ++it;

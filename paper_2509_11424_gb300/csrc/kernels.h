@@ -29,10 +29,13 @@ void dot(const C<T> *x, const C<T> *y, int64_t n, int nrhs, double2 *out, RedScr
 template <typename T>
 void multi_dot(const C<T> *V, int64_t vstride, int k, const C<T> *w, int64_t n, int nrhs,
                double2 *h, int ldh, RedScratch scr, cudaStream_t s);
-// w_r += sign * sum_{j<k} h[r * ldh + j] V_j,r
+// double2 entries of scr.partial per right-hand side for the norms below
+int64_t norm_scratch(int64_t n);
+// w_r += sign * sum_{j<k} h[r * ldh + j] V_j,r; nrm (may be null): also nrm[r].x
+// = <w_r, w_r> of the result
 template <typename T>
 void multi_axpy(const C<T> *V, int64_t vstride, int k, C<T> *w, int64_t n, int nrhs,
-                const double2 *h, int ldh, double sign, cudaStream_t s);
+                const double2 *h, int ldh, double sign, cudaStream_t s, double2 *nrm = nullptr, RedScratch scr = {});
 // d = a - b
 template <typename T>
 void subtract(const C<T> *a, const C<T> *b, C<T> *d, int64_t n, cudaStream_t s);
@@ -40,8 +43,7 @@ void subtract(const C<T> *a, const C<T> *b, C<T> *d, int64_t n, cudaStream_t s);
 // right-hand side r at v + (j nrhs + r) n, the exponents of its tiles at e +
 // (j nrhs + r) digit_tiles(n).  normalise_digits: v_r = w_r inv[r] (may be in
 // place) and the same into `slot`; the products are those of multi_dot and
-// multi_axpy, nrm (may be null) receives <w_r, w_r> of the updated w (scr:
-// digit_tiles(n) doubles per right-hand side).
+// multi_axpy.
 struct DigitBasis {
   int4 *v;
   short *e;

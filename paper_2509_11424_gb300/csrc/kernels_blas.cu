@@ -102,6 +102,37 @@ __device__ __forceinline__ bool block_finish(double mine, double *__restrict__ p
   return true;
 }
 
+// A thread's own entries of the vectors j, j + 1, ... of a basis pass through a
+// ring of kRing slots of 16 TILE bytes in shared memory by asynchronous copies:
+// kRing vectors' entries are in flight per thread (64 KB per block and three
+// blocks per SM at TILE = 1024, 32 KB and six at 512) without a register for
+// them, and without a barrier, since every thread reads only what it copied.
+// FP64 digits, n = 786 k, 16 right-hand sides, 1 .. 20 vectors: updates 364 us on
+// average, 6.9 TB/s, 20 dots 756 us; with the loads of one vector at a time in
+// registers 707 and 1225 us, waiting for memory.
+constexpr int kRing = 4;
+template <int TILE> struct Ring {
+  int4 *slot;  // [kRing][TILE]
+  __device__ __forceinline__ void fetch(int s, const int4 *src, int64_t left) const {
+#pragma unroll
+    for (int u = 0; u < TILE / RB; ++u) {
+      int4 *d = slot + s * TILE + u * RB + threadIdx.x;
+      if (u * RB + (int)threadIdx.x < left)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(d)),
+                     "l"(src + u * RB + threadIdx.x)
+                     : "memory");
+      else *d = make_int4(0, 0, 0, 0);
+    }
+  }
+  __device__ __forceinline__ static void commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+  // the oldest of the last kRing groups has landed
+  __device__ __forceinline__ static void wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 1) : "memory"); }
+  __device__ __forceinline__ int4 get(int s, int u) const { return slot[s * TILE + u * RB + threadIdx.x]; }
+  __device__ __forceinline__ float4 getf(int s, int u) const {
+    return *reinterpret_cast<const float4 *>(slot + s * TILE + u * RB + threadIdx.x);
+  }
+};
+
 // element pairs of FP32 vectors as one 16-byte load where the operands allow
 template <bool VEC>
 __device__ __forceinline__ float4 ld2(const float2 *__restrict__ p, int64_t i, int64_t end) {
@@ -142,6 +173,69 @@ __global__ void __launch_bounds__(RB) dot_f32_kernel(const float2 *__restrict__ 
           ar[j] = fmaf(a.x, c[u].x, fmaf(a.y, c[u].y, fmaf(a.z, c[u].z, fmaf(a.w, c[u].w, ar[j]))));
           ai[j] = fmaf(a.x, c[u].y, fmaf(-a.y, c[u].x, fmaf(a.z, c[u].w, fmaf(-a.w, c[u].z, ai[j]))));
         }
+      }
+    }
+  }
+  WarpSumF ws;
+#pragma unroll
+  for (int j = 0; j < JG; ++j) {
+    if (j < kg) {
+      ws.add(2 * j, ar[j]);
+      ws.add(2 * j + 1, ai[j]);
+    }
+  }
+  double s;
+  const int64_t g = (int64_t)r * gridDim.z + blockIdx.z;
+  double *part = reinterpret_cast<double *>(partial) + ((int64_t)r * k + j0) * 2 * gridDim.x;
+  if (block_finish<2 * JG>(ws.get(), part, ticket + g, 2 * kg, s) && (int)threadIdx.x < 2 * kg)
+    reinterpret_cast<double *>(out + r * ldh + j0)[threadIdx.x] = s;
+}
+
+// The same sums in the same order with the vectors through the ring, for 16-byte
+// aligned FP32 vectors of even length.  n = 786 k, 8 right-hand sides, 9 .. 16
+// vectors: 144 us on average (168 us from registers).
+constexpr int kTileF = 512;  // 1024 elements
+template <int JG>
+__global__ void __launch_bounds__(RB) dot_f32_ring_kernel(const int4 *__restrict__ x, int64_t xstride, int k,
+                                                          const float4 *__restrict__ y, int64_t n, int64_t chunk,
+                                                          double2 *__restrict__ partial,
+                                                          unsigned *__restrict__ ticket, double2 *__restrict__ out,
+                                                          int ldh) {
+  constexpr int U = kTileF / RB;
+  using R = Ring<kTileF>;
+  const int r = blockIdx.y, j0 = blockIdx.z * JG, kg = min(JG, k - j0);
+  const int4 *xr = x + j0 * xstride + r * n;  // n, strides, chunk in pairs of elements
+  const float4 *yr = y + r * n;
+  const int64_t beg = (int64_t)blockIdx.x * chunk, end = min(beg + chunk, n);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const R ring{reinterpret_cast<int4 *>(smem_raw)};
+  float ar[JG], ai[JG];
+#pragma unroll
+  for (int j = 0; j < JG; ++j) ar[j] = ai[j] = 0.f;
+  for (int64_t t0 = beg; t0 < end; t0 += kTileF) {
+#pragma unroll
+    for (int j = 0; j < kRing; ++j) {
+      if (j < kg) ring.fetch(j, xr + j * xstride + t0, end - t0);
+      R::commit();
+    }
+    float4 c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = t0 + threadIdx.x + RB * u;
+      c[u] = i < end ? __ldg(yr + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int j = 0; j < JG; ++j) {
+      if (j < kg) {
+        R::wait();
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float4 a = ring.getf(j % kRing, u);
+          ar[j] = fmaf(a.x, c[u].x, fmaf(a.y, c[u].y, fmaf(a.z, c[u].z, fmaf(a.w, c[u].w, ar[j]))));
+          ai[j] = fmaf(a.x, c[u].y, fmaf(-a.y, c[u].x, fmaf(a.z, c[u].w, fmaf(-a.w, c[u].z, ai[j]))));
+        }
+        if (j + kRing < kg) ring.fetch(j % kRing, xr + (j + kRing) * xstride + t0, end - t0);
+        R::commit();
       }
     }
   }
@@ -235,33 +329,6 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
 // conversions took two thirds of the instructions of the kernels above).
 constexpr int kTile = 1024;
 
-// A thread's own entries of the vectors j, j + 1, ... pass through a ring of
-// kRing slots in shared memory by asynchronous copies: kRing vectors' entries
-// are in flight per thread (64 KB per block, three blocks per SM) without a
-// register for them, and without a barrier, since every thread reads only
-// what it copied.  n = 786 k, 16 right-hand sides, 1 .. 20 vectors: updates 364
-// us on average, 6.9 TB/s, 20 dots 756 us; with the loads of one vector at a
-// time in registers 707 and 1225 us, waiting for memory.
-constexpr int kRing = 4;
-struct Ring {
-  int4 *slot;  // [kRing][kTile]
-  __device__ __forceinline__ void fetch(int s, const int4 *src, int64_t left) const {
-#pragma unroll
-    for (int u = 0; u < kTile / RB; ++u) {
-      int4 *d = slot + s * kTile + u * RB + threadIdx.x;
-      if (u * RB + (int)threadIdx.x < left)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(d)),
-                     "l"(src + u * RB + threadIdx.x)
-                     : "memory");
-      else *d = make_int4(0, 0, 0, 0);
-    }
-  }
-  __device__ __forceinline__ static void commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-  // the oldest of the last kRing groups has landed
-  __device__ __forceinline__ static void wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 1) : "memory"); }
-  __device__ __forceinline__ int4 get(int s, int u) const { return slot[s * kTile + u * RB + threadIdx.x]; }
-};
-
 // v = w inv[r], its digits and the exponent field of each tile's unit
 __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2 *v, int4 *__restrict__ vf,
                                                        short *__restrict__ ev, const double *__restrict__ inv,
@@ -310,14 +377,14 @@ __global__ void __launch_bounds__(RB) dot_digits_kernel(const int4 *__restrict__
   const double2 *yr = y + r * n;
   const int64_t beg = (int64_t)blockIdx.x * chunk, end = min(beg + chunk, n);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const Ring ring{reinterpret_cast<int4 *>(smem_raw)};
+  const Ring<kTile> ring{reinterpret_cast<int4 *>(smem_raw)};
   double acc = 0.0;
   for (int64_t t0 = beg; t0 < end; t0 += kTile) {
     const int64_t i0 = t0 + threadIdx.x, tile = t0 / kTile;
 #pragma unroll
     for (int j = 0; j < kRing; ++j) {
       if (j < kg) ring.fetch(j, xr + j * xstride + t0, end - t0);
-      Ring::commit();
+      Ring<kTile>::commit();
     }
     int4 c[U];
     int Ey = 0;
@@ -338,11 +405,11 @@ __global__ void __launch_bounds__(RB) dot_digits_kernel(const int4 *__restrict__
       if (j < kg) {
         const int Ex = ev[((int64_t)(j0 + j) * nrhs + r) * nt + tile];
         long long hr = 0, hi = 0, mr = 0, mi = 0;
-        Ring::wait();
+        Ring<kTile>::wait();
 #pragma unroll
         for (int u = 0; u < U; ++u) macc(ring.get(j % kRing, u), c[u], hr, hi, mr, mi);
         if (j + kRing < kg) ring.fetch(j % kRing, xr + (j + kRing) * xstride + t0, end - t0);
-        Ring::commit();
+        Ring<kTile>::commit();
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
         const bool bad = Ex == fx::kBadExp || Ey == fx::kBadExp;
         ws.add(2 * j, fx::fold(hr, mr), e, bad);
@@ -441,7 +508,6 @@ __global__ void __launch_bounds__(RB) dot_qr_f64_kernel(const double2 *__restric
 }
 
 // w_r += sign sum_j h[r * ldh + j] V_j,r
-template <bool VEC>
 __global__ void __launch_bounds__(256) multi_axpy_f32_kernel(const float2 *__restrict__ V, int64_t vstride, int k,
                                                              float2 *__restrict__ w, int64_t n,
                                                              const double2 *__restrict__ h, int ldh, double sign) {
@@ -454,21 +520,73 @@ __global__ void __launch_bounds__(256) multi_axpy_f32_kernel(const float2 *__res
   __syncthreads();
   float2 *wr = w + r * n;
   const float2 *Vr = V + r * n;
-  for (int64_t i = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); i < n; i += 2 * (int64_t)gridDim.x * blockDim.x) {
-    float4 t = ld2<VEC>(wr, i, n);
-    float2 a = make_float2(t.x, t.y), b = make_float2(t.z, t.w);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    float2 a = wr[i];
 #pragma unroll 4
-    for (int j = 0; j < k; ++j) {
-      const float4 v = ld2<VEC>(Vr + j * vstride, i, n);
-      a = cfma(coef[j], make_float2(v.x, v.y), a);
-      b = cfma(coef[j], make_float2(v.z, v.w), b);
+    for (int j = 0; j < k; ++j) a = cfma(coef[j], Vr[j * vstride + i], a);
+    wr[i] = a;
+  }
+}
+
+// The same sums through the ring for 16-byte aligned vectors of even length: one
+// tile of 1024 elements per block.  NORM: also nrm[r].x = <w_r, w_r> of the
+// result, in the order of the dots.  n = 786 k, 8 right-hand sides, 1 .. 16
+// vectors: 82 us on average with the norm (71 and 30 us as two launches).
+template <bool NORM>
+__global__ void __launch_bounds__(RB) multi_axpy_f32_ring_kernel(const int4 *__restrict__ V, int64_t vs, int k,
+                                                                 float4 *__restrict__ w, int64_t n,
+                                                                 const double2 *__restrict__ h, int ldh, double sign,
+                                                                 double *__restrict__ partial,
+                                                                 unsigned *__restrict__ ticket,
+                                                                 double2 *__restrict__ nrm) {
+  constexpr int U = kTileF / RB;
+  using R = Ring<kTileF>;
+  __shared__ float2 coef[128];
+  const int r = blockIdx.y;
+  const int64_t t0 = (int64_t)blockIdx.x * kTileF, i0 = t0 + threadIdx.x;  // pairs of elements, as n and vs
+  float4 *wr = w + r * n;
+  const int4 *Vr = V + r * n + t0;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const R ring{reinterpret_cast<int4 *>(smem_raw)};
+#pragma unroll
+  for (int j = 0; j < kRing; ++j) {
+    if (j < k) ring.fetch(j, Vr + j * vs, n - t0);
+    R::commit();
+  }
+  float4 acc[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) acc[u] = i0 + u * RB < n ? wr[i0 + u * RB] : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int j = threadIdx.x; j < k; j += RB) {
+    const double2 c = h[r * ldh + j];
+    coef[j] = make_float2((float)(sign * c.x), (float)(sign * c.y));
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int j = 0; j < k; ++j) {
+    const float2 c = coef[j];
+    R::wait();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float4 v = ring.getf(j % kRing, u);
+      const float2 a = cfma(c, make_float2(v.x, v.y), make_float2(acc[u].x, acc[u].y));
+      const float2 b = cfma(c, make_float2(v.z, v.w), make_float2(acc[u].z, acc[u].w));
+      acc[u] = make_float4(a.x, a.y, b.x, b.y);
     }
-    if (VEC) {
-      *reinterpret_cast<float4 *>(wr + i) = make_float4(a.x, a.y, b.x, b.y);
-    } else {
-      wr[i] = a;
-      if (i + 1 < n) wr[i + 1] = b;
-    }
+    if (j + kRing < k) ring.fetch(j % kRing, Vr + (j + kRing) * vs, n - t0);
+    R::commit();
+  }
+  float q = 0.f;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (i0 + u * RB < n) wr[i0 + u * RB] = acc[u];
+    q = fmaf(acc[u].x, acc[u].x, fmaf(acc[u].y, acc[u].y, fmaf(acc[u].z, acc[u].z, fmaf(acc[u].w, acc[u].w, q))));
+  }
+  if constexpr (NORM) {
+    WarpSumF ws;
+    ws.add(0, q);
+    double s;
+    if (block_finish<4>(ws.get(), partial + (int64_t)r * gridDim.x, ticket + r, 1, s) && threadIdx.x == 0)
+      nrm[r] = make_double2(s, 0.0);
   }
 }
 
@@ -599,11 +717,11 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
   double2 *wr = w + r * n;
   const int4 *Vr = V + r * n;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const Ring ring{reinterpret_cast<int4 *>(smem_raw)};
+  const Ring<kTile> ring{reinterpret_cast<int4 *>(smem_raw)};
 #pragma unroll
   for (int j = 0; j < kRing; ++j) {
     if (j < k) ring.fetch(j, Vr + j * vs + t0, n - t0);
-    Ring::commit();
+    Ring<kTile>::commit();
   }
   double2 acc[U];
 #pragma unroll
@@ -618,9 +736,9 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
       // FP64 from the digits (an entry is then NaN or scaled twice)
       for (int j = 0; j < kg; ++j) {
         // the ring keeps its order
-        Ring::wait();
+        Ring<kTile>::wait();
         if (j0 + j + kRing < k) ring.fetch((j0 + j) % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
-        Ring::commit();
+        Ring<kTile>::commit();
         const bool bad = ce[j0 + j] >= 1 << 20;
         const int Ev = ev[((int64_t)(j0 + j) * nrhs + r) * nt + blockIdx.x] - 1022 - fx::kVecBits;
         for (int u = 0; u < U; ++u) {
@@ -642,7 +760,7 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
       if (j < kg) {
         const int4 c = cd[j0 + j];
         const int sh = min(S - ce[j0 + j], 63);
-        Ring::wait();
+        Ring<kTile>::wait();
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           long long hr = 0, hi = 0, mr = 0, mi = 0;
@@ -651,7 +769,7 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
           si[u] += fx::fold(hi, mi) >> sh;
         }
         if (j0 + j + kRing < k) ring.fetch(j % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
-        Ring::commit();
+        Ring<kTile>::commit();
       }
     }
     static_assert(JG % kRing == 0, "ring slots of a group");
@@ -1048,10 +1166,16 @@ void launch_dot(const C<T> *V, int64_t vstride, int k, const C<T> *w, int64_t n,
   const int64_t chunk = reduce_chunk(n);
   if constexpr (sizeof(T) == 8) {
     dot_f64_kernel<JG><<<grid, RB, 0, s>>>(V, vstride, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
-  } else if (aligned16(n | vstride, V, w)) {
+  } else if (!aligned16(n | vstride, V, w)) {
+    dot_f32_kernel<JG, false><<<grid, RB, 0, s>>>(V, vstride, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
+  } else if constexpr (JG == 1) {
     dot_f32_kernel<JG, true><<<grid, RB, 0, s>>>(V, vstride, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
   } else {
-    dot_f32_kernel<JG, false><<<grid, RB, 0, s>>>(V, vstride, k, w, n, chunk, scr.partial, scr.ticket, h, ldh);
+    constexpr int sm = kRing * kTileF * (int)sizeof(int4);
+    smem_optin((const void *)dot_f32_ring_kernel<JG>, sm);
+    dot_f32_ring_kernel<JG><<<grid, RB, sm, s>>>(reinterpret_cast<const int4 *>(V), vstride / 2, k,
+                                                 reinterpret_cast<const float4 *>(w), n / 2, chunk / 2, scr.partial,
+                                                 scr.ticket, h, ldh);
   }
   MG_LAUNCH_CHECK();
 }
@@ -1065,6 +1189,10 @@ void normalise_digits(const double2 *w, double2 *v, DigitBasis b, int slot, cons
   MG_LAUNCH_CHECK();
 }
 int64_t digit_tiles(int64_t n) { return (n + kTile - 1) / kTile; }
+// a double per tile (FP32 tiles are of 2 kTileF = kTile elements, too), or the
+// partials of a dot
+static_assert(2 * kTileF == kTile, "tiles");
+int64_t norm_scratch(int64_t n) { return std::max<int64_t>(reduce_blocks(n), (digit_tiles(n) + 1) / 2); }
 
 void multi_dot_digits(DigitBasis V, int k, const double2 *w, int64_t n, int nrhs, double2 *h, int ldh, RedScratch scr,
                       cudaStream_t s) {
@@ -1133,19 +1261,31 @@ void multi_dot(const C<T> *V, int64_t vstride, int k, const C<T> *w, int64_t n, 
 
 template <typename T>
 void multi_axpy(const C<T> *V, int64_t vstride, int k, C<T> *w, int64_t n, int nrhs,
-                const double2 *h, int ldh, double sign, cudaStream_t s) {
-  if (k <= 0) return;
+                const double2 *h, int ldh, double sign, cudaStream_t s, double2 *nrm, RedScratch scr) {
   if (k > 128) throw Error(1, "multi_axpy: k > 128");
-  // two elements per thread, at most 32 blocks per SM over all right-hand sides
-  const dim3 grid((unsigned)std::min<int64_t>(div_up(n, 512), std::max(1, sm_count() * 32 / nrhs)), nrhs);
-  if constexpr (sizeof(T) == 8) {
-    multi_axpy_f64_kernel<<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
-  } else if (aligned16(n | vstride, V, w)) {
-    multi_axpy_f32_kernel<true><<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
-  } else {
-    multi_axpy_f32_kernel<false><<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
+  if constexpr (sizeof(T) == 4) {
+    if (k > 0 && aligned16(n | vstride, V, w)) {
+      constexpr int sm = kRing * kTileF * (int)sizeof(int4);
+      auto go = [&](auto kernel) {
+        smem_optin((const void *)kernel, sm);
+        kernel<<<dim3(div_up(n, 2 * kTileF), nrhs), RB, sm, s>>>(
+            reinterpret_cast<const int4 *>(V), vstride / 2, k, reinterpret_cast<float4 *>(w), n / 2, h, ldh, sign,
+            reinterpret_cast<double *>(scr.partial), scr.ticket, nrm);
+      };
+      if (nrm) go(multi_axpy_f32_ring_kernel<true>);
+      else go(multi_axpy_f32_ring_kernel<false>);
+      MG_LAUNCH_CHECK();
+      return;
+    }
   }
-  MG_LAUNCH_CHECK();
+  if (k > 0) {
+    // at most 32 blocks per SM over all right-hand sides
+    const dim3 grid((unsigned)std::min<int64_t>(div_up(n, 512), std::max(1, sm_count() * 32 / nrhs)), nrhs);
+    if constexpr (sizeof(T) == 8) multi_axpy_f64_kernel<<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
+    else multi_axpy_f32_kernel<<<grid, 256, 0, s>>>(V, vstride, k, w, n, h, ldh, sign);
+    MG_LAUNCH_CHECK();
+  }
+  if (nrm) dot<T>(w, w, n, nrhs, nrm, scr, s);
 }
 
 namespace {
@@ -1257,7 +1397,7 @@ void gmres_solve(GmresState st, cudaStream_t s) {
   template void multi_dot<T>(const C<T> *, int64_t, int, const C<T> *, int64_t, int, double2 *,  \
                              int, RedScratch, cudaStream_t);                                     \
   template void multi_axpy<T>(const C<T> *, int64_t, int, C<T> *, int64_t, int, const double2 *, \
-                              int, double, cudaStream_t);                                        \
+                              int, double, cudaStream_t, double2 *, RedScratch);                                        \
   template void axpby<T>(double, const C<T> *, double, C<T> *, int64_t, int, cudaStream_t);      \
   template void scale_rhs<T>(const C<T> *, C<T> *, const double *, int64_t, int, cudaStream_t);  \
   template void mr_update<T>(C<T> *, C<T> *, const C<T> *, const double2 *, const double2 *,     \
