@@ -147,6 +147,30 @@ struct WarpSumD : WarpSumI {
     WarpSumI::add(v, to_fixed(p, min(E, kBadExp - 1)), E - 1022 - kVecBits, E == kBadExp);
   }
 };
+// the sum of n FP64 values by one warp, in lane 0: the 256 values of a step are
+// added as integers in the unit of their largest (one by one in FP64, the 256
+// partial sums of a reduction cost more than the reduction)
+__device__ __forceinline__ double warp_total(const double *__restrict__ p, int n) {
+  constexpr int U = 8;
+  const int lane = threadIdx.x & 31;
+  double t = 0.0;
+  for (int b = 0; b < n; b += 32 * U) {
+    double x[U];
+    int E = 1;
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = b + 32 * u + lane < n ? __ldcg(p + b + 32 * u + lane) : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) E = max(E, exp_field(x[u]));
+    E = __reduce_max_sync(0xffffffffu, E);
+    long long X = 0;  // 8 values below 2^kVecBits
+#pragma unroll
+    for (int u = 0; u < U; ++u) X += to_fixed(x[u], min(E, kBadExp - 1));
+    WarpSumI ws;
+    ws.add(0, X, E - 1022 - kVecBits, E == kBadExp);
+    t += ws.get();
+  }
+  return t;
+}
 __device__ __forceinline__ int4 digits(double2 v, int E) {
   const long long a = to_fixed(v.x, E), b = to_fixed(v.y, E);
   return make_int4(digit_hi(a), digit_lo(a), digit_hi(b), digit_lo(b));

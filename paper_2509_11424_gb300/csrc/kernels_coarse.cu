@@ -657,21 +657,15 @@ __global__ void __launch_bounds__(288, 2)
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // 288 / (6 RP) threads per value, each over consecutive sites
-    constexpr int NV = 6 * RP, K = 288 / NV;
-    static_assert(K <= 48, "threads per value");
-    double *tail = reinterpret_cast<double *>(&xbuf[0][0]);  // [K][NV]
-    const int v = threadIdx.x % NV, c = threadIdx.x / NV;
-    if (c < K) {
-      const int per = (g.V + K - 1) / K, b0 = c * per, b1 = min(g.V, b0 + per);
-      double t = 0.0;
-      for (int q = b0; q < b1; ++q) t += __ldcg(partial + (int64_t)v * g.V + q);
-      tail[c * NV + v] = t;
+    constexpr int NV = 6 * RP;
+    double *tot = reinterpret_cast<double *>(&xbuf[0][0]);
+    for (int v = d; v < NV; v += 9) {
+      const double t = fx::warp_total(partial + (int64_t)v * g.V, g.V);
+      if (lane == 0) tot[v] = t;
     }
     __syncthreads();
     if (threadIdx.x < NV) {
-      double t = tail[threadIdx.x];
-      for (int q = 1; q < K; ++q) t += tail[q * NV + threadIdx.x];
+      const double t = tot[threadIdx.x];
       const int r = 2 * (threadIdx.x / 6) + (threadIdx.x % 6) / 3, w = threadIdx.x % 3;
       if (r < nrhs) {
         if (w == 0) oqx[r].x = t;
