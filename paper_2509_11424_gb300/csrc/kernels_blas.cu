@@ -915,7 +915,10 @@ __global__ void convert_scale_kernel(const C<From> *__restrict__ in, C<To> *__re
 // move whole lines: 16-byte chunks in the structure-of-arrays order, and
 // consecutive entries in the canonical one (8-byte accesses where a buffer is
 // not aligned to 16).  Bound: memory; with scattered 8-byte accesses on one
-// side and no staging it moved 1.4 TB/s.
+// side and no staging it moved 1.4 TB/s.  Without scale factors nothing is
+// multiplied: FP32 to FP32 through an FP64 product by one kept the FP64 pipe
+// busy for most of the launch (9 us for 35 k sites; a one-sweep smoothing of
+// 12^3 x 20 with two of them 56 us, now 48).
 constexpr int kRelayoutSites = 128;
 
 template <typename T, bool VEC> __device__ __forceinline__ Pack<T, 2> ld_pair(const C<T> *p) {
@@ -948,7 +951,8 @@ __global__ void __launch_bounds__(256) relayout_kernel(const C<From> *__restrict
       const Pack<From, 2> v = ld_pair<From, VEC>(src);
       Pack<To, 2> o;
 #pragma unroll
-      for (int j = 0; j < 2; ++j) o.v[j] = mk<To>((To)(v.v[j].x * f), (To)(v.v[j].y * f));
+      for (int j = 0; j < 2; ++j)
+        o.v[j] = scal ? mk<To>((To)(v.v[j].x * f), (To)(v.v[j].y * f)) : mk<To>((To)v.v[j].x, (To)v.v[j].y);
       sh[k][site] = o;
     }
   }
