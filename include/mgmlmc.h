@@ -572,9 +572,10 @@ mgmlmc_status mgmlmc_profile_stats(mgmlmc_ctx *ctx, int kernel_class, int64_t *l
  * identical to variant 3; up to 8 right-hand sides at 32 dofs per site,
  * variant 0 otherwise); 7 = variant 6 with one thread block per coarse site
  * and a warp per direction (more parallel work on coarse lattices with few
- * sites; identical results).  Variant 0 runs up to 8 right-hand sides at 32 dofs per site in
- * a pipelined kernel (persistent blocks, a two-stage ring of bulk copies
- * over sites) with results identical to the one-site-per-block kernels.
+ * sites; identical results).  Variant 0 runs up to 8 right-hand sides at 32 dofs per site
+ * with one thread block per site and row-chunked FP32 blocks where there is
+ * at least one site per SM, else in a pipelined kernel (persistent blocks, a
+ * two-stage ring of bulk copies over sites); the results of all are identical.
  * -2 = autotune among 0, 1, 3, 4, 5, 6 and 7 per (level, nrhs) on the first call
  * outside graph capture (opt-in,
  * since the choice changes the rounding).  Inside a solve the variant applies

@@ -459,8 +459,8 @@ int Engine::stencil_variant(int l, int nrhs) const {
   return it == stencil_tuned_.end() ? -2 : it->second;
 }
 
-// 0: FP32 (the pipelined kernel where it applies, same sums as the
-// one-site-per-CTA kernels); 1, 2: tensor cores (TF32); 3: BF16-stored
+// 0: FP32 (one block per site with row-chunked blocks, or the pipelined kernel
+// below one site per SM, or the staged ones: the same sums); 1, 2: tensor cores (TF32); 3: BF16-stored
 // blocks, FP32 arithmetic (pipelined kernel, up to 8 right-hand sides);
 // 4: tensor cores with BF16 operands; 5: 4 as a persistent pipelined kernel;
 // 6: 3's sums with one warp per site streaming the row-chunked blocks;

@@ -935,8 +935,7 @@ __global__ void __launch_bounds__(256 * RS, (sizeof(T) == 4 && RS == 1) ? 2 : 1)
 
 // The boundary pass over the sites of the blocks of colour `color` only
 // (whole warps of one colour, instead of half the lanes of every warp idle),
-// one load set per direction where the block extent allows it; the same sum
-// as sap_boundary_kernel.  Right-hand side fastest over the grid.
+// one load set per direction where the block extent allows it.  Right-hand side fastest over the grid.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) sap_face_kernel(const C<T> *rin, C<T> *r, const C<T> *__restrict__ e,
                                                        const C<T> *__restrict__ U, SapGeom sg, int color,
