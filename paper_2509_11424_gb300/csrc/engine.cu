@@ -788,6 +788,14 @@ template <typename T> void Engine::smooth_apply(int l, const C<T> *in, C<T> *out
       return;
     }
   }
+  // the kernels of a first step read 16 bytes at a time: any other right-hand
+  // side is copied before it is smoothed
+  if (reinterpret_cast<uintptr_t>(in) & 15) {
+    MG_CUDA(cudaMemcpyAsync(res, in, sizeof(C<T>) * n * nrhs, cudaMemcpyDeviceToDevice, stream));
+    MG_CUDA(cudaMemsetAsync(out, 0, sizeof(C<T>) * n * nrhs, stream));
+    smooth<T>(l, out, res, nrhs);
+    return;
+  }
   smooth<T>(l, out, res, nrhs, in);
 }
 template void Engine::smooth_apply<double>(int, const C<double> *, C<double> *, int, bool);
