@@ -13,6 +13,8 @@
 #include "fixed.cuh"
 #include "kernels.h"
 
+#include <type_traits>
+
 namespace mg {
 
 namespace {
@@ -277,55 +279,57 @@ __global__ void __launch_bounds__(kWgradThreads) glayer_wgrad_kernel(const C<T> 
   __shared__ double sh[OG][32][NW];
   const int ch = blockIdx.y / 9, h = blockIdx.y % 9, o0 = blockIdx.z * OG;
   const int64_t n = g.n();
-  C<T> acc[OG][16];
-#pragma unroll
-  for (int q = 0; q < OG; ++q)
-#pragma unroll
-    for (int k = 0; k < 16; ++k) acc[q][k] = mk<T>((T)0, (T)0);
-  const int beg = blockIdx.x * chunk, end = min(g.V, beg + chunk);
-  for (int s = beg + threadIdx.x; s < end; s += blockDim.x) {
-    int cc[4];
-    g.coords(s, cc);
-    for (int b = 0; b < B; ++b) {
-      C<T> t[12];
-      transported<T>(in + ((int64_t)b * Cin + ch) * n, U, g, s, cc, h, t);
-#pragma unroll
-      for (int q = 0; q < OG; ++q) {
-        if (o0 + q >= Cout) break;
-        const C<T> *gp = gin + ((int64_t)b * Cout + o0 + q) * n;
-        C<T> gv[12];
-        load_fine_site<T>(gp, s, g.V, gv);
-#pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-          for (int sq = 0; sq < 4; ++sq)
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-              acc[q][sp * 4 + sq] = cfmac(t[sq * 3 + a], gv[sp * 3 + a], acc[q][sp * 4 + sq]);  // g conj(t)
-      }
-    }
-  }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  // FP32: a thread's sums run over 16 sites of every sample, then go on in FP64
+  // (16 x 128 of the 4096 sites that a block takes above 2^18)
+  constexpr int kSub = 16 * kWgradThreads;
+  const int beg = blockIdx.x * chunk, end = min(g.V, beg + chunk);
+  double mine[OG];
 #pragma unroll
-  for (int q = 0; q < OG; ++q) {
-    if constexpr (sizeof(T) == 4) {
-      fx::WarpSumF ws;
+  for (int q = 0; q < OG; ++q) mine[q] = 0.0;
+#pragma unroll 1
+  for (int sub = beg, last; sub < end; sub = last) {
+    last = sizeof(T) == 4 ? min(sub + kSub, end) : end;
+    C<T> acc[OG][16];
+#pragma unroll
+    for (int q = 0; q < OG; ++q)
+#pragma unroll
+      for (int k = 0; k < 16; ++k) acc[q][k] = mk<T>((T)0, (T)0);
+    for (int s = sub + threadIdx.x; s < last; s += blockDim.x) {
+      int cc[4];
+      g.coords(s, cc);
+      for (int b = 0; b < B; ++b) {
+        C<T> t[12];
+        transported<T>(in + ((int64_t)b * Cin + ch) * n, U, g, s, cc, h, t);
+#pragma unroll
+        for (int q = 0; q < OG; ++q) {
+          if (o0 + q >= Cout) break;
+          const C<T> *gp = gin + ((int64_t)b * Cout + o0 + q) * n;
+          C<T> gv[12];
+          load_fine_site<T>(gp, s, g.V, gv);
+#pragma unroll
+          for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+            for (int sq = 0; sq < 4; ++sq)
+#pragma unroll
+              for (int a = 0; a < 3; ++a)
+                acc[q][sp * 4 + sq] = cfmac(t[sq * 3 + a], gv[sp * 3 + a], acc[q][sp * 4 + sq]);  // g conj(t)
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < OG; ++q) {
+      std::conditional_t<sizeof(T) == 4, fx::WarpSumF, fx::WarpSumD> ws;
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         ws.add(2 * k, acc[q][k].x);
         ws.add(2 * k + 1, acc[q][k].y);
       }
-      sh[q][l][w] = ws.get();
-    } else {
-      fx::WarpSumD ws;
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        ws.add(2 * k, acc[q][k].x);
-        ws.add(2 * k + 1, acc[q][k].y);
-      }
-      sh[q][l][w] = ws.get();
+      mine[q] += ws.get();
     }
   }
+#pragma unroll
+  for (int q = 0; q < OG; ++q) sh[q][l][w] = mine[q];
   __syncthreads();
   for (int e = threadIdx.x; e < OG * 32; e += blockDim.x) {
     const int q = e >> 5, v = e & 31;
