@@ -88,6 +88,14 @@ __device__ __forceinline__ double scaled(double v, int e) {
   return e > -1000 && e < 1000 ? v * __longlong_as_double((long long)(e + 1023) << 52) : scalbn(v, e);
 }
 
+// the sum over a warp of values some of which are Inf or NaN
+__device__ __forceinline__ double warp_bad(double p) {
+  const double inf = __longlong_as_double(0x7ff0000000000000ll);
+  const bool pos = __any_sync(0xffffffffu, p == inf), neg = __any_sync(0xffffffffu, p == -inf);
+  const bool nan = __any_sync(0xffffffffu, p != p) || (pos && neg);
+  return nan ? __longlong_as_double(0x7ff8000000000000ll) : pos ? inf : -inf;
+}
+
 // ---- exact sums over a warp.  Every lane calls add() for value 0, 1, ... in
 // turn; get() then gives lane v the sum of value v.
 //
@@ -105,8 +113,9 @@ struct WarpSumF {
     const int s = min(max(E, 1) - x, 60);
     long long X = (long long)(((unsigned long long)m << 27) >> s);
     X = (int)b < 0 ? -X : X;
-    const unsigned l = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
+    unsigned l = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
     const int h = __reduce_add_sync(0xffffffffu, (int)(X >> 26));
+    if (E == 0xff) l = __float_as_uint((float)warp_bad(p));
     if ((int)(threadIdx.x & 31) == v) {
       lo = l;
       hi = h;
@@ -115,7 +124,7 @@ struct WarpSumF {
   }
   __device__ __forceinline__ double get() const {
     const double d = scaled((double)(((long long)hi << 26) + lo), max(e, 1) - (127 + 23 + 27));
-    return e == 0xff ? __longlong_as_double(0x7ff8000000000000ll) : d;
+    return e == 0xff ? (double)__uint_as_float(lo) : d;
   }
 };
 // 64-bit integers in units of 2^unit (the same in every lane): three words
@@ -142,10 +151,16 @@ struct WarpSumI {
 __device__ __forceinline__ int warp_exp(int e) { return max(__reduce_max_sync(0xffffffffu, e), 1); }
 // the sum over a warp's lanes of FP64 values, value v to lane v
 struct WarpSumD : WarpSumI {
+  double bad = 0.0;
   __device__ __forceinline__ void add(int v, double p) {
     const int E = max(__reduce_max_sync(0xffffffffu, exp_field(p)), 1);
     WarpSumI::add(v, to_fixed(p, min(E, kBadExp - 1)), E - 1022 - kVecBits, E == kBadExp);
+    if (E == kBadExp) {
+      const double b = warp_bad(p);
+      if ((int)(threadIdx.x & 31) == v) bad = b;
+    }
   }
+  __device__ __forceinline__ double get() const { return e == 1 << 20 ? bad : WarpSumI::get(); }
 };
 // the sum of n FP64 values by one warp, in lane 0: the 256 values of a step are
 // added as integers in the unit of their largest (one by one in FP64, the 256
@@ -162,11 +177,17 @@ __device__ __forceinline__ double warp_total(const double *__restrict__ p, int n
 #pragma unroll
     for (int u = 0; u < U; ++u) E = max(E, exp_field(x[u]));
     E = __reduce_max_sync(0xffffffffu, E);
+    if (E == kBadExp) {
+      double bad = 0.0;
+      for (int u = 0; u < U; ++u) bad += exp_field(x[u]) == kBadExp ? x[u] : 0.0;
+      t += warp_bad(bad);
+      continue;
+    }
     long long X = 0;  // 8 values below 2^kVecBits
 #pragma unroll
-    for (int u = 0; u < U; ++u) X += to_fixed(x[u], min(E, kBadExp - 1));
+    for (int u = 0; u < U; ++u) X += to_fixed(x[u], E);
     WarpSumI ws;
-    ws.add(0, X, E - 1022 - kVecBits, E == kBadExp);
+    ws.add(0, X, E - 1022 - kVecBits, false);
     t += ws.get();
   }
   return t;

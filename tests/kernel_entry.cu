@@ -3,6 +3,8 @@
 // the weight gradient of csrc/kernels_learned.cu.
 #include "kernels.h"
 
+#include <vector>
+
 using namespace mg;
 
 namespace {
@@ -67,6 +69,29 @@ int k_multi_axpy(int fp32, const void *V, int64_t vstride, int k, void *w, int64
     if (fp32) multi_axpy<float>(in<float>(V), vstride, k, static_cast<float2 *>(w), n, nrhs, h, k, sign, 0, nrm, t.s);
     else multi_axpy<double>(in<double>(V), vstride, k, static_cast<double2 *>(w), n, nrhs, h, k, sign, 0, nrm, t.s);
     MG_CUDA(cudaDeviceSynchronize());
+  });
+}
+
+// FP32 coarse operator of 32 dofs per site whose only block is `diag` times the
+// identity at every site, and its dots with the input
+int k_site_dots(const void *x, void *y, float diag, int V, int nrhs, double2 *qx, double2 *qq) {
+  return run([&] {
+    Geom g{{V, 1, 1, 1}, V, 32};
+    if (!stencil_rows_supported(g, nrhs)) throw Error(1, "not supported");
+    std::vector<double2> A((size_t)V * 9 * 1024, make_double2(0.0, 0.0));
+    for (int X = 0; X < V; ++X)
+      for (int i = 0; i < 32; ++i) A[((size_t)X * 9 * 32 + i) * 32 + i].x = diag;
+    double2 *Ad;
+    float4 *AR;
+    MG_CUDA(cudaMalloc(&Ad, A.size() * sizeof(double2)));
+    MG_CUDA(cudaMalloc(&AR, A.size() * sizeof(float2)));
+    MG_CUDA(cudaMemcpy(Ad, A.data(), A.size() * sizeof(double2), cudaMemcpyHostToDevice));
+    stencil_to_rows(Ad, AR, (int64_t)A.size(), 0);
+    Scratch t(stencil_dots_scratch(g, nrhs));
+    stencil_apply_rows_dots(in<float>(x), static_cast<float2 *>(y), AR, g, nrhs, t.s, qx, qq, 0);
+    MG_CUDA(cudaDeviceSynchronize());
+    cudaFree(Ad);
+    cudaFree(AR);
   });
 }
 

@@ -38,3 +38,41 @@ def test_fp32_chain(n):
     V = torch.stack([a, 1j * a])
     assert L.k_multi_dot(1, ptr(V), n, 2, ptr(a), n, 1, ptr(out)) == 0
     assert abs(complex(out[0]) - want) <= bound and abs(complex(out[1]) + 1j * want) <= bound
+
+
+def test_fp32_infinite_sums():
+    """A sum that leaves the range of FP32, or takes in an infinite entry, is
+    infinite; only sums of both signs and of NaN are NaN."""
+    L = kernels()
+    n = 5000
+    a = torch.ones(n, dtype=torch.complex64, device='cuda')
+    out = _out(4)
+    for bad, j in ((1e30, 17), (float('inf'), 4321)):
+        q = a.clone()
+        q[j] = bad
+        assert L.k_dot_qr(1, ptr(q), ptr(q), n, 1, ptr(out), ptr(out[1:])) == 0
+        assert out[1].real == float('inf')
+        w = q.clone()
+        h = _out(1)
+        assert L.k_multi_axpy(1, ptr(a), n, 1, ptr(w), n, 1, ptr(h), 1.0, ptr(out)) == 0
+        assert out[0].real == float('inf')
+    x, y = a.clone(), a.clone()
+    x[3], y[3] = 1e30, -1e30
+    assert L.k_dot(1, ptr(x), ptr(y), n, 1, ptr(out)) == 0
+    assert out[0].real == float('-inf') and out[0].imag == 0.0
+    x[4], y[4] = 1e30, 1e30  # the same warp, another thread
+    x[7], y[7] = 1e30, 1e30
+    assert L.k_dot(1, ptr(x), ptr(y), n, 1, ptr(out)) == 0
+    assert torch.isnan(out[0].real)
+
+
+@pytest.mark.parametrize('nrhs', [1, 4, 7])
+def test_site_stencil_infinite_sums(nrhs):
+    V = 300
+    x = torch.ones(nrhs, V, 32, dtype=torch.complex64, device='cuda')
+    x[0, 299, 5] = 1e30
+    y, qx, qq = torch.empty_like(x), _out(nrhs), _out(nrhs)
+    assert kernels().k_site_dots(ptr(x), ptr(y), 2.0, V, nrhs, ptr(qx), ptr(qq)) == 0
+    assert qx[0].real == float('inf') and qq[0].real == float('inf')
+    for r in range(1, nrhs):
+        assert qx[r] == 2.0 * 32 * V and qq[r] == 4.0 * 32 * V
