@@ -62,6 +62,19 @@ template <int BITS = kVecBits> FX_HD int64_t to_fixed(double v, int E) {
   return (x ^ sg) - sg;
 }
 
+// the same to nearest, BITS <= 61; |result| <= 2^BITS
+template <int BITS = kVecBits> FX_HD int64_t to_nearest(double v, int E) {
+  const int64_t b = bits_of(v);
+  int e = (int)((b >> 52) & 0x7ff);
+  const uint64_t m = ((uint64_t)b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
+  if (e == 0) e = 1;
+  int s = E - e + 63 - BITS;  // >= 2
+  if (s > 64) s = 64;
+  const int64_t x = (int64_t)((((m << 10) >> (s - 1)) + 1) >> 1);
+  const int64_t sg = b >> 63;
+  return (x ^ sg) - sg;
+}
+
 // centred digits of X: X = hi(X) 2^28 + lo(X), -2^27 <= lo < 2^27
 FX_HD int digit_lo(int64_t X) { return (int)((uint32_t)X << 4) >> 4; }
 FX_HD int digit_hi(int64_t X) { return (int)((X + (1 << (kDigit - 1))) >> kDigit); }
@@ -127,11 +140,14 @@ struct WarpSumF {
     return e == 0xff ? (double)__uint_as_float(lo) : d;
   }
 };
-// 64-bit integers in units of 2^unit (the same in every lane): three words
+// 64-bit integers in units of 2^unit (the same in every lane): three words.
+// add() returns, in every lane, whether the sum is below 2^kSmallBits (or just
+// above it).
+constexpr int kSmallBits = 2 * kVecBits - 2 * kDigit - 4;
 struct WarpSumI {
   unsigned w0 = 0, w1 = 0;
   int w2 = 0, e = 0;
-  __device__ __forceinline__ void add(int v, long long X, int unit, bool bad) {
+  __device__ __forceinline__ bool add(int v, long long X, int unit) {
     const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
     const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(X >> 26) & 0x3ffffffu);
     const int c = __reduce_add_sync(0xffffffffu, (int)(X >> 52));
@@ -139,12 +155,14 @@ struct WarpSumI {
       w0 = a;
       w1 = b;
       w2 = c;
-      e = bad ? 1 << 20 : unit;
+      e = unit;
     }
+    // the lower words add 0 .. 31 units of 2^52
+    constexpr int t = 1 << (kSmallBits - 52);
+    return (unsigned)(c + (int)(b >> 26) + t) < 2u * t;
   }
   __device__ __forceinline__ double get() const {
-    const double d = fma((double)w2, 0x1p52, (double)(((long long)w1 << 26) + w0));
-    return e == 1 << 20 ? __longlong_as_double(0x7ff8000000000000ll) : scaled(d, e);
+    return scaled(fma((double)w2, 0x1p52, (double)(((long long)w1 << 26) + w0)), e);
   }
 };
 
@@ -154,7 +172,7 @@ struct WarpSumD : WarpSumI {
   double bad = 0.0;
   __device__ __forceinline__ void add(int v, double p) {
     const int E = max(__reduce_max_sync(0xffffffffu, exp_field(p)), 1);
-    WarpSumI::add(v, to_fixed(p, min(E, kBadExp - 1)), E - 1022 - kVecBits, E == kBadExp);
+    WarpSumI::add(v, to_fixed(p, min(E, kBadExp - 1)), E == kBadExp ? 1 << 20 : E - 1022 - kVecBits);
     if (E == kBadExp) {
       const double b = warp_bad(p);
       if ((int)(threadIdx.x & 31) == v) bad = b;
@@ -187,13 +205,13 @@ __device__ __forceinline__ double warp_total(const double *__restrict__ p, int n
 #pragma unroll
     for (int u = 0; u < U; ++u) X += to_fixed(x[u], E);
     WarpSumI ws;
-    ws.add(0, X, E - 1022 - kVecBits, false);
+    ws.add(0, X, E - 1022 - kVecBits);
     t += ws.get();
   }
   return t;
 }
 __device__ __forceinline__ int4 digits(double2 v, int E) {
-  const long long a = to_fixed(v.x, E), b = to_fixed(v.y, E);
+  const long long a = to_nearest(v.x, E), b = to_nearest(v.y, E);
   return make_int4(digit_hi(a), digit_lo(a), digit_hi(b), digit_lo(b));
 }
 #endif

@@ -255,6 +255,34 @@ __global__ void __launch_bounds__(RB) dot_f32_ring_kernel(const int4 *__restrict
     reinterpret_cast<double *>(out + r * ldh + j0)[threadIdx.x] = s;
 }
 
+// What a group of 128 entries (one warp's of a step) adds to an FP64 dot product
+// is kept in fixed point only where it is at least 2^-4 of the product S of the
+// two scales, in its real or imaginary part.  Then the group's sum of |x y| is
+// at least that, and what the digits lose, 256 products x (2 x 2^-58 + 2^-60) S
+// at most, is within 2^-44.8 of it: the bound of the 256 FP64 additions, 2^-45.
+// Any other group (large entries of one vector meet only small or no ones of
+// the other; Inf or NaN) is added in FP64, out of line: 0.1 to 1% of the groups
+// of normal vectors.  The groups where one vector is zero are not among them.
+// t: the group's sums so far (lane v: value v); bits of redo: the vectors.
+__device__ __noinline__ double redo_groups(double t, unsigned redo, const double2 *__restrict__ x, int64_t xstride,
+                                           const double2 *__restrict__ y, int64_t i0, int64_t end) {
+  const int lane = threadIdx.x & 31;
+  for (; redo; redo &= redo - 1) {
+    const int j = __ffs(redo) - 1;
+    double sr = 0.0, si = 0.0;
+    for (int64_t i = i0; i < min(end, i0 + 4 * RB); i += RB) {
+      const double2 a = x[j * xstride + i], c = y[i];
+      sr = fma(a.x, c.x, fma(a.y, c.y, sr));
+      si = fma(a.x, c.y, fma(-a.y, c.x, si));
+    }
+    fx::WarpSumD ws;
+    ws.add(2 * j, sr);
+    ws.add(2 * j + 1, si);
+    if (lane >> 1 == j) t = ws.get();
+  }
+  return t;
+}
+
 // The same for FP64 vectors on the integer pipe: every warp scales its 128
 // elements of y and of each x_j by their own largest entry; 12 integer
 // multiply-adds per element and vector, exact sums, one conversion per warp,
@@ -281,12 +309,15 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
       a[u] = i0 + RB * u < end ? __ldg(yr + i0 + RB * u) : zero;
       Ey = max(Ey, exp2of(a[u]));
     }
-    Ey = warp_exp(Ey);
+    Ey = __reduce_max_sync(0xffffffffu, Ey);
+    const bool ny = Ey > 0;  // y is not zero here
+    Ey = max(Ey, 1);
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = digits(a[u], min(Ey, fx::kBadExp - 1));
 #pragma unroll
     for (int u = 0; u < U; ++u) a[u] = i0 + RB * u < end ? __ldg(xr + i0 + RB * u) : zero;
     WarpSumI ws;
+    unsigned redo = 0;
 #pragma unroll
     for (int j = 0; j < JG; ++j) {
       if (j < kg) {
@@ -302,19 +333,22 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
           for (int u = 0; u < U; ++u)
             a[u] = i0 + RB * u < end ? __ldg(xr + (j + 1) * xstride + i0 + RB * u) : zero;
         }
-        Ex = warp_exp(Ex);
+        Ex = __reduce_max_sync(0xffffffffu, Ex);
+        const bool nx = Ex > 0;
+        Ex = max(Ex, 1);
         long long hr = 0, hi = 0, mr = 0, mi = 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           macc(digits(b[u], min(Ex, fx::kBadExp - 1)), c[u], hr, hi, mr, mi);
         }
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
-        const bool bad = Ex == fx::kBadExp || Ey == fx::kBadExp;
-        ws.add(2 * j, fx::fold(hr, mr), e, bad);
-        ws.add(2 * j + 1, fx::fold(hi, mi), e, bad);
+        const bool small = ws.add(2 * j, fx::fold(hr, mr), e) & ws.add(2 * j + 1, fx::fold(hi, mi), e);
+        if (Ex == fx::kBadExp || Ey == fx::kBadExp || (small && nx && ny)) redo |= 1u << j;
       }
     }
-    acc += ws.get();
+    double t = ws.get();
+    if (redo) t = redo_groups(t, redo, xr, xstride, yr, i0, end);
+    acc += t;
   }
   double s;
   const int64_t g = (int64_t)r * gridDim.z + blockIdx.z;
@@ -363,10 +397,40 @@ __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2
   }
 }
 
+// an entry of a digit vector; ev: the exponent field of its tile's unit, kBadExp
+// for a tile with Inf or NaN
+__device__ __forceinline__ double2 from_digits(int4 q, int ev) {
+  if (ev == fx::kBadExp) return make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+  const int e = max(ev, 1) - 1022 - fx::kVecBits;
+  return make_double2(scalbn((double)(((long long)q.x << fx::kDigit) + q.y), e),
+                      scalbn((double)(((long long)q.z << fx::kDigit) + q.w), e));
+}
+
+// redo_groups with the vectors as digits (ev: their tiles' exponents, es apart)
+__device__ __noinline__ double redo_digits(double t, unsigned redo, const int4 *__restrict__ x,
+                                           const short *__restrict__ ev, int64_t es, int64_t xstride,
+                                           const double2 *__restrict__ y, int64_t i0, int64_t end) {
+  const int lane = threadIdx.x & 31;
+  for (; redo; redo &= redo - 1) {
+    const int j = __ffs(redo) - 1;
+    double sr = 0.0, si = 0.0;
+    for (int64_t i = i0; i < min(end, i0 + kTile); i += RB) {
+      const double2 a = from_digits(x[j * xstride + i], ev[j * es]), c = y[i];
+      sr = fma(a.x, c.x, fma(a.y, c.y, sr));
+      si = fma(a.x, c.y, fma(-a.y, c.x, si));
+    }
+    fx::WarpSumD ws;
+    ws.add(2 * j, sr);
+    ws.add(2 * j + 1, si);
+    if (lane >> 1 == j) t = ws.get();
+  }
+  return t;
+}
+
 // dot_f64_kernel with the vectors x_j as digits (ev: their tiles' exponents,
 // [j][r][tile])
 template <int JG>
-__global__ void __launch_bounds__(RB) dot_digits_kernel(const int4 *__restrict__ x, const short *__restrict__ ev,
+__global__ void __launch_bounds__(RB, 3) dot_digits_kernel(const int4 *__restrict__ x, const short *__restrict__ ev,
                                                         int64_t xstride, int k, const double2 *__restrict__ y,
                                                         int64_t n, int64_t chunk, double2 *__restrict__ partial,
                                                         unsigned *__restrict__ ticket, double2 *__restrict__ out,
@@ -396,11 +460,14 @@ __global__ void __launch_bounds__(RB) dot_digits_kernel(const int4 *__restrict__
         a[u] = i0 + RB * u < end ? __ldg(yr + i0 + RB * u) : make_double2(0.0, 0.0);
         Ey = max(Ey, exp2of(a[u]));
       }
-      Ey = warp_exp(Ey);
+      Ey = __reduce_max_sync(0xffffffffu, Ey);
 #pragma unroll
-      for (int u = 0; u < U; ++u) c[u] = digits(a[u], min(Ey, fx::kBadExp - 1));
+      for (int u = 0; u < U; ++u) c[u] = digits(a[u], min(max(Ey, 1), fx::kBadExp - 1));
     }
+    const bool ny = Ey > 0;  // y is not zero here
+    Ey = max(Ey, 1);
     WarpSumI ws;
+    unsigned redo = 0;
 #pragma unroll
     for (int j = 0; j < JG; ++j) {
       if (j < kg) {
@@ -412,12 +479,13 @@ __global__ void __launch_bounds__(RB) dot_digits_kernel(const int4 *__restrict__
         if (j + kRing < kg) ring.fetch(j % kRing, xr + (j + kRing) * xstride + t0, end - t0);
         Ring<kTile>::commit();
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
-        const bool bad = Ex == fx::kBadExp || Ey == fx::kBadExp;
-        ws.add(2 * j, fx::fold(hr, mr), e, bad);
-        ws.add(2 * j + 1, fx::fold(hi, mi), e, bad);
+        const bool small = ws.add(2 * j, fx::fold(hr, mr), e) & ws.add(2 * j + 1, fx::fold(hi, mi), e);
+        if (Ex == fx::kBadExp || Ey == fx::kBadExp || (small && Ex > 1 && ny)) redo |= 1u << j;
       }
     }
-    acc += ws.get();
+    double t = ws.get();
+    if (redo) t = redo_digits(t, redo, xr, ev + ((int64_t)j0 * nrhs + r) * nt + tile, nrhs * nt, xstride, yr, i0, end);
+    acc += t;
   }
   double s;
   const int64_t g = (int64_t)r * gridDim.z + blockIdx.z;
@@ -480,8 +548,11 @@ __global__ void __launch_bounds__(RB) dot_qr_f64_kernel(const double2 *__restric
       Ea = max(Ea, exp2of(a[u]));
       Ec = max(Ec, exp2of(c[u]));
     }
-    Ea = warp_exp(Ea);
-    Ec = warp_exp(Ec);
+    Ea = __reduce_max_sync(0xffffffffu, Ea);
+    Ec = __reduce_max_sync(0xffffffffu, Ec);
+    const bool nz = Ea > 0 && Ec > 0;
+    Ea = max(Ea, 1);
+    Ec = max(Ec, 1);
     long long hr = 0, hi = 0, mr = 0, mi = 0, hq = 0, mq = 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -494,10 +565,19 @@ __global__ void __launch_bounds__(RB) dot_qr_f64_kernel(const double2 *__restric
     const int eq = 2 * fx::kDigit + 2 * Ea - 2 * (1022 + fx::kVecBits);
     const bool ba = Ea == fx::kBadExp, bc = ba || Ec == fx::kBadExp;
     WarpSumI ws;
-    ws.add(0, fx::fold(hr, mr), e, bc);
-    ws.add(1, fx::fold(hi, mi), e, bc);
-    ws.add(2, fx::fold(hq, mq), eq, ba);
-    acc += ws.get();
+    const bool small = ws.add(0, fx::fold(hr, mr), e) & ws.add(1, fx::fold(hi, mi), e);
+    ws.add(2, fx::fold(hq, mq), eq);  // at least 2^-2 of its scale
+    double t = ws.get();
+    const int64_t i0 = t0 + threadIdx.x;
+    if (bc || (small && nz)) {
+      const double p = redo_groups(t, 1u, qr, 0, xr, i0, end);
+      if ((threadIdx.x & 31) < 2) t = p;
+    }
+    if (ba) {
+      const double p = redo_groups(t, 2u, qr, 0, qr, i0, end);  // value 2: the real part
+      if ((threadIdx.x & 31) == 2) t = p;
+    }
+    acc += t;
   }
   double s;
   double *part = reinterpret_cast<double *>(partial) + (int64_t)r * 4 * gridDim.x;
@@ -800,9 +880,17 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
       mq = fx::madw(2 * q.w, q.z, fx::madw(2 * q.y, q.x, mq));
     }
     WarpSumI ws;
-    ws.add(0, fx::fold(hq, mq), 2 * fx::kDigit + 2 * E - 2 * (1022 + fx::kVecBits), E == fx::kBadExp);
+    ws.add(0, fx::fold(hq, mq), 2 * fx::kDigit + 2 * E - 2 * (1022 + fx::kVecBits));
+    double t = ws.get();
+    if (E == fx::kBadExp) {  // acc holds Inf or NaN
+      double q = 0.0;
+      for (int u = 0; u < U; ++u) q = fma(acc[u].x, acc[u].x, fma(acc[u].y, acc[u].y, q));
+      fx::WarpSumD wd;
+      wd.add(0, q);
+      t = wd.get();
+    }
     double s;
-    if (block_finish<4>(ws.get(), partial + (int64_t)r * nt, ticket + r, 1, s) && threadIdx.x == 0)
+    if (block_finish<4>(t, partial + (int64_t)r * nt, ticket + r, 1, s) && threadIdx.x == 0)
       nrm[r] = make_double2(s, 0.0);
   }
 }

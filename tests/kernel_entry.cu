@@ -61,6 +61,26 @@ int k_dot_qr(int fp32, const void *q, const void *r, int64_t n, int nrhs, double
   });
 }
 
+// conj(x) y of FP64 vectors x whose digits are formed first
+int k_multi_dot_digits(const void *V, int k, const void *w, int64_t n, int nrhs, double2 *h) {
+  return run([&] {
+    Scratch t((size_t)reduce_blocks(n) * nrhs * k);
+    DigitBasis b;
+    double *inv;
+    double2 *v;
+    std::vector<double> one(nrhs, 1.0);
+    MG_CUDA(cudaMalloc(&b.v, (size_t)k * nrhs * n * sizeof(int4)));
+    MG_CUDA(cudaMalloc(&b.e, (size_t)k * nrhs * digit_tiles(n) * sizeof(short)));
+    MG_CUDA(cudaMalloc(&v, (size_t)nrhs * n * sizeof(double2)));
+    MG_CUDA(cudaMalloc(&inv, nrhs * sizeof(double)));
+    MG_CUDA(cudaMemcpy(inv, one.data(), nrhs * sizeof(double), cudaMemcpyHostToDevice));
+    for (int j = 0; j < k; ++j) normalise_digits(in<double>(V) + (int64_t)j * nrhs * n, v, b, j, inv, n, nrhs, 0);
+    multi_dot_digits(b, k, in<double>(w), n, nrhs, h, k, t.s, 0);
+    MG_CUDA(cudaDeviceSynchronize());
+    for (void *p : {(void *)b.v, (void *)b.e, (void *)v, (void *)inv}) cudaFree(p);
+  });
+}
+
 // w += sign sum_j h[j] V_j; nrm (may be null): the norms of the result
 int k_multi_axpy(int fp32, const void *V, int64_t vstride, int k, void *w, int64_t n, int nrhs, const double2 *h,
                  double sign, double2 *nrm) {

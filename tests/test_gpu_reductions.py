@@ -76,3 +76,62 @@ def test_site_stencil_infinite_sums(nrhs):
     assert qx[0].real == float('inf') and qq[0].real == float('inf')
     for r in range(1, nrhs):
         assert qx[r] == 2.0 * 32 * V and qq[r] == 4.0 * 32 * V
+
+
+def _exact(x, y):
+    """sum conj(x) y and sum |x||y| over the last axis, in long double."""
+    x, y = x.cpu().numpy().astype(np.clongdouble), y.cpu().numpy().astype(np.clongdouble)
+    return (x.conj() * y).sum(-1), (abs(x) * abs(y)).sum(-1)
+
+
+def _graded(seed, *shape):
+    """x of entries 1 .. 2^-100, y small where x is large: all products about 2^-100."""
+    r = np.random.default_rng(seed)
+    e = r.integers(0, 101, shape)
+    cn = lambda: r.standard_normal(shape) + 1j * r.standard_normal(shape)  # noqa: E731
+    to = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    return to(cn() * 2.0 ** -e), to(cn() * 2.0 ** (e - 100.0))
+
+
+# n below and above a step of a block (1024), a warp's group ending raggedly;
+# vectors read one, up to four and up to eight at a time
+@pytest.mark.parametrize('n,k', [(1, 1), (100, 2), (1025, 5), (3000, 1), (3000, 3), (3000, 9)])
+def test_fp64_graded_dots(n, k):
+    """Vectors whose large entries meet only small ones of the other, equal
+    ones, and ones with zeros: each sum of n <= 3000 complex products within
+    FP64's bound for it, (256 + 3 steps and blocks) 2^-53 of sum |x||y|, taken
+    as 2^-44."""
+    L = kernels()
+    x, y = _graded(91, 2, n)
+    g = torch.Generator(device='cuda').manual_seed(92)
+    V = torch.randn(k, 2, n, dtype=torch.complex128, device='cuda', generator=g)
+    V[k // 2] = x
+    V[0, :, n // 3:] = 0.0
+    h = _out(2 * k)
+    assert L.k_multi_dot(0, ptr(V), 2 * n, k, ptr(y), n, 2, ptr(h)) == 0
+    got = h.cpu().numpy().reshape(2, k).T
+    want, top = _exact(V, y[None])
+    assert np.all(abs(got - want) <= 2.0 ** -44 * top)
+    qq = _out(2)
+    assert L.k_dot_qr(0, ptr(x), ptr(y), n, 2, ptr(h), ptr(qq)) == 0
+    want, top = _exact(x, y)
+    assert np.all(abs(h[:2].cpu().numpy() - want) <= 2.0 ** -44 * top)
+    assert np.all(abs(qq.cpu().numpy() - _exact(x, x)[0]) <= 2.0 ** -44 * _exact(x, x)[1])
+    assert L.k_dot(0, ptr(x), ptr(y), n, 2, ptr(h)) == 0
+    assert np.all(abs(h[:2].cpu().numpy() - want) <= 2.0 ** -44 * top)
+
+
+def test_fp64_infinite_sums():
+    L = kernels()
+    n = 2000
+    x = torch.ones(n, dtype=torch.complex128, device='cuda')
+    y = x.clone()
+    y[1500] = float('inf')
+    h, qq = _out(1), _out(1)
+    assert L.k_dot_qr(0, ptr(y), ptr(y), n, 1, ptr(h), ptr(qq)) == 0
+    assert qq[0].real == float('inf')
+    assert L.k_dot(0, ptr(x), ptr(y), n, 1, ptr(h)) == 0
+    assert h[0].real == float('inf')
+    y[3] = complex(float('nan'), 0.0)
+    assert L.k_dot(0, ptr(x), ptr(y), n, 1, ptr(h)) == 0
+    assert torch.isnan(h[0].real)
