@@ -675,10 +675,14 @@ __global__ void __launch_bounds__(RB) multi_axpy_f32_ring_kernel(const int4 *__r
 // added as integers in the unit of the largest coefficient times entry of
 // the warp's 64 elements, then once to w in FP64.  n = 786 k, 16 right-hand
 // sides, 1 .. 20 vectors: 705 us on average (3.6 TB/s) against 931 us in FP64.
+// The digits lose up to 2^-53 of the group's largest product (16 real products x
+// 2^-57); an element whose own largest is more than 2^-kFar below that, its
+// entries far smaller than its neighbours', is added in FP64 instead: 0.02% of
+// the elements of normal vectors where one coefficient dominates, none else.
 __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__restrict__ V, int64_t vstride, int k,
                                                              double2 *__restrict__ w, int64_t n,
                                                              const double2 *__restrict__ h, int ldh, double sign) {
-  constexpr int JG = 8, U = 2;
+  constexpr int JG = 8, U = 2, kFar = 8;
   __shared__ int4 cd[128];
   __shared__ int ce[128];
   __shared__ double2 coef[128];
@@ -714,18 +718,26 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
           const int64_t i = i0 + (int64_t)u * blockDim.x;
           v[j][u] = j < kg && i < n ? __ldg(Vr + (j0 + j) * vstride + i) : make_double2(0.0, 0.0);
         }
-      int S = 2;  // largest exponent sum of a coefficient and its entries
+      // largest exponent sum of a coefficient and its entries, by element
+      int top[U];
       bool bad = false;
+#pragma unroll
+      for (int u = 0; u < U; ++u) top[u] = 0;
 #pragma unroll
       for (int j = 0; j < JG; ++j) {
         if (j < kg) {
-          int e = 1;
+          bad |= ce[j0 + j] == fx::kBadExp;
 #pragma unroll
-          for (int u = 0; u < U; ++u) e = max(e, exp2of(v[j][u]));
-          bad |= e == fx::kBadExp || ce[j0 + j] == fx::kBadExp;
-          S = max(S, e + ce[j0 + j]);
+          for (int u = 0; u < U; ++u) {
+            const int e = max(exp2of(v[j][u]), 1);
+            bad |= e == fx::kBadExp;
+            if (v[j][u].x != 0.0 || v[j][u].y != 0.0) top[u] = max(top[u], e + ce[j0 + j]);
+          }
         }
       }
+      int S = 2;
+#pragma unroll
+      for (int u = 0; u < U; ++u) S = max(S, top[u]);
       S = __reduce_max_sync(0xffffffffu, S);
       const int ex = S - 2 * (1022 + fx::kVecBits) + 2 * fx::kDigit;
       if (__any_sync(0xffffffffu, bad) || ex < -1000 || ex > 900) {
@@ -755,6 +767,12 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
       const double f = __longlong_as_double((long long)(ex + 1023) << 52);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
+        if (top[u] && S - top[u] > kFar) {
+#pragma unroll
+          for (int j = 0; j < JG; ++j)
+            if (j < kg) acc[u] = cfma(coef[j0 + j], v[j][u], acc[u]);
+          continue;
+        }
         acc[u].x = fma(f, (double)fx::fold(hr[u], mr[u]), acc[u].x);
         acc[u].y = fma(f, (double)fx::fold(hi[u], mi[u]), acc[u].y);
       }

@@ -135,3 +135,21 @@ def test_fp64_infinite_sums():
     y[3] = complex(float('nan'), 0.0)
     assert L.k_dot(0, ptr(x), ptr(y), n, 1, ptr(h)) == 0
     assert torch.isnan(h[0].real)
+
+
+# one vector and up to two groups of eight, n below and above the 512 entries of a block
+@pytest.mark.parametrize('n,k', [(1, 1), (100, 3), (700, 8), (1300, 11)])
+def test_fp64_graded_update(n, k):
+    """w -= V h with entries of very different size beside one another: each
+    entry within 2^-44 of its own sum of products (2^(8 - 53) of its largest
+    product, or the rounding of FP64 sums)."""
+    r = np.random.default_rng(93)
+    cn = lambda *s: r.standard_normal(s) + 1j * r.standard_normal(s)  # noqa: E731
+    V = cn(k, 2, n) * 2.0 ** -r.integers(0, 101, (1, 2, n))
+    V[:, :, ::7] = 0.0
+    h, w = cn(2, k), cn(2, n) * 2.0 ** -r.integers(60, 101, (2, n))
+    to = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    wd, Vd, hd = to(w), to(V), to(h)
+    assert kernels().k_multi_axpy(0, ptr(Vd), 2 * n, k, ptr(wd), n, 2, ptr(hd), -1.0, None) == 0
+    P = V.astype(np.clongdouble) * h.T[:, :, None]
+    assert np.all(abs(wd.cpu().numpy() - (w - P.sum(0))) <= 2.0 ** -44 * (abs(P).sum(0) + abs(w)))
