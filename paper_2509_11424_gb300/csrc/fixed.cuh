@@ -113,7 +113,9 @@ __device__ __forceinline__ double warp_bad(double p) {
 // turn; get() then gives lane v the sum of value v.
 //
 // FP32 lanes: integers of 51 bits in the unit of the largest lane's exponent,
-// as two words whose 32-fold sums fit 32 bits.
+// as two words whose 32-fold sums fit 32 bits.  Where bad() says so (in every
+// lane), Inf or NaN were among the values: fix() for each of them, with the
+// same arguments, before get().
 struct WarpSumF {
   unsigned lo = 0;
   int hi = 0, e = 0;
@@ -126,14 +128,19 @@ struct WarpSumF {
     const int s = min(max(E, 1) - x, 60);
     long long X = (long long)(((unsigned long long)m << 27) >> s);
     X = (int)b < 0 ? -X : X;
-    unsigned l = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
+    const unsigned l = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
     const int h = __reduce_add_sync(0xffffffffu, (int)(X >> 26));
-    if (E == 0xff) l = __float_as_uint((float)warp_bad(p));
     if ((int)(threadIdx.x & 31) == v) {
       lo = l;
       hi = h;
       e = E;
     }
+  }
+  __device__ __forceinline__ bool bad() const { return __any_sync(0xffffffffu, e == 0xff); }
+  __device__ __forceinline__ void fix(int v, float p) {
+    if (__shfl_sync(0xffffffffu, e, v) != 0xff) return;
+    const float b = (float)warp_bad((p - p == 0.f) ? 0.0 : (double)p);
+    if ((int)(threadIdx.x & 31) == v) lo = __float_as_uint(b);
   }
   __device__ __forceinline__ double get() const {
     const double d = scaled((double)(((long long)hi << 26) + lo), max(e, 1) - (127 + 23 + 27));
@@ -195,18 +202,19 @@ __device__ __forceinline__ double warp_total(const double *__restrict__ p, int n
 #pragma unroll
     for (int u = 0; u < U; ++u) E = max(E, exp_field(x[u]));
     E = __reduce_max_sync(0xffffffffu, E);
-    if (E == kBadExp) {
-      double bad = 0.0;
-      for (int u = 0; u < U; ++u) bad += exp_field(x[u]) == kBadExp ? x[u] : 0.0;
-      t += warp_bad(bad);
-      continue;
-    }
     long long X = 0;  // 8 values below 2^kVecBits
 #pragma unroll
-    for (int u = 0; u < U; ++u) X += to_fixed(x[u], E);
+    for (int u = 0; u < U; ++u) X += to_fixed(x[u], min(E, kBadExp - 1));
     WarpSumI ws;
     ws.add(0, X, E - 1022 - kVecBits);
-    t += ws.get();
+    double d = ws.get();
+    if (E == kBadExp) {
+      double bad = 0.0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) bad += exp_field(x[u]) == kBadExp ? x[u] : 0.0;
+      d = warp_bad(bad);
+    }
+    t += d;
   }
   return t;
 }

@@ -185,6 +185,15 @@ __global__ void __launch_bounds__(RB) dot_f32_kernel(const float2 *__restrict__ 
       ws.add(2 * j + 1, ai[j]);
     }
   }
+  if (ws.bad()) {
+#pragma unroll
+    for (int j = 0; j < JG; ++j) {
+      if (j < kg) {
+        ws.fix(2 * j, ar[j]);
+        ws.fix(2 * j + 1, ai[j]);
+      }
+    }
+  }
   double s;
   const int64_t g = (int64_t)r * gridDim.z + blockIdx.z;
   double *part = reinterpret_cast<double *>(partial) + ((int64_t)r * k + j0) * 2 * gridDim.x;
@@ -246,6 +255,15 @@ __global__ void __launch_bounds__(RB) dot_f32_ring_kernel(const int4 *__restrict
     if (j < kg) {
       ws.add(2 * j, ar[j]);
       ws.add(2 * j + 1, ai[j]);
+    }
+  }
+  if (ws.bad()) {
+#pragma unroll
+    for (int j = 0; j < JG; ++j) {
+      if (j < kg) {
+        ws.fix(2 * j, ar[j]);
+        ws.fix(2 * j + 1, ai[j]);
+      }
     }
   }
   double s;
@@ -518,6 +536,11 @@ __global__ void __launch_bounds__(RB) dot_qr_f32_kernel(const float2 *__restrict
   ws.add(0, sr);
   ws.add(1, si);
   ws.add(2, sq);
+  if (ws.bad()) {
+    ws.fix(0, sr);
+    ws.fix(1, si);
+    ws.fix(2, sq);
+  }
   double s;
   double *part = reinterpret_cast<double *>(partial) + (int64_t)r * 4 * gridDim.x;
   if (block_finish<4>(ws.get(), part, ticket + r, 3, s) && threadIdx.x < 3) {
@@ -665,6 +688,7 @@ __global__ void __launch_bounds__(RB) multi_axpy_f32_ring_kernel(const int4 *__r
   if constexpr (NORM) {
     WarpSumF ws;
     ws.add(0, q);
+    if (ws.bad()) ws.fix(0, q);
     double s;
     if (block_finish<4>(ws.get(), partial + (int64_t)r * gridDim.x, ticket + r, 1, s) && threadIdx.x == 0)
       nrm[r] = make_double2(s, 0.0);

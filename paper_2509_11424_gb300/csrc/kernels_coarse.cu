@@ -639,13 +639,16 @@ __global__ void __launch_bounds__(288, 2)
     if (2 * rp < nrhs) out[(int64_t)(2 * rp) * n + (int64_t)X * 32 + lane] = make_float2(re.x, im.x);
     if (2 * rp + 1 < nrhs) out[(int64_t)(2 * rp + 1) * n + (int64_t)X * 32 + lane] = make_float2(re.y, im.y);
     if (DOTS) {
+      // conj(q) x, then |q|^2, of both right-hand sides
+      const float p[6] = {fmaf(re.x, x0.x, im.x * x0.z), fmaf(re.x, x0.z, -im.x * x0.x), fmaf(re.x, re.x, im.x * im.x),
+                          fmaf(re.y, x0.y, im.y * x0.w), fmaf(re.y, x0.w, -im.y * x0.y), fmaf(re.y, re.y, im.y * im.y)};
       fx::WarpSumF ws;
-      ws.add(0, fmaf(re.x, x0.x, im.x * x0.z));  // conj(q) x, then |q|^2, of both right-hand sides
-      ws.add(1, fmaf(re.x, x0.z, -im.x * x0.x));
-      ws.add(2, fmaf(re.x, re.x, im.x * im.x));
-      ws.add(3, fmaf(re.y, x0.y, im.y * x0.w));
-      ws.add(4, fmaf(re.y, x0.w, -im.y * x0.y));
-      ws.add(5, fmaf(re.y, re.y, im.y * im.y));
+#pragma unroll
+      for (int k = 0; k < 6; ++k) ws.add(k, p[k]);
+      if (ws.bad()) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) ws.fix(k, p[k]);
+      }
       if (lane < 6) partial[((int64_t)rp * 6 + lane) * g.V + X] = ws.get();
     }
   }

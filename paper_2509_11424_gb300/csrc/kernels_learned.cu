@@ -325,6 +325,15 @@ __global__ void __launch_bounds__(kWgradThreads) glayer_wgrad_kernel(const C<T> 
         ws.add(2 * k, acc[q][k].x);
         ws.add(2 * k + 1, acc[q][k].y);
       }
+      if constexpr (sizeof(T) == 4) {
+        if (ws.bad()) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            ws.fix(2 * k, acc[q][k].x);
+            ws.fix(2 * k + 1, acc[q][k].y);
+          }
+        }
+      }
       mine[q] += ws.get();
     }
   }
