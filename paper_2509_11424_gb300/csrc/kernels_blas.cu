@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
 // conversions took two thirds of the instructions of the kernels above).
 constexpr int kTile = 1024;
 
-// v = w inv[r], its digits and the exponent field of each tile's unit
+// v = w inv[r], its digits and the exponent field of each tile's unit (0 for a
+// tile of zeros)
 __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2 *v, int4 *__restrict__ vf,
                                                        short *__restrict__ ev, const double *__restrict__ inv,
                                                        int64_t n) {
@@ -397,9 +398,9 @@ __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2
   for (int u = 0; u < U; ++u) {
     const int64_t i = i0 + u * RB;
     x[u] = i < n ? cscale(w[r * n + i], f) : make_double2(0.0, 0.0);
-    E = max(E, exp2of(x[u]));
+    if (x[u].x != 0.0 || x[u].y != 0.0) E = max(E, max(exp2of(x[u]), 1));
   }
-  E = warp_exp(E);
+  E = __reduce_max_sync(0xffffffffu, E);
   if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = E;
   __syncthreads();
 #pragma unroll
@@ -410,7 +411,7 @@ __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2
     const int64_t i = i0 + u * RB;
     if (i < n) {
       v[r * n + i] = x[u];
-      vf[r * n + i] = digits(x[u], min(E, fx::kBadExp - 1));
+      vf[r * n + i] = digits(x[u], min(max(E, 1), fx::kBadExp - 1));
     }
   }
 }
@@ -498,7 +499,7 @@ __global__ void __launch_bounds__(RB, 3) dot_digits_kernel(const int4 *__restric
         Ring<kTile>::commit();
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
         const bool small = ws.add(2 * j, fx::fold(hr, mr), e) & ws.add(2 * j + 1, fx::fold(hi, mi), e);
-        if (Ex == fx::kBadExp || Ey == fx::kBadExp || (small && Ex > 1 && ny)) redo |= 1u << j;
+        if (Ex == fx::kBadExp || Ey == fx::kBadExp || (small && Ex > 0 && ny)) redo |= 1u << j;
       }
     }
     double t = ws.get();
@@ -695,6 +696,9 @@ __global__ void __launch_bounds__(RB) multi_axpy_f32_ring_kernel(const int4 *__r
   }
 }
 
+// exponent of a zero coefficient or tile: its products take no part in a scale
+constexpr int kNone = -(1 << 20);
+
 // The same for FP64 vectors on the integer pipe: JG vectors at a time are
 // added as integers in the unit of the largest coefficient times entry of
 // the warp's 64 elements, then once to w in FP64.  n = 786 k, 16 right-hand
@@ -716,7 +720,7 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
     c = make_double2(sign * c.x, sign * c.y);
     const int E = max(exp2of(c), 1);
     coef[j] = c;
-    ce[j] = E;
+    ce[j] = c.x == 0.0 && c.y == 0.0 ? kNone : E;
     cd[j] = digits(c, min(E, fx::kBadExp - 1));
   }
   __syncthreads();
@@ -759,12 +763,14 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
           }
         }
       }
-      int S = 2;
+      int S = 0;
 #pragma unroll
       for (int u = 0; u < U; ++u) S = max(S, top[u]);
       S = __reduce_max_sync(0xffffffffu, S);
       const int ex = S - 2 * (1022 + fx::kVecBits) + 2 * fx::kDigit;
-      if (__any_sync(0xffffffffu, bad) || ex < -1000 || ex > 900) {
+      const bool any_bad = __any_sync(0xffffffffu, bad);
+      if (S == 0 && !any_bad) continue;  // only products with zeros
+      if (any_bad || ex < -1000 || ex > 900) {
 #pragma unroll
         for (int j = 0; j < JG; ++j)
           if (j < kg)
@@ -832,7 +838,7 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
     c = make_double2(sign * c.x, sign * c.y);
     const int E = max(exp2of(c), 1), Ev = ev[((int64_t)j * nrhs + r) * nt + blockIdx.x];
     coef[j] = c;
-    ce[j] = E == fx::kBadExp || Ev == fx::kBadExp ? 1 << 20 : E + Ev;
+    ce[j] = E == fx::kBadExp || Ev == fx::kBadExp ? 1 << 20 : Ev == 0 || (c.x == 0.0 && c.y == 0.0) ? kNone : E + Ev;
     cd[j] = digits(c, min(E, fx::kBadExp - 1));
   }
   __syncthreads();
@@ -851,27 +857,23 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
   for (int u = 0; u < U; ++u) acc[u] = i0 + u * RB < n ? wr[i0 + u * RB] : make_double2(0.0, 0.0);
   for (int j0 = 0; j0 < k; j0 += JG) {
     const int kg = min(JG, k - j0);
-    int S = 2;
+    int S = kNone;
     for (int j = 0; j < kg; ++j) S = max(S, ce[j0 + j]);
     const int ex = S - 2 * (1022 + fx::kVecBits) + 2 * fx::kDigit;
     if (S >= 1 << 20 || ex < -1000 || ex > 900) {
-      // Inf or NaN among them, or products near the ends of the range: in
-      // FP64 from the digits (an entry is then NaN or scaled twice)
+      // only products with zeros; or Inf or NaN among them, or products near the
+      // ends of the range: in FP64 from the digits (an entry is then NaN or
+      // scaled twice).  The ring keeps its order
       for (int j = 0; j < kg; ++j) {
-        // the ring keeps its order
         Ring<kTile>::wait();
-        if (j0 + j + kRing < k) ring.fetch((j0 + j) % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
-        Ring<kTile>::commit();
-        const bool bad = ce[j0 + j] >= 1 << 20;
-        const int Ev = ev[((int64_t)(j0 + j) * nrhs + r) * nt + blockIdx.x] - 1022 - fx::kVecBits;
-        for (int u = 0; u < U; ++u) {
-          if (i0 + u * RB >= n) continue;
-          const int4 q = Vr[(j0 + j) * vs + i0 + u * RB];
-          double2 x = make_double2(scalbn((double)(((long long)q.x << fx::kDigit) + q.y), Ev),
-                                   scalbn((double)(((long long)q.z << fx::kDigit) + q.w), Ev));
-          if (bad) x.x = x.y = __longlong_as_double(0x7ff8000000000000ll);
-          acc[u] = cfma(coef[j0 + j], x, acc[u]);
+        if (S != kNone) {
+          const int Ev = ev[((int64_t)(j0 + j) * nrhs + r) * nt + blockIdx.x];
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (i0 + u * RB < n) acc[u] = cfma(coef[j0 + j], from_digits(ring.get(j % kRing, u), Ev), acc[u]);
         }
+        if (j0 + j + kRing < k) ring.fetch(j % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
+        Ring<kTile>::commit();
       }
       continue;
     }

@@ -3,6 +3,7 @@
 // the weight gradient of csrc/kernels_learned.cu.
 #include "kernels.h"
 
+#include <algorithm>
 #include <vector>
 
 using namespace mg;
@@ -61,10 +62,11 @@ int k_dot_qr(int fp32, const void *q, const void *r, int64_t n, int nrhs, double
   });
 }
 
-// conj(x) y of FP64 vectors x whose digits are formed first
-int k_multi_dot_digits(const void *V, int k, const void *w, int64_t n, int nrhs, double2 *h) {
+// the same for FP64 vectors V held as a Krylov basis: h = V^H w where nothing is
+// to be added (sign 0), else w += sign V h
+int k_basis(const void *V, int k, void *w, int64_t n, int nrhs, double2 *h, double sign, double2 *nrm) {
   return run([&] {
-    Scratch t((size_t)reduce_blocks(n) * nrhs * k);
+    Scratch t(std::max((size_t)reduce_blocks(n) * nrhs * k, (size_t)norm_scratch(n) * nrhs));
     DigitBasis b;
     double *inv;
     double2 *v;
@@ -75,7 +77,8 @@ int k_multi_dot_digits(const void *V, int k, const void *w, int64_t n, int nrhs,
     MG_CUDA(cudaMalloc(&inv, nrhs * sizeof(double)));
     MG_CUDA(cudaMemcpy(inv, one.data(), nrhs * sizeof(double), cudaMemcpyHostToDevice));
     for (int j = 0; j < k; ++j) normalise_digits(in<double>(V) + (int64_t)j * nrhs * n, v, b, j, inv, n, nrhs, 0);
-    multi_dot_digits(b, k, in<double>(w), n, nrhs, h, k, t.s, 0);
+    if (sign == 0.0) multi_dot_digits(b, k, in<double>(w), n, nrhs, h, k, t.s, 0);
+    else multi_axpy_digits(b, k, static_cast<double2 *>(w), n, nrhs, h, k, sign, 0, nrm, t.s);
     MG_CUDA(cudaDeviceSynchronize());
     for (void *p : {(void *)b.v, (void *)b.e, (void *)v, (void *)inv}) cudaFree(p);
   });

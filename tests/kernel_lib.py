@@ -25,7 +25,7 @@ def kernels():
     P, i64, i32, f64 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_double
     L.k_dot.argtypes = [i32, P, P, i64, i32, P]
     L.k_multi_dot.argtypes = [i32, P, i64, i32, P, i64, i32, P]
-    L.k_multi_dot_digits.argtypes = [P, i32, P, i64, i32, P]
+    L.k_basis.argtypes = [P, i32, P, i64, i32, P, f64, P]
     L.k_dot_qr.argtypes = [i32, P, P, i64, i32, P, P]
     L.k_multi_axpy.argtypes = [i32, P, i64, i32, P, i64, i32, P, f64, P]
     L.k_wgrad_f32.argtypes = [P, P, P, P, i32, i32, i32, P]

@@ -153,3 +153,32 @@ def test_fp64_graded_update(n, k):
     assert kernels().k_multi_axpy(0, ptr(Vd), 2 * n, k, ptr(wd), n, 2, ptr(hd), -1.0, None) == 0
     P = V.astype(np.clongdouble) * h.T[:, :, None]
     assert np.all(abs(wd.cpu().numpy() - (w - P.sum(0))) <= 2.0 ** -44 * (abs(P).sum(0) + abs(w)))
+
+
+# below and above a tile of 1024 entries, one group and two groups of eight vectors
+@pytest.mark.parametrize('n,k', [(700, 3), (2500, 8), (2500, 13)])
+@pytest.mark.parametrize('basis', [False, True])
+def test_fp64_update_zeros(n, k, basis):
+    """Right-hand sides all of whose coefficients are zero (one that has
+    converged), groups of them, and vectors that are zero over a whole tile:
+    the update is exact where there is nothing to add and as accurate as ever
+    beside it, with 2^-48 of the largest product for the entries' digits."""
+    r = np.random.default_rng(94)
+    cn = lambda *s: r.standard_normal(s) + 1j * r.standard_normal(s)  # noqa: E731
+    V, h, w = cn(k, 3, n), cn(3, k), cn(3, n)
+    h[0] = 0.0
+    h[1, :8] = 0.0
+    V[:, 2, :1024] = 0.0
+    to = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    wd, Vd, hd, nrm = to(w), to(V), to(h), _out(3)
+    L = kernels()
+    if basis:
+        assert L.k_basis(ptr(Vd), k, ptr(wd), n, 3, ptr(hd), -1.0, ptr(nrm)) == 0
+    else:
+        assert L.k_multi_axpy(0, ptr(Vd), 3 * n, k, ptr(wd), n, 3, ptr(hd), -1.0, ptr(nrm)) == 0
+    got = wd.cpu().numpy()
+    P = V.astype(np.clongdouble) * h.T[:, :, None]
+    want = w - P.sum(0)
+    assert np.array_equal(got[0], w[0]) and np.array_equal(got[2, :1024], w[2, :1024])
+    assert np.all(abs(got - want) <= 2.0 ** -48 * (abs(P).max((0, 2))[:, None] + abs(w)))
+    assert np.allclose(nrm.cpu().numpy().real, (abs(got) ** 2).sum(1), rtol=1e-14, atol=0.0)
