@@ -379,8 +379,13 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
 // much as the FP64 entries), 57 bits of the largest entry of every tile of
 // kTile entries: the vector is converted once, when it is normalised, instead
 // of in each of the four passes of its every later orthogonalisation (the
-// conversions took two thirds of the instructions of the kernels above).
-constexpr int kTile = 1024;
+// conversions took two thirds of the instructions of the kernels above).  A
+// tile with a nonzero entry more than 2^-kFarTile below its largest, or with
+// Inf or NaN, stays as it is in FP64 and is added in FP64; so every entry keeps
+// 45 bits at least and most of them 54 or more.  Normal vectors: 0.05% of their
+// tiles.
+constexpr int kTile = 1024, kFarTile = 12;
+constexpr int kRawTile = -1;  // in place of the exponent field of the unit
 
 // v = w inv[r], its digits and the exponent field of each tile's unit (0 for a
 // tile of zeros)
@@ -388,41 +393,54 @@ __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2
                                                        short *__restrict__ ev, const double *__restrict__ inv,
                                                        int64_t n) {
   constexpr int U = kTile / RB;
-  __shared__ int top[RB / 32];
+  __shared__ int top[RB / 32], low[RB / 32];
   const int r = blockIdx.y;
   const double f = inv[r];
   const int64_t i0 = (int64_t)blockIdx.x * kTile + threadIdx.x;
   double2 x[U];
-  int E = 0;
+  int E = 0, lo = fx::kBadExp;
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int64_t i = i0 + u * RB;
     x[u] = i < n ? cscale(w[r * n + i], f) : make_double2(0.0, 0.0);
-    if (x[u].x != 0.0 || x[u].y != 0.0) E = max(E, max(exp2of(x[u]), 1));
+    if (x[u].x != 0.0 || x[u].y != 0.0) {
+      const int e = max(exp2of(x[u]), 1);
+      E = max(E, e);
+      lo = min(lo, e);
+    }
   }
   E = __reduce_max_sync(0xffffffffu, E);
-  if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = E;
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  if ((threadIdx.x & 31) == 0) {
+    top[threadIdx.x >> 5] = E;
+    low[threadIdx.x >> 5] = lo;
+  }
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < RB / 32; ++q) E = max(E, top[q]);
-  if (threadIdx.x == 0) ev[(int64_t)r * gridDim.x + blockIdx.x] = (short)E;
+  for (int q = 0; q < RB / 32; ++q) {
+    E = max(E, top[q]);
+    lo = min(lo, low[q]);
+  }
+  const bool raw = E == fx::kBadExp || E - lo > kFarTile;
+  if (threadIdx.x == 0) ev[(int64_t)r * gridDim.x + blockIdx.x] = (short)(raw ? kRawTile : E);
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int64_t i = i0 + u * RB;
     if (i < n) {
       v[r * n + i] = x[u];
-      vf[r * n + i] = digits(x[u], min(max(E, 1), fx::kBadExp - 1));
+      vf[r * n + i] = raw ? make_int4(__double2loint(x[u].x), __double2hiint(x[u].x), __double2loint(x[u].y),
+                                      __double2hiint(x[u].y))
+                          : digits(x[u], max(E, 1));
     }
   }
 }
 
-// an entry of a digit vector; ev: the exponent field of its tile's unit, kBadExp
-// for a tile with Inf or NaN
+// an entry of a basis vector; ev: the exponent field of its tile's unit
 __device__ __forceinline__ double2 from_digits(int4 q, int ev) {
-  if (ev == fx::kBadExp) return make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+  if (ev == kRawTile) return make_double2(__hiloint2double(q.y, q.x), __hiloint2double(q.w, q.z));
   const int e = max(ev, 1) - 1022 - fx::kVecBits;
-  return make_double2(scalbn((double)(((long long)q.x << fx::kDigit) + q.y), e),
-                      scalbn((double)(((long long)q.z << fx::kDigit) + q.w), e));
+  return make_double2(fx::scaled((double)(((long long)q.x << fx::kDigit) + q.y), e),
+                      fx::scaled((double)(((long long)q.z << fx::kDigit) + q.w), e));
 }
 
 // redo_groups with the vectors as digits (ev: their tiles' exponents, es apart)
@@ -499,7 +517,7 @@ __global__ void __launch_bounds__(RB, 3) dot_digits_kernel(const int4 *__restric
         Ring<kTile>::commit();
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
         const bool small = ws.add(2 * j, fx::fold(hr, mr), e) & ws.add(2 * j + 1, fx::fold(hi, mi), e);
-        if (Ex == fx::kBadExp || Ey == fx::kBadExp || (small && Ex > 0 && ny)) redo |= 1u << j;
+        if (Ex == kRawTile || Ey == fx::kBadExp || (small && Ex > 0 && ny)) redo |= 1u << j;
       }
     }
     double t = ws.get();
@@ -815,6 +833,9 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
   }
 }
 
+// in place of it: an Inf or NaN coefficient, a coefficient of a tile in FP64
+constexpr int kBadCoef = 1 << 20, kRawCoef = -(1 << 21);
+
 // The same with the vectors as digits: one tile of kTile elements per block,
 // whose units are the vectors' own, so a product is shifted to the largest
 // unit of its group of JG before it is added.  NORM: also nrm[r].x = <w_r, w_r>
@@ -838,7 +859,7 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
     c = make_double2(sign * c.x, sign * c.y);
     const int E = max(exp2of(c), 1), Ev = ev[((int64_t)j * nrhs + r) * nt + blockIdx.x];
     coef[j] = c;
-    ce[j] = E == fx::kBadExp || Ev == fx::kBadExp ? 1 << 20 : Ev == 0 || (c.x == 0.0 && c.y == 0.0) ? kNone : E + Ev;
+    ce[j] = E == fx::kBadExp ? kBadCoef : Ev == kRawTile ? kRawCoef : Ev == 0 || (c.x == 0.0 && c.y == 0.0) ? kNone : E + Ev;
     cd[j] = digits(c, min(E, fx::kBadExp - 1));
   }
   __syncthreads();
@@ -860,17 +881,15 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
     int S = kNone;
     for (int j = 0; j < kg; ++j) S = max(S, ce[j0 + j]);
     const int ex = S - 2 * (1022 + fx::kVecBits) + 2 * fx::kDigit;
-    if (S >= 1 << 20 || ex < -1000 || ex > 900) {
-      // only products with zeros; or Inf or NaN among them, or products near the
-      // ends of the range: in FP64 from the digits (an entry is then NaN or
-      // scaled twice).  The ring keeps its order
+    if (ex < -1000 || ex > 900) {
+      // only products with zeros or tiles in FP64, Inf or NaN coefficients, or
+      // products near the ends of the range: in FP64.  The ring keeps its order
       for (int j = 0; j < kg; ++j) {
         Ring<kTile>::wait();
-        if (S != kNone) {
+        if (ce[j0 + j] != kNone) {
           const int Ev = ev[((int64_t)(j0 + j) * nrhs + r) * nt + blockIdx.x];
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (i0 + u * RB < n) acc[u] = cfma(coef[j0 + j], from_digits(ring.get(j % kRing, u), Ev), acc[u]);
+          for (int u = 0; u < U; ++u) acc[u] = cfma(coef[j0 + j], from_digits(ring.get(j % kRing, u), Ev), acc[u]);
         }
         if (j0 + j + kRing < k) ring.fetch(j % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
         Ring<kTile>::commit();
@@ -886,12 +905,18 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
         const int4 c = cd[j0 + j];
         const int sh = min(S - ce[j0 + j], 63);
         Ring<kTile>::wait();
+        if (ce[j0 + j] != kRawCoef) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          long long hr = 0, hi = 0, mr = 0, mi = 0;
-          mac(c, ring.get(j % kRing, u), hr, hi, mr, mi);  // j0 is a multiple of kRing
-          sr[u] += fx::fold(hr, mr) >> sh;
-          si[u] += fx::fold(hi, mi) >> sh;
+          for (int u = 0; u < U; ++u) {
+            long long hr = 0, hi = 0, mr = 0, mi = 0;
+            mac(c, ring.get(j % kRing, u), hr, hi, mr, mi);  // j0 is a multiple of kRing
+            sr[u] += fx::fold(hr, mr) >> sh;
+            si[u] += fx::fold(hi, mi) >> sh;
+          }
+        } else {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            acc[u] = cfma(coef[j0 + j], from_digits(ring.get(j % kRing, u), kRawTile), acc[u]);
         }
         if (j0 + j + kRing < k) ring.fetch(j % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
         Ring<kTile>::commit();

@@ -182,3 +182,34 @@ def test_fp64_update_zeros(n, k, basis):
     assert np.array_equal(got[0], w[0]) and np.array_equal(got[2, :1024], w[2, :1024])
     assert np.all(abs(got - want) <= 2.0 ** -48 * (abs(P).max((0, 2))[:, None] + abs(w)))
     assert np.allclose(nrm.cpu().numpy().real, (abs(got) ** 2).sum(1), rtol=1e-14, atol=0.0)
+
+
+# below and above a tile of 1024 entries, groups of up to eight vectors
+@pytest.mark.parametrize('n,k', [(1, 1), (700, 3), (2500, 8), (2500, 13)])
+def test_fp64_graded_basis(n, k):
+    """A Krylov basis whose vectors hold entries of very different size beside
+    one another (every third one), zeros, and equally scaled entries, dotted
+    with graded vectors and subtracted from them: dots within FP64's bound (as
+    above), entries of an update within 2^-44 of their own sum of products."""
+    L = kernels()
+    r = np.random.default_rng(95)
+    cn = lambda *s: r.standard_normal(s) + 1j * r.standard_normal(s)  # noqa: E731
+    to = lambda a: torch.from_numpy(a).cuda()  # noqa: E731
+    x, y = _graded(96, 2, n)
+    V = cn(k, 2, n)
+    V[::3] = x.cpu().numpy() * 2.0 ** r.integers(-3, 3, (len(V[::3]), 1, 1))
+    V[k // 2, 0] *= 2.0 ** -700
+    V[:, :, ::5] = 0.0
+    Vd, h = to(V), _out(2 * k)
+    assert L.k_basis(ptr(Vd), k, ptr(y), n, 2, ptr(h), 0.0, None) == 0
+    want, top = _exact(Vd, y[None])
+    assert np.all(abs(h.cpu().numpy().reshape(2, k).T - want) <= 2.0 ** -44 * top)
+    c, w = cn(2, k), cn(2, n) * 2.0 ** -r.integers(60, 101, (2, n))
+    c[1, 1:] = 0.0
+    w[1] *= 2.0 ** -40
+    wd, cd, nrm = to(w), to(c), _out(2)
+    assert L.k_basis(ptr(Vd), k, ptr(wd), n, 2, ptr(cd), -1.0, ptr(nrm)) == 0
+    got = wd.cpu().numpy()
+    P = V.astype(np.clongdouble) * c.T[:, :, None]
+    assert np.all(abs(got - (w - P.sum(0))) <= 2.0 ** -44 * (abs(P).sum(0) + abs(w)))
+    assert np.allclose(nrm.cpu().numpy().real, (abs(got) ** 2).sum(1), rtol=1e-14, atol=0.0)
