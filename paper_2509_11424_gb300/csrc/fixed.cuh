@@ -148,13 +148,11 @@ struct WarpSumF {
   }
 };
 // 64-bit integers in units of 2^unit (the same in every lane): three words.
-// add() returns, in every lane, whether the sum is below 2^kSmallBits (or just
-// above it).
-constexpr int kSmallBits = 2 * kVecBits - 2 * kDigit - 4;
+constexpr int kSmallBits = 2 * kVecBits - 2 * kDigit - 5;
 struct WarpSumI {
   unsigned w0 = 0, w1 = 0;
   int w2 = 0, e = 0;
-  __device__ __forceinline__ bool add(int v, long long X, int unit) {
+  __device__ __forceinline__ void add(int v, long long X, int unit) {
     const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)X & 0x3ffffffu);
     const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(X >> 26) & 0x3ffffffu);
     const int c = __reduce_add_sync(0xffffffffu, (int)(X >> 52));
@@ -164,14 +162,21 @@ struct WarpSumI {
       w2 = c;
       e = unit;
     }
-    // the lower words add 0 .. 31 units of 2^52
+  }
+  // whether the lane's sum is between -2^kSmallBits and 2^kSmallBits
+  __device__ __forceinline__ bool small() const {
     constexpr int t = 1 << (kSmallBits - 52);
-    return (unsigned)(c + (int)(b >> 26) + t) < 2u * t;
+    return (unsigned)(w2 + (int)(w1 >> 26) + t) < 2u * t;
   }
   __device__ __forceinline__ double get() const {
     return scaled(fma((double)w2, 0x1p52, (double)(((long long)w1 << 26) + w0)), e);
   }
 };
+// bit 2 j: pred holds in lanes 2 j and 2 j + 1
+__device__ __forceinline__ unsigned ballot_pairs(bool pred) {
+  const unsigned m = __ballot_sync(0xffffffffu, pred);
+  return m & (m >> 1) & 0x55555555u;
+}
 
 __device__ __forceinline__ int warp_exp(int e) { return max(__reduce_max_sync(0xffffffffu, e), 1); }
 // the sum over a warp's lanes of FP64 values, value v to lane v

@@ -274,19 +274,20 @@ __global__ void __launch_bounds__(RB) dot_f32_ring_kernel(const int4 *__restrict
 }
 
 // What a group of 128 entries (one warp's of a step) adds to an FP64 dot product
-// is kept in fixed point only where it is at least 2^-4 of the product S of the
+// is kept in fixed point only where it is at least 2^-5 of the product S of the
 // two scales, in its real or imaginary part.  Then the group's sum of |x y| is
 // at least that, and what the digits lose, 256 products x (2 x 2^-58 + 2^-60) S
-// at most, is within 2^-44.8 of it: the bound of the 256 FP64 additions, 2^-45.
+// at most, is within 2^-43.8 of it, near the bound of 256 FP64 additions, 2^-45.
 // Any other group (large entries of one vector meet only small or no ones of
-// the other; Inf or NaN) is added in FP64, out of line: 0.1 to 1% of the groups
-// of normal vectors.  The groups where one vector is zero are not among them.
-// t: the group's sums so far (lane v: value v); bits of redo: the vectors.
+// the other; Inf or NaN) is added in FP64, out of line: 0.1% of the groups of a
+// set-up's vectors (below 2^-4: 0.4%, and 3% of the dots' time, since a block
+// waits for its last warp).  Groups where one vector is zero are not among them.
+// t: the group's sums so far (lane v: value v); bits 2 j of redo: the vectors j.
 __device__ __noinline__ double redo_groups(double t, unsigned redo, const double2 *__restrict__ x, int64_t xstride,
                                            const double2 *__restrict__ y, int64_t i0, int64_t end) {
   const int lane = threadIdx.x & 31;
   for (; redo; redo &= redo - 1) {
-    const int j = __ffs(redo) - 1;
+    const int j = (__ffs(redo) - 1) >> 1;
     double sr = 0.0, si = 0.0;
     for (int64_t i = i0; i < min(end, i0 + 4 * RB); i += RB) {
       const double2 a = x[j * xstride + i], c = y[i];
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
 #pragma unroll
     for (int u = 0; u < U; ++u) a[u] = i0 + RB * u < end ? __ldg(xr + i0 + RB * u) : zero;
     WarpSumI ws;
-    unsigned redo = 0;
+    unsigned nz = 0, bad = 0;  // bits 2 j
 #pragma unroll
     for (int j = 0; j < JG; ++j) {
       if (j < kg) {
@@ -352,7 +353,8 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
             a[u] = i0 + RB * u < end ? __ldg(xr + (j + 1) * xstride + i0 + RB * u) : zero;
         }
         Ex = __reduce_max_sync(0xffffffffu, Ex);
-        const bool nx = Ex > 0;
+        nz |= Ex > 0 ? 1u << 2 * j : 0u;
+        bad |= Ex == fx::kBadExp ? 1u << 2 * j : 0u;
         Ex = max(Ex, 1);
         long long hr = 0, hi = 0, mr = 0, mi = 0;
 #pragma unroll
@@ -360,11 +362,13 @@ __global__ void __launch_bounds__(RB) dot_f64_kernel(const double2 *__restrict__
           macc(digits(b[u], min(Ex, fx::kBadExp - 1)), c[u], hr, hi, mr, mi);
         }
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
-        const bool small = ws.add(2 * j, fx::fold(hr, mr), e) & ws.add(2 * j + 1, fx::fold(hi, mi), e);
-        if (Ex == fx::kBadExp || Ey == fx::kBadExp || (small && nx && ny)) redo |= 1u << j;
+        ws.add(2 * j, fx::fold(hr, mr), e);
+        ws.add(2 * j + 1, fx::fold(hi, mi), e);
       }
     }
     double t = ws.get();
+    unsigned redo = bad | (ny ? nz & fx::ballot_pairs(ws.small()) : 0u);
+    if (Ey == fx::kBadExp) redo = 0x55555555u & ((2u << (2 * kg - 1)) - 1u);
     if (redo) t = redo_groups(t, redo, xr, xstride, yr, i0, end);
     acc += t;
   }
@@ -409,6 +413,9 @@ __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2
       lo = min(lo, e);
     }
   }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (i0 + u * RB < n) v[r * n + i0 + u * RB] = x[u];
   E = __reduce_max_sync(0xffffffffu, E);
   lo = __reduce_min_sync(0xffffffffu, lo);
   if ((threadIdx.x & 31) == 0) {
@@ -426,12 +433,10 @@ __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int64_t i = i0 + u * RB;
-    if (i < n) {
-      v[r * n + i] = x[u];
+    if (i < n)
       vf[r * n + i] = raw ? make_int4(__double2loint(x[u].x), __double2hiint(x[u].x), __double2loint(x[u].y),
                                       __double2hiint(x[u].y))
                           : digits(x[u], max(E, 1));
-    }
   }
 }
 
@@ -449,7 +454,7 @@ __device__ __noinline__ double redo_digits(double t, unsigned redo, const int4 *
                                            const double2 *__restrict__ y, int64_t i0, int64_t end) {
   const int lane = threadIdx.x & 31;
   for (; redo; redo &= redo - 1) {
-    const int j = __ffs(redo) - 1;
+    const int j = (__ffs(redo) - 1) >> 1;
     double sr = 0.0, si = 0.0;
     for (int64_t i = i0; i < min(end, i0 + kTile); i += RB) {
       const double2 a = from_digits(x[j * xstride + i], ev[j * es]), c = y[i];
@@ -504,7 +509,6 @@ __global__ void __launch_bounds__(RB, 3) dot_digits_kernel(const int4 *__restric
     const bool ny = Ey > 0;  // y is not zero here
     Ey = max(Ey, 1);
     WarpSumI ws;
-    unsigned redo = 0;
 #pragma unroll
     for (int j = 0; j < JG; ++j) {
       if (j < kg) {
@@ -516,11 +520,16 @@ __global__ void __launch_bounds__(RB, 3) dot_digits_kernel(const int4 *__restric
         if (j + kRing < kg) ring.fetch(j % kRing, xr + (j + kRing) * xstride + t0, end - t0);
         Ring<kTile>::commit();
         const int e = 2 * fx::kDigit + Ex + Ey - 2 * (1022 + fx::kVecBits);
-        const bool small = ws.add(2 * j, fx::fold(hr, mr), e) & ws.add(2 * j + 1, fx::fold(hi, mi), e);
-        if (Ex == kRawTile || Ey == fx::kBadExp || (small && Ex > 0 && ny)) redo |= 1u << j;
+        ws.add(2 * j, fx::fold(hr, mr), e);
+        ws.add(2 * j + 1, fx::fold(hi, mi), e);
       }
     }
     double t = ws.get();
+    // the lane's Ex (0 in the lanes past the last vector, as in a tile of zeros)
+    const int lane = threadIdx.x & 31;
+    const int ex = lane < 2 * kg ? ws.e - (2 * fx::kDigit + Ey - 2 * (1022 + fx::kVecBits)) : 0;
+    const unsigned redo =
+        fx::ballot_pairs(ex == kRawTile || (ex > 0 && ny && ws.small()) || (Ey == fx::kBadExp && lane < 2 * kg));
     if (redo) t = redo_digits(t, redo, xr, ev + ((int64_t)j0 * nrhs + r) * nt + tile, nrhs * nt, xstride, yr, i0, end);
     acc += t;
   }
@@ -607,16 +616,17 @@ __global__ void __launch_bounds__(RB) dot_qr_f64_kernel(const double2 *__restric
     const int eq = 2 * fx::kDigit + 2 * Ea - 2 * (1022 + fx::kVecBits);
     const bool ba = Ea == fx::kBadExp, bc = ba || Ec == fx::kBadExp;
     WarpSumI ws;
-    const bool small = ws.add(0, fx::fold(hr, mr), e) & ws.add(1, fx::fold(hi, mi), e);
+    ws.add(0, fx::fold(hr, mr), e);
+    ws.add(1, fx::fold(hi, mi), e);
     ws.add(2, fx::fold(hq, mq), eq);  // at least 2^-2 of its scale
     double t = ws.get();
     const int64_t i0 = t0 + threadIdx.x;
-    if (bc || (small && nz)) {
+    if (bc || (nz && (fx::ballot_pairs(ws.small()) & 1u))) {
       const double p = redo_groups(t, 1u, qr, 0, xr, i0, end);
       if ((threadIdx.x & 31) < 2) t = p;
     }
     if (ba) {
-      const double p = redo_groups(t, 2u, qr, 0, qr, i0, end);  // value 2: the real part
+      const double p = redo_groups(t, 4u, qr, 0, qr, i0, end);  // value 2: the real part
       if ((threadIdx.x & 31) == 2) t = p;
     }
     acc += t;
@@ -833,8 +843,9 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
   }
 }
 
-// in place of it: an Inf or NaN coefficient, a coefficient of a tile in FP64
-constexpr int kBadCoef = 1 << 20, kRawCoef = -(1 << 21);
+// in place of it: a product that is added in FP64 (tile in FP64, Inf or NaN
+// coefficient, near the ends of the range)
+constexpr int kInFp64 = -(1 << 21);
 
 // The same with the vectors as digits: one tile of kTile elements per block,
 // whose units are the vectors' own, so a product is shifted to the largest
@@ -854,15 +865,18 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
   __shared__ double2 coef[128];
   const int r = blockIdx.y, nrhs = gridDim.y;
   const int64_t nt = gridDim.x;
+  int slow = 0;  // some products are left to FP64 (ce = kInFp64)
   for (int j = threadIdx.x; j < k; j += blockDim.x) {
     double2 c = h[r * ldh + j];
     c = make_double2(sign * c.x, sign * c.y);
     const int E = max(exp2of(c), 1), Ev = ev[((int64_t)j * nrhs + r) * nt + blockIdx.x];
     coef[j] = c;
-    ce[j] = E == fx::kBadExp ? kBadCoef : Ev == kRawTile ? kRawCoef : Ev == 0 || (c.x == 0.0 && c.y == 0.0) ? kNone : E + Ev;
-    cd[j] = digits(c, min(E, fx::kBadExp - 1));
+    const bool fp64 = E == fx::kBadExp || Ev == kRawTile;
+    ce[j] = fp64 ? kInFp64 : Ev == 0 || (c.x == 0.0 && c.y == 0.0) ? kNone : E + Ev;
+    cd[j] = fp64 ? make_int4(0, 0, 0, 0) : digits(c, E);
+    slow |= fp64;
   }
-  __syncthreads();
+  slow = __syncthreads_or(slow);
   const int64_t t0 = (int64_t)blockIdx.x * kTile, i0 = t0 + threadIdx.x;
   double2 *wr = w + r * n;
   const int4 *Vr = V + r * n;
@@ -879,21 +893,19 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
   for (int j0 = 0; j0 < k; j0 += JG) {
     const int kg = min(JG, k - j0);
     int S = kNone;
-    for (int j = 0; j < kg; ++j) S = max(S, ce[j0 + j]);
+    for (int j = 0; j < kg; ++j) S = max(S, ce[j0 + j]);  // kInFp64 is below all
     const int ex = S - 2 * (1022 + fx::kVecBits) + 2 * fx::kDigit;
     if (ex < -1000 || ex > 900) {
-      // only products with zeros or tiles in FP64, Inf or NaN coefficients, or
-      // products near the ends of the range: in FP64.  The ring keeps its order
+      // only products with zeros or left to FP64, as those near the ends of the
+      // range; the ring keeps its order
       for (int j = 0; j < kg; ++j) {
         Ring<kTile>::wait();
-        if (ce[j0 + j] != kNone) {
-          const int Ev = ev[((int64_t)(j0 + j) * nrhs + r) * nt + blockIdx.x];
-#pragma unroll
-          for (int u = 0; u < U; ++u) acc[u] = cfma(coef[j0 + j], from_digits(ring.get(j % kRing, u), Ev), acc[u]);
-        }
         if (j0 + j + kRing < k) ring.fetch(j % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
         Ring<kTile>::commit();
       }
+      __syncthreads();
+      if ((int)threadIdx.x < kg && ce[j0 + threadIdx.x] != kNone) ce[j0 + threadIdx.x] = kInFp64;
+      slow |= S != kNone;
       continue;
     }
     long long sr[U], si[U];
@@ -905,18 +917,12 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
         const int4 c = cd[j0 + j];
         const int sh = min(S - ce[j0 + j], 63);
         Ring<kTile>::wait();
-        if (ce[j0 + j] != kRawCoef) {
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            long long hr = 0, hi = 0, mr = 0, mi = 0;
-            mac(c, ring.get(j % kRing, u), hr, hi, mr, mi);  // j0 is a multiple of kRing
-            sr[u] += fx::fold(hr, mr) >> sh;
-            si[u] += fx::fold(hi, mi) >> sh;
-          }
-        } else {
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            acc[u] = cfma(coef[j0 + j], from_digits(ring.get(j % kRing, u), kRawTile), acc[u]);
+        for (int u = 0; u < U; ++u) {
+          long long hr = 0, hi = 0, mr = 0, mi = 0;
+          mac(c, ring.get(j % kRing, u), hr, hi, mr, mi);  // j0 is a multiple of kRing
+          sr[u] += fx::fold(hr, mr) >> sh;
+          si[u] += fx::fold(hi, mi) >> sh;
         }
         if (j0 + j + kRing < k) ring.fetch(j % kRing, Vr + (j0 + j + kRing) * vs + t0, n - t0);
         Ring<kTile>::commit();
@@ -928,6 +934,17 @@ __global__ void __launch_bounds__(RB) multi_axpy_digits_kernel(const int4 *__res
     for (int u = 0; u < U; ++u) {
       acc[u].x = fma(f, (double)sr[u], acc[u].x);
       acc[u].y = fma(f, (double)si[u], acc[u].y);
+    }
+  }
+  if (slow) {
+    __syncthreads();
+#pragma unroll 1
+    for (int j = 0; j < k; ++j) {
+      if (ce[j] != kInFp64) continue;
+      const int Ev = ev[((int64_t)j * nrhs + r) * nt + blockIdx.x];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * RB < n) acc[u] = cfma(coef[j], from_digits(Vr[j * vs + i0 + u * RB], Ev), acc[u]);
     }
   }
 #pragma unroll
