@@ -46,6 +46,9 @@ FX_HD int64_t bits_of(double v) {
 // below 2^(e - 1022)
 FX_HD int exp_field(double v) { return (int)((bits_of(v) >> 52) & 0x7ff); }
 
+// not +-0, on the integer pipe
+FX_HD bool nonzero(double v) { return ((uint64_t)bits_of(v) << 1) != 0; }
+
 // round toward zero of v 2^(BITS - (E - 1022)), BITS = 53 .. 62; |result| <
 // 2^BITS for every v whose exponent field is at most E (1 <= E < 2047)
 template <int BITS = kVecBits> FX_HD int64_t to_fixed(double v, int E) {

@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(RB) normalise_kernel(const double2 *w, double2
   for (int u = 0; u < U; ++u) {
     const int64_t i = i0 + u * RB;
     x[u] = i < n ? cscale(w[r * n + i], f) : make_double2(0.0, 0.0);
-    if (x[u].x != 0.0 || x[u].y != 0.0) {
+    if (fx::nonzero(x[u].x) || fx::nonzero(x[u].y)) {
       const int e = max(exp2of(x[u]), 1);
       E = max(E, e);
       lo = min(lo, e);
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(256) multi_axpy_f64_kernel(const double2 *__re
           for (int u = 0; u < U; ++u) {
             const int e = max(exp2of(v[j][u]), 1);
             bad |= e == fx::kBadExp;
-            if (v[j][u].x != 0.0 || v[j][u].y != 0.0) top[u] = max(top[u], e + ce[j0 + j]);
+            if (fx::nonzero(v[j][u].x) || fx::nonzero(v[j][u].y)) top[u] = max(top[u], e + ce[j0 + j]);
           }
         }
       }

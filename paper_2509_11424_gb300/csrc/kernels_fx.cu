@@ -220,18 +220,31 @@ void launch(const double2 *in, double2 *out, const int4 *AF, const short *unit, 
 // (integer additions), the link product (12 multiply-adds per complex product
 // on 56- and 57-bit operands), and adds it in the unit of the largest of the
 // nine sites; the result is one conversion per component plus the diagonal
-// term in FP64.  24^4 x 3 right-hand sides: 58 + 480 us, against 1.57 ms of
+// term in FP64.  24^4 x 3 right-hand sides: 62 + 497 us, against 1.57 ms of
 // the FP64 kernel (888 instructions of the FP64 pipe per site, at its rate);
 // the integer pipe is 53% busy, the rest waits for loads (16 warps per SM).
+//
+// An entry keeps 55 bits of the largest of its spinor and, in the sum over the
+// hops, of the largest of the eight neighbours: as many as FP64 sums keep where
+// that entry takes part in the sum.  Where it does not (spinors whose components
+// differ much beside links that do not mix them, a site beside a far larger one)
+// the row's own hop terms are all small: a site with a row whose four forward
+// hops are below 2^-4 of the scale (normal entries: one site in 30 000), or below
+// 2^-23 beside entries below 2^-kFarHop of it, is formed in FP64 instead.  Looking
+// at all eight hops cost 5% of the kernel, at four of them 3%.
 constexpr int kSiteBits = 61;   // stored components
 constexpr int kHopShift = 6;    // of which the link products use 55 bits
+// A link entry of 1 takes the scale to 2^55 (2^56 where no link holds a 1); in
+// units of 2^32
+constexpr int kSmallHop = 1 << (55 - 4 - 32);
+constexpr int kFarHop = 6;
 
 // first entry of site s in the tiled order with N entries per site
 template <int N> __device__ __forceinline__ int64_t tiled(int s) { return (int64_t)(s >> 5) * (N * 32) + (s & 31); }
 inline int64_t tiles(int V) { return (V + 31) / 32; }
 
 __global__ void __launch_bounds__(128) spinor_digits_kernel(const double2 *__restrict__ in,
-                                                            longlong2 *__restrict__ xs, short *__restrict__ ex,
+                                                            longlong2 *__restrict__ xs, short2 *__restrict__ ex,
                                                             int V) {
   __shared__ double2 sh[128 * 13];  // 13: a site's rows fall on different banks
   const int r = blockIdx.y, s0 = blockIdx.x * 128;
@@ -240,19 +253,21 @@ __global__ void __launch_bounds__(128) spinor_digits_kernel(const double2 *__res
   for (int e = threadIdx.x; e < ns * 12; e += 128) sh[e / 12 * 13 + e % 12] = __ldg(p + e);
   __syncthreads();
   if ((int)threadIdx.x >= ns) return;
-  int E = 1;
+  int E = 1, lo = fx::kBadExp;
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     const double2 v = sh[threadIdx.x * 13 + k];
-    E = max(E, max(fx::exp_field(v.x), fx::exp_field(v.y)));
+    const int e = max(fx::exp_field(v.x), fx::exp_field(v.y));
+    E = max(E, e);
+    if (fx::nonzero(v.x) || fx::nonzero(v.y)) lo = min(lo, e);
   }
   const int64_t s = s0 + threadIdx.x;
-  ex[(int64_t)r * V + s] = (short)E;
+  ex[(int64_t)r * V + s] = make_short2((short)E, (short)lo);
   longlong2 *o = xs + r * ((V + 31) / 32) * (int64_t)384 + tiled<12>((int)s);
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     const double2 v = sh[threadIdx.x * 13 + k];
-    o[k * 32] = E < fx::kBadExp ? make_longlong2(fx::to_fixed<kSiteBits>(v.x, E), fx::to_fixed<kSiteBits>(v.y, E))
+    o[k * 32] = E < fx::kBadExp ? make_longlong2(fx::to_nearest<kSiteBits>(v.x, E), fx::to_nearest<kSiteBits>(v.y, E))
                                         : make_longlong2(0, 0);
   }
 }
@@ -281,7 +296,7 @@ __global__ void link_digits_kernel(const double2 *__restrict__ U, int4 *__restri
     const int64_t s = i / 36;
     const int q = (int)(i - s * 36), mu = q / 9;
     const double2 u = U[i];
-    const long long a = fx::to_fixed(u.x, E), b = fx::to_fixed(u.y, E);
+    const long long a = fx::to_nearest(u.x, E), b = fx::to_nearest(u.y, E);
     UF[mu * ((V + 31) / 32) * (int64_t)288 + tiled<9>((int)s) + (q - mu * 9) * 32] = make_int4(fx::digit_hi(a), fx::digit_lo(a), fx::digit_hi(b), fx::digit_lo(b));
   }
 }
@@ -333,8 +348,8 @@ __device__ __forceinline__ int2 hop_digits(long long t) {
   return make_int2((int)(ladd(t, 1ll << (kHopShift + fx::kDigit - 1)) >> 32) >> (kHopShift + fx::kDigit - 32), lo);
 }
 
-// D at a site with an Inf or NaN among the nine spinors, from the spinors and
-// links themselves (out of line: rare)
+// D at a site with Inf or NaN or very different entries among the neighbours,
+// from the spinors and links themselves (out of line: rare)
 __device__ __noinline__ void special_site(const double2 *in, const double2 *U, const Geom &g, int s, double diag,
                                           double2 *o) {
   for (int i = 0; i < 12; ++i) o[i] = cscale(in[(int64_t)s * 12 + i], diag);
@@ -431,9 +446,20 @@ __device__ __forceinline__ void hop_row(const longlong2 *__restrict__ x, int row
   }
 }
 
+// top[k] |= the magnitudes of v[k], in units of 2^32
+__device__ __forceinline__ void largest(int (&top)[3], const longlong2 (&v)[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int x = (int)(v[k].x >> 32), y = (int)(v[k].y >> 32);
+    top[k] |= (x ^ (x >> 31)) | (y ^ (y >> 31));
+  }
+}
+
 // Row A of the eight hops: up (row A of the upper half) and its parts of the
 // lower rows (cross: row 1 - A, from x and y; same: row A, from z and t), in
-// units of the common scale E.
+// units of the common scale E.  Returns the sizes of the terms of up: for the
+// forward hops in x and y, bit k: term k is at least kSmallHop in one of them, bit
+// 4 + k: not zero (both in units of 2^32); the same from bit 8 for z and t.
 //
 // Chiral basis of the other Wilson kernels, B = -i sigma_k, B_4 = 1: row A of
 // u + sg B_mu l takes one row of l, and row A of a product v enters one row
@@ -441,9 +467,11 @@ __device__ __forceinline__ void hop_row(const longlong2 *__restrict__ x, int row
 // with a power of i.  The loop over mu stays rolled: eight unrolled hops for
 // either row are more instructions than the caches hold (5 of 15 cycles per
 // issue went to fetching them).
-__device__ __forceinline__ void hops(const longlong2 *__restrict__ xs, const int4 *__restrict__ UF,
-                                     const short *__restrict__ er, const Geom &g, int s, int A, int E,
+__device__ __forceinline__ unsigned hops(const longlong2 *__restrict__ xs, const int4 *__restrict__ UF,
+                                     const short2 *__restrict__ er, const Geom &g, int s, int A, int E,
                                      longlong2 (&up)[3], longlong2 (&cross)[3], longlong2 (&same)[3]) {
+  int top[3] = {0, 0, 0};
+  unsigned sizes = 0;
   int stride = 1, rest = s;
   const int4 *u = UF;
 #pragma unroll 1
@@ -457,15 +485,16 @@ __device__ __forceinline__ void hops(const longlong2 *__restrict__ xs, const int
     const int pb = mu == 0 ? 3 : mu == 1 ? (A == 0 ? 2 : 0) : mu == 2 ? (A == 0 ? 3 : 1) : 0;
     const int ph = mu == 0 ? 1 : mu == 1 ? (B == 0 ? 0 : 2) : mu == 2 ? (B == 0 ? 1 : 3) : 0;
     longlong2 v[3];
-    hop_row<true>(xs + tiled<12>(sf) + 96 * A, rows, u + tiled<9>(s), (pb + 2) & 3, E - er[sf], v);
+    hop_row<true>(xs + tiled<12>(sf) + 96 * A, rows, u + tiled<9>(s), (pb + 2) & 3, E - er[sf].x, v);
     if (mu == 3 && c + 1 == L) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) v[k] = make_longlong2(-v[k].x, -v[k].y);
     }
+    largest(top, v);
     add3<0, false>(up, v);
     if (mu < 2) add3<false>(cross, v, (ph + 2) & 3);
     else add3<false>(same, v, (ph + 2) & 3);
-    hop_row<false>(xs + tiled<12>(sb) + 96 * A, rows, u + tiled<9>(sb), pb, E - er[sb], v);
+    hop_row<false>(xs + tiled<12>(sb) + 96 * A, rows, u + tiled<9>(sb), pb, E - er[sb].x, v);
     if (mu == 3 && c == 0) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) v[k] = make_longlong2(-v[k].x, -v[k].y);
@@ -476,7 +505,22 @@ __device__ __forceinline__ void hops(const longlong2 *__restrict__ xs, const int
     rest = next;
     stride *= L;
     u += ((g.V + 31) / 32) * (int64_t)288;
+    if (mu & 1) {
+      sizes >>= 8;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        sizes |= (top[k] >= kSmallHop ? 0x100u << k : 0u) | (top[k] ? 0x1000u << k : 0u);
+        top[k] = 0;
+      }
+    }
   }
+  return sizes;
+}
+
+// whether one of a row's three entries is small in all of these hops, or nearly
+// zero in them beside entries that the scale may have lost (far)
+__device__ __forceinline__ bool small_row(unsigned sizes, bool far) {
+  return ((sizes >> 4) & ~sizes & 7u) || (far && (~(sizes >> 4) & 7u));
 }
 
 constexpr int kWilsonSites = 64;  // per block
@@ -488,11 +532,12 @@ constexpr int kWilsonSites = 64;  // per block
 // the 15 loads of a hop in flight without spills (five: 520 us).
 __global__ void __launch_bounds__(2 * kWilsonSites, 4)
     wilson_fx_kernel(const double2 *__restrict__ in, double2 *__restrict__ out, const longlong2 *__restrict__ xs,
-                     const short *__restrict__ ex, const int4 *__restrict__ UF, const double2 *__restrict__ U, Geom g,
+                     const short2 *__restrict__ ex, const int4 *__restrict__ UF, const double2 *__restrict__ U, Geom g,
                      double diag, int EU, int nrhs) {
   constexpr int S = kWilsonSites;
   __shared__ double2 sh[S * 13];
   __shared__ longlong2 other[2][3][S];
+  __shared__ unsigned sizes[2][S];
   // the right-hand side fastest: the blocks of a site range share its links
   const int sb = (int)(blockIdx.x / (unsigned)nrhs), r = (int)(blockIdx.x - (unsigned)sb * nrhs);
   const int half = (int)threadIdx.x / S, ls = (int)threadIdx.x - half * S;
@@ -503,19 +548,29 @@ __global__ void __launch_bounds__(2 * kWilsonSites, 4)
     const double2 *pi = in + ((int64_t)r * V + s0) * 12;
     for (int q = threadIdx.x; q < ns * 12; q += 2 * S) sh[q / 12 * 13 + q % 12] = __ldg(pi + q);
   }
-  const short *er = ex + (int64_t)r * V;
+  const short2 *er = ex + (int64_t)r * V;
   longlong2 up[3], cross[3], same[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) up[k] = cross[k] = same[k] = make_longlong2(0, 0);
-  int E = 1;
+  int E = 1, lo = fx::kBadExp;
 #pragma unroll 1
-  for (int d = 1; d < 9; ++d) E = max(E, (int)er[g.neighbor(s, d)]);
-  hops(xs + r * ((g.V + 31) / 32) * (int64_t)384, UF, er, g, s, half, E, up, cross, same);
+  for (int d = 1; d < 9; ++d) {
+    const short2 e = er[g.neighbor(s, d)];
+    E = max(E, (int)e.x);
+    lo = min(lo, (int)e.y);
+  }
+  const bool far = E - lo > kFarHop;
+  sizes[half][ls] = hops(xs + r * ((g.V + 31) / 32) * (int64_t)384, UF, er, g, s, half, E, up, cross, same);
 #pragma unroll
   for (int k = 0; k < 3; ++k) other[half][k][ls] = cross[k];
   __syncthreads();
   double2 *o = sh + ls * 13 + 3 * half;
-  if (E < fx::kBadExp) {
+  // an upper row takes all eight hops of its half, a lower row z and t of its own
+  // half and x and y of the other
+  const unsigned z0 = sizes[0][ls], z1 = sizes[1][ls];
+  const bool graded = E > 1 && (small_row(z0 | z0 >> 8, far) || small_row(z1 | z1 >> 8, far) ||
+                                small_row(z0 >> 8 | z1, far) || small_row(z1 >> 8 | z0, far));
+  if (E < fx::kBadExp && !graded) {
     // value = diag psi - 1/2 sum 2^(56 + (E - 1022 - 55) + (EU - 1022 - 57))
     const int ea = 2 * fx::kDigit + (E - 1022 - (kSiteBits - kHopShift)) + (EU - 1022 - fx::kVecBits);
     const bool plain = ea > -1000 && ea < 900;
@@ -583,14 +638,14 @@ int wilson_fx_group(int V, int nrhs) {
 }
 size_t wilson_fx_elems(int V, int nrhs) {
   const size_t g = wilson_fx_group(V, nrhs);
-  return g * tiles(V) * 384 + (g * V * sizeof(short) + 15) / 16;
+  return g * tiles(V) * 384 + (g * V * sizeof(short2) + 15) / 16;
 }
 
 void wilson_apply_fx(const double2 *in, double2 *out, const int4 *UF, const double2 *U, int EU, double2 *work, Geom g,
                      double m0, int nrhs, cudaStream_t s) {
   const int grp = wilson_fx_group(g.V, nrhs);
   longlong2 *xs = reinterpret_cast<longlong2 *>(work);
-  short *ex = reinterpret_cast<short *>(xs + (size_t)grp * tiles(g.V) * 384);
+  short2 *ex = reinterpret_cast<short2 *>(xs + (size_t)grp * tiles(g.V) * 384);
   for (int r0 = 0; r0 < nrhs; r0 += grp) {
     const int k = std::min(grp, nrhs - r0);
     const int64_t off = (int64_t)r0 * g.n();
