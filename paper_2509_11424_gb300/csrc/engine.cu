@@ -577,7 +577,7 @@ template <typename T> void Engine::apply_D(int l, const C<T> *in, C<T> *out, int
     // bytes of one complex block entry as stored (BF16 variants: 4)
     double bs = cs;
     if constexpr (sizeof(T) == 8) {
-      stencil_apply_fx(in, out, L.AF, L.AFu, L.g, nrhs, stream);
+      stencil_apply_fx(in, out, L.AF, L.AFu, L.A64, L.g, nrhs, stream);
     } else {
       const int v = stencil_pick(l, nrhs, in, out);
       stencil_run(l, v, in, out, nrhs);

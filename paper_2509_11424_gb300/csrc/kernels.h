@@ -163,10 +163,10 @@ void stencil_apply(const float2 *in, float2 *out, const float2 *AT, Geom g, int 
                    cudaStream_t s);
 // FP64 coarse stencil in fixed point on the integer pipe (fixed.cuh), up to
 // 256 dofs per site: AF, unit from stencil_digits (transposed like AT, 16
-// bytes per entry, one exponent per row)
+// bytes per entry, one exponent per row), A itself for the rows that need FP64
 void stencil_digits(const double2 *A, int4 *AF, short *unit, const Geom &g, cudaStream_t s);
-void stencil_apply_fx(const double2 *in, double2 *out, const int4 *AF, const short *unit, Geom g, int nrhs,
-                      cudaStream_t s);
+void stencil_apply_fx(const double2 *in, double2 *out, const int4 *AF, const short *unit, const double2 *A, Geom g,
+                      int nrhs, cudaStream_t s);
 // Tensor-core (tcgen05 kind::tf32) coarse stencil for 32 dofs per site:
 // ATC holds each site's nine stacked [Re A_d; Im A_d] tiles in the MMA's
 // shared-memory image (stencil_tile_tc builds it from the canonical A);

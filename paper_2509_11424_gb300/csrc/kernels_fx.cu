@@ -39,7 +39,7 @@ __global__ void stencil_digits_kernel(const double2 *__restrict__ A, int4 *__res
     frexp(sum * 1.0001, &es);  // the rounding of the sum above stays below
     u = fx::row_unit(em, es);
   }
-  if (lane == 0) unit[row] = ok ? (short)u : (short)0x7fff;  // an overflowed row gives NaN
+  if (lane == 0) unit[row] = ok ? (short)u : (short)0x7fff;  // a row with Inf or NaN: in FP64
   for (int e = lane; e < 9 * m; e += 32) {
     const int d = e / m, j = e - d * m;
     const double2 a = AX[((int64_t)d * m + i) * m + j];
@@ -52,13 +52,6 @@ __global__ void stencil_digits_kernel(const double2 *__restrict__ A, int4 *__res
   }
 }
 
-// one entry of the operator back as a double pair
-__device__ __forceinline__ double2 entry(int4 a, int u) {
-  return make_double2(scalbn((double)(((long long)a.x << fx::kDigit) + a.y), u),
-                      scalbn((double)(((long long)a.z << fx::kDigit) + a.w), u));
-}
-
-
 // complex product of digits: high and middle sums of the real and imaginary
 // parts
 __device__ __forceinline__ void mac(int4 a, int4 x, long long &hr, long long &hi, long long &mr, long long &mi) {
@@ -69,14 +62,20 @@ __device__ __forceinline__ void mac(int4 a, int4 x, long long &hr, long long &hi
   mi = fx::madw(a.w, x.x, fx::madw(a.z, x.y, fx::madw(a.y, x.z, fx::madw(a.x, x.w, mi))));
 }
 
-// one row for a right-hand side with an Inf or NaN among the neighbours, in
-// FP64 from the operator's digits (out of line: rare)
-__device__ __noinline__ double2 special_row(const double2 *x, const int4 *A, int u, const Geom &g, int X) {
+// one row in FP64 from the operator itself, A[X][d][i][j] of site X and row i, by
+// a whole warp (out of line: rare; a lane by itself took 60 us of load latency)
+__device__ __noinline__ double2 special_row(const double2 *x, const double2 *A, const Geom &g, int X) {
   const int m = g.dof;
   double2 v = make_double2(0.0, 0.0);
+#pragma unroll 3
   for (int d = 0; d < 9; ++d) {
-    const double2 *xn = x + (int64_t)g.neighbor(X, d) * m;
-    for (int j = 0; j < m; ++j) v = cfma(entry(A[((int64_t)d * m + j) * m], u), xn[j], v);
+    const double2 *xn = x + (int64_t)g.neighbor(X, d) * m, *Ad = A + (int64_t)d * m * m;
+    for (int j = threadIdx.x & 31; j < m; j += 32) v = cfma(Ad[j], xn[j], v);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
   }
   return v;
 }
@@ -95,10 +94,20 @@ __device__ __noinline__ double2 special_row(const double2 *x, const int4 *A, int
 // this kernel took 340 us, bound by the FP64 pipe (which now converts one
 // result per row).  Two columns per step with the next two in flight: four
 // with predicates for ragged rows took 88 us.
+//
+// The digits keep 2^-59 of the row's largest entry (2^-62 of its 1-norm) and
+// 2^-58 of a site vector's largest, below what FP64 additions lose where these
+// entries meet.  Where they meet only small or no ones, a row's nine partial sums
+// are all small: a row with none above 2^-12 of |row|_1 max|x| (blocks and
+// vectors of random entries: 2^-8 to 2^-10, 18 numbers), or Inf or NaN, is formed
+// in FP64 from the canonical blocks A instead.  2^-11 takes one row in 10^4 of a
+// diagonally dominant operator and 7 us of the 74.
+constexpr int kSmallRow = 1 << (61 + 57 - 2 * fx::kDigit - 12 - 32);  // in units of 2^32
+
 template <int RG>
 __global__ void __launch_bounds__(288, 2)
     stencil_fx_kernel(const double2 *__restrict__ in, double2 *__restrict__ out, const int4 *__restrict__ AF,
-                      const short *__restrict__ unit, Geom g, int nrhs) {
+                      const short *__restrict__ unit, const double2 *__restrict__ A, Geom g, int nrhs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int emax[9][RG];
   const int m = g.dof;
@@ -134,7 +143,7 @@ __global__ void __launch_bounds__(288, 2)
         if (m > 32 && r < rg) v = __ldg(xd + r * n + j);
         int4 q = make_int4(0, 0, 0, 0);
         if (E < fx::kBadExp) {
-          const long long a = fx::to_fixed(v.x, E), b = fx::to_fixed(v.y, E);
+          const long long a = fx::to_nearest(v.x, E), b = fx::to_nearest(v.y, E);
           q = make_int4(fx::digit_hi(a), fx::digit_lo(a), fx::digit_hi(b), fx::digit_lo(b));
         }
         xq[r * m + j] = q;
@@ -174,40 +183,44 @@ __global__ void __launch_bounds__(288, 2)
 #pragma unroll
   for (int r = 0; r < RG; ++r) part[(d * RG + r) * 32 + lane] = make_longlong2(hr[r], hi[r]);
   __syncthreads();
-  if (d >= rg || i >= m) return;
+  if (d >= rg) return;
   // warp d adds the partial rows of right-hand side d
-  const int r = d, u = unit[(int64_t)X * m + i];
+  const int r = d, u = unit[(int64_t)X * m + (i < m ? i : i0)];
   int E = emax[0][r];
 #pragma unroll
   for (int dd = 1; dd < 9; ++dd) E = max(E, emax[dd][r]);
   double2 v;
-  if (u == 0x7fff) {
-    v = make_double2(nan(""), nan(""));
-  } else if (E < fx::kBadExp) {
-    long long sr = 0, si = 0;
+  long long sr = 0, si = 0;
+  int top = 0;
 #pragma unroll
-    for (int dd = 0; dd < 9; ++dd) {
-      const longlong2 t = part[(dd * RG + r) * 32 + lane];
-      const int sh = min(E - emax[dd][r], 63);
-      sr += t.x >> sh;
-      si += t.y >> sh;
-    }
-    const int e = 2 * fx::kDigit + u + (E - 1022 - fx::kVecBits);
-    v = make_double2(scalbn((double)sr, e), scalbn((double)si, e));
-  } else {
-    v = special_row(in + r * n, AF + (int64_t)X * 9 * m * m + i, u, g, X);
+  for (int dd = 0; dd < 9; ++dd) {
+    const longlong2 t = part[(dd * RG + r) * 32 + lane];
+    const int sh = min(E - emax[dd][r], 63);
+    const long long a = t.x >> sh, b = t.y >> sh;
+    top |= ((int)(a >> 32) ^ (int)(a >> 63)) | ((int)(b >> 32) ^ (int)(b >> 63));
+    sr += a;
+    si += b;
   }
-  out[r * n + (int64_t)X * m + i] = v;
+  const int e = 2 * fx::kDigit + u + (E - 1022 - fx::kVecBits);
+  v = make_double2(scalbn((double)sr, e), scalbn((double)si, e));
+  const bool in_fp64 = u == 0x7fff || E == fx::kBadExp || (top < kSmallRow && E > 1);
+  for (unsigned rows = __ballot_sync(0xffffffffu, i < m && in_fp64); rows; rows &= rows - 1) {
+    const int k = __ffs(rows) - 1;
+    const double2 w = special_row(in + r * n, A + ((int64_t)X * 9 * m + i0 + k) * m, g, X);
+    if (lane == k) v = w;
+  }
+  if (i < m) out[r * n + (int64_t)X * m + i] = v;
 }
 
 template <int RG>
-void launch(const double2 *in, double2 *out, const int4 *AF, const short *unit, Geom g, int nrhs, cudaStream_t s) {
+void launch(const double2 *in, double2 *out, const int4 *AF, const short *unit, const double2 *A, Geom g, int nrhs,
+            cudaStream_t s) {
   const int m = g.dof, ng = (nrhs + RG - 1) / RG;
   const size_t sm = (size_t)9 * RG * (m + 32) * 16;
   if ((int64_t)g.V * ng > 0x7fffffff) throw Error(1, "coarse stencil: too many right-hand sides for one launch");
   smem_optin((const void *)stencil_fx_kernel<RG>, 200 * 1024);
   stencil_fx_kernel<RG>
-      <<<dim3((unsigned)g.V * (unsigned)ng, (m + 31) / 32), 288, sm, s>>>(in, out, AF, unit, g, nrhs);
+      <<<dim3((unsigned)g.V * (unsigned)ng, (m + 31) / 32), 288, sm, s>>>(in, out, AF, unit, A, g, nrhs);
   MG_LAUNCH_CHECK();
 }
 
@@ -603,14 +616,14 @@ void stencil_digits(const double2 *A, int4 *AF, short *unit, const Geom &g, cuda
   MG_LAUNCH_CHECK();
 }
 
-void stencil_apply_fx(const double2 *in, double2 *out, const int4 *AF, const short *unit, Geom g, int nrhs,
-                      cudaStream_t s) {
+void stencil_apply_fx(const double2 *in, double2 *out, const int4 *AF, const short *unit, const double2 *A, Geom g,
+                      int nrhs, cudaStream_t s) {
   // right-hand sides per block: 4 leave room for two blocks per SM; the
   // digits of 4 right-hand sides at 256 dofs fill 166 KB
   if (g.dof > 256) throw Error(1, "coarse stencil: too many dofs per site");
-  if (nrhs == 1) launch<1>(in, out, AF, unit, g, nrhs, s);
-  else if (nrhs == 2) launch<2>(in, out, AF, unit, g, nrhs, s);
-  else launch<4>(in, out, AF, unit, g, nrhs, s);
+  if (nrhs == 1) launch<1>(in, out, AF, unit, A, g, nrhs, s);
+  else if (nrhs == 2) launch<2>(in, out, AF, unit, A, g, nrhs, s);
+  else launch<4>(in, out, AF, unit, A, g, nrhs, s);
 }
 
 size_t link_digits_elems(int V) { return (size_t)tiles(V) * 4 * 288; }

@@ -79,3 +79,71 @@ def test_wilson(dims, links):
     for r in range(5):
         want = Dl @ x[r].astype(np.clongdouble)
         assert np.all(abs(got[r] - want) <= 100 * 2.0 ** -53 * _moduli(U, x[r], -0.3, dims))
+
+
+def _check_coarse(M, ctx, lat, m, kinds, nrhs):
+    """OP_D of level 1 on multiples of each of `kinds`: 9 m complex products an
+    entry, 4 real ones each, of the blocks that the library holds."""
+    V = int(np.prod(lat))
+    blocks = np.zeros(2 * V * 9 * m * m)
+    M.mgmlmc_get_coarse_op(ctx, 1, blocks)
+    blocks = blocks.view(complex).reshape(V, 9, m, m).astype(np.clongdouble)
+    for kind in kinds:
+        y = torch.empty((nrhs, V * m), dtype=torch.complex128, device='cuda')
+        M.mgmlmc_apply(ctx, M.OP_D, 1, M.FP64, dev(np.stack([kind * 2.0 ** k for k in range(nrhs)])), y, nrhs)
+        got = host(y)
+        f = kind.reshape(*lat[::-1], m).astype(np.clongdouble)
+        want, top = 0, 0
+        for d in range(9):
+            nb = f if d == 0 else np.roll(f, -1 if d % 2 else 1, 3 - (d - 1) // 2)
+            nb = nb.reshape(V, 1, m)
+            want = want + (blocks[:, d] * nb).sum(-1)
+            top = top + (abs(blocks[:, d]) * abs(nb)).sum(-1)
+        for r in range(nrhs):
+            assert np.all(abs(got[r] - 2.0 ** r * want.ravel()) <= 36 * m * 2.0 ** -53 * 2.0 ** r * top.ravel())
+
+
+# rows below and above a tile of 32, right-hand sides in groups of 1, 2 and 4
+@pytest.mark.parametrize('ntv,nrhs', [(3, 1), (16, 2), (17, 5)])
+def test_coarse_stencil(ntv, nrhs):
+    """Vectors of graded entries, of one entry per site (columns of the
+    operator), of one site far above the others."""
+    s = Setup((4, 6, 4, 4), [(2, 3, 2, 2)], [ntv], eps=0.4, m0=-0.2, gseed=61, oracle=False)
+    try:
+        m = 2 * ntv
+        n1, rng = 16 * m, np.random.default_rng(73)
+        kinds = np.zeros((3, n1), dtype=complex)
+        kinds[0] = (rng.standard_normal(n1) + 1j * rng.standard_normal(n1)) * 2.0 ** -rng.integers(0, 101, n1)
+        kinds[1, np.arange(16) * m + rng.integers(0, m, 16)] = 2.0 ** -rng.integers(0, 61, 16)
+        kinds[2] = rng.standard_normal(n1) * 2.0 ** -70
+        kinds[2, 5 * m:5 * m + 2] = 1.0
+        _check_coarse(s.M, s.ctx, (2, 2, 2, 2), m, kinds, nrhs)
+    finally:
+        s.close()
+
+
+@pytest.mark.parametrize('nrhs', [1, 3])
+def test_coarse_stencil_decoupled(nrhs):
+    """Unit links and test vectors of one colour each: the operator does not mix
+    them, so a row meets only the entries of its own colour, here 2^-60 and
+    2^-30 of the others'."""
+    M = require_lib()
+    dims = (4, 4, 4, 6)
+    V = dirac.volume(dims)
+    tv = np.zeros((3, V, 4, 3), dtype=complex)
+    rng = np.random.default_rng(74)
+    for k in range(3):
+        tv[k, :, :, k] = rng.standard_normal((V, 4)) + 1j * rng.standard_normal((V, 4))
+    ctx = M.mgmlmc_create(dims, torch.cuda.current_stream())
+    try:
+        M.mgmlmc_set_gauge(ctx, _unit(dims))
+        M.mgmlmc_set_mass(ctx, -0.3)
+        M.mgmlmc_set_test_vectors(ctx, 0, tv.reshape(3, -1).copy(), 3, 12 * V)
+        M.mgmlmc_build_hierarchy(ctx, M.mg_params([(2, 2, 2, 2)], [3], setup_rounds=0))
+        lat = (2, 2, 2, 3)
+        x = rng.standard_normal((24, 2, 3)) + 1j * rng.standard_normal((24, 2, 3))
+        x[..., 1] *= 2.0 ** -60
+        x[..., 2] *= 2.0 ** -30
+        _check_coarse(M, ctx, lat, 6, [x.reshape(-1)], nrhs)
+    finally:
+        M.mgmlmc_destroy(ctx)
