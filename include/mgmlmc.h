@@ -590,9 +590,11 @@ mgmlmc_status mgmlmc_profile_stats(mgmlmc_ctx *ctx, int kernel_class, int64_t *l
  * site, the block's links staged in shared memory by asynchronous copies that
  * overlap the residual load; 1 = with two or more right-hand sides, one
  * thread per site carrying two of them in packed FP32 pairs (.f32x2
- * instructions).  Other cases, and 2 = throughout, the general kernels.  Every variant updates the
- * faces of each colour in a separate pass over that colour's sites, and all
- * compute the same sums in the same order: identical results. */
+ * instructions).  With blocks of 2^4 sites: 0 = a half warp per block and
+ * right-hand side.  Other cases, and 2 = throughout, the general kernels.
+ * Every variant updates the faces of each colour in a separate pass over that
+ * colour's sites, and all compute the same sums in the same order: identical
+ * results. */
 #define MGMLMC_VARIANT_SAP_FP32 2
 /* FP32 restriction P_l^H and prolongation P_l (Sec. 2.2): 0 (default) = P in
  * FP32; 1 = P stored as BF16 (round to nearest, relative error <= 2^-9 per

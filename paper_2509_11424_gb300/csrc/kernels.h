@@ -227,9 +227,9 @@ bool sap_feasible(const Geom &g, const int b[4]);
 template <typename T> size_t sap_smem_bytes(const int b[4], int rs);
 // one red/black sweep: r (residual, exact on exit), z += correction, e scratch;
 // FP32: structure-of-arrays vectors and links (UDs), FP64: canonical.
-// variant 0: the staged FP32 block kernels where they apply (two or more
-// right-hand sides, blocks 8 x 4 x 4 x 2 or 4^4), 1: the paired ones there,
-// 2: the general kernels throughout; all give identical results.  r0: the
+// variant 0: the staged FP32 block kernels (blocks 8 x 4 x 4 x 2 or 4^4) or the
+// half-warp one (2^4) where they apply, 1: the paired ones for two or more
+// right-hand sides, 2: the general kernels throughout; identical results.  r0: the
 // residual of z = 0, read in r's place and left as it is, z being written
 // without a read (no copy of r0 and no clearing of z before the first sweep)
 int sap_variants();

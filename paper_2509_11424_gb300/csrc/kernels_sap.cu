@@ -15,16 +15,18 @@
 // sites after each colour's blocks: red blocks, face pass on the black
 // sites, black blocks, face pass on the red sites (four launches per sweep).
 //
-// Three block kernels, for FP32 blocks of 256 sites with every extent >= 2
-// (8 x 4 x 4 x 2 and 4^4): the staged one (the default) takes one block and
+// Four block kernels.  For FP32 blocks of 256 sites with every extent >= 2
+// (8 x 4 x 4 x 2 and 4^4) the staged one (the default) takes one block and
 // right-hand side per CTA, two CTAs per SM, the links arriving in shared
 // memory by asynchronous copies that overlap the residual load; the paired
 // one (two or more right-hand sides) gives each thread one site and two
 // right-hand sides held in the two lanes of packed registers (.f32x2
 // arithmetic: one instruction and one link read from shared memory serve
 // both; fewer instructions, but its 197 KB of shared memory leaves 8 warps
-// per SM).  The general one below serves FP64 and other block shapes.  All
-// compute the same sums in the same order.
+// per SM).  For FP32 blocks of 2^4 sites a half warp per block and right-hand
+// side, everything in registers.  The general one below serves FP64 and other
+// block shapes, and every shape on request (variant 2).  All compute the same
+// sums in the same order.
 //
 // One CTA per (active block, rhs), one thread per site of the block; the
 // right-hand side varies fastest over the grid, so the CTAs of a block share
@@ -1039,7 +1041,6 @@ void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4],
   bool b8 = false, b4 = false, b2 = false;
   const unsigned half = (unsigned)(nblocks / 2);
   if constexpr (sizeof(T) == 4) {
-    // the staged kernel's copies and its 16-byte chunks want aligned vectors
     b8 = b[0] == 8 && b[1] == 4 && b[2] == 4 && b[3] == 2;
     b4 = b[0] == 4 && b[1] == 4 && b[2] == 4 && b[3] == 4;
     b2 = b[0] == 2 && b[1] == 2 && b[2] == 2 && b[3] == 2;
@@ -1064,7 +1065,7 @@ void sap_sweep(C<T> *r, C<T> *z, C<T> *e, const C<T> *U, Geom g, const int b[4],
       else if (variant == 0 && b4) launch_staged<4, 4, 4, 4>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, half, s);
       else if (variant == 1 && two && b8) launch_pair<8, 4, 4, 2>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, grid, s);
       else if (variant == 1 && two && b4) launch_pair<4, 4, 4, 4>(rin, r, z, e, U, sg, dg, color, block_iters, nrhs, zero, grid, s);
-      else if (b2) {
+      else if (variant == 0 && b2) {
         sap_small_kernel<<<(unsigned)div_up((int64_t)half * nrhs, 8), 128, 0, s>>>(rin, r, z, e, U, sg, dg, color,
                                                                                   block_iters, nrhs, zero);
       } else if (two) {

@@ -40,3 +40,26 @@ def test_small_blocks(dims, nrhs, sweeps):
             assert rel(got[r], want) < 1e-4
     finally:
         M.mgmlmc_destroy(ctx)
+
+
+@pytest.mark.parametrize('dims,nrhs', [((4, 4, 4, 4), 1), ((12, 4, 4, 12), 3)])
+def test_small_blocks_match_general_kernel(dims, nrhs):
+    """Variant 2 runs the general block kernel on these blocks as on any other:
+    the same sums in the same order, the same bits."""
+    M = require_lib()
+    n = dirac.volume(dims) * 12
+    ctx = M.mgmlmc_create(dims, torch.cuda.current_stream())
+    try:
+        M.mgmlmc_set_gauge(ctx, synth.gauge_field(dims, 0.4, 53))
+        M.mgmlmc_set_mass(ctx, 0.1)
+        M.mgmlmc_set_solver(ctx, smoother=M.SMOOTHER_SAP, smoother_steps=2, sap_iters=3)
+        b = dev(synth.complex_normal((nrhs, n), 54), torch.complex64)
+        outs = []
+        for v in range(M.mgmlmc_kernel_variants(M.VARIANT_SAP_FP32)):
+            M.mgmlmc_set_kernel_variant(ctx, M.VARIANT_SAP_FP32, v)
+            out = torch.empty_like(b)
+            M.mgmlmc_apply(ctx, M.OP_SMOOTH, 0, M.FP32, b, out, nrhs)
+            outs.append(host(out))
+        assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[0], outs[2])
+    finally:
+        M.mgmlmc_destroy(ctx)
