@@ -326,6 +326,7 @@ class Engine {
   void stencil_run(int l, int v, const float2 *in, float2 *out, int nrhs);
   int dslash_pick(int nrhs, const float2 *in, float2 *out);
   static constexpr int64_t kDirectSites = 1 << 15;
+  static constexpr int64_t kFxEager = 1 << 18;
 };
 
 }  // namespace mg
