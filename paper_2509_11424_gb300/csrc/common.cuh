@@ -251,6 +251,11 @@ __device__ __forceinline__ unsigned long long global_ns() {
 void set_staging_extra_bytes(unsigned bytes);
 unsigned staging_extra_bytes();
 
+// cudaMalloc; for tests, the next `n` ones of at least `bytes` fail as if there
+// were no memory (0 in normal operation)
+cudaError_t device_malloc(void **p, size_t bytes);
+void set_alloc_failures(int n, size_t bytes);
+
 // Raise the dynamic shared-memory limit of kernel `func` to `bytes` on the
 // current device.  The attribute is per device, so the call is made once per
 // (kernel, device) and remembered under a lock: launchers may run on several

@@ -18,7 +18,18 @@ namespace mg {
 namespace {
 template <typename T> T *dalloc(size_t count) {
   void *p = nullptr;
-  MG_CUDA(cudaMalloc(&p, count * sizeof(T) + 64));
+  MG_CUDA(device_malloc(&p, count * sizeof(T) + 64));
+  return static_cast<T *>(p);
+}
+// the same, or nullptr where the memory does not allow it
+template <typename T> T *dalloc_optional(size_t count) {
+  void *p = nullptr;
+  const cudaError_t e = device_malloc(&p, count * sizeof(T) + 64);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  MG_CUDA(e);
   return static_cast<T *>(p);
 }
 template <typename T> void dfree(T *&p) {
@@ -121,7 +132,7 @@ Engine::Engine(const int dims[4], cudaStream_t s) : user_stream(s) {
     MG_CUDA(cudaEventCreateWithFlags(&ev_enter_, cudaEventDisableTiming));
     MG_CUDA(cudaEventCreateWithFlags(&ev_leave_, cudaEventDisableTiming));
     levels_[0].U64 = dalloc<double2>((size_t)V * 36);
-    levels_[0].UF = dalloc<int4>(link_digits_elems((int)V));
+    levels_[0].UF = dalloc_optional<int4>(link_digits_elems((int)V));
     levels_[0].UD32 = dalloc<float2>((size_t)V * 36);
     levels_[0].Ub16 = dalloc<float>((size_t)V * 36);  // 36 bf16 pairs of 4 bytes per site
     scal_ = dalloc<double2>(4096);
@@ -131,7 +142,8 @@ Engine::Engine(const int dims[4], cudaStream_t s) : user_stream(s) {
     MG_CUDA(cudaMemset(tickets_, 0, kTickets * sizeof(unsigned)));
     // the digits of the FP64 operator (at most 201 MB), so that its first call
     // does not allocate them: 8^4 and 40 right-hand sides, 201 us with, 127 without
-    if (V <= kFxEager) ws<double>("fxw", 0, wilson_fx_elems((int)V, 1 << 30));
+    int group;
+    if (V <= kFxEager) fx_work(1 << 30, group);
   } catch (...) {
     release();
     throw;
@@ -268,7 +280,8 @@ RedScratch Engine::partials(size_t count) {
     drop_graphs();
     sync();
     dfree(partial_);
-    partial_ = dalloc<double2>(count);
+    partial_cap_ = 0;
+    partial_ = alloc<double2>(count);
     partial_cap_ = count;
   }
   return RedScratch{partial_, tickets_};
@@ -286,10 +299,65 @@ template <typename T> C<T> *Engine::ws(const std::string &name, int l, size_t co
     cudaFree(it->second.first);
     ws_.erase(it);
   }
-  void *p = nullptr;
-  MG_CUDA(cudaMalloc(&p, bytes + 256));
+  void *p = alloc<char>(bytes + 256);
   ws_[key] = {p, bytes};
   return static_cast<C<T> *>(p);
+}
+
+template <typename T> T *Engine::alloc(size_t count) {
+  T *p = dalloc_optional<T>(count);
+  if (p) return p;
+  reclaim();
+  return dalloc<T>(count);
+}
+
+// Give back what only makes calls faster: the link digits and the workspace of
+// the FP64 Wilson operator (the FP64 kernel needs neither) and the row-chunked
+// FP32 blocks (the pipelined kernel reads AT32).  Whether there was anything.
+bool Engine::reclaim() {
+  if (capturing_) return false;
+  bool any = levels_[0].UF != nullptr || ws_.count(kFxWork);
+  for (const Level &L : levels_) any |= L.AR32 != nullptr;
+  if (!any) return false;
+  drop_graphs();
+  sync();
+  levels_[0].UFe = 0;
+  dfree(levels_[0].UF);
+  auto it = ws_.find(kFxWork);
+  if (it != ws_.end()) {
+    cudaFree(it->second.first);
+    ws_.erase(it);
+  }
+  for (Level &L : levels_) dfree(L.AR32);
+  return true;
+}
+
+// The digits of the FP64 Wilson operator for `group` right-hand sides at a time:
+// as many as are wanted, or as the memory allows (nullptr: none).
+double2 *Engine::fx_work(int nrhs, int &group) {
+  const int V = levels_[0].g.V, want = wilson_fx_group(V, nrhs);
+  auto it = ws_.find(kFxWork);
+  int have = it == ws_.end() ? 0 : fx_group_;
+  if (have < want && want < fx_refused_ && !capturing_) {
+    if (it != ws_.end()) {
+      drop_graphs();
+      sync();
+      cudaFree(it->second.first);
+      ws_.erase(it);
+    }
+    for (have = want; have > 0; have /= 2) {
+      const size_t n = wilson_fx_elems(V, have);
+      if (double2 *p = dalloc_optional<double2>(n)) {
+        ws_[kFxWork] = {p, n * sizeof(double2)};
+        fx_group_ = have;
+        break;
+      }
+      fx_refused_ = have;
+    }
+    it = ws_.find(kFxWork);
+  }
+  group = std::min(have, want);
+  return group > 0 ? static_cast<double2 *>(it->second.first) : nullptr;
 }
 
 void Engine::ws_release(const std::string &name, int l, bool dbl) {
@@ -347,7 +415,8 @@ void Engine::gauge_derived() {
   convert<float, double>(levels_[0].U64, u32.p, (int64_t)cnt, stream);
   link_soa(u32.p, levels_[0].UD32, fine_.V, stream);
   link_bf16(u32.p, levels_[0].Ub16, fine_.V, stream);
-  levels_[0].UFe = link_digits(levels_[0].U64, levels_[0].UF, flag_dev_ + 8, fine_.V, stream);
+  if (!levels_[0].UF) levels_[0].UF = dalloc_optional<int4>(link_digits_elems(fine_.V));
+  levels_[0].UFe = levels_[0].UF ? link_digits(levels_[0].U64, levels_[0].UF, flag_dev_ + 8, fine_.V, stream) : 0;
   sync();
   have_gauge_ = true;
   free_hierarchy();
@@ -560,11 +629,12 @@ template <typename T> void Engine::apply_D(int l, const C<T> *in, C<T> *out, int
   int cls;
   if (L.fine) {
     if constexpr (sizeof(T) == 8) {
-      // fixed point wherever the links allow (332 k sites x 3: 1.57 ms in the
-      // FP64 kernel, bound by the FP64 pipe)
-      if (L.UFe) {
-        double2 *work = ws<double>("fxw", 0, wilson_fx_elems(L.g.V, nrhs));
-        wilson_apply_fx(in, out, L.UF, L.U64, L.UFe, work, L.g, m0_, nrhs, stream);
+      // fixed point wherever the links and the memory allow (332 k sites x 3:
+      // 1.57 ms in the FP64 kernel, bound by the FP64 pipe)
+      int group = 0;
+      double2 *work = L.UFe ? fx_work(nrhs, group) : nullptr;
+      if (work) {
+        wilson_apply_fx(in, out, L.UF, L.U64, L.UFe, work, group, L.g, m0_, nrhs, stream);
       } else {
         wilson_apply<double>(in, out, L.U64, nullptr, L.g, m0_, nrhs, -1, stream);
       }
@@ -698,9 +768,11 @@ template <typename T> void Engine::apply_D_dots(int l, const C<T> *x, C<T> *q, i
   const Level &L = levels_[l];
   const int64_t n = L.g.n();
   if constexpr (sizeof(T) == 4) {
-    if (!L.fine && L.AR32 && stencil_rows_supported(L.g, nrhs) && L.g.V <= 2048 && stencil_pick(l, nrhs, x, q) == 0) {
+    const bool rows = !L.fine && stencil_rows_supported(L.g, nrhs) && L.g.V <= 2048;
+    const RedScratch scr = rows ? partials(stencil_dots_scratch(L.g, nrhs)) : RedScratch{};  // may give AR32 back
+    if (rows && L.AR32 && stencil_pick(l, nrhs, x, q) == 0) {
       cudaEvent_t a = prof_begin();
-      stencil_apply_rows_dots(x, q, L.AR32, L.g, nrhs, partials(stencil_dots_scratch(L.g, nrhs)), d, d + nrhs, stream);
+      stencil_apply_rows_dots(x, q, L.AR32, L.g, nrhs, scr, d, d + nrhs, stream);
       const double m = L.g.dof;
       prof_end(a, K_STENCIL32, (double)L.g.V * (9.0 * m * m + 2.0 * m * nrhs) * sizeof(float2),
                72.0 * m * m * L.g.V * nrhs);
@@ -1214,10 +1286,10 @@ void Engine::galerkin(int l) {
   double2 *out9 = ws<double>("gal9", l, (size_t)9 * nf);
   double2 *cols = ws<double>("galc", l, (size_t)9 * nc);
   const size_t acnt = (size_t)c.g.V * 9 * dofc * dofc;
-  c.A64 = dalloc<double2>(acnt);
-  c.AF = dalloc<int4>(acnt);
-  c.AFu = dalloc<short>((size_t)c.g.V * dofc);
-  c.AT32 = dalloc<float2>(acnt);
+  c.A64 = alloc<double2>(acnt);
+  c.AF = alloc<int4>(acnt);
+  c.AFu = alloc<short>((size_t)c.g.V * dofc);
+  c.AT32 = alloc<float2>(acnt);
   for (int col = 0; col < dofc; ++col) {
     probe_column(probe, f.P64, m, col, stream);
     if (f.fine) wilson_split<double>(probe, out9, f.U64, f.g, m0_, m.b, stream);
@@ -1228,19 +1300,19 @@ void Engine::galerkin(int l) {
   stencil_digits(c.A64, c.AF, c.AFu, c.g, stream);
   stencil_transpose(c.A64, c.AT32, (int64_t)c.g.V * 9, dofc, stream);
   if (stencil_tc_supported(c.g)) {
-    c.ATC = dalloc<float>(stencil_tc_elems(c.g));
+    c.ATC = alloc<float>(stencil_tc_elems(c.g));
     stencil_tile_tc(c.A64, c.ATC, false, c.g, stream);
-    c.ATCB = dalloc<float>((stencil_tc_elems(c.g) + 1) / 2);  // BF16 elements, two per float slot
+    c.ATCB = alloc<float>((stencil_tc_elems(c.g) + 1) / 2);  // BF16 elements, two per float slot
     stencil_tile_tc(c.A64, c.ATCB, true, c.g, stream);
   }
   if (stencil_rows_supported(c.g, 1)) {
-    c.AR32 = dalloc<float4>((acnt + 1) / 2);
-    stencil_to_rows(c.A64, c.AR32, (int64_t)acnt, stream);
+    c.AR32 = dalloc_optional<float4>((acnt + 1) / 2);
+    if (c.AR32) stencil_to_rows(c.A64, c.AR32, (int64_t)acnt, stream);
   }
   if (stencil_pipe_supported(c.g)) {
-    c.ATB16 = dalloc<float>(acnt);  // one bf16 pair (4 bytes) per complex entry
+    c.ATB16 = alloc<float>(acnt);  // one bf16 pair (4 bytes) per complex entry
     stencil_to_bf16(c.AT32, c.ATB16, (int64_t)acnt, stream);
-    c.ATS = dalloc<float>(acnt);
+    c.ATS = alloc<float>(acnt);
     stencil_to_stream(c.AT32, c.ATS, (int64_t)acnt, stream);
   }
 }
@@ -1305,9 +1377,9 @@ void Engine::build_hierarchy(const mgmlmc_mg_params &p) {
       z4_noise<double>(V, f.g, p.seed, 0, 96 + l, 0, -1, ntv, stream);
       if (p.setup_rounds > 0) setup_test_vectors(l, V, ntv, p);
     }
-    f.P64 = dalloc<double2>((size_t)ntv * n);
-    f.P32 = dalloc<float2>((size_t)ntv * n);
-    f.PB16 = dalloc<float>((size_t)ntv * n);
+    f.P64 = alloc<double2>((size_t)ntv * n);
+    f.P32 = alloc<float2>((size_t)ntv * n);
+    f.PB16 = alloc<float>((size_t)ntv * n);
     MG_CUDA(cudaMemsetAsync(flag_dev_, 0, sizeof(int), stream));
     build_prolongator(V, f.P64, f.agg, flag_dev_, stream);
     convert<float, double>(f.P64, f.P32, (int64_t)ntv * n, stream);
@@ -1325,8 +1397,8 @@ void Engine::build_hierarchy(const mgmlmc_mg_params &p) {
     // one level only: the coarsest operator is the Wilson operator itself
     throw Error(MGMLMC_ERR_ARG, "n_levels must be >= 2");
   }
-  c.Dinv64 = dalloc<double2>((size_t)n * n);
-  c.Dinv32 = dalloc<float2>((size_t)n * n);
+  c.Dinv64 = alloc<double2>((size_t)n * n);
+  c.Dinv32 = alloc<float2>((size_t)n * n);
   double2 *work = ws<double>("gj", 0, (size_t)2 * n * n + n + 8);
   dense_from_stencil(c.A64, c.Dinv64, c.g, stream);
   MG_CUDA(cudaMemsetAsync(flag_dev_, 0, sizeof(int), stream));
@@ -1431,6 +1503,7 @@ void Engine::release_workspaces() {
     cudaFree(it->second.first);
     it = ws_.erase(it);
   }
+  fx_refused_ = 1 << 30;
 }
 
 // ------------------------------------------------------------------ estimators
@@ -1642,7 +1715,7 @@ void Engine::deflation_build(int k, int iters, double tol, uint64_t seed,
   dfree(defl_V_);
   defl_V_ = nullptr;
   defl_k_ = 0;
-  double2 *V = dalloc<double2>((size_t)k * n);
+  double2 *V = alloc<double2>((size_t)k * n);
   try {
     double2 *g = ws<double>("dfg", 0, (size_t)8 * n);
     double2 *W = ws<double>("dfw", 0, (size_t)k * n);

@@ -218,6 +218,13 @@ class Engine {
   int transfer_variant() const { return transfer_variant_; }
 
  private:
+  // device memory; where it runs out, what only makes calls faster is given back
+  template <typename T> T *alloc(size_t count);
+  bool reclaim();
+  double2 *fx_work(int nrhs, int &group);
+  static constexpr const char *kFxWork = "fxw#0d";
+  int fx_group_ = 0;            // right-hand sides that the workspace holds
+  int fx_refused_ = 1 << 30;    // fewest for which there was no memory
   template <typename T> C<T> *ws(const std::string &name, int l, size_t count);
   // free one named workspace (only for buffers no captured graph uses)
   void ws_release(const std::string &name, int l, bool dbl);

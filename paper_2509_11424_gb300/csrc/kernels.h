@@ -138,9 +138,12 @@ void gauge_generate(double2 *U, int64_t nlinks, double eps, uint64_t seed, cudaS
 // one (range: two ints of device scratch; synchronises).
 size_t link_digits_elems(int V);
 int link_digits(const double2 *U, int4 *UF, int *range, int V, cudaStream_t s);
-size_t wilson_fx_elems(int V, int nrhs);
-void wilson_apply_fx(const double2 *in, double2 *out, const int4 *UF, const double2 *U, int EU, double2 *work, Geom g,
-                     double m0, int nrhs, cudaStream_t s);
+// (work: of wilson_fx_elems for `group` right-hand sides, which are converted at
+// a time; wilson_fx_group: as many as gain by it)
+int wilson_fx_group(int V, int nrhs);
+size_t wilson_fx_elems(int V, int group);
+void wilson_apply_fx(const double2 *in, double2 *out, const int4 *UF, const double2 *U, int EU, double2 *work,
+                     int group, Geom g, double m0, int nrhs, cudaStream_t s);
 // BF16 storage, FP32 arithmetic: D psi for nrhs vectors of complex bf16 in
 // the chunked structure-of-arrays order (pair ((i/4) V + s) * 4 + i % 4),
 // links Ub from link_bf16; 16-byte aligned

@@ -1302,6 +1302,21 @@ std::atomic<unsigned> g_staging_extra{0};
 void set_staging_extra_bytes(unsigned bytes) { g_staging_extra.store(bytes); }
 unsigned staging_extra_bytes() { return g_staging_extra.load(); }
 
+namespace {
+std::atomic<int> g_alloc_failures{0};
+std::atomic<size_t> g_alloc_failure_bytes{0};
+}
+void set_alloc_failures(int n, size_t bytes) {
+  g_alloc_failure_bytes.store(bytes);
+  g_alloc_failures.store(n);
+}
+cudaError_t device_malloc(void **p, size_t bytes) {
+  if (g_alloc_failures.load(std::memory_order_relaxed) > 0 && bytes >= g_alloc_failure_bytes.load() &&
+      g_alloc_failures.fetch_sub(1) > 0)
+    return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+
 void smem_optin(const void *func, int bytes) {
   static std::mutex mu;
   static std::map<std::pair<const void *, int>, int> done;  // (kernel, device) -> bytes set

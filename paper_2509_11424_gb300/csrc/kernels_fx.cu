@@ -644,19 +644,19 @@ int link_digits(const double2 *U, int4 *UF, int *range, int V, cudaStream_t s) {
 }
 
 int wilson_fx_group(int V, int nrhs) {
-  // right-hand sides converted together: 4 share a link read from memory;
-  // small lattices take more, up to 2^18 sites
+  // right-hand sides converted together: 4 share a link read from memory; small
+  // lattices take more, up to 2^18 sites
   const int g = std::max(4, (1 << 18) / V);
   return std::min(g, nrhs);
 }
-size_t wilson_fx_elems(int V, int nrhs) {
-  const size_t g = wilson_fx_group(V, nrhs);
+size_t wilson_fx_elems(int V, int group) {
+  const size_t g = group;
   return g * tiles(V) * 384 + (g * V * sizeof(short2) + 15) / 16;
 }
 
-void wilson_apply_fx(const double2 *in, double2 *out, const int4 *UF, const double2 *U, int EU, double2 *work, Geom g,
-                     double m0, int nrhs, cudaStream_t s) {
-  const int grp = wilson_fx_group(g.V, nrhs);
+void wilson_apply_fx(const double2 *in, double2 *out, const int4 *UF, const double2 *U, int EU, double2 *work,
+                     int group, Geom g, double m0, int nrhs, cudaStream_t s) {
+  const int grp = std::min(group, nrhs);
   longlong2 *xs = reinterpret_cast<longlong2 *>(work);
   short2 *ex = reinterpret_cast<short2 *>(xs + (size_t)grp * tiles(g.V) * 384);
   for (int r0 = 0; r0 < nrhs; r0 += grp) {

@@ -35,6 +35,8 @@ template <typename T> const C<T> *in(const void *p) { return static_cast<const C
 
 extern "C" {
 
+void k_alloc_failures(int n, int64_t bytes) { set_alloc_failures(n, (size_t)bytes); }
+
 int k_dot(int fp32, const void *x, const void *y, int64_t n, int nrhs, double2 *out) {
   return run([&] {
     Scratch t((size_t)reduce_blocks(n) * nrhs);

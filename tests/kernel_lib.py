@@ -30,6 +30,8 @@ def kernels():
     L.k_multi_axpy.argtypes = [i32, P, i64, i32, P, i64, i32, P, f64, P]
     L.k_wgrad_f32.argtypes = [P, P, P, P, i32, i32, i32, P]
     L.k_site_dots.argtypes = [P, P, ctypes.c_float, i32, i32, P, P]
+    L.k_alloc_failures.argtypes = [i32, i64]
+    L.k_alloc_failures.restype = None
     return L
 
 
