@@ -783,6 +783,10 @@ template <typename T> void Engine::apply_D_dots(int l, const C<T> *x, C<T> *q, i
   dot_qr<T>(q, x, n, nrhs, d, d + nrhs, partials((size_t)reduce_blocks(n) * nrhs * 2), stream);
 }
 
+void Engine::need_network() const {
+  if (!net_.C) throw Error(MGMLMC_ERR_STATE, "network smoother selected but the network is not initialised");
+}
+
 template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs, const C<T> *r0) {
   const int64_t n = levels_[l].g.n();
   const bool learned = l == 0 && sp_.smoother == MGMLMC_SMOOTHER_LEARNED;
@@ -795,7 +799,7 @@ template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs, c
   if (net) {
     // the network in place of SAP: smoother_steps residual-minimising steps
     // z += alpha N(res), res -= alpha D N(res)
-    if (!net_.C) throw Error(MGMLMC_ERR_STATE, "network smoother selected but the network is not initialised");
+    need_network();
     C<T> *e = ws<T>("sape", l, (size_t)n * nrhs);
     C<T> *q = ws<T>("smq", l, (size_t)n * nrhs);
     double2 *d = ws<double>("netd", l, 2 * (size_t)nrhs);
@@ -901,6 +905,7 @@ template <typename T> void Engine::precond(int l, const C<T> *r, C<T> *z, int nr
   C<T> *q = ws<T>("smq", l, (size_t)n * nrhs);
   C<T> *rc = ws<T>("mgrc", l + 1, (size_t)nc * nrhs);
   C<T> *ec = ws<T>("mgec", l + 1, (size_t)nc * nrhs);
+  if (l == 0 && sp_.smoother == MGMLMC_SMOOTHER_NET && !sp_.post_smoothing_only) need_network();
   // without pre-smoothing the residual is r itself and z = 0 is never stored
   const bool pre = !(sp_.post_smoothing_only && l == 0) && n_steps > 0;
   if (pre) smooth<T>(l, z, res, nrhs, r);

@@ -238,6 +238,7 @@ class Engine {
   // q = D_l x and the two dots of a minimal-residual step, d[r] = <q_r, x_r>,
   // d[nrhs + r] = <q_r, q_r>
   template <typename T> void apply_D_dots(int l, const C<T> *x, C<T> *q, int nrhs, double2 *d);
+  void need_network() const;  // throws where the network smoother has none
   // r0: the smoothing starts from z = 0 with the residual r0 (left as it is;
   // z and res hold nothing yet)
   template <typename T> void smooth(int l, C<T> *z, C<T> *res, int nrhs, const C<T> *r0 = nullptr);
