@@ -762,13 +762,15 @@ void Engine::noise(int l, uint64_t seed, uint64_t sample0, uint64_t term, uint64
 // (MGMLMC_SMOOTHER_SAP), followed for MGMLMC_SMOOTHER_LEARNED by one learned
 // step z += alpha N(res) with the residual-minimising alpha (so the step can
 // only lower ||res||); other levels / MR: minimal-residual steps.
-// One launch where the FP32 row-chunked stencil applies and its last block can
-// add every site's sums in the time of another launch (V <= 2048), else two.
+// One launch where the FP32 row-chunked stencil applies and its last block adds
+// every site's sums sooner than another launch would: four steps on 256 coarse
+// sites, 1 and 4 right-hand sides, 54 and 66 us (74 and 74 with a launch for the
+// dots), on 512 74 and 90 (81 and 90), on 1024 103 and 124 (87 and 109).
 template <typename T> void Engine::apply_D_dots(int l, const C<T> *x, C<T> *q, int nrhs, double2 *d) {
   const Level &L = levels_[l];
   const int64_t n = L.g.n();
   if constexpr (sizeof(T) == 4) {
-    const bool rows = !L.fine && stencil_rows_supported(L.g, nrhs) && L.g.V <= 2048;
+    const bool rows = !L.fine && stencil_rows_supported(L.g, nrhs) && L.g.V <= 512;
     const RedScratch scr = rows ? partials(stencil_dots_scratch(L.g, nrhs)) : RedScratch{};  // may give AR32 back
     if (rows && L.AR32 && stencil_pick(l, nrhs, x, q) == 0) {
       cudaEvent_t a = prof_begin();
