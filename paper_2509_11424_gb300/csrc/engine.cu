@@ -671,7 +671,8 @@ template <typename T> void Engine::apply_D(int l, const C<T> *in, C<T> *out, int
 
 // The caller's order in one launch where the two reordering passes around the
 // operator would cost more than its strided accesses: up to kDirectSites
-// sites times right-hand sides, once the autotuned choice for nrhs is made
+// sites times right-hand sides (2^13 sites 6.4 us, reordering 14.8; 2^15 8.8 and
+// 16.5; at 2^17, 18.8 and 30.5, it would still be ahead), once the autotuned choice for nrhs is made
 // (it stays what mgmlmc_get_kernel_variant reports), 16-byte aligned.
 void Engine::apply_D_canonical(const float2 *in, float2 *out, int nrhs) {
   const Level &L = levels_[0];
@@ -758,14 +759,10 @@ void Engine::noise(int l, uint64_t seed, uint64_t sample0, uint64_t term, uint64
 }
 
 // ------------------------------------------------------------------ MG cycle
-// Smoothing: res holds r - D z on entry and exit.  Level 0: SAP sweeps
-// (MGMLMC_SMOOTHER_SAP), followed for MGMLMC_SMOOTHER_LEARNED by one learned
-// step z += alpha N(res) with the residual-minimising alpha (so the step can
-// only lower ||res||); other levels / MR: minimal-residual steps.
 // One launch where the FP32 row-chunked stencil applies and its last block adds
 // every site's sums sooner than another launch would: four steps on 256 coarse
-// sites, 1 and 4 right-hand sides, 54 and 66 us (74 and 74 with a launch for the
-// dots), on 512 74 and 90 (81 and 90), on 1024 103 and 124 (87 and 109).
+// sites, 1 and 4 right-hand sides, 54 and 62 us (74 and 74 with a launch for the
+// dots), on 512 74 and 87 (81 and 90), on 1024 103 and 124 (87 and 109).
 template <typename T> void Engine::apply_D_dots(int l, const C<T> *x, C<T> *q, int nrhs, double2 *d) {
   const Level &L = levels_[l];
   const int64_t n = L.g.n();
@@ -789,6 +786,10 @@ void Engine::need_network() const {
   if (!net_.C) throw Error(MGMLMC_ERR_STATE, "network smoother selected but the network is not initialised");
 }
 
+// Smoothing: res holds r - D z on entry and exit.  Level 0: SAP sweeps
+// (MGMLMC_SMOOTHER_SAP), followed for MGMLMC_SMOOTHER_LEARNED by one learned
+// step z += alpha N(res) with the residual-minimising alpha (so the step can
+// only lower ||res||); other levels / MR: minimal-residual steps.
 template <typename T> void Engine::smooth(int l, C<T> *z, C<T> *res, int nrhs, const C<T> *r0) {
   const int64_t n = levels_[l].g.n();
   const bool learned = l == 0 && sp_.smoother == MGMLMC_SMOOTHER_LEARNED;

@@ -8,10 +8,14 @@
 // keeps three of its four digit products,
 //   a x = a1 x1 2^56 + (a1 x0 + a0 x1) 2^28 + a0 x0,  |a0 x0| <= 2^54 dropped,
 // each an exact 64-bit integer multiply-add: sums are exact (whatever their
-// order) and rounded to a double once.  What is lost is the dropped term
-// (2^-60 of the product of the two scales) and the operands' last bit (2^-57
-// of their group's largest entry), below the 2^-53 that every single FP64
-// addition of the same sum rounds off.
+// order) and rounded to a double once.  What is lost of a sum of K products is
+// the dropped term and the operands' rounding, at most K (2 x 2^-58 + 2^-60) of
+// the product of the two groups' largest entries.  Where these meet, that is less
+// than what FP64 additions round off (2^-53 of every partial sum).  Where they
+// meet only small entries, or none, it is not: an entry 2^-k of its group's
+// largest keeps 57 - k bits and below 2^-58 nothing.  So every kernel compares
+// its sums (or the entries' exponents) with the scale, and forms those that are
+// small against it in FP64.
 //
 // Plain C++ apart from the decorations, so that a host test can compile it.
 #pragma once

@@ -5,7 +5,7 @@
 // only) writes partial sums that the last block to finish adds in block
 // order, so a result never depends on scheduling.  FP32 products are summed
 // in FP32 within a thread, FP64 ones as integers (fixed.cuh); the sums over
-// the lanes of a warp are exact integer ones (52 bits of the largest lane for
+// the lanes of a warp are exact integer ones (51 bits of the largest lane for
 // FP32), and across warps and blocks FP64.  FP64 additions are kept to those:
 // a warp's shuffle reduction of one complex number in FP64 takes 640 cycles
 // of the FP64 pipe, as long as 64 FP32 multiply-adds per lane.
@@ -110,7 +110,8 @@ __device__ __forceinline__ bool block_finish(double mine, double *__restrict__ p
 // them, and without a barrier, since every thread reads only what it copied.
 // FP64 digits, n = 786 k, 16 right-hand sides, 1 .. 20 vectors: updates 364 us on
 // average, 6.9 TB/s, 20 dots 756 us; with the loads of one vector at a time in
-// registers 707 and 1225 us, waiting for memory.
+// registers 707 and 1225 us, waiting for memory.  (The checks for graded entries
+// have added 2.5% since.)
 constexpr int kRing = 4;
 template <int TILE> struct Ring {
   int4 *slot;  // [kRing][TILE]

@@ -645,7 +645,8 @@ int link_digits(const double2 *U, int4 *UF, int *range, int V, cudaStream_t s) {
 
 int wilson_fx_group(int V, int nrhs) {
   // right-hand sides converted together: 4 share a link read from memory; small
-  // lattices take more, up to 2^18 sites
+  // lattices take more, up to 2^18 sites (8^4 and 64 right-hand sides: 155 us, 195
+  // in groups of 16; 16^4 and 16: 642, 585 in one group, for 201 MB of digits)
   const int g = std::max(4, (1 << 18) / V);
   return std::min(g, nrhs);
 }
